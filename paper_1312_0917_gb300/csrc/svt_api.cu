@@ -165,13 +165,13 @@ int svt_create(svt_ctx **out, int device, const svt_limits *lim)
     d.max_combs = L.max_combinations;
     d.hash_mask = L.hash_slots - 1;
     d.small_n4 = N4_SMALL_MAX;
-    d.run_roads = WARP_ROADS;
+    d.run_roads = RUN_ROADS;
     bool ok =
         !dalloc(c, &d.ctrl, 1) && !dalloc(c, const_cast<svt_const_set **>(&d.consts), N_SETS) &&
         !dalloc(c, &d.span_ee, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.span_ep, MAX_SPANS + MAX_GRID) &&
         !dalloc(c, &d.span_seg, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.ev_road_end, L.max_events) && !dalloc(c, &d.ev_big, L.max_events) &&
         !dalloc(c, &d.roads, L.max_roads) && !dalloc(c, &d.coords, (size_t)L.max_roads * 40) &&
-        !dalloc(c, &d.xmask, L.max_roads) && !dalloc(c, &d.big_list, L.max_roads) &&
+        !dalloc(c, &d.xmask, L.max_roads) && !dalloc(c, &d.box_list, L.max_roads) &&
         !dalloc(c, &d.cand_bits, L.max_roads / 32 + 1) && !dalloc(c, &d.fitc, N_SETS * SET_INT4) &&
         !dalloc(c, &d.surv_pool, (size_t)L.max_roads * SURV_SLOTS) &&
         !dalloc(c, &d.surv_cnt, L.max_roads) &&
@@ -457,7 +457,7 @@ static void apply_launch(svt_ctx *c, const svt_launch &L)
     c->block = L.block ? L.block : 256;
     c->blocks_per_sm = L.blocks_per_sm;
     c->d.small_n4 = L.small_n4 ? L.small_n4 : N4_SMALL_MAX;
-    c->d.run_roads = L.run_roads ? L.run_roads : WARP_ROADS;
+    c->d.run_roads = L.run_roads ? L.run_roads : RUN_ROADS;
     c->max_ctas = L.max_ctas;
 }
 
@@ -501,7 +501,7 @@ int svt_autotune(svt_ctx *c, int reps, svt_tune_point *points, uint32_t cap, uin
         return SVT_E_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     static const int kSmall[] = {64, 128, N4_SMALL_MAX};
-    static const int kRun[] = {4, WARP_ROADS, RUN_ROADS_MAX};
+    static const int kRun[] = {4, RUN_ROADS, RUN_ROADS_MAX};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (cudaEventCreate(&e0) || cudaEventCreate(&e1))
         return SVT_E_CUDA;

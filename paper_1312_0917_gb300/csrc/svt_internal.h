@@ -17,11 +17,10 @@ constexpr int N_LAYERS = 5;
 constexpr int N_SETS = 360;                // 12 wedges x 6 barrels x 5 excluded layers
 constexpr int SURV_SLOTS = 64;             // survivors per road are <= 64 (see box_road)
 constexpr int ROAD_CHUNK = 256;            // roads per output work item
-constexpr int WARP_ROADS = 8;              // roads a fitting warp takes into its tables at once
 constexpr int P2W_ROADS = 64;              // events of at most this many roads: one warp each in P2
-constexpr int RUN_ROADS_MAX = 16;          // roads per queue claim of a fitting warp (run_roads)
-constexpr int N4_SMALL_MAX = 256;          // largest road a single warp takes
-constexpr int QTAB_SMALL = 160;            // the same sum for any road with N4 <= 256
+constexpr int RUN_ROADS = 8;               // default of svt_launch::run_roads
+constexpr int RUN_ROADS_MAX = 16;          // and its largest value
+constexpr int N4_SMALL_MAX = 256;          // distinct fits of the largest road the group path takes
 constexpr unsigned long long NO_KEY = ~0ull;
 
 // fault ranks: at one word a format/grammar fault outranks a limit fault;
@@ -63,13 +62,12 @@ struct Ctrl {
     unsigned int n_ep;            // EP words in the stream
     unsigned int has_tail;        // words after the last EE
     unsigned int n_roads;         // roads of complete events
-    unsigned int n_big;           // roads fitted by a whole CTA (list length)
     unsigned int n_big_ev;        // events of more than P2W_ROADS roads (list length)
     unsigned int hash_used;       // claimed slots of the group table
+    unsigned int n_box;           // roads of the box path (list length)
     unsigned int q[12];           // work-queue heads
     unsigned int bar;             // grid barrier arrivals
     unsigned int done[4];         // last-block-done counters
-    unsigned int pad0;
     unsigned long long n_comb, n_pass, n_out;
     unsigned long long pad1[2];
     unsigned long long t_phase[8];   // persistent kernel: globaltimer at its start, after each
@@ -83,9 +81,14 @@ struct RoadRec {
     uint32_t pk;
     int16_t curv, phi;
     uint16_t set;
-    uint16_t cta;   // bit 0: fitted by a whole CTA (listed in big_list), not by a warp's run;
-                    // bit 1: a coordinate repeated within a layer
+    uint16_t fit;   // written in P2: the fitted slots by falling hit count, two bits each, the fit
+                    // class in bits 8..10, bit 11: a coordinate repeated within a layer
 };
+
+// Fit classes of the roads: the group path's
+// classes by the two largest hit counts of the fitted layers, (2, 2), (4, 2),
+// (4, 4), (8, 2), (8, 4) at most, then the box path, then no fit at all.
+constexpr int N_GROUP_CLS = 5, CLS_BOX = 5, CLS_NONE = 6;
 
 // Cross-road group table slot: key = (event + 1, triple, three coordinates),
 // val_inv = ~(lowest track key of the group), 0 = empty.
@@ -109,7 +112,7 @@ struct Dev {
     RoadRec *roads;                                               // [max_roads]
     uint16_t *coords;                                             // [max_roads][5][8]
     unsigned long long *xmask;                                    // [max_roads]
-    uint32_t *big_list;                                           // [max_roads]
+    uint32_t *box_list;                                           // [max_roads]
     int4 *fitc;            // [N_SETS][SET_INT4]: the constants as int32 in 16-byte words, written
                            // with the constants (fit_words); read-only in the kernels
     uint32_t *cand_bits;                                          // [max_roads / 32 + 1] cross-road
@@ -129,7 +132,7 @@ struct Dev {
     svt_road *road_out;                                           // [max_roads] (svt_get_roads)
     long long cut;
     int small_n4;
-    int run_roads;         // roads per queue claim of the fit stage's runs: 4, 8 or 16
+    int run_roads;         // claim of a warp of the group path: max(run_roads / 8, 1) warp steps
     int skip_arrival;
     unsigned long long wait_ns;
 };

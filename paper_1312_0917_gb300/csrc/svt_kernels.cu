@@ -368,7 +368,7 @@ __device__ __forceinline__ void stamp(const Dev &d, unsigned k)
 }
 
 // work-queue indices (Ctrl::q)
-enum { Q_P0 = 0, Q_P1, Q_P2, Q_BIG, Q_SMALL, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
+enum { Q_P0 = 0, Q_P1, Q_P2, Q_BOX, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
 
 // ---------------------------------------------------------------------------
 // P0 / P1: the word stream, one warp per span.  The stream is cut into
@@ -586,7 +586,7 @@ __device__ __forceinline__ unsigned long long decode_batch(const Dev &d, P1Warp 
             r.curv = (int16_t)(cw & 0xFFFFu);
             r.phi = (int16_t)(pw & 0xFFFFu);
             r.set = (uint16_t)((wedge * 6 + barrel) * 5 + excl);
-            r.cta = 0;
+            r.fit = 0;
             d.roads[g] = r;
             if (ee && ev < d.max_events) {   // the event's last road
                 d.ev_road_end[ev] = g + 1;
@@ -898,6 +898,69 @@ __device__ void pair_exact_warp(P2Smem &s, unsigned r, unsigned t)
     }
 }
 
+// The four fitted layers' hit counts of a road record, slot j in bits 4j ..
+// 4j + 3 (the excluded layer's count taken out).
+__device__ __forceinline__ unsigned fitted_counts(uint32_t pk)
+{
+    const unsigned m = (1u << (4 * min((pk >> 20) & 7u, 4u))) - 1u;
+    return (pk & m) | ((pk >> 4) & 0xFFFFu & ~m);
+}
+
+// Fit class of a road with N combinations and N4 distinct fits, and its slots
+// by falling hit count (perm).  The box path takes roads with more than
+// small_n4 distinct fits, with more than four hits on two fitted layers, or
+// with a coordinate repeated within a layer (rep: it works on canonical hits).
+__device__ __forceinline__ unsigned road_class(uint32_t pk, unsigned N, unsigned N4, unsigned small_n4, bool rep,
+                                               unsigned &perm)
+{
+    const unsigned nf = fitted_counts(pk);
+    unsigned v[4];
+#pragma unroll
+    for (unsigned j = 0; j < 4; ++j)
+        v[j] = (((nf >> (4 * j)) & 15u) << 2) | j;
+    const auto order = [&v](unsigned i, unsigned j) {
+        const unsigned hi = max(v[i], v[j]), lo = min(v[i], v[j]);
+        v[i] = hi;
+        v[j] = lo;
+    };
+    order(0, 1);
+    order(2, 3);
+    order(0, 2);
+    order(1, 3);
+    order(1, 2);
+    perm = (v[0] & 3u) | (v[1] & 3u) << 2 | (v[2] & 3u) << 4 | (v[3] & 3u) << 6;
+    const unsigned ma = v[0] >> 2, mb = v[1] >> 2;
+    if (N == 0)
+        return CLS_NONE;
+    if (rep || N4 > small_n4 || mb > 4)
+        return CLS_BOX;
+    return ma > 4 ? (mb > 2 ? 4u : 3u) : ma > 2 ? (mb > 2 ? 2u : 1u) : 0u;
+}
+
+// The end of P2 for road g (record r, flagged hits xm, rep: a coordinate
+// repeated within a layer): the record's candidate bit and fit path; a road of
+// the box path joins its list.  Returns the road's combinations.
+__device__ __forceinline__ unsigned finish_road(const Dev &d, unsigned g, RoadRec r, unsigned long long xm, bool rep)
+{
+    const bool cand = xm != 0ull;
+    unsigned N, N4, perm;
+    road_sizes(r.pk, N, N4);
+    const unsigned cls = road_class(r.pk, N, N4, (unsigned)d.small_n4, rep, perm);
+    r.pk |= cand ? (1u << 23) : 0u;
+    r.fit = (uint16_t)(perm | cls << 8 | (rep ? 1u << 11 : 0u));
+    d.roads[g] = r;
+    d.xmask[g] = xm;
+    d.surv_cnt[g] = 0;
+    if (cls == CLS_BOX) {
+        const unsigned i = atomicAdd(&d.ctrl->n_box, 1u);
+        if (i < d.max_roads)
+            d.box_list[i] = g;
+    }
+    if (N > 0 && cand)   // checked against the other roads' groups after the fit
+        atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
+    return N;
+}
+
 // Flags of event e (roads r0 .. r0 + nr - 1); adds its combinations to n_comb.
 __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, unsigned char *smem,
                          unsigned long long &n_comb)
@@ -985,31 +1048,8 @@ __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, uns
         pair_exact_warp(s, s.cp[k] & 0xFFFFu, s.cp[k] >> 16);
     __syncthreads();
     // the road records: candidate bit and fit path
-    for (unsigned k = threadIdx.x; k < nr; k += BLOCK) {
-        const unsigned g = r0 + k;
-        RoadRec r = s.rec[k];
-        const unsigned long long xm = ((unsigned long long)s.xhi[k] << 32) | s.xlo[k];
-        const bool cand = xm != 0ull, rep = s.rep[k] != 0;
-        unsigned N, N4;
-        road_sizes(r.pk, N, N4);
-        // fitted by one warp each (the box path): roads with more distinct
-        // fits than a warp's run takes, and cross-road candidates with a
-        // repeated coordinate (they publish over canonical hits)
-        const bool big = N > 0 && (N4 > (unsigned)d.small_n4 || (cand && rep));
-        r.pk |= cand ? (1u << 23) : 0u;
-        r.cta = (big ? 1 : 0) | (rep ? 2 : 0);
-        d.roads[g] = r;
-        d.xmask[g] = xm;
-        d.surv_cnt[g] = 0;
-        if (big) {
-            unsigned i = atomicAdd(&d.ctrl->n_big, 1u);
-            if (i < d.max_roads)
-                d.big_list[i] = g;
-        }
-        if (N > 0 && cand)   // checked against the other roads' groups after the fit
-            atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
-        n_comb += N;
-    }
+    for (unsigned k = threadIdx.x; k < nr; k += BLOCK)
+        n_comb += finish_road(d, r0 + k, s.rec[k], ((unsigned long long)s.xhi[k] << 32) | s.xlo[k], s.rep[k] != 0);
     __syncthreads();   // the shared arrays are refilled for the next event
 }
 
@@ -1157,27 +1197,8 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, unsig
 #pragma unroll
     for (unsigned h = 0; h < 2; ++h) {
         const unsigned k = lane + 32 * h;
-        if (k >= nr)
-            continue;
-        const unsigned g = r0 + k;
-        RoadRec r = ldcg(d.roads + g);
-        const bool cand = xm[h] != 0ull;
-        unsigned N, N4;
-        road_sizes(r.pk, N, N4);
-        const bool big = N > 0 && (N4 > (unsigned)d.small_n4 || (cand && rep[h]));
-        r.pk |= cand ? (1u << 23) : 0u;
-        r.cta = (big ? 1 : 0) | (rep[h] ? 2 : 0);
-        d.roads[g] = r;
-        d.xmask[g] = xm[h];
-        d.surv_cnt[g] = 0;
-        if (big) {
-            unsigned i = atomicAdd(&d.ctrl->n_big, 1u);
-            if (i < d.max_roads)
-                d.big_list[i] = g;
-        }
-        if (N > 0 && cand)
-            atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
-        n_comb += N;
+        if (k < nr)
+            n_comb += finish_road(d, r0 + k, ldcg(d.roads + r0 + k), xm[h], rep[h]);
     }
     __syncwarp();   // the state is refilled for the next event
 }
@@ -1333,593 +1354,216 @@ __device__ __forceinline__ unsigned nth_bit(unsigned mask, unsigned n)
 }
 
 // ---------------------------------------------------------------------------
-// P3, flat path: a warp fits a run of small roads together, one lane per
-// table entry across the roads of the run (fit, pair tables, survivors), so
-// the per-road work is spread over the lanes instead of repeated per road.
-// A coordinate repeated within a fitted layer makes the pair tables take
-// canonical hits (the lowest index with the same coordinate); a cross-road
-// candidate with a repeated coordinate goes through the box path.
+// P3, group path: a warp fits several small roads at once, a group of lanes
+// per road.  The four fitted slots get roles by falling hit count, (a, b, c,
+// e).  A road's class bounds the hits of a by A = 2^LA, those of b and c by B
+// = YN 2^LY and those of e by W, and its group is A x 2^LY lanes: lane (x, yl)
+// holds hit x of slot a and the YN hits y = yl + j 2^LY of slot b, and runs
+// over the hits z and w of slots c and e.
+//
+// A distinct fit survives the road-local warrior iff no passing fit of the
+// road with a lower key shares two of its four hits.  Fits are compared by a
+// 32-bit word, the chi-square shifted right until the cut fits 31 bits.  Each
+// of the lane's pairs (x, y) keeps its lowest fit; it survives iff its word is
+// the minimum of the other five pair tables.  At each z the tables (a, c),
+// (b, c) and (c, e) are complete after a shuffle minimum over the group's
+// other y, other x, and all its lanes; (a, e) and (b, e) follow after the
+// loop from the minima over z.  No table is kept in memory.  Without two
+// passing fits of one word that meet in a minimum (a tie) the words order the
+// fits as the keys do; a road with a tie (0.3 % of the roads at random: hits
+// that differ by one or two often give the same floors) is left to the box
+// path, which compares whole keys.
+//
+// Bound: issue slots.  Several hits of slot b per lane (YN = 2) share the
+// road's set-up, the loads and the shuffles of (a, c) and (c, e); with one
+// hit per lane a warp step took 700 instructions for half the roads.
 // ---------------------------------------------------------------------------
 
-constexpr unsigned FLAT_K = N4_SMALL_MAX, FLAT_Q = QTAB_SMALL, FLAT_A = 64;
+// Key of a fit from its summed partials s: (chi2, road bits and comb), or
+// NO_KEY when it fails the cut.  s.x, s.y, s.z are 4096 times the three
+// chi-square components before the floor (exact in int32, see the header);
+// s.w is road << 15 | comb.
+__device__ __forceinline__ unsigned long long box_key(const int4 &s, long long cut, bool &pass)
+{
+    const long long chi2 = sq(s.x >> 12) + sq(s.y >> 12) + sq(s.z >> 12);
+    pass = chi2 <= cut;
+    return pass ? (((unsigned long long)chi2 << 23) | (unsigned)s.w) : NO_KEY;
+}
 
-// One road of a run, in the warp's shared memory.  The fields the per-entry
-// passes read are grouped in 16-byte words (vector loads).
-struct alignas(16) FlatRoad {
-    unsigned kb, ab, qb, key_hi;  // first key, partial sum and pair-table entry; road bits of a key
-    unsigned m[4], st[4], SL[4], aoff[4];   // aoff: first partial sum of fitted slot j
-    unsigned off[6];              // first entry of pair table p (aoff and off are rebased on the
-                                  // sub-run's tables in the shared copy)
-    unsigned M[3];                // magic divisors of m[0..2]
-    unsigned xl;                  // excluded layer (bits 0..2), cross-road candidate (bit 3), hits
-                                  // of the excluded layer (bits 4..7), layer of fitted slot j
-                                  // (bits 8 + 3j .. 10 + 3j)
-    unsigned g, N4, E, set;
-    unsigned event, nl, Se;       // nl: hits per layer, 4 bits each; Se: comb stride of excl
-    int curv, phi;
-    unsigned pad;
-    unsigned cm[4];               // canonical hit (the lowest index with the same coordinate) of
-                                  // each hit of fitted slot j, 3 bits each
-    unsigned long long cb;        // plain mode: first combination of the road
-    unsigned long long xm;        // cross-road candidates: the road's flagged hits (xmask)
-};
-static_assert(offsetof(FlatRoad, m) % 16 == 0 && offsetof(FlatRoad, off) % 16 == 0 &&
-                  offsetof(FlatRoad, cm) % 16 == 0,
-              "16-byte groups");
-__device__ __forceinline__ unsigned fr_excl(const FlatRoad &r) { return r.xl & 7u; }
-__device__ __forceinline__ unsigned fr_ne(const FlatRoad &r) { return (r.xl >> 4) & 15u; }
-__device__ __forceinline__ unsigned fr_layer(const FlatRoad &r, unsigned j) { return (r.xl >> (8 + 3 * j)) & 7u; }
-constexpr unsigned CANON_ID = 0xFAC688u;   // hit x -> x for x < 8, 3 bits each
-
-struct P3Flat {
-    int4 A[FLAT_A];                       // partial chi-square sums, [aoff[j] + hit]
-    unsigned long long K[FLAT_K];         // keys of distinct fits, [kb + f]
-    unsigned Qh[FLAT_Q], Ql[FLAT_Q];      // pair tables, [qb + off[p] + x * m_b + y]: high and
-                                          // low word of the minimum key (all ones = none)
-    uint16_t dig[FLAT_K];                 // the fit's four slot hits (3 bits each), its road's lane
-    FlatRoad rd[WARP_ROADS];
-    uint16_t co[WARP_ROADS][40];
-    unsigned cnt[WARP_ROADS];             // survivors found so far
-};
-static_assert(offsetof(P3Flat, co) % 16 == 0, "coordinate rows are copied in 16-byte words");
+__device__ __forceinline__ int4 add4(const int4 &a, const int4 &b)
+{
+    return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
 
 // the six pairs of fitted slots (a, b)
 __device__ __forceinline__ unsigned pair_a(unsigned p) { return (0x211000u >> (4 * p)) & 15u; }
 __device__ __forceinline__ unsigned pair_b(unsigned p) { return (0x332321u >> (4 * p)) & 15u; }
 
-// The roads of a sub-run, in order, are the set bits of `sub` (lanes of the
-// run).  A table over the sub-run packs the first entry of its k-th road in
-// half-word k of w (0xFFFF past the last road) and the road's lane in nibble
-// k of `lanes`.
-struct FlatIndex {
-    unsigned w[4], lanes;
-    // lane of the road that owns entry t
-    __device__ unsigned owner(unsigned t) const
+constexpr unsigned GROUP_HITS = 128;   // hits of a warp's roads at most (sixteen roads of class 0)
+struct P3Group {
+    int4 A[GROUP_HITS];   // a road's hits in role order: chi-square partial sums (x, y, z) and comb
+                          // part (w); role a also carries curvature, phi, 4096 k and the road bits
+};
+
+// A road as a group reads it, 16 bytes in shared memory: RoadRec::pk, the
+// fitted slots by falling hit count (perm), and its index.
+struct alignas(16) RoadItem {
+    uint32_t g, pk;
+    int16_t curv, phi;
+    uint16_t set, perm;
+};
+
+// The shape of a class and one lane's view of its group's road.
+template <unsigned LA_, unsigned LY_, unsigned YN_, unsigned W_>
+struct GroupRoad {
+    static constexpr unsigned A = 1u << LA_, YL = 1u << LY_, YN = YN_, B = YN * YL, W = W_;
+    static constexpr unsigned G = A * YL, ROADS = 32 / G, HITS = A + 2 * B + W;   // W <= B
+    static_assert(ROADS * HITS <= GROUP_HITS, "the warp's hits fit its table");
+    RoadItem it;
+    const int4 *hit;            // the road's hits
+    unsigned nf, excl;          // hits per fitted slot (4 bits each), excluded layer
+    unsigned mb, mc, me;        // hits of slots b, c, e
+    unsigned x, yl;             // the lane's hits
+    bool live;                  // hit x exists
+    unsigned long long cb;      // plain mode: first combination of the road
+    __device__ unsigned slot(unsigned role) const { return (it.perm >> (2 * role)) & 3u; }
+    __device__ unsigned m(unsigned s) const { return (nf >> (4 * s)) & 15u; }
+    __device__ unsigned y(unsigned j) const { return yl + j * YL; }
+    __device__ bool has(unsigned j) const { return live && y(j) < mb; }
+    // first hit of fitted slot s in the table
+    __device__ unsigned first(unsigned s) const
     {
-        unsigned k = t >= (w[0] >> 16);
-#pragma unroll
-        for (unsigned q = 1; q < 4; ++q)
-            k += (t >= (w[q] & 0xFFFFu)) + (t >= (w[q] >> 16));
-        return (lanes >> (4 * k)) & 15u;
+        return s == slot(0) ? 0u : A + B * (s == slot(1) ? 0u : s == slot(2) ? 1u : 2u);
+    }
+    template <bool PLAIN>
+    __device__ unsigned long long key(const Dev &d, long long cut, const int4 &s) const
+    {
+        if (PLAIN)
+            return ldcg(d.fit_key + cb + (unsigned)s.w);
+        bool pass;
+        return box_key(s, cut, pass);
+    }
+    // the lane's fit at its hit j of slot b and hits z, w of slots c and e
+    template <bool PLAIN>
+    __device__ unsigned long long key_at(const Dev &d, long long cut, unsigned j, unsigned z, unsigned w) const
+    {
+        return key<PLAIN>(d, cut, add4(add4(hit[x], hit[A + y(j)]), add4(hit[A + B + z], hit[A + 2 * B + w])));
     }
 };
 
-// Build the index from each road lane's first entry (every lane calls it).
-__device__ __forceinline__ FlatIndex flat_index(unsigned first, unsigned sub)
+// a fit's hits by role in one word
+__device__ __forceinline__ unsigned pack_fit(unsigned x, unsigned y, unsigned z, unsigned w)
 {
-    FlatIndex x{{0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu}, 0u};
-    unsigned rest = sub;
-#pragma unroll
-    for (unsigned k = 0; k < WARP_ROADS; ++k) {
-        const unsigned ln = rest ? __ffs(rest) - 1 : 0u;
-        const unsigned v = __shfl_sync(FULL_MASK, first, ln) & 0xFFFFu;
-        if (rest) {
-            const unsigned sh = 16 * (k & 1u);
-            x.w[k >> 1] = (x.w[k >> 1] & ~(0xFFFFu << sh)) | (v << sh);
-            x.lanes |= ln << (4 * k);
-        }
-        rest &= rest - 1;
-    }
-    return x;
+    return x | (y << 3) | (z << 6) | (w << 9);
 }
 
-// Publish, for road ri of a flat sub-run (no repeated coordinate in a layer,
-// so every hit index is canonical), the minimum key of every group (layer
-// triple, three coordinates) whose three hits are flagged as shared with
-// another road of the event.  The whole warp takes the groups.
-__device__ void flat_publish(const Dev &d, const P3Flat &F, unsigned ri)
+// What a lane has found of its road's survivors: those of its pairs (flag,
+// key, place among the road's survivors by comb), and the road's number.
+template <unsigned YN>
+struct GroupFound {
+    bool surv[YN];
+    unsigned long long key[YN];
+    unsigned rank[YN], cnt;
+};
+
+// The survivors' places by comb (whole warp).
+template <unsigned YN>
+__device__ __forceinline__ void group_rank(GroupFound<YN> &f, unsigned gmask)
 {
-    const FlatRoad &r = F.rd[ri];
-    const unsigned excl = fr_excl(r);
-    // flagged hits of layer l: byte l of flp (no arrays indexed at run time)
-    unsigned long long flp = 0;
+    const unsigned lane = lane_id();
 #pragma unroll
-    for (unsigned l = 0; l < N_LAYERS; ++l) {
-        const unsigned n = (r.nl >> (4 * l)) & 15u;
-        flp |= (r.xm & ((unsigned long long)((1u << n) - 1u) << (8 * l)));
+    for (unsigned j = 0; j < YN; ++j)
+        f.rank[j] = 0;
+#pragma unroll
+    for (unsigned i = 0; i < YN; ++i) {
+        unsigned rest = __ballot_sync(FULL_MASK, f.surv[i]) & gmask;
+        while (__any_sync(FULL_MASK, rest != 0u)) {
+            const unsigned other = __shfl_sync(FULL_MASK, (unsigned)f.key[i] & 0x7FFFu, rest ? __ffs(rest) - 1 : lane);
+#pragma unroll
+            for (unsigned j = 0; j < YN; ++j)
+                f.rank[j] += rest && other < ((unsigned)f.key[j] & 0x7FFFu);
+            rest &= rest - 1;
+        }
     }
-    const auto fl = [flp](unsigned l) { return (unsigned)(flp >> (8 * l)) & 0xFFu; };
-    const auto groups = [&fl](unsigned t) {   // groups of triple t
-        return __popc(fl(triple_l(t, 0))) * __popc(fl(triple_l(t, 1))) * __popc(fl(triple_l(t, 2)));
-    };
-    unsigned total = 0;
+}
+
+// Publish, for each cross-road candidate among the warp's roads (no repeated
+// coordinate in a layer, so every hit is canonical), the minimum key of every
+// group (layer triple, three coordinates) whose three hits are flagged as
+// shared with another road of the event: the road's lanes take its groups.
+template <bool PLAIN, class Road>
+__device__ __noinline__ void group_publish(const Dev &d, const Road &r, bool publish)
+{
+    const unsigned g = r.it.g, excl = r.excl;
+    if (publish) {
+        const unsigned long long xm = ldcg(d.xmask + g);   // flagged hits of layer l: byte l
+        const unsigned event = ldcg(&d.roads[g].event);
+        unsigned Se = 1;   // comb stride of the excluded layer
+        for (unsigned l = 0; l < excl; ++l)
+            Se *= (r.it.pk >> (4 * l)) & 15u;
+        const auto fl = [xm](unsigned l) { return (unsigned)(xm >> (8 * l)) & 0xFFu; };
+        const auto groups = [&fl](unsigned t) {   // groups of triple t
+            return __popc(fl(triple_l(t, 0))) * __popc(fl(triple_l(t, 1))) * __popc(fl(triple_l(t, 2)));
+        };
+        unsigned total = 0;
 #pragma unroll
-    for (unsigned t = 0; t < 10; ++t)
-        total += groups(t);
-    for (unsigned gi = lane_id(); gi < total; gi += 32) {
-        unsigned t = 0, rem = gi;
-        bool found = false;
+        for (unsigned t = 0; t < 10; ++t)
+            total += groups(t);
+        for (unsigned gi = lane_id() % Road::G; gi < total; gi += Road::G) {
+            unsigned t = 0, rem = gi;
+            bool found = false;
 #pragma unroll
-        for (unsigned tt = 0; tt < 10; ++tt) {   // the triple of group gi
-            const unsigned c = groups(tt);
-            if (!found) {
-                if (rem < c) {
-                    t = tt;
-                    found = true;
-                } else {
-                    rem -= c;
+            for (unsigned tt = 0; tt < 10; ++tt) {   // the triple of group gi
+                const unsigned c = groups(tt);
+                if (!found) {
+                    if (rem < c) {
+                        t = tt;
+                        found = true;
+                    } else {
+                        rem -= c;
+                    }
                 }
             }
-        }
-        const unsigned lt[3] = {triple_l(t, 0), triple_l(t, 1), triple_l(t, 2)};
-        const unsigned f0 = fl(lt[0]), f1 = fl(lt[1]), f2 = fl(lt[2]);
-        const unsigned p0 = __popc(f0), p1 = __popc(f1);
-        const unsigned dsel[3] = {nth_bit(f0, rem % p0), nth_bit(f1, (rem / p0) % p1), nth_bit(f2, rem / (p0 * p1))};
-        unsigned long long mn = NO_KEY;
-        if (lt[0] != excl && lt[1] != excl && lt[2] != excl) {
-            // the free fitted slot runs over its hits, the three others are fixed
-            unsigned fb = 0, free_slot = 0 + 1 + 2 + 3;
-#pragma unroll
-            for (unsigned q = 0; q < 3; ++q) {
-                const unsigned sq_ = lt[q] - (lt[q] > excl);
-                free_slot -= sq_;
-                fb += dsel[q] * r.st[sq_];
-            }
-            for (unsigned z = 0; z < r.m[free_slot]; ++z) {
-                const unsigned long long k = F.K[r.kb + fb + z * r.st[free_slot]];
-                mn = k < mn ? k : mn;
-            }
-        } else {
-            // the excluded layer in the triple: its lowest hit index of the
-            // coordinate (the index itself, canonical) and the pair table
-            unsigned de = 0, fa = 4, fb = 4, da = 0, db = 0;
+            const unsigned lt[3] = {triple_l(t, 0), triple_l(t, 1), triple_l(t, 2)};
+            const unsigned f0 = fl(lt[0]), f1 = fl(lt[1]), f2 = fl(lt[2]);
+            const unsigned p0 = __popc(f0), p1 = __popc(f1);   // at most 8 each: the quotients are divm's
+            const unsigned r1 = divm(rem, c_magic[p0]), r2 = divm(r1, c_magic[p1]);
+            const unsigned dsel[3] = {nth_bit(f0, rem - r1 * p0), nth_bit(f1, r1 - r2 * p1), nth_bit(f2, r2)};
+            // the triple's fitted slots are fixed, the other fitted slots
+            // (one, or two when the triple has the excluded layer) run over
+            // their hits
+            int4 base = make_int4(0, 0, 0, 0);
+            unsigned de = 0, rest = 0xFu;
 #pragma unroll
             for (unsigned q = 0; q < 3; ++q) {
                 if (lt[q] == excl) {
                     de = dsel[q];
-                } else if (fa == 4) {
-                    fa = lt[q] - (lt[q] > excl);
-                    da = dsel[q];
                 } else {
-                    fb = lt[q] - (lt[q] > excl);
-                    db = dsel[q];
+                    const unsigned s = lt[q] - (lt[q] > excl);
+                    base = add4(base, r.hit[r.first(s) + dsel[q]]);
+                    rest &= ~(1u << s);
                 }
             }
-            unsigned p = 0;
-            while (p < 5 && !(pair_a(p) == fa && pair_b(p) == fb))
-                ++p;
-            const unsigned idx = r.off[p] + da * r.m[fb] + db;
-            mn = ((unsigned long long)F.Qh[idx] << 32) | F.Ql[idx];
-            if (mn != NO_KEY)
-                mn += (unsigned long long)de * r.Se;
+            const unsigned su = __ffs(rest) - 1, sv = 31 - __clz(rest);   // the same slot when one is free
+            const unsigned mv = su == sv ? 1u : r.m(sv);
+            unsigned long long mn = NO_KEY;
+            for (unsigned u = 0; u < r.m(su); ++u) {
+                const int4 bu = add4(base, r.hit[r.first(su) + u]);
+                for (unsigned v = 0; v < mv; ++v) {
+                    const unsigned long long k = r.template key<PLAIN>(d, d.cut, su == sv ? bu : add4(bu, r.hit[r.first(sv) + v]));
+                    mn = k < mn ? k : mn;
+                }
+            }
+            if (mn != NO_KEY) {   // the excluded layer's hit of the group, or its lowest
+                const uint16_t *co = d.coords + (size_t)g * 40;
+                hash_min(d, group_key(event, t, ldcg(co + lt[0] * 8 + dsel[0]), ldcg(co + lt[1] * 8 + dsel[1]),
+                                      ldcg(co + lt[2] * 8 + dsel[2])),
+                         mn + (unsigned long long)de * Se);
+            }
         }
-        if (mn != NO_KEY)
-            hash_min(d, group_key(r.event, t, F.co[ri][lt[0] * 8 + dsel[0]], F.co[ri][lt[1] * 8 + dsel[1]],
-                                  F.co[ri][lt[2] * 8 + dsel[2]]),
-                     mn);
     }
     __syncwarp();
 }
-
-// Survivors of one pass of a flat sub-run (every lane of the warp calls it):
-// lane flags `surv` with its key and its road's lane ri (entries in order).
-// A road's survivors take its slots in entry order.
-__device__ __forceinline__ void flat_emit(const Dev &d, P3Flat &F, bool surv, unsigned ri,
-                                          unsigned long long key)
-{
-    const unsigned lane = lane_id();
-    if (!surv)
-        ri = WARP_ROADS + lane;   // distinct per lane unless a survivor
-    const unsigned sv = __ballot_sync(FULL_MASK, surv);
-    if (!sv)
-        return;
-    const unsigned same = __match_any_sync(FULL_MASK, ri) & sv;
-    unsigned pos = 0;
-    if (surv)
-        pos = F.cnt[ri] + __popc(same & lanemask_lt());
-    __syncwarp();
-    if (surv) {
-        if (pos < SURV_SLOTS)
-            d.surv_pool[surv_at(d, F.rd[ri].g, pos)] = key;
-        else
-            raise_flag(d, FLAG_INTERNAL);
-        if ((same >> lane) == 1u)   // the last survivor of its road in this pass
-            F.cnt[ri] = pos + 1;
-    }
-    __syncwarp();
-}
-
-// Fit roads g0 .. g0 + R - 1 (R <= WARP_ROADS) with one warp; `region` is
-// the warp's shared memory.  Roads marked in P2 for a whole CTA are skipped.
-template <bool PLAIN>
-__device__ void fit_run(const Dev &d, unsigned char *region, unsigned g0, unsigned R,
-                        unsigned long long &npass)
-{
-    P3Flat &F = *reinterpret_cast<P3Flat *>(region);
-    const unsigned lane = lane_id();
-    unsigned np32 = 0;   // passing combinations of the run (at most 8 x 256 x 8)
-
-    // the run's records and coordinates
-    RoadRec rec = {};
-    unsigned N = 0, N4 = 0;
-    if (lane < R) {
-        rec = ldcg(d.roads + g0 + lane);
-        road_sizes(rec.pk, N, N4);
-    }
-    {   // 80 bytes per road, five 16-byte words
-        const uint4 *src = reinterpret_cast<const uint4 *>(d.coords + (size_t)g0 * 40);
-        uint4 *dst = reinterpret_cast<uint4 *>(&F.co[0][0]);
-        for (unsigned idx = lane; idx < R * N_LAYERS; idx += 32)
-            dst[idx] = ldcg(src + idx);
-    }
-    __syncwarp();
-
-    // lane i < R: the shape of road i (a road the CTAs fit is skipped),
-    // written straight into the road's record in shared memory (slot i in
-    // every sub-run), so that no per-lane array needs local memory
-    const bool small = lane < R && N > 0 && !(rec.cta & 1u);
-    unsigned E = 0, asum = 0, xl = 0;
-    bool flat = false, dup_fit = false;
-    if (small) {
-        FlatRoad &w = F.rd[lane];
-        const uint32_t pk = rec.pk;
-        const unsigned excl = min((pk >> 20) & 7u, 4u);
-        // fitted slots: the layers other than excl, in order.  Canonical hits
-        // of each fitted layer: a repeated coordinate makes the pair tables
-        // take canonical indices (dup_fit)
-        unsigned S = 1, Se = 1, ne = 0, j = 0, st = 1;
-        xl = excl | (((pk >> 23) & 1u) << 3);
-        for (unsigned l = 0; l < N_LAYERS; ++l) {
-            const unsigned nl_ = min((pk >> (4 * l)) & 15u, (unsigned)MAX_HITS);
-            if (l == excl) {
-                Se = S;
-                ne = nl_;
-            } else {
-                xl |= l << (8 + 3 * j);
-                unsigned map = CANON_ID;
-                for (unsigned x = 1; x < ((rec.cta & 2u) ? nl_ : 0u); ++x) {   // P2 flags repeated coordinates
-                    unsigned c = x;
-                    for (unsigned y = x; y-- > 0;)   // the lowest equal index wins
-                        c = F.co[lane][l * 8 + x] == F.co[lane][l * 8 + y] ? y : c;
-                    map = (map & ~(7u << (3 * x))) | (c << (3 * x));
-                }
-                w.cm[j] = map;
-                dup_fit = dup_fit || map != CANON_ID;
-                w.m[j] = nl_;
-                w.st[j] = st;
-                w.SL[j] = S;
-                w.aoff[j] = asum;
-                asum += nl_;
-                st *= nl_;
-                ++j;
-            }
-            S *= nl_;
-        }
-        xl |= ne << 4;
-        for (unsigned p = 0; p < 6; ++p) {
-            w.off[p] = E;
-            E += w.m[pair_a(p)] * w.m[pair_b(p)];
-        }
-        for (unsigned q = 0; q < 3; ++q)
-            w.M[q] = c_magic[w.m[q]];
-        w.g = g0 + lane;
-        w.event = rec.event;
-        w.xl = xl;
-        w.nl = pk & 0xFFFFFu;
-        w.Se = Se;
-        w.N4 = N4;
-        w.E = E;
-        w.key_hi = rec.pk >> 24;
-        w.set = min((unsigned)rec.set, (unsigned)(N_SETS - 1));
-        w.curv = rec.curv;
-        w.phi = rec.phi;
-        w.cb = PLAIN ? ldcg(d.comb_off + g0 + lane) : 0ull;
-        w.xm = ((pk >> 23) & 1u) ? ldcg(d.xmask + g0 + lane) : 0ull;   // loaded with the run
-        // every road a warp takes fits the tables: N4 <= small_n4 <= FLAT_K,
-        // and then E <= QTAB_SMALL and asum <= 32
-        flat = N4 <= FLAT_K && E <= FLAT_Q && asum <= FLAT_A;
-        if (!flat)
-            raise_flag(d, FLAG_INTERNAL);
-    }
-
-    // flat sub-runs: a prefix of the remaining flat roads that fits the tables
-    unsigned todo = __ballot_sync(FULL_MASK, flat);
-    while (todo) {
-        const bool mine = (todo >> lane) & 1u;
-        unsigned ik = mine ? N4 : 0u, iq = mine ? E : 0u, ia = mine ? asum : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {   // inclusive prefix sums over the lanes
-            const unsigned uk = __shfl_up_sync(FULL_MASK, ik, o);
-            const unsigned uq = __shfl_up_sync(FULL_MASK, iq, o);
-            const unsigned ua = __shfl_up_sync(FULL_MASK, ia, o);
-            if ((int)lane >= o) {
-                ik += uk;
-                iq += uq;
-                ia += ua;
-            }
-        }
-        const bool take = mine && ik <= FLAT_K && iq <= FLAT_Q && ia <= FLAT_A;
-        const unsigned sub = __ballot_sync(FULL_MASK, take);   // the first roads left
-        const bool sdup = __any_sync(FULL_MASK, take && dup_fit);
-        const unsigned s1 = 31 - __clz(sub);
-        const unsigned nk = __shfl_sync(FULL_MASK, ik, s1), nq = __shfl_sync(FULL_MASK, iq, s1),
-                       na = __shfl_sync(FULL_MASK, ia, s1);
-        if (take) {   // the road's record joins the sub-run: offsets rebased on its tables
-            FlatRoad &w = F.rd[lane];
-            const unsigned qb = iq - E, ab = ia - asum;
-            w.kb = ik - N4;
-            w.qb = qb;
-            w.ab = ab;
-#pragma unroll
-            for (unsigned p = 0; p < 6; ++p)
-                w.off[p] += qb;
-#pragma unroll
-            for (unsigned jj = 0; jj < 4; ++jj)
-                w.aoff[jj] += ab;
-            F.cnt[lane] = 0;
-        }
-        const FlatIndex xk = flat_index(ik - N4, sub), xa = flat_index(ia - asum, sub);
-        __syncwarp();
-
-        // partial chi-square sums of every fitted hit of every road
-        if (!PLAIN) {
-            for (unsigned t = lane; t < na; t += 32) {
-                const unsigned ri = xa.owner(t);
-                const FlatRoad &r = F.rd[ri];
-                const unsigned j = (t >= r.aoff[1]) + (t >= r.aoff[2]) + (t >= r.aoff[3]);
-                const unsigned dd = t - r.aoff[j];
-                const int h = F.co[ri][fr_layer(r, j) * 8 + dd];
-                // column j of the set's C (one 16-byte load; columns 4, 5 and k for slot 0)
-                const int4 *cc = d.fitc + SET_INT4 * r.set + SET_C;
-                const int4 cj = __ldg(cc + j);
-                int4 a;
-                a.x = cj.x * h;
-                a.y = cj.y * h;
-                a.z = cj.z * h;
-                a.w = 0;
-                if (j == 0) {   // curvature, phi and 4096 * offset ride on slot 0
-                    const int4 c4 = __ldg(cc + 4), c5 = __ldg(cc + 5), kk = __ldg(cc + 6);
-                    a.x += c4.x * r.curv + c5.x * r.phi + 4096 * kk.x;
-                    a.y += c4.y * r.curv + c5.y * r.phi + 4096 * kk.y;
-                    a.z += c4.z * r.curv + c5.z * r.phi + 4096 * kk.z;
-                }
-                F.A[t] = a;
-            }
-            __syncwarp();
-        }
-
-        // pair tables start empty (the low words once they are needed)
-        for (unsigned t = lane; t < nq; t += 32)
-            F.Qh[t] = 0xFFFFFFFFu;
-        __syncwarp();
-
-        // keys of the distinct fits.  The pair tables hold the minimum key of
-        // the fits with the same hits on two fitted slots; a 64-bit minimum
-        // is taken in two 32-bit steps: the high words here, then, only if
-        // a table has two keys with its minimum high word (a tie), the low
-        // words of the keys whose high word is the minimum.  A key that
-        // finds a lower high word already in one of its tables cannot be a
-        // table's minimum there; the others ("maybe" keys) are listed in
-        // entry order over the low words, unused until a tie.  The second
-        // of two keys with the minimum high word of a table always finds
-        // it there, so every tie at a minimum is seen.
-        const long long cut = d.cut;
-        uint16_t *ml = reinterpret_cast<uint16_t *>(F.Ql);
-        static_assert(sizeof(F.Ql) >= FLAT_K * sizeof(uint16_t), "maybe list fits over Ql");
-        unsigned nmaybe = 0;
-        bool tie = false;
-        for (unsigned base = 0; base < nk; base += 32) {
-            const unsigned t = base + lane;
-            bool maybe = false;
-            if (t < nk) {
-                const unsigned ri = xk.owner(t);
-                const FlatRoad &r = F.rd[ri];
-                const unsigned f = t - r.kb;
-                const unsigned q0 = divm(f, r.M[0]), f0 = f - q0 * r.m[0];
-                const unsigned q1 = divm(q0, r.M[1]), f1 = q0 - q1 * r.m[1];
-                const unsigned f3 = divm(q1, r.M[2]), f2 = q1 - f3 * r.m[2];
-                const unsigned comb = f0 * r.SL[0] + f1 * r.SL[1] + f2 * r.SL[2] + f3 * r.SL[3];
-                unsigned long long key;
-                if (PLAIN) {
-                    key = ldcg(d.fit_key + r.cb + comb);
-                } else {
-                    const int4 a0 = F.A[r.aoff[0] + f0], a1 = F.A[r.aoff[1] + f1];
-                    const int4 a2 = F.A[r.aoff[2] + f2], a3 = F.A[r.aoff[3] + f3];
-                    const int sx = a0.x + a1.x + a2.x + a3.x;
-                    const int sy = a0.y + a1.y + a2.y + a3.y;
-                    const int sz = a0.z + a1.z + a2.z + a3.z;
-                    const long long chi2 = sq(sx >> 12) + sq(sy >> 12) + sq(sz >> 12);
-                    const bool pass = chi2 <= cut;
-                    np32 += pass ? fr_ne(r) : 0u;
-                    key = pass ? make_key(chi2, r.key_hi, comb) : NO_KEY;
-                }
-                // pair tables take canonical hits (a sub-run with a repeated
-                // coordinate maps them; elsewhere they are the hits)
-                unsigned fd[4] = {f0, f1, f2, f3};
-                if (sdup) {
-#pragma unroll
-                    for (unsigned jj = 0; jj < 4; ++jj)
-                        fd[jj] = (r.cm[jj] >> (3 * fd[jj])) & 7u;
-                }
-                F.K[t] = key;
-                F.dig[t] = (uint16_t)(fd[0] | (fd[1] << 3) | (fd[2] << 6) | (fd[3] << 9) | (ri << 12));
-                if (key != NO_KEY) {
-                    const unsigned hi = (unsigned)(key >> 32);
-                    maybe = true;
-#pragma unroll
-                    for (unsigned p = 0; p < 6; ++p) {
-                        const unsigned a = pair_a(p), b = pair_b(p);
-                        const unsigned old = atomicMin(&F.Qh[r.off[p] + fd[a] * r.m[b] + fd[b]], hi);
-                        maybe = maybe && old >= hi;
-                        tie = tie || old == hi;
-                    }
-                }
-            }
-            const unsigned mb = __ballot_sync(FULL_MASK, maybe);
-            if (maybe)
-                ml[nmaybe + __popc(mb & lanemask_lt())] = (uint16_t)t;
-            nmaybe += __popc(mb);
-        }
-        const bool ties = __any_sync(FULL_MASK, tie);
-        __syncwarp();
-
-        // candidates: keys whose high word is the minimum of all six
-        // tables.  Without a tie a candidate is a survivor and is written at
-        // once; after a tie the candidates are listed in entry order over the
-        // partial sums (no longer needed) for the low-word test.
-        uint16_t *cl = reinterpret_cast<uint16_t *>(F.A);
-        static_assert(sizeof(F.A) >= FLAT_K * sizeof(uint16_t), "candidate list fits over A");
-        unsigned ncand = 0;
-        if (!ties) {
-            for (unsigned base = 0; base < nmaybe; base += 32) {
-                const unsigned i = base + lane;
-                bool cand = false;
-                unsigned t = 0;
-                unsigned long long key = NO_KEY;
-                unsigned ri = 0;
-                if (i < nmaybe) {
-                    t = ml[i];
-                    key = F.K[t];
-                    const unsigned hi = (unsigned)(key >> 32);
-                    const unsigned dg = F.dig[t];
-                    ri = dg >> 12;
-                    const FlatRoad &r = F.rd[ri];
-                    const unsigned fd[4] = {dg & 7u, (dg >> 3) & 7u, (dg >> 6) & 7u, (dg >> 9) & 7u};
-                    cand = true;
-#pragma unroll
-                    for (unsigned p = 0; p < 6; ++p) {
-                        const unsigned a = pair_a(p), b = pair_b(p);
-                        cand = cand && F.Qh[r.off[p] + fd[a] * r.m[b] + fd[b]] == hi;
-                    }
-                }
-                // without a tie a candidate is a survivor: written now (the
-                // maybe keys are in entry order)
-                flat_emit(d, F, cand, ri, key);
-            }
-        } else {
-            // a tie: the low words start empty (the list over them is
-            // dropped) and every key with a table's minimum high word
-            // takes part in that table's low-word minimum
-            for (unsigned t = lane; t < nq; t += 32)
-                F.Ql[t] = 0xFFFFFFFFu;
-            __syncwarp();
-            for (unsigned base = 0; base < nk; base += 32) {
-                const unsigned t = base + lane;
-                bool cand = false;
-                if (t < nk) {
-                    const unsigned long long key = F.K[t];
-                    if (key != NO_KEY) {
-                        const unsigned dg = F.dig[t];
-                        const FlatRoad &r = F.rd[dg >> 12];
-                        const unsigned fd[4] = {dg & 7u, (dg >> 3) & 7u, (dg >> 6) & 7u, (dg >> 9) & 7u};
-                        const unsigned hi = (unsigned)(key >> 32), lo = (unsigned)key;
-                        cand = true;
-#pragma unroll
-                        for (unsigned p = 0; p < 6; ++p) {
-                            const unsigned a = pair_a(p), b = pair_b(p);
-                            const unsigned idx = r.off[p] + fd[a] * r.m[b] + fd[b];
-                            if (F.Qh[idx] == hi)
-                                atomicMin(&F.Ql[idx], lo);
-                            else
-                                cand = false;
-                        }
-                    }
-                }
-                const unsigned cb = __ballot_sync(FULL_MASK, cand);
-                if (cand)
-                    cl[ncand + __popc(cb & lanemask_lt())] = (uint16_t)t;
-                ncand += __popc(cb);
-            }
-        }
-        __syncwarp();
-
-        // after a tie: survivors are the candidates that also hold the low
-        // word of all six tables (in entry order)
-        for (unsigned base = 0; base < ncand; base += 32) {
-            const unsigned i = base + lane;
-            unsigned ri = 0;
-            bool surv = false;
-            unsigned long long key = NO_KEY;
-            if (i < ncand) {
-                const unsigned t = cl[i];
-                const unsigned dg = F.dig[t];
-                ri = dg >> 12;
-                const FlatRoad &r = F.rd[ri];
-                const unsigned fd[4] = {dg & 7u, (dg >> 3) & 7u, (dg >> 6) & 7u, (dg >> 9) & 7u};
-                key = F.K[t];
-                const unsigned lo = (unsigned)key;
-                surv = true;
-#pragma unroll
-                for (unsigned p = 0; p < 6; ++p) {
-                    const unsigned a = pair_a(p), b = pair_b(p);
-                    surv = surv && F.Ql[r.off[p] + fd[a] * r.m[b] + fd[b]] == lo;
-                }
-            }
-            flat_emit(d, F, surv, ri, key);
-        }
-        {
-            // survivor counts of the sub-run's roads, and their sums per road
-            // chunk (a run spans at most two chunks)
-            const bool in_sub = (sub >> lane) & 1u;
-            const unsigned v = in_sub ? min(F.cnt[lane], (unsigned)SURV_SLOTS) : 0u;
-            if (in_sub)
-                d.surv_cnt[g0 + lane] = (uint8_t)v;
-            const unsigned ch0 = g0 / ROAD_CHUNK;
-            const bool second = (g0 + lane) / ROAD_CHUNK != ch0;
-            const unsigned s0 = __reduce_add_sync(FULL_MASK, second ? 0u : v);
-            const unsigned s1 = __reduce_add_sync(FULL_MASK, second ? v : 0u);
-            if (lane == 0 && s0)
-                atomicAdd(&d.rchunk_sum[ch0], s0);
-            if (lane == 0 && s1)
-                atomicAdd(&d.rchunk_sum[ch0 + 1], s1);
-        }
-        // cross-road candidates of the sub-run publish their group minima,
-        // which read whole keys from the pair tables.  Without a tie the low
-        // words were not taken: each table's minimum high word belongs to
-        // one key, which writes its low word.
-        const unsigned cands = __ballot_sync(FULL_MASK, ((sub >> lane) & 1u) && (xl & 8u));
-        if (cands && !ties) {
-            for (unsigned t = lane; t < nq; t += 32)
-                F.Ql[t] = 0xFFFFFFFFu;
-            __syncwarp();
-            for (unsigned t = lane; t < nk; t += 32) {
-                const unsigned long long key = F.K[t];
-                if (key == NO_KEY)
-                    continue;
-                const unsigned dg = F.dig[t];
-                const FlatRoad &r = F.rd[dg >> 12];
-                const unsigned fd[4] = {dg & 7u, (dg >> 3) & 7u, (dg >> 6) & 7u, (dg >> 9) & 7u};
-                const unsigned hi = (unsigned)(key >> 32);
-#pragma unroll
-                for (unsigned p = 0; p < 6; ++p) {
-                    const unsigned a = pair_a(p), b = pair_b(p);
-                    const unsigned idx = r.off[p] + fd[a] * r.m[b] + fd[b];
-                    if (F.Qh[idx] == hi)
-                        F.Ql[idx] = (unsigned)key;
-                }
-            }
-            __syncwarp();
-        }
-        for (unsigned c = cands; c; c &= c - 1)
-            flat_publish(d, F, __ffs(c) - 1);
-        todo &= ~sub;
-        __syncwarp();
-    }
-    npass += np32;
-}
-
-// shared memory of one warp in the warp part of P3
-constexpr size_t P3_WARP_BYTES = (sizeof(P3Flat) + 15) / 16 * 16;
 
 // ---------------------------------------------------------------------------
 // P3, box path: one warp fits one listed road (more distinct fits than
@@ -1960,12 +1604,25 @@ enum { T_AB = 0, T_CE, T_AC, T_BC, T_AE, T_BE, N_TAB };
 // different u in different banks
 constexpr unsigned TS = 9;
 
+// The float pass's partials by role (see box_float).
+struct P3Float {
+    float4 hit[4][8];      // (x, y, z): a quarter of the components' sums / 4096, the first role less 0.5
+    float2 c[8][4];        // role c again, each component twice
+    float ex[8], ey[8], ez[8];   // role e again, by component
+};
+
 struct P3Box {
-    unsigned long long T[2][8 * TS];   // T_ab, T_ce: [u * TS + v] (u: the first role's hit); T_ce
-                                       // only where needed (box_tce)
-    unsigned H[2][4][8 * TS];          // T_ac, T_bc of pass 0 and pass 1: high words; T_ae, T_be:
-                                       // the entries taken on demand for the publish step (pass 0)
-    unsigned L[2][4][8 * TS];          // and low words (of the keys with the minimum high word)
+    union {
+        struct {
+            unsigned long long T[2][8 * TS];   // T_ab, T_ce: [u * TS + v] (u: the first role's hit);
+                                               // T_ce only where needed (box_tce)
+            unsigned H[2][4][8 * TS];          // T_ac, T_bc of pass 0 and pass 1: high words; T_ae,
+                                               // T_be: the entries taken on demand for the publish
+                                               // step (pass 0)
+            unsigned L[2][4][8 * TS];          // and low words (of the keys with the minimum high word)
+        };
+        P3Float F;
+    };
     int4 A[4][8];                      // slot j, canonical hit k: chi-square partial sums (x, y,
                                        // z) and comb part (w); slot 0 also carries curvature, phi,
                                        // 4096 k and the road bits of the key
@@ -1974,7 +1631,8 @@ struct P3Box {
     uint8_t rank[4][8];                // canonical hit (class) of raw hit d of slot j
     uint8_t mult[4][8];                // raw hits sharing the coordinate of canonical hit k
 };
-static_assert(offsetof(P3Box, A) % 16 == 0 && offsetof(P3Box, co) % 16 == 0, "16-byte rows");
+static_assert(offsetof(P3Box, A) % 16 == 0 && offsetof(P3Box, co) % 16 == 0 && sizeof(P3Float) % 16 == 0,
+              "16-byte rows");
 
 __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b)
 {
@@ -2009,22 +1667,6 @@ __device__ __forceinline__ void fold_lo(P3Box &B, unsigned q, unsigned t, unsign
 __device__ __forceinline__ unsigned hits_of(uint32_t pk, unsigned l)
 {
     return min((pk >> (4 * l)) & 15u, (unsigned)MAX_HITS);
-}
-
-// Key of a fit from its summed partials s: (chi2, road bits and comb), or
-// NO_KEY when it fails the cut.  s.x, s.y, s.z are 4096 times the three
-// chi-square components before the floor (exact in int32, see the header);
-// s.w is road << 15 | comb.
-__device__ __forceinline__ unsigned long long box_key(const int4 &s, long long cut, bool &pass)
-{
-    const long long chi2 = sq(s.x >> 12) + sq(s.y >> 12) + sq(s.z >> 12);
-    pass = chi2 <= cut;
-    return pass ? (((unsigned long long)chi2 << 23) | (unsigned)s.w) : NO_KEY;
-}
-
-__device__ __forceinline__ int4 add4(const int4 &a, const int4 &b)
-{
-    return make_int4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
 }
 
 // Shape of a road in the box path, the same in every lane.
@@ -2191,9 +1833,322 @@ __device__ __forceinline__ unsigned box_tab(const BoxShape &sh, unsigned p, unsi
     return r1 == 0 && r2 == 1 ? T_AB : r1 == 2 ? T_CE : r2 == 2 ? (r1 == 0 ? T_AC : T_BC) : (r1 == 0 ? T_AE : T_BE);
 }
 
-// Fit road g with one warp (see above); adds its passing combinations to npass.
+// ---------------------------------------------------------------------------
+// P3, box path, float pass: the road's chi-squares in float, two fits per
+// instruction, with a bound on their error; whole numbers decide only where
+// floats cannot.
+//
+// With v the float sums of the per-hit partials / 4096, less 0.5, each
+// component differs from the floor a by at most 0.62: 0.5 from the floor, and
+// 0.11 from the conversions (2^-5 in all), the 0.5 (2^-5) and three sums (2^-6
+// each) of numbers below 2^19.  So | |v| - |a| | <= sqrt(3) 0.62 < 1.075, and
+// the float c of |v|^2 is off by a relative 2.5e-7 at most.  Hence, for the
+// chi-squares X of two fits with floats c:
+//   X1 <= X2  =>  c1 <= float_thr(c2)           (near: not certainly larger)
+//   X <= cut  =>  c <= float_hi,   X > cut  =>  c >= float_lo
+//
+// Lane (x, yl) holds hit x of slot a (eight) and hits yl, yl + 4 of slot b and
+// runs over the hits z and w of slots c and e.  The passing fits are those
+// below float_lo; a fit in [float_lo, float_hi] (one road in twenty) makes the
+// warp count again in whole numbers.  A pair (x, y) is a candidate when its
+// lowest row is near the minima of tables (a, c) and (b, c) there, which are
+// shuffle minima; each candidate's fits that share two hits with it (about
+// 320) are then taken in float, and only if one is near the candidate without
+// being certainly lower do the whole keys of box_min2 decide.
+//
+// Bound: issue slots, nine instructions per fit; in whole numbers (three
+// sums, floors and squares of 64 bits, 64-bit keys and minima) it took 48.
+// ---------------------------------------------------------------------------
+
+constexpr long long FLOAT_CUT = 1ll << 24;   // a smaller cut's band [lo, hi] is a visible share of the fits
+constexpr float FLOAT_PAD = 1e18f;           // component of a missing hit: its fits are far above every cut
+constexpr unsigned FLOAT_CANDS = 8;          // candidates the float pass follows up (more: the integer passes)
+
+// two floats, added and multiplied by one instruction each
+__device__ __forceinline__ float2 f2_add(float2 a, float2 b)
+{
+    float2 r;
+    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; add.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_mul(float2 a, float2 b)
+{
+    float2 r;
+    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mul.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c)
+{
+    float2 r;
+    asm("{ .reg .b64 x, y, z, w; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mov.b64 w, {%6, %7}; fma.rn.f32x2 z, x, y, w; mov.b64 {%0, %1}, z; }"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+__device__ __forceinline__ float sqrt_approx(float x)
+{
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// At least c2 + 4.3 sqrt(c2) + 4.7 and a little: what a fit not above c2 stays
+// below.  4.32 sqrt(c2) <= e c2 + 4.67 / e for every e; e = 9 / sqrt(cut) makes
+// that equal near 0.06 cut, where a road's minima lie (eps = 1.000002 + e, off =
+// 4.8 + 0.53 sqrt(cut)).
+#define float_thr(c2) fmaf((c2), eps, off)
+
+// float chi-square of a fit given by its four partials
+__device__ __forceinline__ float float_chi(const float4 &a, const float4 &b, const float4 &c, const float4 &e)
+{
+    const float x = a.x + b.x + c.x + e.x, y = a.y + b.y + c.y + e.y, z = a.z + b.z + c.z + e.z;
+    return fmaf(z, z, fmaf(y, y, x * x));
+}
+
+// The hits z and w (z << 3 | w) of slots c and e of the pair (x, y)'s fit whose
+// comb bits are those of `low` (the fit exists: it is the pair's minimum).
+__device__ __forceinline__ unsigned box_arg(const P3Box &B, const BoxShape &sh, unsigned x, unsigned y, unsigned low)
+{
+    const unsigned base = (unsigned)(B.A[sh.ra][x].w + B.A[sh.rb][y].w);
+    const unsigned lane = lane_id();
+    unsigned hit = 0;
+    for (unsigned i = 0; i < 2; ++i) {
+        const unsigned z = (lane >> 3) + 4 * i, w = lane & 7u;
+        if (z < sh.mc && w < sh.me && ((base + (unsigned)(B.A[sh.rc][z].w + B.A[sh.re][w].w) - low) & 0x7FFFu) == 0)
+            hit = z << 3 | w;
+    }
+    return __reduce_max_sync(FULL_MASK, hit);
+}
+
+// Fit road g (record rec) with one warp; false when it is left to the integer
+// passes.  The shape's slots are roles here, by falling hit count.
+__device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
+{
+    P3Box &B = *reinterpret_cast<P3Box *>(region);
+    P3Float &F = B.F;
+    const unsigned lane = lane_id();
+    const RoadRec rec = ldcg(d.roads + g);
+    const uint32_t pk = rec.pk;
+    if (((pk >> 23) & 1u) || ((rec.fit >> 11) & 1u))   // publishes, or repeats a coordinate
+        return false;
+    const unsigned excl = min((pk >> 20) & 7u, 4u), nf = fitted_counts(pk);
+    BoxShape sh;
+    sh.ra = 0;
+    sh.rb = 1;
+    sh.rc = 2;
+    sh.re = 3;
+    sh.ma = (nf >> (4 * (rec.fit & 3u))) & 15u;
+    sh.mb = (nf >> (4 * ((rec.fit >> 2) & 3u))) & 15u;
+    sh.mc = (nf >> (4 * ((rec.fit >> 4) & 3u))) & 15u;
+    sh.me = (nf >> (4 * ((rec.fit >> 6) & 3u))) & 15u;
+    sh.mpk = sh.ma | sh.mb << 4 | sh.mc << 8 | sh.me << 12;
+    sh.ne = hits_of(pk, excl);
+    sh.cb = 0;
+    __syncwarp();   // the region's previous user is done
+    {   // lane 8 role + k: hit k
+        const unsigned role = lane >> 3, k = lane & 7u, s = (rec.fit >> (2 * role)) & 3u;
+        float4 v = make_float4(FLOAT_PAD, 0.f, 0.f, 0.f);
+        if (k < sh.m(role)) {
+            const unsigned L = s + (s >= excl);
+            const int h = ldcg(d.coords + (size_t)g * 40 + L * 8 + k);
+            const int4 *cc = d.fitc + SET_INT4 * min((unsigned)rec.set, (unsigned)(N_SETS - 1)) + SET_C;
+            const int4 cj = __ldg(cc + s);
+            unsigned S = 1;   // comb stride of layer L
+            for (unsigned l = 0; l < L; ++l)
+                S *= (pk >> (4 * l)) & 15u;
+            int4 a = make_int4(cj.x * h, cj.y * h, cj.z * h, (int)(k * S));
+            float o = 0.f;
+            if (role == 0) {   // curvature, phi, 4096 * offset and the road bits
+                const int4 c4 = __ldg(cc + 4), c5 = __ldg(cc + 5), kk = __ldg(cc + 6);
+                a.x += c4.x * rec.curv + c5.x * rec.phi + 4096 * kk.x;
+                a.y += c4.y * rec.curv + c5.y * rec.phi + 4096 * kk.y;
+                a.z += c4.z * rec.curv + c5.z * rec.phi + 4096 * kk.z;
+                a.w += (int)((pk >> 24) << 15);
+                o = -0.5f;
+            }
+            B.A[role][k] = a;
+            v = make_float4(fmaf((float)a.x, 1.f / 4096.f, o), fmaf((float)a.y, 1.f / 4096.f, o),
+                            fmaf((float)a.z, 1.f / 4096.f, o), 0.f);
+        }
+        F.hit[role][k] = v;
+        if (role == 2) {
+            F.c[k][0] = make_float2(v.x, v.x);
+            F.c[k][1] = make_float2(v.y, v.y);
+            F.c[k][2] = make_float2(v.z, v.z);
+        }
+        if (role == 3) {
+            F.ex[k] = v.x;
+            F.ey[k] = v.y;
+            F.ez[k] = v.z;
+        }
+    }
+    __syncwarp();
+    // the cut's band
+    const float cut = (float)min(d.cut, 1ll << 38), root = sqrt_approx(cut);
+    const float band = fmaf(2.2f, root, 8.f);
+    const float eps = 1.000002f + 9.f / root, off = fmaf(0.53f, root, 4.8f);   // of float_thr
+    const float float_lo = cut * 0.999999f - band, float_hi = cut * 1.000001f + band;
+    const unsigned lo = __float_as_uint(float_lo), width = __float_as_uint(float_hi) + 1 - lo;
+
+    const unsigned x = lane & 7u, yl = lane >> 3;
+    float2 px[2], py[2], pz[2];
+#pragma unroll
+    for (unsigned j = 0; j < 2; ++j) {
+        const float4 a = F.hit[0][x], b = F.hit[1][yl + 4 * j];
+        px[j] = make_float2(a.x + b.x, a.x + b.x);
+        py[j] = make_float2(a.y + b.y, a.y + b.y);
+        pz[j] = make_float2(a.z + b.z, a.z + b.z);
+    }
+    unsigned np = 0, near_cut = ~0u;
+    float q[2] = {3e38f, 3e38f}, qok[2] = {3e38f, 3e38f};   // a pair's lowest row, and its lowest near one
+    const unsigned nw = (sh.me + 1) / 2, nj = sh.mb > 4 ? 2u : 1u;
+    for (unsigned z = 0; z < sh.mc; ++z) {
+        const float2 cx = F.c[z][0], cy = F.c[z][1], cz = F.c[z][2];
+        float rz[2] = {3e38f, 3e38f};
+#pragma unroll
+        for (unsigned j = 0; j < 2; ++j) {
+            if (j >= nj)
+                break;
+            const float2 zx = f2_add(px[j], cx), zy = f2_add(py[j], cy), zz = f2_add(pz[j], cz);
+#pragma unroll
+            for (unsigned h = 0; h < 4; ++h) {
+                if (h >= nw)
+                    break;
+                const float2 vx = f2_add(zx, *reinterpret_cast<const float2 *>(F.ex + 2 * h));
+                const float2 vy = f2_add(zy, *reinterpret_cast<const float2 *>(F.ey + 2 * h));
+                const float2 vz = f2_add(zz, *reinterpret_cast<const float2 *>(F.ez + 2 * h));
+                const float2 c = f2_fma(vz, vz, f2_fma(vy, vy, f2_mul(vx, vx)));
+                const unsigned d0 = __float_as_uint(c.x) - lo, d1 = __float_as_uint(c.y) - lo;
+                np += d0 >> 31;
+                np += d1 >> 31;
+                near_cut = min(near_cut, min(d0, d1));
+                rz[j] = fminf(rz[j], fminf(c.x, c.y));
+            }
+        }
+        float ac = fminf(rz[0], rz[1]);   // (a, c) at x, z
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 8));
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 16));
+#pragma unroll
+        for (unsigned j = 0; j < 2; ++j) {
+            if (j >= nj)
+                break;
+            float bc = rz[j];   // (b, c) at y, z
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 1));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 2));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 4));
+            q[j] = fminf(q[j], rz[j]);
+            qok[j] = rz[j] <= float_thr(fminf(ac, bc)) ? fminf(qok[j], rz[j]) : qok[j];
+        }
+    }
+    unsigned cand[2], n_cand = 0;
+#pragma unroll
+    for (unsigned j = 0; j < 2; ++j) {
+        cand[j] = __ballot_sync(FULL_MASK, qok[j] <= float_thr(q[j]) && q[j] <= float_hi);
+        n_cand += __popc(cand[j]);
+    }
+    if (n_cand > FLOAT_CANDS)
+        return false;
+    if (__any_sync(FULL_MASK, near_cut < width)) {   // count in whole numbers
+        np = 0;
+        for (unsigned j = 0; j < nj; ++j) {
+            const unsigned y = yl + 4 * j;
+            if (x >= sh.ma || y >= sh.mb)
+                continue;
+            const int4 pab = add4(B.A[sh.ra][x], B.A[sh.rb][y]);
+            for (unsigned z = 0; z < sh.mc; ++z) {
+                const int4 p = add4(pab, B.A[sh.rc][z]);
+                for (unsigned w = 0; w < sh.me; ++w) {
+                    bool pass;
+                    box_key(add4(p, B.A[sh.re][w]), d.cut, pass);
+                    np += pass;
+                }
+            }
+        }
+    }
+    npass += (unsigned long long)np * sh.ne;
+
+    // the candidates, one after the other; lane i keeps survivor i
+    unsigned n_surv = 0;
+    unsigned long long mine = NO_KEY;
+    const unsigned u = lane >> 3, v = lane & 7u;   // the lane's two hits of a table: u, u + 4 and v
+    for (unsigned j = 0; j < 2; ++j)
+        for (unsigned bits = cand[j]; bits; bits &= bits - 1) {
+            const unsigned src = __ffs(bits) - 1, cx = src & 7u, cy = (src >> 3) + 4 * j;
+            const float4 ha = F.hit[0][cx], hb = F.hit[1][cy];
+            // the pair's lowest fit
+            const float c0 = float_chi(ha, hb, F.hit[2][u], F.hit[3][v]);
+            const float c1 = float_chi(ha, hb, F.hit[2][u + 4], F.hit[3][v]);
+            const float cf = __uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(fminf(c0, c1))));
+            const float thr = float_thr(cf);
+            const unsigned n0 = __ballot_sync(FULL_MASK, c0 <= thr), n1 = __ballot_sync(FULL_MASK, c1 <= thr);
+            unsigned cz, cw;
+            int verdict = -1;   // 1 survives, 0 dropped, -1 undecided
+            if (__popc(n0) + __popc(n1) == 1 && cf < float_lo) {
+                const unsigned at = __ffs(n0 | n1) - 1;
+                cz = (at >> 3) + (n0 ? 0u : 4u);
+                cw = at & 7u;
+                const float4 hc = F.hit[2][cz], he = F.hit[3][cw];
+                float m = 3e38f;   // the lowest other fit that shares two hits with it
+#pragma unroll
+                for (unsigned i = 0; i < 2; ++i) {
+                    const unsigned w = u + 4 * i;
+                    const float4 a = F.hit[0][w], b = F.hit[1][w], bv = F.hit[1][v], c = F.hit[2][w], e = F.hit[3][v];
+                    const float ac = float_chi(ha, b, hc, e), bc = float_chi(a, hb, hc, e);
+                    const float ae = float_chi(ha, bv, c, he), be = float_chi(F.hit[0][v], hb, c, he);
+                    const float ce = float_chi(a, bv, hc, he);
+                    m = fminf(m, w == cy && v == cw ? 3e38f : ac);
+                    m = fminf(m, w == cx && v == cw ? 3e38f : bc);
+                    m = fminf(m, v == cy && w == cz ? 3e38f : ae);
+                    m = fminf(m, v == cx && w == cz ? 3e38f : be);
+                    m = fminf(m, w == cx && v == cy ? 3e38f : ce);
+                }
+                m = __uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(m)));
+                verdict = m > thr ? 1 : float_thr(m) < cf ? 0 : -1;
+            }
+            unsigned long long key = NO_KEY;
+            if (verdict == 1) {
+                bool pass;
+                key = box_key(add4(add4(B.A[sh.ra][cx], B.A[sh.rb][cy]), add4(B.A[sh.rc][cz], B.A[sh.re][cw])), d.cut,
+                              pass);
+            } else if (verdict < 0) {   // whole keys: the pair's minimum against the other five tables
+                key = box_min2<false>(d, B, sh, sh.ra, cx, sh.rb, cy);
+                if (key != NO_KEY) {
+                    const unsigned t = box_arg(B, sh, cx, cy, (unsigned)key);
+                    cz = t >> 3;
+                    cw = t & 7u;
+                    bool ok = box_min2<false>(d, B, sh, sh.ra, cx, sh.rc, cz) == key;
+                    ok = ok && box_min2<false>(d, B, sh, sh.rb, cy, sh.rc, cz) == key;
+                    ok = ok && box_min2<false>(d, B, sh, sh.ra, cx, sh.re, cw) == key;
+                    ok = ok && box_min2<false>(d, B, sh, sh.rb, cy, sh.re, cw) == key;
+                    ok = ok && box_tce<false>(d, B, sh, cz, cw) == key;
+                    key = ok ? key : NO_KEY;
+                }
+            }
+            if (key != NO_KEY) {
+                if (lane == n_surv)
+                    mine = key;
+                ++n_surv;
+            }
+        }
+    // in comb order
+    unsigned rank = 0;
+    for (unsigned i = 0; i < n_surv; ++i)
+        rank += ((unsigned)__shfl_sync(FULL_MASK, mine, i) & 0x7FFFu) < ((unsigned)mine & 0x7FFFu);
+    if (lane < n_surv)
+        d.surv_pool[surv_at(d, g, rank)] = mine;
+    if (lane == 0) {
+        d.surv_cnt[g] = (uint8_t)n_surv;
+        if (n_surv)
+            atomicAdd(&d.rchunk_sum[g / ROAD_CHUNK], n_surv);
+    }
+    __syncwarp();
+    return true;
+}
+
+// Fit a listed road with one warp (see above); adds its passing combinations to npass.
 template <bool PLAIN>
-__device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
+__device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
     P3Box &B = *reinterpret_cast<P3Box *>(region);
     const unsigned lane = lane_id();
@@ -2203,10 +2158,6 @@ __device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsign
     __syncwarp();   // the region's previous user is done
     if (lane < N_LAYERS)   // 80 bytes of coordinates, five 16-byte words
         reinterpret_cast<uint4 *>(B.co)[lane] = ldcg(reinterpret_cast<const uint4 *>(d.coords + (size_t)g * 40) + lane);
-    for (unsigned i = lane; i < 2 * 8 * TS; i += 32)
-        (&B.T[0][0])[i] = NO_KEY;
-    for (unsigned i = lane; i < 2 * 2 * 4 * 8 * TS; i += 32)   // H and L
-        (&B.H[0][0][0])[i] = 0xFFFFFFFFu;
     __syncwarp();
 
     // lane 8 j + h: raw hit h of fitted slot j.  Canonical hits, their ranks
@@ -2260,6 +2211,10 @@ __device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsign
         }
         B.A[j][k] = a;
     }
+    for (unsigned i = lane; i < 2 * 8 * TS; i += 32)
+        (&B.T[0][0])[i] = NO_KEY;
+    for (unsigned i = lane; i < 2 * 2 * 4 * 8 * TS; i += 32)   // H and L
+        (&B.H[0][0][0])[i] = 0xFFFFFFFFu;
     // roles: the pair (a, b) that needs the fewest lane steps, then c before
     // e with e (the unrolled inner loop) the larger
     {
@@ -2401,6 +2356,7 @@ __device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsign
         }
         const unsigned cmx = __ballot_sync(FULL_MASK, xv && xc == lane) & 0xFFu;
         const unsigned long long xm = ldcg(d.xmask + g);
+        const unsigned event = rec.event;
         unsigned long long flp = 0;
 #pragma unroll
         for (unsigned l = 0; l < N_LAYERS; ++l) {
@@ -2508,7 +2464,7 @@ __device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsign
                     mn += (unsigned long long)de * Se;
             }
             if (mn != NO_KEY)
-                hash_min(d, group_key(rec.event, t, B.co[lt[0] * 8 + dsel[0]], B.co[lt[1] * 8 + dsel[1]],
+                hash_min(d, group_key(event, t, B.co[lt[0] * 8 + dsel[0]], B.co[lt[1] * 8 + dsel[1]],
                                       B.co[lt[2] * 8 + dsel[2]]),
                          mn);
         }
@@ -2516,43 +2472,438 @@ __device__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsign
     __syncwarp();
 }
 
-static_assert(sizeof(P3Box) <= P3_WARP_BYTES, "the box path uses a warp's region of the flat path");
-
-// The roads listed in P2 (more than small_n4 distinct fits, or a cross-road
-// candidate with a repeated coordinate) are fitted first, one warp each
-// (box_road); then every warp claims runs of d.run_roads consecutive roads
-// (4, 8 or 16) and fits the others itself, WARP_ROADS at a time (fit_run).
-// Each warp works in its own region of shared memory, so no stage of P3
-// waits for the whole CTA.
 template <bool PLAIN>
-__device__ void p3_phase(const Dev &d, unsigned char *smem, int qbig, int qsmall)
+__device__ __forceinline__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
-    const unsigned n_big = min(ldcg(&d.ctrl->n_big), d.max_roads);
-    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
-    unsigned long long npass = 0;
-    unsigned char *region = smem + warp_id() * P3_WARP_BYTES;
-    // a warp's first item of each queue is its own index; the queue hands out the rest
-    const unsigned n_warps = gridDim.x * WARPS;
-    for (unsigned i = blockIdx.x * WARPS + warp_id(); i < n_big;) {
-        box_road<PLAIN>(d, region, min(ldcg(d.big_list + i), d.max_roads - 1), npass);
-        unsigned ni = 0;
-        if (lane_id() == 0)
-            ni = n_warps + atomicAdd(&d.ctrl->q[qbig], 1u);
-        i = __shfl_sync(FULL_MASK, ni, 0);
+    if (PLAIN || d.cut < FLOAT_CUT || !box_float(d, region, g, npass))
+        box_integer<PLAIN>(d, region, g, npass);
+}
+
+constexpr size_t P3_BOX_BYTES = (sizeof(P3Box) + 15) / 16 * 16;   // a warp's region of the box path
+
+// The group path's shared memory: a slice of the roads, sorted.
+constexpr unsigned P3_ROADS = 2 * BLOCK;      // roads of a slice at most
+constexpr unsigned P3_BUCKETS = 16 * N_GROUP_CLS;
+struct P3Slice {
+    P3Group warp[WARPS];
+    RoadItem item[P3_ROADS];
+    unsigned n[P3_BUCKETS];                      // roads of each bucket, then its first place
+    unsigned end[2 * N_GROUP_CLS];               // place after each half class's last road
+    unsigned csum[P3_ROADS / ROAD_CHUNK + 2];    // survivors of the slice's road chunks
+    unsigned q;                                  // steps handed out
+    unsigned g0, sh;                             // first road; the shift of the 32-bit words
+    // what every step reads of the kernel's argument (a load through its
+    // address takes an L1 miss)
+    const uint16_t *coords;
+    const int4 *fitc;
+    unsigned long long *surv_pool;
+    uint8_t *surv_cnt;
+    long long cut;
+    size_t max_roads;
+};
+static_assert(offsetof(P3Slice, item) % 16 == 0, "16-byte items");
+// the slice's roads left to the box path, after the warps' regions of that path
+struct P3Redo {
+    uint16_t road[P3_ROADS];
+    unsigned n;
+};
+constexpr size_t P3_REDO = WARPS * P3_BOX_BYTES > sizeof(P3Slice) ? WARPS * P3_BOX_BYTES : (sizeof(P3Slice) + 15) / 16 * 16;
+
+// The classes' shapes (lanes of slot a, of slot b, hits of b per lane, hits of
+// e).  Most roads of classes 2 and 4 have two hits at most in slot e: they
+// take a loop of half the length.
+using GroupCls0 = GroupRoad<1, 0, 2, 2>;    // (2, 2) hits: 16 roads a step
+using GroupCls1 = GroupRoad<2, 0, 2, 2>;    // (4, 2): 8
+using GroupCls2 = GroupRoad<2, 1, 2, 2>;    // (4, 4): 4
+using GroupCls2e = GroupRoad<2, 1, 2, 4>;   // and more than two hits in slot e
+using GroupCls3 = GroupRoad<3, 0, 2, 2>;    // (8, 2): 4
+using GroupCls4 = GroupRoad<3, 1, 2, 2>;    // (8, 4): 2
+using GroupCls4e = GroupRoad<3, 1, 2, 4>;
+
+// Fit the roads first .. first + ROADS - 1 of the slice's list (below n) with
+// one warp; returns the lane's passing combinations.  Not inlined: a register
+// allocation per class (in one function the five classes spilled 220 bytes).
+template <bool PLAIN, class Road>
+__device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, unsigned first, unsigned n)
+{
+    P3Slice &S = *reinterpret_cast<P3Slice *>(smem);
+    const unsigned sh = S.sh, g0 = S.g0;
+    constexpr unsigned A = Road::A, YL = Road::YL, YN = Road::YN, B = Road::B, W = Road::W, G = Road::G,
+                       HITS = Road::HITS;
+    const unsigned lane = lane_id(), gl = lane % G, gi = lane / G;
+    const unsigned gmask = G == 32 ? FULL_MASK : ((1u << (G & 31u)) - 1u) << (gi * G);
+    Road r;
+    const bool on = first + gi < n;
+    r.it = RoadItem{};
+    if (on)
+        r.it = S.item[first + gi];
+    const uint32_t pk = r.it.pk;
+    const size_t g = r.it.g;
+    r.excl = min((pk >> 20) & 7u, 4u);
+    r.nf = fitted_counts(pk);   // no road: no hits
+    r.mb = r.m(r.slot(1));
+    r.mc = r.m(r.slot(2));
+    r.me = r.m(r.slot(3));
+    r.x = gl % A;
+    r.yl = gl / A;
+    r.live = r.x < r.m(r.slot(0));
+    r.cb = PLAIN && on ? ldcg(d.comb_off + g) : 0ull;
+    int4 *hit = S.warp[warp_id()].A + gi * HITS;
+    r.hit = hit;
+    __syncwarp();   // the table's previous readers are done
+    {
+        // comb strides of the layers
+        const unsigned S1 = pk & 15u, S2 = S1 * ((pk >> 4) & 15u), S3 = S2 * ((pk >> 8) & 15u),
+                       S4 = S3 * ((pk >> 12) & 15u);
+        // The road's hits, N per lane.  Every load is issued before the first
+        // is used, without a branch (a missing hit reads its row's slot, whose
+        // value is not used): one wait for L2 instead of one per round.
+        constexpr unsigned N = (HITS + G - 1) / G;
+        unsigned at[N];   // slot | k << 4, and bit 31: the hit exists
+        int v[N];
+        int4 cj[N];
+        const int4 *cc = S.fitc + SET_INT4 * min((unsigned)r.it.set, (unsigned)(N_SETS - 1)) + SET_C;
+        const uint16_t *row = S.coords + g * 40;
+#pragma unroll
+        for (unsigned i = 0; i < N; ++i) {
+            const unsigned h = i * G + gl;
+            const unsigned role = h < A ? 0u : h < A + B ? 1u : h < A + 2 * B ? 2u : 3u;
+            const unsigned k = (h - (role == 0 ? 0u : A + (role - 1) * B)) & 7u, s = r.slot(role);
+            at[i] = s | k << 4 | (k < r.m(s) && h < HITS ? 0x80000000u : 0u);
+            v[i] = ldcg(row + (s + (s >= r.excl)) * 8 + k);
+            if (!PLAIN)
+                cj[i] = __ldg(cc + s);
+        }
+        int4 c4, c5, kk;
+        if (!PLAIN) {
+            c4 = __ldg(cc + 4);
+            c5 = __ldg(cc + 5);
+            kk = __ldg(cc + 6);
+        }
+#pragma unroll
+        for (unsigned i = 0; i < N; ++i) {
+            const unsigned s = at[i] & 15u, k = (at[i] >> 4) & 7u, L = s + (s >= r.excl);
+            const unsigned S = L == 0 ? 1u : L == 1 ? S1 : L == 2 ? S2 : L == 3 ? S3 : S4;
+            int4 a = make_int4(0, 0, 0, (int)(k * S));
+            if (!PLAIN) {
+                a.x = cj[i].x * v[i];
+                a.y = cj[i].y * v[i];
+                a.z = cj[i].z * v[i];
+                if (i * G < A) {   // role a: curvature, phi, 4096 * offset and the road bits
+                    const bool ra = i * G + gl < A;
+                    const int curv = ra ? r.it.curv : 0, phi = ra ? r.it.phi : 0, off = ra ? 4096 : 0;
+                    a.x += c4.x * curv + c5.x * phi + kk.x * off;
+                    a.y += c4.y * curv + c5.y * phi + kk.y * off;
+                    a.z += c4.z * curv + c5.z * phi + kk.z * off;
+                    a.w += ra ? (int)((pk >> 24) << 15) : 0;
+                }
+            }
+            if (at[i] >> 31)
+                hit[i * G + gl] = a;
+        }
     }
     __syncwarp();
-    {
-        const unsigned rr = (unsigned)d.run_roads;
-        const unsigned n_runs = (n_roads + rr - 1) / rr;
-        for (unsigned c = blockIdx.x * WARPS + warp_id(); c < n_runs;) {
-            const unsigned ge = min(c * rr + rr, n_roads);
-            for (unsigned g0 = c * rr; g0 < ge; g0 += WARP_ROADS)
-                fit_run<PLAIN>(d, region, g0, min((unsigned)WARP_ROADS, ge - g0), npass);
-            unsigned nc = 0;
-            if (lane_id() == 0)
-                nc = n_warps + atomicAdd(&d.ctrl->q[qsmall], 1u);
-            c = __shfl_sync(FULL_MASK, nc, 0);
+
+    // The lane's fits.  A failing or missing fit's word is its own, above
+    // every passing one's, so that two equal words are always two passing fits.
+    const unsigned mcw = __reduce_max_sync(FULL_MASK, r.mc), mew = __reduce_max_sync(FULL_MASK, r.me);
+    const long long cut = S.cut;
+    int4 pab[YN];
+    unsigned q[YN], code[YN], cw[YN][W], np = 0;   // a pair's lowest word, its fit and state; minima over z
+    bool tie = false, tie2 = false, tie3 = false, tie4 = false;   // (several: no long chain of one flag)
+    // minimum of t over the lanes that differ in bits [o0, o1) of the lane
+    const auto fold = [](bool &tie, unsigned t, unsigned o0, unsigned o1) {
+#pragma unroll
+        for (unsigned o = o0; o < o1; o <<= 1) {
+            const unsigned u = __shfl_xor_sync(FULL_MASK, t, o);
+            tie = tie | (u == t);
+            t = min(t, u);
         }
+        return t;
+    };
+    const auto meet = [](bool &tie, unsigned t, unsigned u) {
+        tie = tie | (u == t);
+        return min(t, u);
+    };
+#pragma unroll
+    for (unsigned j = 0; j < YN; ++j) {
+        pab[j] = add4(hit[r.x], hit[A + r.y(j)]);   // unspecified unless the hits exist
+        q[j] = 0xE0000000u | (lane << 8) | j;
+        code[j] = 0;
+#pragma unroll
+        for (unsigned w = 0; w < W; ++w)
+            cw[j][w] = 0xC0000000u | (lane << 8) | (j * W + w);
+    }
+    for (unsigned z = 0; z < mcw; ++z) {
+        const int4 az = hit[A + B + z];
+        const unsigned none = 0x80000000u | (lane << 8) | (z << 4);
+        unsigned word[YN][W], rz[YN], ce[W];
+#pragma unroll
+        for (unsigned w = 0; w < W; ++w) {
+            if (w >= 2 && w >= mew) {   // no road of the warp has hit w
+                ce[w] = 0;
+                continue;
+            }
+            const int4 aw = hit[A + 2 * B + w];
+            const bool zw = r.live & (z < r.mc) & (w < r.me);
+#pragma unroll
+            for (unsigned j = 0; j < YN; ++j) {
+                const bool in = zw & (r.y(j) < r.mb);
+                if (PLAIN) {
+                    const unsigned long long k =
+                        in ? ldcg(d.fit_key + r.cb + (unsigned)(pab[j].w + az.w + aw.w)) : NO_KEY;
+                    word[j][w] = k == NO_KEY ? none + (j * W + w) : (unsigned)((k >> 23) >> sh);
+                } else {
+                    const long long chi2 = sq((pab[j].x + az.x + aw.x) >> 12) + sq((pab[j].y + az.y + aw.y) >> 12) +
+                                           sq((pab[j].z + az.z + aw.z) >> 12);
+                    const bool pass = in & (chi2 <= cut);
+                    np += pass;
+                    word[j][w] = pass ? (unsigned)((unsigned long long)chi2 >> sh) : none + (j * W + w);
+                }
+                cw[j][w] = meet(tie, cw[j][w], word[j][w]);
+                rz[j] = w == 0 ? word[j][w] : meet(tie2, rz[j], word[j][w]);
+            }
+            // (c, e) at z, w
+            ce[w] = word[0][w];
+#pragma unroll
+            for (unsigned j = 1; j < YN; ++j)
+                ce[w] = meet(tie3, ce[w], word[j][w]);
+            ce[w] = fold(tie3, ce[w], 1, G);
+        }
+        unsigned ac = rz[0];   // (a, c) at x, z
+#pragma unroll
+        for (unsigned j = 1; j < YN; ++j)
+            ac = meet(tie4, ac, rz[j]);
+        ac = fold(tie4, ac, A, G);
+#pragma unroll
+        for (unsigned j = 0; j < YN; ++j) {
+            const unsigned t = min(ac, fold(tie4, rz[j], 1, A));   // and (b, c) at y, z
+            bool ok = false;
+            unsigned ws = 0;
+#pragma unroll
+            for (unsigned w = 0; w < W; ++w) {
+                if (w >= 2 && w >= mew)
+                    continue;
+                const bool here = word[j][w] == rz[j];
+                ws = here ? w : ws;
+                ok = here ? ce[w] == rz[j] : ok;
+            }
+            tie2 = tie2 | (rz[j] == q[j]);
+            if (rz[j] < q[j]) {
+                q[j] = rz[j];
+                code[j] = z << 2 | ws | (ok && t == rz[j] ? 0x80u : 0u);
+            }
+        }
+    }
+
+    // (a, e) and (b, e), then the survivors
+    GroupFound<YN> f;
+    unsigned te[YN];
+#pragma unroll
+    for (unsigned j = 0; j < YN; ++j)
+        te[j] = 0;
+#pragma unroll
+    for (unsigned w = 0; w < W; ++w) {
+        if (w >= 2 && w >= mew)
+            continue;
+        unsigned ae = cw[0][w];
+#pragma unroll
+        for (unsigned j = 1; j < YN; ++j)
+            ae = meet(tie3, ae, cw[j][w]);
+        ae = fold(tie3, ae, A, G);
+#pragma unroll
+        for (unsigned j = 0; j < YN; ++j) {
+            const unsigned t = min(ae, fold(tie4, cw[j][w], 1, A));
+            te[j] = (code[j] & 3u) == w ? t : te[j];
+        }
+    }
+    const bool tied = (__ballot_sync(FULL_MASK, tie | tie2 | tie3 | tie4) & gmask) != 0u;   // the road has a tie
+    f.cnt = 0;
+#pragma unroll
+    for (unsigned j = 0; j < YN; ++j) {
+        f.surv[j] = !tied && code[j] >= 0x80u && te[j] == q[j] && q[j] < 0x80000000u;
+        f.key[j] = NO_KEY;
+        f.rank[j] = 0;
+        f.cnt += __popc(__ballot_sync(FULL_MASK, f.surv[j]) & gmask);
+    }
+#pragma unroll
+    for (unsigned j = 0; j < YN; ++j)
+        if (f.surv[j])
+            f.key[j] = r.template key_at<PLAIN>(d, cut, j, (code[j] >> 2) & 3u, code[j] & 3u);
+    if (__any_sync(FULL_MASK, f.cnt > 1))
+        group_rank(f, gmask);
+#pragma unroll
+    for (unsigned j = 0; j < YN; ++j)
+        if (f.surv[j])
+            S.surv_pool[f.rank[j] * S.max_roads + g] = f.key[j];
+    if (on && gl == 0) {
+        if (tied) {
+            P3Redo &R = *reinterpret_cast<P3Redo *>(smem + P3_REDO);
+            R.road[atomicAdd(&R.n, 1u)] = (uint16_t)(g - g0);
+        } else {
+            S.surv_cnt[g] = (uint8_t)f.cnt;
+            if (f.cnt)
+                atomicAdd(&S.csum[g / ROAD_CHUNK - g0 / ROAD_CHUNK], f.cnt);
+        }
+    }
+    np = tied ? 0u : np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
+    const bool publish = ((pk >> 23) & 1u) && !tied;
+    if (__any_sync(FULL_MASK, publish)) {   // on a copy, so that the road stays in registers
+        const Road rc = r;
+        group_publish<PLAIN>(d, rc, publish);
+    }
+    return np;
+}
+
+// The group path: every CTA takes an equal share of the roads, P3_ROADS at
+// most at a time, and sorts them in shared memory by class, widest first, and
+// by the hits of slots c and e, so that a warp's roads loop alike.  (Lists of
+// the whole batch in device memory, with an atomic per class and warp, made
+// the flag stage of 10,000 events wait 8 us on the counters.)  A step is one
+// warp's roads of one class; the warps claim the steps from a queue in shared
+// memory.  Not inlined: the stages before and after it keep a register
+// allocation of their own (inlined, the decode and the box path took 10 % and
+// 3 % longer).
+template <bool PLAIN>
+__device__ __noinline__ void p3_groups(const Dev &d, unsigned char *smem, unsigned long long &npass)
+{
+    P3Slice &S = *reinterpret_cast<P3Slice *>(smem);
+    P3Redo &R = *reinterpret_cast<P3Redo *>(smem + P3_REDO);
+    const unsigned lane = lane_id();
+    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
+    const unsigned lo = (unsigned)((unsigned long long)n_roads * blockIdx.x / gridDim.x);
+    const unsigned hi = (unsigned)((unsigned long long)n_roads * (blockIdx.x + 1) / gridDim.x);
+    const unsigned cl = max((unsigned)d.run_roads / 8, 1u);
+    const unsigned parts = (hi - lo + P3_ROADS - 1) / P3_ROADS;
+    unsigned long long np = 0;
+    for (unsigned part = 0; part < parts; ++part) {
+        const unsigned g0 = lo + (unsigned)((unsigned long long)(hi - lo) * part / parts);
+        const unsigned g1 = lo + (unsigned)((unsigned long long)(hi - lo) * (part + 1) / parts);
+        // counting sort, two roads per thread
+        for (unsigned i = threadIdx.x; i < P3_BUCKETS; i += BLOCK)
+            S.n[i] = 0;
+        if (threadIdx.x < P3_ROADS / ROAD_CHUNK + 2)
+            S.csum[threadIdx.x] = 0;
+        if (threadIdx.x == 0) {
+            S.q = R.n = 0;
+            S.g0 = g0;
+            S.coords = d.coords;
+            S.fitc = d.fitc;
+            S.surv_pool = d.surv_pool;
+            S.surv_cnt = d.surv_cnt;
+            S.cut = d.cut;
+            S.max_roads = d.max_roads;
+            // the shift that brings the cut below 2^31 (a chi-square is below 2^38)
+            const unsigned long long cut = min((unsigned long long)max(d.cut, 0ll), (1ull << 38) - 1);
+            S.sh = cut >> 31 ? 33 - __clzll((long long)cut) : 0u;
+        }
+        __syncthreads();
+        RoadItem it[2];
+        unsigned bucket[2], place[2];
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h) {
+            const unsigned g = g0 + h * BLOCK + threadIdx.x;
+            bucket[h] = P3_BUCKETS;
+            if (g < g1) {
+                const RoadRec r = ldcg(d.roads + g);
+                const unsigned perm = r.fit & 0xFFu, cls = (r.fit >> 8) & 7u;
+                it[h] = RoadItem{g, r.pk, r.curv, r.phi, r.set, (uint16_t)perm};
+                if (cls < N_GROUP_CLS) {   // a fitted road has 1 .. 4 hits in slots c and e
+                    const unsigned nf = fitted_counts(r.pk);
+                    const unsigned mc = (nf >> (4 * ((perm >> 4) & 3u))) & 15u, me = (nf >> (4 * (perm >> 6))) & 15u;
+                    bucket[h] = 16 * (N_GROUP_CLS - 1 - cls) + (me > 2 ? 0u : 8u) + 2 * ((4 - mc) & 3u) + (me & 1u);
+                    place[h] = atomicAdd(&S.n[bucket[h]], 1u);
+                }
+            }
+        }
+        __syncthreads();
+        if (warp_id() == 0) {   // first places: an exclusive scan of the counts, class by class
+            unsigned run = 0;
+#pragma unroll
+            for (unsigned c = 0; c < N_GROUP_CLS; ++c) {
+                const unsigned v = lane < 16 ? S.n[16 * c + lane] : 0u;
+                unsigned inc = v;
+#pragma unroll
+                for (unsigned o = 1; o < 16; o <<= 1) {
+                    const unsigned u = __shfl_up_sync(FULL_MASK, inc, o);
+                    inc += lane >= o ? u : 0u;
+                }
+                if (lane < 16)
+                    S.n[16 * c + lane] = run + inc - v;
+                if (lane == 7 || lane == 15)
+                    S.end[2 * c + (lane >> 3)] = run + inc;
+                run += __shfl_sync(FULL_MASK, inc, 15);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h)
+            if (bucket[h] < P3_BUCKETS)
+                S.item[S.n[bucket[h]] + place[h]] = it[h];
+        __syncthreads();
+        // steps of the classes 4, 3, .. 0
+        const auto steps = [&](unsigned i, unsigned roads) {
+            return (S.end[i] - (i ? S.end[i - 1] : 0u) + roads - 1) / roads;
+        };
+        const unsigned e4e = steps(0, GroupCls4e::ROADS), e4 = e4e + steps(1, GroupCls4::ROADS),
+                       e3 = e4 + steps(3, GroupCls3::ROADS), e2e = e3 + steps(4, GroupCls2e::ROADS),
+                       e2 = e2e + steps(5, GroupCls2::ROADS), e1 = e2 + steps(7, GroupCls1::ROADS),
+                       e0 = e1 + steps(9, GroupCls0::ROADS);
+        for (;;) {
+            unsigned s0 = 0;
+            if (lane == 0)
+                s0 = atomicAdd(&S.q, cl);
+            s0 = __shfl_sync(FULL_MASK, s0, 0);
+            if (s0 >= e0)
+                break;
+            for (unsigned s = s0; s < min(s0 + cl, e0); ++s) {
+                if (s < e4e)
+                    np += group_item<PLAIN, GroupCls4e>(d, smem, s * GroupCls4e::ROADS, S.end[0]);
+                else if (s < e4)
+                    np += group_item<PLAIN, GroupCls4>(d, smem, S.end[0] + (s - e4e) * GroupCls4::ROADS, S.end[1]);
+                else if (s < e3)
+                    np += group_item<PLAIN, GroupCls3>(d, smem, S.end[2] + (s - e4) * GroupCls3::ROADS, S.end[3]);
+                else if (s < e2e)
+                    np += group_item<PLAIN, GroupCls2e>(d, smem, S.end[3] + (s - e3) * GroupCls2e::ROADS, S.end[4]);
+                else if (s < e2)
+                    np += group_item<PLAIN, GroupCls2>(d, smem, S.end[4] + (s - e2e) * GroupCls2::ROADS, S.end[5]);
+                else if (s < e1)
+                    np += group_item<PLAIN, GroupCls1>(d, smem, S.end[6] + (s - e2) * GroupCls1::ROADS, S.end[7]);
+                else
+                    np += group_item<PLAIN, GroupCls0>(d, smem, S.end[8] + (s - e1) * GroupCls0::ROADS, S.end[9]);
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < P3_ROADS / ROAD_CHUNK + 2 && S.csum[threadIdx.x])
+            atomicAdd(&d.rchunk_sum[g0 / ROAD_CHUNK + threadIdx.x], S.csum[threadIdx.x]);
+        __syncthreads();   // the slice's memory becomes the warps' regions, then is refilled
+        for (unsigned i = warp_id(); i < R.n; i += WARPS)
+            box_road<PLAIN>(d, smem + warp_id() * P3_BOX_BYTES, g0 + R.road[i], np);
+        __syncthreads();
+    }
+    npass += np;
+}
+
+// P3: the group path's roads, then the roads listed in P2 for the box path
+// (one warp each, a warp's first by its own index, neighbouring indices on
+// different SMs, the rest from a queue, which evens out the group path's
+// shares too).
+template <bool PLAIN>
+__device__ void p3_phase(const Dev &d, unsigned char *smem, int qbox)
+{
+    unsigned long long npass = 0;
+    p3_groups<PLAIN>(d, smem, npass);
+    __syncthreads();   // the shared memory becomes the warps' regions
+    unsigned char *region = smem + warp_id() * P3_BOX_BYTES;
+    const unsigned n_warps = gridDim.x * WARPS, n_box = min(ldcg(&d.ctrl->n_box), d.max_roads);
+    for (unsigned i = warp_id() * gridDim.x + blockIdx.x; i < n_box;) {
+        box_road<PLAIN>(d, region, min(ldcg(d.box_list + i), d.max_roads - 1), npass);
+        if (n_box <= n_warps)
+            break;
+        unsigned ni = 0;
+        if (lane_id() == 0)
+            ni = n_warps + atomicAdd(&d.ctrl->q[qbox], 1u);
+        i = __shfl_sync(FULL_MASK, ni, 0);
     }
     npass = block_sum(npass);
     if (!PLAIN && threadIdx.x == 0 && npass)
@@ -2967,7 +3318,7 @@ __device__ void clear_hash(const Dev &d)
 // ---------------------------------------------------------------------------
 
 
-__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_persistent(Dev d)
+__global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 2 : 768 / BLOCK) k_persistent(const __grid_constant__ Dev d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     if (d.skip_arrival == 1 && blockIdx.x == 0)
@@ -2991,7 +3342,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) k_persistent(Dev d)
     if (ldcg(&d.ctrl->err_inv) != 0ull)
         return;   // a data fault: no tracks
 
-    p3_phase<false>(d, smem, Q_BIG, Q_SMALL);
+    p3_phase<false>(d, smem, Q_BOX);
     if (d.skip_arrival == 2 && blockIdx.x == 0)
         return;   // test hook: this CTA leaves after publishing, the others' waits run out
     if (!grid_sync(d))
@@ -3145,12 +3496,12 @@ __global__ void __launch_bounds__(BLOCK) k_fit_plain(Dev d)
         atomicAdd(&d.ctrl->n_pass, npass);
 }
 
-__global__ void __launch_bounds__(BLOCK) k_warrior_plain(Dev d)
+__global__ void __launch_bounds__(BLOCK) k_warrior_plain(const __grid_constant__ Dev d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     if (stop_after_unpack(d))
         return;
-    p3_phase<true>(d, smem, Q_BIG, Q_SMALL);
+    p3_phase<true>(d, smem, Q_BOX);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p4(Dev d)
@@ -3208,7 +3559,10 @@ __global__ void __launch_bounds__(BLOCK) k_export_roads(Dev d)
 
 static size_t p1_smem() { return WARPS * sizeof(P1Warp); }
 static size_t p2_smem() { return sizeof(P2Smem) > WARPS * P2W_BYTES ? sizeof(P2Smem) : WARPS * P2W_BYTES; }
-static size_t p3_smem() { return WARPS * P3_WARP_BYTES; }
+static size_t p3_smem()
+{
+    return P3_REDO + sizeof(P3Redo);
+}
 
 size_t persistent_smem_bytes()
 {

@@ -41,8 +41,8 @@ constexpr size_t OFF_EV = OFF_SPAN + up256(3 * sizeof(uint32_t) * S_SPANS);     
 constexpr size_t OFF_ROADS = OFF_EV + up256(2 * sizeof(uint32_t) * S_EVENTS);
 constexpr size_t OFF_COORDS = OFF_ROADS + up256(sizeof(RoadRec) * S_ROADS);
 constexpr size_t OFF_XMASK = OFF_COORDS + up256(sizeof(uint16_t) * 40 * S_ROADS);
-constexpr size_t OFF_BIG = OFF_XMASK + up256(sizeof(unsigned long long) * S_ROADS);
-constexpr size_t OFF_CAND = OFF_BIG + up256(sizeof(uint32_t) * S_ROADS);
+constexpr size_t OFF_BOX = OFF_XMASK + up256(sizeof(unsigned long long) * S_ROADS);
+constexpr size_t OFF_CAND = OFF_BOX + up256(sizeof(uint32_t) * S_ROADS);
 constexpr size_t OFF_FITC = OFF_CAND + up256(sizeof(uint32_t) * (S_ROADS / 32 + 1));
 constexpr size_t OFF_SURV = OFF_FITC + up256(sizeof(int4) * SET_INT4 * N_SETS);
 constexpr size_t OFF_SCNT = OFF_SURV + up256(sizeof(unsigned long long) * SURV_SLOTS * S_ROADS);
@@ -127,7 +127,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     d.roads = reinterpret_cast<RoadRec *>(b + OFF_ROADS);
     d.coords = reinterpret_cast<uint16_t *>(b + OFF_COORDS);
     d.xmask = reinterpret_cast<unsigned long long *>(b + OFF_XMASK);
-    d.big_list = reinterpret_cast<uint32_t *>(b + OFF_BIG);
+    d.box_list = reinterpret_cast<uint32_t *>(b + OFF_BOX);
     d.cand_bits = reinterpret_cast<uint32_t *>(b + OFF_CAND);
     d.fitc = reinterpret_cast<int4 *>(b + OFF_FITC);
     d.surv_pool = reinterpret_cast<unsigned long long *>(b + OFF_SURV);
@@ -144,7 +144,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     d.tracks = d_tracks;
     d.cut = chi2_cut;
     d.small_n4 = N4_SMALL_MAX;
-    d.run_roads = WARP_ROADS;
+    d.run_roads = RUN_ROADS;
     d.wait_ns = 2000000000ull;
 
     // what must start at zero: the control block every batch, the group

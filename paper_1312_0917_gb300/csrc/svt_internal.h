@@ -26,7 +26,9 @@ constexpr unsigned long long NO_KEY = ~0ull;
 // fault ranks: at one word a format/grammar fault outranks a limit fault;
 // truncation is reported at position n_words, after every word
 enum : unsigned { RANK_BAD = 1, RANK_LIMIT = 2, RANK_TRUNC = 3 };
-enum : unsigned { FLAG_CAPACITY = 1, FLAG_TIMEOUT = 2, FLAG_INTERNAL = 4 };
+// FLAG_FAULT: the stream has a fault (err_inv is set); FLAG_GROUPS: the group
+// table has an entry
+enum : unsigned { FLAG_CAPACITY = 1, FLAG_TIMEOUT = 2, FLAG_INTERNAL = 4, FLAG_FAULT = 8, FLAG_GROUPS = 16 };
 
 // The kernels' copy of each set's constants as int32 in 16-byte words, 14
 // per set: words 0..5 hold F row by row, then q and three zeros (the output
@@ -57,6 +59,7 @@ inline void fit_words(const svt_const_set *sets, int32_t *out)
 // arrivals of the persistent kernel.
 struct Ctrl {
     unsigned long long err_inv;   // max over faults of ~((pos << 8) | rank); 0 = none
+    unsigned int bar;             // grid barrier arrivals; its polls read the flags with it
     unsigned int flags;           // FLAG_*
     unsigned int n_events;        // complete events (EE words)
     unsigned int n_ep;            // EP words in the stream
@@ -66,7 +69,6 @@ struct Ctrl {
     unsigned int hash_used;       // claimed slots of the group table
     unsigned int n_box;           // roads of the box path (list length)
     unsigned int q[12];           // work-queue heads
-    unsigned int bar;             // grid barrier arrivals
     unsigned int done[4];         // last-block-done counters
     unsigned long long n_comb, n_pass, n_out;
     unsigned long long pad1[2];

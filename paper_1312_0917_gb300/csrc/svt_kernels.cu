@@ -78,17 +78,10 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
     return t;
 }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p)
 {
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned ld_relaxed(const unsigned *p)
-{
-    unsigned v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -105,12 +98,14 @@ __device__ __forceinline__ RoadRec ldcg(const RoadRec *p)
     return r;
 }
 
-__device__ __forceinline__ void report(const Dev &d, unsigned long long pos, unsigned rank)
-{
-    atomicMax(&d.ctrl->err_inv, ~((pos << 8) | rank));
-}
-
 __device__ __forceinline__ void raise_flag(const Dev &d, unsigned f) { atomicOr(&d.ctrl->flags, f); }
+
+// a fault of the stream at word err >> 8 of rank err & 255
+__device__ __forceinline__ void report(const Dev &d, unsigned long long err)
+{
+    atomicMax(&d.ctrl->err_inv, ~err);
+    raise_flag(d, FLAG_FAULT);
+}
 
 // Survivor slot s of road g.  Slots are slot-major, so the first survivors
 // of consecutive roads are adjacent (the output stage reads them in road
@@ -321,44 +316,55 @@ __device__ __forceinline__ unsigned grab_after_first(const Dev &d, int q)
     return gridDim.x + grab(d, q);
 }
 
-// Grid barrier of the persistent kernel.  All CTAs are co-resident
+// Grid barrier number k (1, 2, ..) of the persistent kernel; `flags` gets
+// FLAG_* as they are once every CTA has arrived.  All CTAs are co-resident
 // (cooperative launch).  The wait is bounded by d.wait_ns; on expiry the CTA
-// raises FLAG_TIMEOUT and every CTA that sees the flag stops working.
-__device__ bool grid_sync(const Dev &d)
+// raises FLAG_TIMEOUT and every CTA that sees the flag stops working.  Bound:
+// L2 round trips.  The arrival returns nothing, and a poll reads the count and
+// the flags as one word, so that a CTA leaves one trip after the last arrival
+// (with the arrival's old value awaited and the flags loaded after the wait a
+// barrier took 0.9 us more).
+__device__ bool grid_sync(const Dev &d, unsigned k, unsigned &flags)
 {
-    __shared__ int s_ok;
+    __shared__ unsigned s_flags;
     __syncthreads();
     if (threadIdx.x == 0) {
+        static_assert(offsetof(Ctrl, bar) % 8 == 0 && offsetof(Ctrl, flags) == offsetof(Ctrl, bar) + 4,
+                      "count and flags in one word");
+        const unsigned long long *word = reinterpret_cast<const unsigned long long *>(&d.ctrl->bar);
         __threadfence();
-        const unsigned nb = gridDim.x;
-        unsigned old = atomicAdd(&d.ctrl->bar, 1u);
-        unsigned target = (old / nb + 1u) * nb;
-        unsigned long long t0 = globaltimer_ns();
-        int ok = 1;
-        // relaxed polls of the counter (the fence below orders what follows);
-        // the timeout flag and the clock are looked at every 16th poll
-        for (unsigned it = 1; (int)(ld_relaxed(&d.ctrl->bar) - target) < 0; ++it) {
+        atomicAdd(&d.ctrl->bar, 1u);
+        const unsigned target = k * gridDim.x;
+        unsigned long long t0 = 0, v;
+        // relaxed polls (the fence below orders what follows); the clock is
+        // looked at every 16th poll
+        for (unsigned it = 1; v = ld_relaxed(word), (int)((unsigned)v - target) < 0; ++it) {
+            if ((unsigned)(v >> 32) & FLAG_TIMEOUT)
+                break;
             if ((it & 15u) == 0) {
-                if (ld_relaxed(&d.ctrl->flags) & FLAG_TIMEOUT) {
-                    ok = 0;
-                    break;
-                }
-                if (globaltimer_ns() - t0 > d.wait_ns) {
+                const unsigned long long t = globaltimer_ns();
+                t0 = t0 ? t0 : t;
+                if (t - t0 > d.wait_ns) {
                     raise_flag(d, FLAG_TIMEOUT);
-                    ok = 0;
+                    v |= (unsigned long long)FLAG_TIMEOUT << 32;
                     break;
                 }
             }
-            __nanosleep(32);
+            __nanosleep(20);
         }
         __threadfence();
-        if (ld_acquire(&d.ctrl->flags) & FLAG_TIMEOUT)
-            ok = 0;
-        s_ok = ok;
+        s_flags = (unsigned)(v >> 32);
     }
     __syncthreads();
-    return s_ok != 0;
+    flags = s_flags;
+    return !(flags & FLAG_TIMEOUT);
 }
+
+// The batch's counts as every CTA knows them: events and EP words from the
+// totals it sums in P1, the roads of complete events from the control block.
+struct Batch {
+    unsigned n_events, n_ep, n_roads;
+};
 
 // phase timestamp k of the persistent kernel (block 0, thread 0)
 __device__ __forceinline__ void stamp(const Dev &d, unsigned k)
@@ -368,7 +374,7 @@ __device__ __forceinline__ void stamp(const Dev &d, unsigned k)
 }
 
 // work-queue indices (Ctrl::q)
-enum { Q_P0 = 0, Q_P1, Q_P2, Q_BOX, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
+enum { Q_P2 = 0, Q_BOX, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
 
 // ---------------------------------------------------------------------------
 // P0 / P1: the word stream, one warp per span.  The stream is cut into
@@ -469,7 +475,7 @@ __device__ void scan_count(const Dev &d)
     __shared__ unsigned s_cnt[3][WARPS];
     if (lane == 0) {
         if (bad != ~0ull)
-            report(d, bad, RANK_BAD);
+            report(d, (bad << 8) | RANK_BAD);
         d.span_ee[sp] = ee;
         d.span_ep[sp] = ep;
         d.span_seg[sp] = seg;
@@ -684,12 +690,12 @@ __device__ void decode_span(const Dev &d, P1Warp &q, unsigned long long a, unsig
         }
     }
     if (lane == 0 && err != ~0ull)
-        atomicMax(&d.ctrl->err_inv, ~err);   // the first fault of the batch is its status
+        report(d, err);   // the first fault of the batch is its status
 }
 
 // P1; false when the stream does not fit the context (every CTA sees the
 // same totals and stops).  smem: the CTA's shared memory (a P1Warp per warp).
-__device__ bool scan_decode(const Dev &d, unsigned char *smem)
+__device__ bool scan_decode(const Dev &d, unsigned char *smem, Batch &bt)
 {
     const unsigned mine0 = blockIdx.x * WARPS;
     // the CTAs below this one (their aggregates follow the per-warp entries),
@@ -711,6 +717,8 @@ __device__ bool scan_decode(const Dev &d, unsigned char *smem)
     seg = block_seg_fold(seg);
     const unsigned n_ee = (unsigned)(all >> 32), n_ep = (unsigned)all;
     const bool fits = n_ee <= d.max_events && n_ep <= d.max_roads;
+    bt.n_events = n_ee;
+    bt.n_ep = n_ep;
     // the candidate bits of this batch's roads start at zero (P2 sets them)
     if (fits)
         for (unsigned i = blockIdx.x * BLOCK + threadIdx.x; i < n_ep / 32 + 1; i += gridDim.x * BLOCK)
@@ -722,7 +730,7 @@ __device__ bool scan_decode(const Dev &d, unsigned char *smem)
         unsigned tail = 0;
         if (d.n_words > 0 && !(__ldg(d.words + d.n_words - 1) >> 31)) {
             tail = 1;
-            report(d, d.n_words, RANK_TRUNC);
+            report(d, (d.n_words << 8) | RANK_TRUNC);
         }
         c->has_tail = tail;
         if (!fits)
@@ -759,10 +767,9 @@ __device__ bool scan_decode(const Dev &d, unsigned char *smem)
 // cross-road candidate; its marked hits are the ones it publishes and looks
 // up.  The road records get the candidate bit and their fit path.
 //
-// In a batch of many events, events of at most P2W_ROADS roads take one warp
-// each instead (p2_warp), with the same bitmaps, 32-bit signatures, and a
-// lane per road that tests its road against the others and marks its own
-// hits (p2_phase chooses).
+// Events of at most P2W_ROADS roads take one warp each instead (p2_warp), and
+// so do larger ones when there are many, with a bitmap of one layer at a time,
+// 10-bit signatures and a lane per tested pair (p2_phase chooses).
 // ---------------------------------------------------------------------------
 
 constexpr unsigned P2_PAIRS = 1024;   // road pairs queued for the exact test (more: tested in place)
@@ -798,29 +805,87 @@ __device__ __forceinline__ unsigned row_coord(const uint4 &q, unsigned x)
     return (w >> (16 * (x & 1u))) & 0xFFFFu;
 }
 
+// the coordinates of row q from slot n on replaced by 0xFFFF (no coordinate)
+__device__ __forceinline__ uint4 row_clip(uint4 q, unsigned n)
+{
+    const auto word = [n](unsigned w, unsigned i) {
+        return n >= 2 * i + 2 ? w : n == 2 * i + 1 ? w | 0xFFFF0000u : 0xFFFFFFFFu;
+    };
+    return make_uint4(word(q.x, 0), word(q.y, 1), word(q.z, 2), word(q.w, 3));
+}
+
+// slots of row q that hold v (bit x: slot x)
+__device__ __forceinline__ unsigned row_find(const uint4 &q, unsigned v)
+{
+    const unsigned v2 = v | v << 16;
+    const auto eq = [v2](unsigned w) {   // bit 15 and bit 31: the halves equal to v
+        const unsigned x = w ^ v2;
+        return ~(((x & 0x7FFF7FFFu) + 0x7FFF7FFFu) | x) & 0x80008000u;
+    };
+    // halves 2 i and 2 i + 1 of word i to bits 2 i and 2 i + 1
+    const auto two = [](unsigned e) { return (e >> 15 & 1u) | (e >> 30 & 2u); };
+    return two(eq(q.x)) | two(eq(q.y)) << 2 | two(eq(q.z)) << 4 | two(eq(q.w)) << 6;
+}
+
+// A layer's hits (row q, n of them) join the event's bitmap: bit x of the
+// result: hit x found its bit set.  The atomics are in flight together.
+// most: at least every lane's n.
+__device__ __forceinline__ unsigned see_row(uint32_t *seen, const uint4 &q, unsigned n, unsigned most)
+{
+    unsigned old[MAX_HITS], again = 0;
+#pragma unroll
+    for (unsigned x = 0; x < MAX_HITS; ++x) {
+        old[x] = 0;
+        if (x >= 2 && x >= most)
+            continue;
+        const unsigned v = row_coord(q, x);
+        if (x < n)   // the result is not awaited here
+            old[x] = atomicOr(&seen[v >> 5], 1u << (v & 31u)) >> (v & 31u);
+    }
+#pragma unroll
+    for (unsigned x = 0; x < MAX_HITS; ++x)
+        again |= (old[x] & 1u) << x;
+    return again;
+}
+
+// coordinate x (0 .. 7) of a layer's row
+__device__ __forceinline__ unsigned row_at(const uint4 &q, unsigned x)
+{
+    const unsigned w = x < 4 ? (x < 2 ? q.x : q.y) : (x < 6 ? q.z : q.w);
+    return (w >> (16 * (x & 1u))) & 0xFFFFu;
+}
+
 // Hits of one layer of a road (row q) whose coordinate was already in the
 // event's bitmap when the hit set its bit (bit x of `again`): a coordinate
 // of an earlier slot of the same row is a repeat; any other was set by
 // another road and gets the multi bit.  So a coordinate gets the multi bit
 // exactly when two roads hold it.  True when the row repeats a coordinate.
-__device__ __noinline__ bool seen_again(uint32_t *multi, const uint4 &q, unsigned again)
+__device__ __forceinline__ bool seen_again(uint32_t *multi, const uint4 &q, unsigned again)
 {
     bool rep = false;
-#pragma unroll
-    for (unsigned x = 0; x < MAX_HITS; ++x) {
-        if (!((again >> x) & 1u))
-            continue;
-        const unsigned v = row_coord(q, x);
-        bool dup = false;
-#pragma unroll
-        for (unsigned y = 0; y < x; ++y)
-            dup = dup || row_coord(q, y) == v;
-        if (dup)
+    for (; again; again &= again - 1) {
+        const unsigned x = __ffs(again) - 1;
+        const unsigned v = row_at(q, x);
+        if (row_find(q, v) & ((1u << x) - 1u))
             rep = true;
         else
             atomicOr(&multi[v >> 5], 1u << (v & 31u));
     }
     return rep;
+}
+
+// hits of a layer (row q, n of them) whose coordinate two roads hold: bit x
+__device__ __forceinline__ unsigned multi_row(const uint32_t *multi, const uint4 &q, unsigned n, unsigned most)
+{
+    unsigned m = 0;
+#pragma unroll
+    for (unsigned x = 0; x < MAX_HITS; ++x) {
+        if (x >= 4 && x >= most)
+            continue;
+        const unsigned v = row_coord(q, x) & 0xFFFu;
+        m |= ((multi[v >> 5] >> (v & 31u)) & 1u) << x;
+    }
+    return m & ((1u << n) - 1u);
 }
 
 // Roads r and t of the event: the layers on which they hold a common
@@ -990,17 +1055,11 @@ __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, uns
     __syncthreads();
     // coordinates present in >= 2 roads on a layer: each distinct coordinate
     // of a road's layer marks the bitmap, a second road with it the multi bit
-    for (unsigned i = threadIdx.x; i < nr * N_LAYERS; i += BLOCK) {
-        const unsigned k = i / N_LAYERS, l = i - k * N_LAYERS;
-        const unsigned n = (s.rec[k].pk >> (4 * l)) & 15u;
+    for (unsigned i0 = threadIdx.x - lane_id(); i0 < nr * N_LAYERS; i0 += BLOCK) {
+        const unsigned i = min(i0 + lane_id(), nr * N_LAYERS - 1), k = i / N_LAYERS, l = i - k * N_LAYERS;
+        const unsigned n = i0 + lane_id() == i ? (s.rec[k].pk >> (4 * l)) & 15u : 0u;   // <= MAX_HITS
         const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
-        unsigned again = 0;   // bit x: hit x found its bit set
-#pragma unroll
-        for (unsigned x = 0; x < MAX_HITS; ++x) {
-            const unsigned v = row_coord(q, x), bit = 1u << (v & 31u);
-            if (x < n && (atomicOr(&s.seen[l][v >> 5], bit) & bit))
-                again |= 1u << x;
-        }
+        const unsigned again = see_row(s.seen[l], q, n, __reduce_max_sync(FULL_MASK, n));
         if (again && seen_again(s.multi[l], q, again))
             s.rep[k] = 1;
     }
@@ -1012,11 +1071,9 @@ __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, uns
         for (unsigned l = 0; l < N_LAYERS; ++l) {
             const unsigned n = (s.rec[k].pk >> (4 * l)) & 15u;
             unsigned long long sg = 0;
-            for (unsigned x = 0; x < n; ++x) {
-                const unsigned v = s.coord[k][l * 8 + x];
-                if (is_multi(s, l, v))
-                    sg |= 1ull << sig_bit(v);
-            }
+            const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
+            for (unsigned m = multi_row(s.multi[l], q, n, MAX_HITS); m; m &= m - 1)
+                sg |= 1ull << sig_bit(row_at(q, __ffs(m) - 1));
             s.sig[k][l] = sg;
             layers += sg != 0;
         }
@@ -1053,206 +1110,238 @@ __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, uns
     __syncthreads();   // the shared arrays are refilled for the next event
 }
 
-// One warp's state for an event of at most P2W_ROADS roads; the roads'
-// coordinate rows stay in global memory (L2), read a road at a time.
+// One warp's state for an event of its own; the roads' coordinate rows stay in
+// global memory (they are written once, before this stage, so that loads may
+// use L1).
+constexpr unsigned P2_QUEUE = 64;       // queued road pairs: a batch of 32, and what one test may add
 struct P2Warp {
-    uint32_t seen[N_LAYERS][128];           // coordinate bitmaps of the event (12-bit coordinates)
-    uint32_t multi[N_LAYERS][128];          // coordinates present in two or more roads
-    uint32_t sig[P2W_ROADS][N_LAYERS];      // 32-bit signatures of a road's shared coordinates
-    uint32_t pk[P2W_ROADS];
+    uint32_t seen[128];                 // coordinate bitmap of the event, one layer at a time
+    uint32_t multi[128];                // coordinates present in two or more roads
+    uint2 sig[P2W_ROADS];               // signatures of the eligible roads' shared coordinates
+    uint32_t xm[P2W_ROADS][2];          // flagged hits of a road: bit 8 l + d, low and high word
+    uint32_t pair[P2_QUEUE];            // road pairs whose signatures meet on >= 3 layers (r | t << 16)
+    uint8_t elig[P2W_ROADS];            // roads with shared coordinates on >= 3 layers
 };
 constexpr size_t P2W_BYTES = (sizeof(P2Warp) + 15) / 16 * 16;
 
-// signature bit of a coordinate in a 32-bit signature
-__device__ __forceinline__ unsigned sig_bit32(unsigned v) { return (v * 0x9E3779B1u) >> 27; }
-
-// Hits of road g that road h holds too (bit 8 l + x), when they hold common
-// coordinates on three layers or more; 0 otherwise.  pg, ph: their records'
-// pk words.
-__device__ unsigned long long pair_marks(const Dev &d, unsigned g, unsigned h, uint32_t pg, uint32_t ph)
+// Signature of coordinates of layer l, ten bits a layer: layers 0..2 in x,
+// layers 3 and 4 in y.  bit: a multiplicative hash into 0..9.
+__device__ __forceinline__ unsigned sig_bit10(unsigned v) { return ((v * 0x9E3779B1u) >> 16) * 10u >> 16; }
+// layers on which two signatures (their fields ANDed) meet: the top bit of a
+// field is set by adding all ones below it to any bits below it
+__device__ __forceinline__ unsigned sig_layers(unsigned x, unsigned y)
 {
-    const uint4 *rg = reinterpret_cast<const uint4 *>(d.coords + (size_t)g * 40);
-    const uint4 *rh = reinterpret_cast<const uint4 *>(d.coords + (size_t)h * 40);
-    unsigned long long m = 0;
-    unsigned layers = 0;
-    for (unsigned l = 0; l < N_LAYERS; ++l) {
-        const unsigned ng = (pg >> (4 * l)) & 15u, nh = (ph >> (4 * l)) & 15u;   // <= MAX_HITS
-        const uint4 a = ldcg(rg + l), b = ldcg(rh + l);
-        unsigned br = 0;
-#pragma unroll
-        for (unsigned x = 0; x < MAX_HITS; ++x) {
-            const unsigned v = row_coord(a, x);
-            bool hit = false;
-#pragma unroll
-            for (unsigned y = 0; y < MAX_HITS; ++y)
-                hit = hit || (y < nh && row_coord(b, y) == v);
-            br |= (x < ng && hit) ? 1u << x : 0u;
-        }
-        layers += br != 0;
-        m |= (unsigned long long)br << (8 * l);
-    }
-    return layers >= 3 ? m : 0ull;
+    const unsigned m = 0x1FF7FDFFu, t = 0x20080200u;
+    return __popc(((x & m) + m | x) & t) + __popc(((y & m) + m | y) & t & 0xFFFFFu);
 }
 
-// P2 of the event of roads r0 .. r0 + nr - 1 (nr <= P2W_ROADS) by one warp
-// with state `w`; lane i owns roads i and i + 32.  The same steps as
-// p2_event: coordinates present in two roads (bitmaps), signatures of those
-// per road and layer, pairs whose signatures meet on >= 3 layers tested
-// exactly.  A lane tests its eligible road against every other eligible road
-// (a pair whose signatures meet on >= 3 layers has two) and marks only its
-// own road's hits, so each pair is tested from both sides.
+// The queued pairs (n of them, one per lane): hits the two roads of a pair
+// share are flagged in both when they share coordinates on >= 3 layers.
+__device__ __noinline__ void p2_pairs(const uint16_t *coords, const RoadRec *roads, P2Warp &w, unsigned r0, unsigned n)
+{
+    const unsigned lane = lane_id();
+    if (lane < n) {
+        const unsigned p = w.pair[lane], r = p & 0xFFFFu, t = p >> 16;
+        const uint4 *rr = reinterpret_cast<const uint4 *>(coords + (size_t)(r0 + r) * 40);
+        const uint4 *rt = reinterpret_cast<const uint4 *>(coords + (size_t)(r0 + t) * 40);
+        const uint32_t pr = ldcg(&roads[r0 + r].pk), pt = ldcg(&roads[r0 + t].pk);
+        unsigned lo_r = 0, lo_t = 0, hi_r = 0, hi_t = 0, layers = 0;
+        for (unsigned l = 0; l < N_LAYERS; ++l) {
+            const unsigned nr = (pr >> (4 * l)) & 15u, nt = (pt >> (4 * l)) & 15u;   // <= MAX_HITS
+            uint4 a = rr[l];
+            const uint4 b = row_clip(rt[l], nt);
+            unsigned br = 0, bt = 0;
+            for (unsigned x = 0; x < nr; ++x) {
+                const unsigned hit = row_find(b, a.x & 0xFFFFu);
+                br |= hit ? 1u << x : 0u;
+                bt |= hit;
+                a.x = a.x >> 16 | a.y << 16;   // the next slot
+                a.y = a.y >> 16 | a.z << 16;
+                a.z = a.z >> 16 | a.w << 16;
+                a.w >>= 16;
+            }
+            layers += br != 0;
+            if (l < 4) {
+                lo_r |= br << (8 * l);
+                lo_t |= bt << (8 * l);
+            } else {
+                hi_r = br;
+                hi_t = bt;
+            }
+        }
+        if (layers >= 3) {
+            atomicOr(&w.xm[r][0], lo_r);
+            atomicOr(&w.xm[r][1], hi_r);
+            atomicOr(&w.xm[t][0], lo_t);
+            atomicOr(&w.xm[t][1], hi_t);
+        }
+    }
+    __syncwarp();
+}
+
+// P2 of the event of roads r0 .. r0 + nr - 1 (nr <= P2W_ROADS) by one warp with
+// state `w`; lane i owns roads i and i + 32.  The same steps as p2_event:
+// coordinates present in two roads (bitmaps, a layer at a time), signatures of
+// those per road, pairs of roads whose signatures meet on >= 3 layers tested
+// exactly (a lane per pair).  Bound: latency of one warp's chain, so a layer's
+// rows are loaded while the layer before is worked on, and a layer's atomics
+// are in flight together.
 __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, unsigned long long &n_comb)
 {
     const unsigned lane = lane_id();
-    {
-        uint4 *z = reinterpret_cast<uint4 *>(&w.seen[0][0]);   // seen and multi
-        for (unsigned i = lane; i < 2 * N_LAYERS * 128 / 4; i += 32)
-            z[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    bool rep[2] = {false, false};
+    const uint4 *rows = reinterpret_cast<const uint4 *>(d.coords + (size_t)r0 * 40);
+    RoadRec rec[2];
+    uint4 q[2], next[2];
+    unsigned sx[2] = {0u, 0u}, sy[2] = {0u, 0u};   // the roads' signatures (sig_layers)
+    bool rep[2] = {false, false};                  // a coordinate repeated within a layer
 #pragma unroll
     for (unsigned h = 0; h < 2; ++h) {
-        const unsigned k = lane + 32 * h;
+        const unsigned k = min(32 * h + lane, nr - 1);   // a missing road reads the last one and has no hits
+        rec[h] = ldcg(d.roads + r0 + k);
+        next[h] = rows[k * N_LAYERS];
+    }
+    if (lane >= nr)
+        rec[0].pk = 0;
+    if (lane + 32 >= nr)
+        rec[1].pk = 0;
+    w.xm[lane][0] = w.xm[lane][1] = w.xm[lane + 32][0] = w.xm[lane + 32][1] = 0;
+    for (unsigned l = 0; l < N_LAYERS; ++l) {
+        reinterpret_cast<uint4 *>(w.seen)[lane] = make_uint4(0u, 0u, 0u, 0u);
+        reinterpret_cast<uint4 *>(w.multi)[lane] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
+        unsigned n[2];   // <= MAX_HITS
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h) {
+            q[h] = next[h];
+            n[h] = (rec[h].pk >> (4 * l)) & 15u;
+            if (l + 1 < N_LAYERS)
+                next[h] = rows[min(32 * h + lane, nr - 1) * N_LAYERS + l + 1];
+        }
+        const unsigned most = __reduce_max_sync(FULL_MASK, max(n[0], n[1]));
+        unsigned again[2];
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h)
+            again[h] = see_row(w.seen, q[h], n[h], most);
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h)
+            if (seen_again(w.multi, q[h], again[h]))
+                rep[h] = true;
+        __syncwarp();
+#pragma unroll
+        for (unsigned h = 0; h < 2; ++h) {
+            unsigned f = 0;
+            for (unsigned m = multi_row(w.multi, q[h], n[h], most); m; m &= m - 1)
+                f |= 1u << sig_bit10(row_at(q[h], __ffs(m) - 1));
+            if (l < 3)
+                sx[h] |= f << (10 * l);
+            else
+                sy[h] |= f << (10 * (l - 3));
+        }
+        __syncwarp();
+    }
+    // roads with shared coordinates on >= 3 layers, and their signatures
+    unsigned ne = 0;
+#pragma unroll
+    for (unsigned h = 0; h < 2; ++h) {
+        const bool e = sig_layers(sx[h], sy[h]) >= 3;
+        const unsigned m = __ballot_sync(FULL_MASK, e), at = ne + __popc(m & lanemask_lt());
+        if (e) {
+            w.elig[at] = (uint8_t)(32 * h + lane);
+            w.sig[at] = make_uint2(sx[h], sy[h]);
+        }
+        ne += __popc(m);
+    }
+    __syncwarp();
+    // pairs of them whose signatures meet on >= 3 layers
+    unsigned qn = 0;
+    for (unsigned b = 0; b + 1 < ne; b += 32) {
+        const unsigned i = b + lane, r = i < ne ? w.elig[i] : 0u;
+        const uint2 s = i < ne ? w.sig[i] : make_uint2(0u, 0u);
+        for (unsigned j = b + 1; j < ne; ++j) {
+            const unsigned t = w.elig[j];
+            const uint2 u = w.sig[j];
+            const bool hit = j > i && sig_layers(s.x & u.x, s.y & u.y) >= 3;
+            const unsigned m = __ballot_sync(FULL_MASK, hit);
+            if (!m)
+                continue;
+            if (hit)
+                w.pair[qn + __popc(m & lanemask_lt())] = r | t << 16;
+            qn += __popc(m);
+            __syncwarp();
+            if (qn >= 32) {
+                p2_pairs(d.coords, d.roads, w, r0, 32);
+                const unsigned rest = qn - 32, p = lane < rest ? w.pair[32 + lane] : 0u;
+                __syncwarp();
+                if (lane < rest)
+                    w.pair[lane] = p;
+                qn = rest;
+                __syncwarp();
+            }
+        }
+    }
+    if (qn)
+        p2_pairs(d.coords, d.roads, w, r0, qn);
+#pragma unroll
+    for (unsigned h = 0; h < 2; ++h) {
+        const unsigned k = 32 * h + lane;
         if (k < nr)
-            w.pk[k] = ldcg(&d.roads[r0 + k].pk);
-    }
-    __syncwarp();
-    // each distinct coordinate of a road's layer marks the bitmap once; a
-    // second road with it sets the multi bit
-#pragma unroll
-    for (unsigned h = 0; h < 2; ++h) {
-        const unsigned k = lane + 32 * h;
-        if (k >= nr)
-            continue;
-        const uint4 *row = reinterpret_cast<const uint4 *>(d.coords + (size_t)(r0 + k) * 40);
-        const uint32_t pk = w.pk[k];
-        for (unsigned l = 0; l < N_LAYERS; ++l) {
-            const unsigned n = (pk >> (4 * l)) & 15u;
-            const uint4 q = ldcg(row + l);
-#pragma unroll
-            for (unsigned x = 0; x < MAX_HITS; ++x) {
-                const unsigned v = row_coord(q, x);
-                bool first = x < n;
-#pragma unroll
-                for (unsigned y = 0; y < x; ++y)
-                    first = first && row_coord(q, y) != v;
-                if (first) {
-                    const unsigned bit = 1u << (v & 31u);
-                    if (atomicOr(&w.seen[l][v >> 5], bit) & bit)
-                        atomicOr(&w.multi[l][v >> 5], bit);
-                }
-                rep[h] = rep[h] || (x < n && !first);
-            }
-        }
-    }
-    __syncwarp();
-    // signatures of the shared coordinates
-    unsigned elig = 0;   // bit h: the lane's road h has shared coordinates on >= 3 layers
-#pragma unroll
-    for (unsigned h = 0; h < 2; ++h) {
-        const unsigned k = lane + 32 * h;
-        if (k >= nr)
-            continue;
-        const uint4 *row = reinterpret_cast<const uint4 *>(d.coords + (size_t)(r0 + k) * 40);
-        const uint32_t pk = w.pk[k];
-        unsigned layers = 0;
-        for (unsigned l = 0; l < N_LAYERS; ++l) {
-            const unsigned n = (pk >> (4 * l)) & 15u;
-            const uint4 q = ldcg(row + l);
-            uint32_t sl = 0;
-#pragma unroll
-            for (unsigned x = 0; x < MAX_HITS; ++x) {
-                const unsigned v = row_coord(q, x);
-                if (x < n && ((w.multi[l][v >> 5] >> (v & 31u)) & 1u))
-                    sl |= 1u << sig_bit32(v);
-            }
-            w.sig[k][l] = sl;
-            layers += sl != 0u;
-        }
-        elig |= layers >= 3 ? 1u << h : 0u;
-    }
-    __syncwarp();
-    // the other eligible roads t against the lane's eligible roads (their
-    // signatures meet on >= 3 layers first)
-    unsigned long long xm[2] = {0ull, 0ull};
-    unsigned long long em = ((unsigned long long)__ballot_sync(FULL_MASK, (elig >> 1) & 1u) << 32) |
-                            __ballot_sync(FULL_MASK, elig & 1u);
-    if (__popcll(em) >= 2) {
-        for (; em; em &= em - 1) {
-            const unsigned t = (unsigned)__ffsll((long long)em) - 1;
-#pragma unroll
-            for (unsigned h = 0; h < 2; ++h) {
-                const unsigned k = lane + 32 * h;
-                if (!((elig >> h) & 1u) || k == t)
-                    continue;
-                unsigned c = 0;
-#pragma unroll
-                for (unsigned l = 0; l < N_LAYERS; ++l)
-                    c += (w.sig[k][l] & w.sig[t][l]) != 0u;
-                if (c >= 3)
-                    xm[h] |= pair_marks(d, r0 + k, r0 + t, w.pk[k], w.pk[t]);
-            }
-        }
-    }
-#pragma unroll
-    for (unsigned h = 0; h < 2; ++h) {
-        const unsigned k = lane + 32 * h;
-        if (k < nr)
-            n_comb += finish_road(d, r0 + k, ldcg(d.roads + r0 + k), xm[h], rep[h]);
+            n_comb += finish_road(d, r0 + k, rec[h], ((unsigned long long)w.xm[k][1] << 32) | w.xm[k][0], rep[h]);
     }
     __syncwarp();   // the state is refilled for the next event
 }
 
-// P2 over the events.  A batch of at most P2_CTA_EVENTS events per CTA: a
-// CTA per event.  A larger one: first the events of more than P2W_ROADS
-// roads (listed in P1), a CTA each from a queue; then every warp takes the
-// other events from a second queue, one at a time (a warp takes longer over
-// an event than a CTA, but eight of them work at once).  One
-// combination-count atomic per CTA.
-constexpr unsigned P2_CTA_EVENTS = 4;
-
-__device__ void p2_phase(const Dev &d, unsigned char *smem)
+// P2 over the events.  At most one per CTA: a CTA each.  More: those of more
+// than P2W_ROADS roads (listed in P1) a CTA each from a queue, then every warp takes the other events one at a time, its
+// first by its own index (neighbouring indices on different SMs), the rest
+// from a queue.  One combination-count atomic per CTA.
+__device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
 {
-    if (ldcg(&d.ctrl->err_inv) != 0ull)
-        return;   // a data fault (every CTA reads the same word after the barrier): no tracks
-    const unsigned n_events = min(ldcg(&d.ctrl->n_events), d.max_events);
+    // what the stage reads first, in one trip
+    const unsigned n_events = bt.n_events, e0 = blockIdx.x;
+    const unsigned n_big_ev = min(ldcg(&d.ctrl->n_big_ev), n_events);
+    bt.n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
     // survivor totals of the road chunks start at zero (the fit adds to them)
-    const unsigned n_chunks = min((ldcg(&d.ctrl->n_roads) + ROAD_CHUNK - 1) / ROAD_CHUNK, d.max_chunks_r);
+    const unsigned n_chunks = min((bt.n_ep + ROAD_CHUNK - 1) / ROAD_CHUNK, d.max_chunks_r);
     for (unsigned i = blockIdx.x * BLOCK + threadIdx.x; i < n_chunks; i += gridDim.x * BLOCK)
         d.rchunk_sum[i] = 0;
     unsigned long long n_comb = 0;
-    if (n_events <= P2_CTA_EVENTS * gridDim.x) {
-        // few events for the grid: every event a CTA (the shortest time per
-        // event); the CTA's first event is its own index, the queue hands
-        // out the rest
-        for (unsigned e = blockIdx.x; e < n_events; e = grab_after_first(d, Q_P2)) {
-            const unsigned r0 = e == 0 ? 0u : min(ldcg(d.ev_road_end + e - 1), d.max_roads);
-            const unsigned r1 = min(ldcg(d.ev_road_end + e), d.max_roads);
-            p2_event(d, e, r0, min(r1 - min(r0, r1), (unsigned)MAX_ROADS_EV), smem, n_comb);
+    // first road and roads of event e (an event of more than MAX_ROADS_EV
+    // roads is a fault, reported in P1)
+    const auto roads_of = [&d](unsigned e, unsigned &r0) {
+        r0 = e == 0 ? 0u : min(ldcg(d.ev_road_end + e - 1), d.max_roads);
+        const unsigned r1 = min(ldcg(d.ev_road_end + e), d.max_roads);
+        return min(r1 - min(r0, r1), (unsigned)MAX_ROADS_EV);
+    };
+    if (n_events <= gridDim.x) {   // few: a CTA each is the shortest time per event
+        if (e0 < n_events) {
+            unsigned r0;
+            const unsigned nr = roads_of(e0, r0);
+            p2_event(d, e0, r0, nr, smem, n_comb);
         }
         n_comb = block_sum(n_comb);
         if (threadIdx.x == 0 && n_comb)
             atomicAdd(&d.ctrl->n_comb, n_comb);
         return;
     }
-    const unsigned n_big_ev = min(ldcg(&d.ctrl->n_big_ev), n_events);
-    for (unsigned i = blockIdx.x; i < n_big_ev; i = grab_after_first(d, Q_P2)) {
-        const unsigned e = min(ldcg(d.ev_big + i), n_events - 1);
-        const unsigned r0 = e == 0 ? 0u : min(ldcg(d.ev_road_end + e - 1), d.max_roads);
-        const unsigned r1 = min(ldcg(d.ev_road_end + e), d.max_roads);
-        // an event of more than MAX_ROADS_EV roads is a fault (reported in P1)
-        p2_event(d, e, r0, min(r1 - min(r0, r1), (unsigned)MAX_ROADS_EV), smem, n_comb);
+    if (n_big_ev) {
+        for (unsigned i = e0; i < n_big_ev; i = grab_after_first(d, Q_P2)) {
+            const unsigned e = min(ldcg(d.ev_big + i), n_events - 1);
+            unsigned r0;
+            const unsigned nr = roads_of(e, r0);
+            p2_event(d, e, r0, nr, smem, n_comb);
+        }
+        __syncthreads();   // the shared memory becomes the warps' regions
     }
-    __syncthreads();   // the shared memory becomes the warps' regions
     {
         P2Warp &w = *reinterpret_cast<P2Warp *>(smem + warp_id() * P2W_BYTES);
         const unsigned n_warps = gridDim.x * WARPS;
-        for (unsigned e = blockIdx.x * WARPS + warp_id(); e < n_events;) {
-            const unsigned r0 = e == 0 ? 0u : min(ldcg(d.ev_road_end + e - 1), d.max_roads);
-            const unsigned r1 = min(ldcg(d.ev_road_end + e), d.max_roads);
-            const unsigned nr = r1 - min(r0, r1);
-            if (nr <= (unsigned)P2W_ROADS)   // the others were listed
+        for (unsigned e = warp_id() * gridDim.x + blockIdx.x; e < n_events;) {
+            unsigned r0;
+            const unsigned nr = roads_of(e, r0);
+            if (nr && nr <= (unsigned)P2W_ROADS)   // the others were listed
                 p2_warp(d, r0, nr, w, n_comb);
+            if (n_events <= n_warps)
+                break;
             unsigned ne = 0;
             if (lane_id() == 0)
                 ne = n_warps + atomicAdd(&d.ctrl->q[Q_P2W], 1u);
@@ -1310,7 +1399,10 @@ __device__ void hash_min(const Dev &d, unsigned long long gk, unsigned long long
         unsigned long long prev = atomicCAS(&d.hash[h].key, 0ull, gk);
         if (prev == 0ull) {   // a new slot: marked for clearing (no value awaited)
             atomicOr(&d.hash_bits[h >> 5], 1u << (h & 31u));
-            if (atomicAdd(&d.ctrl->hash_used, 1u) >= slots - slots / 4)
+            const unsigned used = atomicAdd(&d.ctrl->hash_used, 1u);
+            if (used == 0)
+                raise_flag(d, FLAG_GROUPS);
+            if (used >= slots - slots / 4)
                 raise_flag(d, FLAG_CAPACITY);
         }
         if (prev == 0ull || prev == gk) {
@@ -2765,12 +2857,11 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, u
 // allocation of their own (inlined, the decode and the box path took 10 % and
 // 3 % longer).
 template <bool PLAIN>
-__device__ __noinline__ void p3_groups(const Dev &d, unsigned char *smem, unsigned long long &npass)
+__device__ __noinline__ void p3_groups(const Dev &d, unsigned char *smem, unsigned n_roads, unsigned long long &npass)
 {
     P3Slice &S = *reinterpret_cast<P3Slice *>(smem);
     P3Redo &R = *reinterpret_cast<P3Redo *>(smem + P3_REDO);
     const unsigned lane = lane_id();
-    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
     const unsigned lo = (unsigned)((unsigned long long)n_roads * blockIdx.x / gridDim.x);
     const unsigned hi = (unsigned)((unsigned long long)n_roads * (blockIdx.x + 1) / gridDim.x);
     const unsigned cl = max((unsigned)d.run_roads / 8, 1u);
@@ -2889,13 +2980,14 @@ __device__ __noinline__ void p3_groups(const Dev &d, unsigned char *smem, unsign
 // different SMs, the rest from a queue, which evens out the group path's
 // shares too).
 template <bool PLAIN>
-__device__ void p3_phase(const Dev &d, unsigned char *smem, int qbox)
+__device__ void p3_phase(const Dev &d, unsigned char *smem, unsigned n_roads, int qbox)
 {
     unsigned long long npass = 0;
-    p3_groups<PLAIN>(d, smem, npass);
+    const unsigned n_box = min(ldcg(&d.ctrl->n_box), d.max_roads);
+    p3_groups<PLAIN>(d, smem, n_roads, npass);
     __syncthreads();   // the shared memory becomes the warps' regions
     unsigned char *region = smem + warp_id() * P3_BOX_BYTES;
-    const unsigned n_warps = gridDim.x * WARPS, n_box = min(ldcg(&d.ctrl->n_box), d.max_roads);
+    const unsigned n_warps = gridDim.x * WARPS;
     for (unsigned i = warp_id() * gridDim.x + blockIdx.x; i < n_box;) {
         box_road<PLAIN>(d, region, min(ldcg(d.box_list + i), d.max_roads - 1), npass);
         if (n_box <= n_warps)
@@ -3121,9 +3213,8 @@ __device__ void p5_item(const Dev &d, unsigned c, unsigned n_roads, unsigned *s_
 // every candidate road checks its survivors at once; bit word w goes to CTA
 // w % grid, so that a few candidates are spread out.  A road that loses
 // survivors takes them off its chunk's total.
-__device__ void p4_cand_phase(const Dev &d)
+__device__ void p4_cand_phase(const Dev &d, unsigned n_roads)
 {
-    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
     const unsigned n_words = (n_roads + 31) / 32;
     const unsigned lane = lane_id();
     for (unsigned w = warp_id() * gridDim.x + blockIdx.x; w < n_words; w += gridDim.x * WARPS) {
@@ -3187,10 +3278,9 @@ __device__ __forceinline__ unsigned long long load_counts8(const Dev &d, unsigne
     return v;
 }
 
-__device__ void p5_phase(const Dev &d, unsigned char *smem)
+__device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads)
 {
     P5Smem &s = *reinterpret_cast<P5Smem *>(smem);
-    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads);
     const unsigned n_chunks = min((n_roads + ROAD_CHUNK - 1) / ROAD_CHUNK, d.max_chunks_r);
     // each thread sums a contiguous range of chunk totals
     const unsigned per = (n_chunks + BLOCK - 1) / BLOCK;
@@ -3325,37 +3415,44 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 2 : 768 / BLOCK) k_persi
         return;   // test hook: this CTA never arrives at the first barrier
     stamp(d, 0);
 
+    unsigned flags;
+    Batch bt;
     scan_count(d);
-    if (!grid_sync(d))
+    if (!grid_sync(d, 1, flags))
         return;
     stamp(d, 1);
-    if (!scan_decode(d, smem))
+    if (!scan_decode(d, smem, bt))
         return;
-    if (!grid_sync(d))
+    if (!grid_sync(d, 2, flags))
         return;
     stamp(d, 2);
-
-    p2_phase(d, smem);
-    if (!grid_sync(d))
+    const bool fault = flags & FLAG_FAULT;   // a fault of the stream: no tracks
+    if (!fault)
+        p2_phase(d, smem, bt);
+    if (!grid_sync(d, 3, flags))
         return;
     stamp(d, 3);
-    if (ldcg(&d.ctrl->err_inv) != 0ull)
-        return;   // a data fault: no tracks
+    if (fault)
+        return;
 
-    p3_phase<false>(d, smem, Q_BOX);
+    p3_phase<false>(d, smem, bt.n_roads, Q_BOX);
     if (d.skip_arrival == 2 && blockIdx.x == 0)
         return;   // test hook: this CTA leaves after publishing, the others' waits run out
-    if (!grid_sync(d))
+    if (!grid_sync(d, 4, flags))
         return;
     stamp(d, 4);
 
-    p4_cand_phase(d);
-    if (!grid_sync(d))
-        return;
+    const bool groups = flags & FLAG_GROUPS;   // no group published: nothing to look up or clear
+    if (groups) {
+        p4_cand_phase(d, bt.n_roads);
+        if (!grid_sync(d, 5, flags))
+            return;
+    }
     stamp(d, 5);
-    p5_phase(d, smem);
+    p5_phase(d, smem, bt.n_roads);
     // every lookup is done (barrier above): leave the group table empty
-    clear_hash(d);
+    if (groups)
+        clear_hash(d);
     if (threadIdx.x == 0)
         atomicMax(&d.ctrl->t_phase[6], globaltimer_ns());
 }
@@ -3370,20 +3467,22 @@ __global__ void __launch_bounds__(BLOCK) k_p0(Dev d) { scan_count(d); }
 __global__ void __launch_bounds__(BLOCK) k_p1(Dev d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    scan_decode(d, smem);
+    Batch bt;
+    scan_decode(d, smem, bt);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p2(Dev d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (ldcg(&d.ctrl->flags) & FLAG_CAPACITY)
+    if (ldcg(&d.ctrl->flags) & (FLAG_CAPACITY | FLAG_FAULT))
         return;
-    p2_phase(d, smem);
+    Batch bt{ldcg(&d.ctrl->n_events), ldcg(&d.ctrl->n_ep), 0u};
+    p2_phase(d, smem, bt);
 }
 
 __device__ __forceinline__ bool stop_after_unpack(const Dev &d)
 {
-    return ldcg(&d.ctrl->err_inv) != 0ull || (ldcg(&d.ctrl->flags) & FLAG_CAPACITY);
+    return ldcg(&d.ctrl->flags) & (FLAG_CAPACITY | FLAG_FAULT);
 }
 
 // combinations per road -> exclusive offsets (the "combine" stage)
@@ -3501,7 +3600,7 @@ __global__ void __launch_bounds__(BLOCK) k_warrior_plain(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem[];
     if (stop_after_unpack(d))
         return;
-    p3_phase<true>(d, smem, Q_BOX);
+    p3_phase<true>(d, smem, min(ldcg(&d.ctrl->n_roads), d.max_roads), Q_BOX);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p4(Dev d)

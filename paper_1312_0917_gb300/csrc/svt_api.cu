@@ -172,6 +172,7 @@ int svt_create(svt_ctx **out, int device, const svt_limits *lim)
         !dalloc(c, &d.span_seg, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.ev_road_end, L.max_events) && !dalloc(c, &d.ev_big, L.max_events) &&
         !dalloc(c, &d.roads, L.max_roads) && !dalloc(c, &d.coords, (size_t)L.max_roads * 40) &&
         !dalloc(c, &d.xmask, L.max_roads) && !dalloc(c, &d.box_list, L.max_roads) &&
+        !dalloc(c, &d.items, (size_t)N_GROUP_CLS * L.max_roads) &&
         !dalloc(c, &d.cand_bits, L.max_roads / 32 + 1) && !dalloc(c, &d.fitc, N_SETS * SET_INT4) &&
         !dalloc(c, &d.surv_pool, (size_t)L.max_roads * SURV_SLOTS) &&
         !dalloc(c, &d.surv_cnt, L.max_roads) &&

@@ -68,6 +68,7 @@ struct Ctrl {
     unsigned int n_big_ev;        // events of more than P2W_ROADS roads (list length)
     unsigned int hash_used;       // claimed slots of the group table
     unsigned int n_box;           // roads of the box path (list length)
+    unsigned int n_seg[10];       // roads of each half class of the group path (list lengths)
     unsigned int q[12];           // work-queue heads
     unsigned int done[4];         // last-block-done counters
     unsigned long long n_comb, n_pass, n_out;
@@ -92,6 +93,14 @@ struct RoadRec {
 // (4, 4), (8, 2), (8, 4) at most, then the box path, then no fit at all.
 constexpr int N_GROUP_CLS = 5, CLS_BOX = 5, CLS_NONE = 6;
 
+// A road as the group path lists it, 16 bytes: RoadRec::pk, the fitted slots by
+// falling hit count (perm, two bits each), and its index.
+struct alignas(16) RoadItem {
+    uint32_t g, pk;
+    int16_t curv, phi;
+    uint16_t set, perm;
+};
+
 // Cross-road group table slot: key = (event + 1, triple, three coordinates),
 // val_inv = ~(lowest track key of the group), 0 = empty.
 struct HashSlot {
@@ -115,6 +124,8 @@ struct Dev {
     uint16_t *coords;                                             // [max_roads][5][8]
     unsigned long long *xmask;                                    // [max_roads]
     uint32_t *box_list;                                           // [max_roads]
+    RoadItem *items;       // [N_GROUP_CLS][max_roads] group path, by class: roads of at most two hits
+                           // in slot e from the front, the others from the back
     int4 *fitc;            // [N_SETS][SET_INT4]: the constants as int32 in 16-byte words, written
                            // with the constants (fit_words); read-only in the kernels
     uint32_t *cand_bits;                                          // [max_roads / 32 + 1] cross-road

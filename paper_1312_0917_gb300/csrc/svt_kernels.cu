@@ -316,6 +316,38 @@ __device__ __forceinline__ unsigned grab_after_first(const Dev &d, int q)
     return gridDim.x + grab(d, q);
 }
 
+// A warp's items out of n for n_warps warps: three quarters are dealt out in
+// turn (warp wi: wi, wi + n_warps, ..), the rest, which evens the warps out,
+// `claim` at a time from queue head q.  (All from the queue, 40,000 claims of
+// one counter were 80 us: L2 takes about one atomic on an address in 2 ns.)
+struct Share {
+    unsigned n, n_warps, claim, dealt, left;   // items dealt out; of the last claim, still to do
+    unsigned *q;
+    __device__ Share(unsigned n_, unsigned n_warps_, unsigned claim_, unsigned *q_)
+        : n(n_), n_warps(n_warps_), claim(claim_),
+          dealt(n_ <= n_warps_ ? n_ : max(n_ / 4 * 3 / n_warps_, 1u) * n_warps_), left(0), q(q_)
+    {
+    }
+    __device__ unsigned first(unsigned wi) const { return wi < dealt ? wi : ~0u; }   // (dealt is 0 or covers a turn)
+    // the item after item i, or one past n
+    __device__ unsigned next(unsigned i)
+    {
+        if (i + n_warps < dealt)
+            return i + n_warps;
+        if (dealt >= n)
+            return ~0u;
+        if (i >= dealt && left) {
+            --left;
+            return i + 1;
+        }
+        unsigned c = 0;
+        if (lane_id() == 0)
+            c = atomicAdd(q, claim);
+        left = claim - 1;
+        return dealt + __shfl_sync(FULL_MASK, c, 0);
+    }
+};
+
 // Grid barrier number k (1, 2, ..) of the persistent kernel; `flags` gets
 // FLAG_* as they are once every CTA has arrived.  All CTAs are co-resident
 // (cooperative launch).  The wait is bounded by d.wait_ns; on expiry the CTA
@@ -374,7 +406,7 @@ __device__ __forceinline__ void stamp(const Dev &d, unsigned k)
 }
 
 // work-queue indices (Ctrl::q)
-enum { Q_P2 = 0, Q_BOX, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
+enum { Q_P2 = 0, Q_BOX, Q_GROUP, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
 
 // ---------------------------------------------------------------------------
 // P0 / P1: the word stream, one warp per span.  The stream is cut into
@@ -1002,32 +1034,132 @@ __device__ __forceinline__ unsigned road_class(uint32_t pk, unsigned N, unsigned
     return ma > 4 ? (mb > 2 ? 4u : 3u) : ma > 2 ? (mb > 2 ? 2u : 1u) : 0u;
 }
 
-// The end of P2 for road g (record r, flagged hits xm, rep: a coordinate
-// repeated within a layer): the record's candidate bit and fit path; a road of
-// the box path joins its list.  Returns the road's combinations.
-__device__ __forceinline__ unsigned finish_road(const Dev &d, unsigned g, RoadRec r, unsigned long long xm, bool rep)
+// The fit stage's lists.  A CTA gathers the group path's roads of its events
+// in shared memory and lists them at the end of the stage, sorted by class and
+// by the hits of the two smallest fitted slots (c, e), so that a warp's roads
+// loop alike: one atomic per half class and CTA.  (An atomic per class and
+// warp made 10,000 events wait 8 us on the counters; lists of each CTA's share
+// in its own shared memory, sorted at the start of the fit stage, left a third
+// of the warps idle at its end, since CTAs of equal shares take 56 to 79 us.)
+// Roads that find the list full are listed directly.
+constexpr unsigned P2_LIST = 3 * BLOCK;        // roads gathered at most
+constexpr unsigned P2_BUCKETS = 16 * N_GROUP_CLS;
+struct P2List {
+    RoadItem item[P2_LIST];                    // perm: bucket in the high byte
+    unsigned cnt[P2_BUCKETS];                  // roads of a bucket, then the first place of each in its half class
+    unsigned base[2 * N_GROUP_CLS];            // first place of the CTA's roads in each half class
+    unsigned n;
+};
+
+// where place i of half class seg lies (odd: at most two hits in slot e)
+__device__ __forceinline__ size_t list_at(const Dev &d, unsigned seg, unsigned i)
 {
+    return (size_t)(seg >> 1) * d.max_roads + ((seg & 1u) ? i : d.max_roads - 1 - i);
+}
+
+// Bucket of a road of class cls: half class (widest class first, then more
+// than two hits in slot e) in units of eight, then the hits of slots c and e,
+// most first.
+__device__ __forceinline__ unsigned road_bucket(uint32_t pk, unsigned perm, unsigned cls)
+{
+    const unsigned nf = fitted_counts(pk);
+    const unsigned mc = (nf >> (4 * ((perm >> 4) & 3u))) & 15u, me = (nf >> (4 * (perm >> 6))) & 15u;   // 1 .. 4
+    return 16 * (N_GROUP_CLS - 1 - cls) + (me > 2 ? 0u : 8u) + 2 * ((4 - mc) & 3u) + (me & 1u);
+}
+
+// The end of P2 for road g (record r, flagged hits xm, rep: a coordinate
+// repeated within a layer), one road per lane, by a whole warp (in: the lane
+// has a road): the record's candidate bit and fit path, and the road joins its
+// list.  Returns the road's combinations.
+__device__ __forceinline__ unsigned finish_road(const Dev &d, P2List &list, bool in, unsigned g, RoadRec r,
+                                                unsigned long long xm, bool rep)
+{
+    const unsigned lane = lane_id(), lt = lanemask_lt();
     const bool cand = xm != 0ull;
     unsigned N, N4, perm;
     road_sizes(r.pk, N, N4);
+    N = in ? N : 0u;
     const unsigned cls = road_class(r.pk, N, N4, (unsigned)d.small_n4, rep, perm);
     r.pk |= cand ? (1u << 23) : 0u;
     r.fit = (uint16_t)(perm | cls << 8 | (rep ? 1u << 11 : 0u));
-    d.roads[g] = r;
-    d.xmask[g] = xm;
-    d.surv_cnt[g] = 0;
-    if (cls == CLS_BOX) {
-        const unsigned i = atomicAdd(&d.ctrl->n_box, 1u);
-        if (i < d.max_roads)
-            d.box_list[i] = g;
+    if (in) {
+        d.roads[g] = r;
+        d.xmask[g] = xm;
+        d.surv_cnt[g] = 0;
+        if (N > 0 && cand)   // checked against the other roads' groups after the fit
+            atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
     }
-    if (N > 0 && cand)   // checked against the other roads' groups after the fit
-        atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
+    const unsigned mg = __ballot_sync(FULL_MASK, cls < N_GROUP_CLS), mb = __ballot_sync(FULL_MASK, cls == CLS_BOX);
+    unsigned at = 0;
+    if (lane == 0 && mg)
+        at = atomicAdd(&list.n, (unsigned)__popc(mg));
+    if (lane == 1 && mb)
+        at = atomicAdd(&d.ctrl->n_box, (unsigned)__popc(mb));
+    const unsigned gat = __shfl_sync(FULL_MASK, at, 0) + __popc(mg & lt);
+    const unsigned bat = __shfl_sync(FULL_MASK, at, 1) + __popc(mb & lt);
+    if (cls == CLS_BOX && bat < d.max_roads)
+        d.box_list[bat] = g;
+    if (cls < N_GROUP_CLS) {
+        const unsigned bucket = road_bucket(r.pk, perm, cls);
+        const RoadItem it{g, r.pk, r.curv, r.phi, r.set, (uint16_t)(perm | bucket << 8)};
+        if (gat < P2_LIST) {
+            list.item[gat] = it;
+        } else {
+            const unsigned i = atomicAdd(&d.ctrl->n_seg[bucket >> 3], 1u);
+            if (i < d.max_roads)
+                d.items[list_at(d, bucket >> 3, i)] = it;
+        }
+    }
     return N;
 }
 
-// Flags of event e (roads r0 .. r0 + nr - 1); adds its combinations to n_comb.
-__device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, unsigned char *smem,
+// The CTA's list goes out (every thread; the list is complete and `cnt` zero).
+__device__ void list_out(const Dev &d, P2List &list)
+{
+    constexpr unsigned EACH = (P2_LIST + BLOCK - 1) / BLOCK;
+    const unsigned lane = lane_id(), n = min(list.n, P2_LIST);
+    if (n == 0)
+        return;
+    unsigned place[EACH];
+#pragma unroll
+    for (unsigned k = 0; k < EACH; ++k) {
+        const unsigned i = k * BLOCK + threadIdx.x;
+        if (i < n)
+            place[k] = atomicAdd(&list.cnt[list.item[i].perm >> 8], 1u);
+    }
+    __syncthreads();
+    if (warp_id() == 0) {   // first places within each half class: eight buckets each
+        for (unsigned c = 0; c < P2_BUCKETS; c += 32) {
+            const unsigned b = c + lane;
+            const unsigned v = b < P2_BUCKETS ? list.cnt[b] : 0u;
+            unsigned inc = v;
+#pragma unroll
+            for (unsigned o = 1; o < 8; o <<= 1) {
+                const unsigned u = __shfl_up_sync(FULL_MASK, inc, o);
+                inc += (lane & 7u) >= o ? u : 0u;
+            }
+            if (b < P2_BUCKETS) {
+                list.cnt[b] = inc - v;
+                if ((lane & 7u) == 7 && inc)
+                    list.base[b >> 3] = atomicAdd(&d.ctrl->n_seg[b >> 3], inc);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (unsigned k = 0; k < EACH; ++k) {
+        const unsigned i = k * BLOCK + threadIdx.x;
+        if (i < n) {
+            const RoadItem it = list.item[i];
+            const unsigned b = it.perm >> 8, at = list.base[b >> 3] + list.cnt[b] + place[k];
+            if (at < d.max_roads)
+                d.items[list_at(d, b >> 3, at)] = it;
+        }
+    }
+}
+
+// Flags of the event of roads r0 .. r0 + nr - 1; adds its combinations to n_comb.
+__device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *smem, P2List &list,
                          unsigned long long &n_comb)
 {
     P2Smem &s = *reinterpret_cast<P2Smem *>(smem);
@@ -1105,8 +1237,11 @@ __device__ void p2_event(const Dev &d, unsigned e, unsigned r0, unsigned nr, uns
         pair_exact_warp(s, s.cp[k] & 0xFFFFu, s.cp[k] >> 16);
     __syncthreads();
     // the road records: candidate bit and fit path
-    for (unsigned k = threadIdx.x; k < nr; k += BLOCK)
-        n_comb += finish_road(d, r0 + k, s.rec[k], ((unsigned long long)s.xhi[k] << 32) | s.xlo[k], s.rep[k] != 0);
+    for (unsigned k0 = threadIdx.x - lane_id(); k0 < nr; k0 += BLOCK) {
+        const unsigned k = min(k0 + lane_id(), nr - 1);
+        n_comb += finish_road(d, list, k0 + lane_id() == k, r0 + k, s.rec[k],
+                              ((unsigned long long)s.xhi[k] << 32) | s.xlo[k], s.rep[k] != 0);
+    }
     __syncthreads();   // the shared arrays are refilled for the next event
 }
 
@@ -1186,7 +1321,7 @@ __device__ __noinline__ void p2_pairs(const uint16_t *coords, const RoadRec *roa
 // exactly (a lane per pair).  Bound: latency of one warp's chain, so a layer's
 // rows are loaded while the layer before is worked on, and a layer's atomics
 // are in flight together.
-__device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, unsigned long long &n_comb)
+__device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2List &list, unsigned long long &n_comb)
 {
     const unsigned lane = lane_id();
     const uint4 *rows = reinterpret_cast<const uint4 *>(d.coords + (size_t)r0 * 40);
@@ -1284,8 +1419,8 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, unsig
 #pragma unroll
     for (unsigned h = 0; h < 2; ++h) {
         const unsigned k = 32 * h + lane;
-        if (k < nr)
-            n_comb += finish_road(d, r0 + k, rec[h], ((unsigned long long)w.xm[k][1] << 32) | w.xm[k][0], rep[h]);
+        n_comb += finish_road(d, list, k < nr, r0 + k, rec[h], ((unsigned long long)w.xm[k][1] << 32) | w.xm[k][0],
+                              rep[h]);
     }
     __syncwarp();   // the state is refilled for the next event
 }
@@ -1294,6 +1429,17 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, unsig
 // than P2W_ROADS roads (listed in P1) a CTA each from a queue, then every warp takes the other events one at a time, its
 // first by its own index (neighbouring indices on different SMs), the rest
 // from a queue.  One combination-count atomic per CTA.
+constexpr size_t P2_LIST_AT = (sizeof(P2Smem) > WARPS * P2W_BYTES ? sizeof(P2Smem) : WARPS * P2W_BYTES) / 16 * 16 + 16;
+
+// The end of P2 in a CTA: its list goes out, its combinations are counted.
+__device__ void p2_finish(const Dev &d, P2List &list, unsigned long long n_comb)
+{
+    n_comb = block_sum(n_comb);   // and every road has joined the list
+    if (threadIdx.x == 0 && n_comb)
+        atomicAdd(&d.ctrl->n_comb, n_comb);
+    list_out(d, list);
+}
+
 __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
 {
     // what the stage reads first, in one trip
@@ -1305,6 +1451,12 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
     for (unsigned i = blockIdx.x * BLOCK + threadIdx.x; i < n_chunks; i += gridDim.x * BLOCK)
         d.rchunk_sum[i] = 0;
     unsigned long long n_comb = 0;
+    P2List &list = *reinterpret_cast<P2List *>(smem + P2_LIST_AT);
+    if (threadIdx.x == 0)
+        list.n = 0;
+    for (unsigned i = threadIdx.x; i < P2_BUCKETS; i += BLOCK)
+        list.cnt[i] = 0;
+    __syncthreads();
     // first road and roads of event e (an event of more than MAX_ROADS_EV
     // roads is a fault, reported in P1)
     const auto roads_of = [&d](unsigned e, unsigned &r0) {
@@ -1316,11 +1468,9 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
         if (e0 < n_events) {
             unsigned r0;
             const unsigned nr = roads_of(e0, r0);
-            p2_event(d, e0, r0, nr, smem, n_comb);
+            p2_event(d, r0, nr, smem, list, n_comb);
         }
-        n_comb = block_sum(n_comb);
-        if (threadIdx.x == 0 && n_comb)
-            atomicAdd(&d.ctrl->n_comb, n_comb);
+        p2_finish(d, list, n_comb);
         return;
     }
     if (n_big_ev) {
@@ -1328,7 +1478,7 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
             const unsigned e = min(ldcg(d.ev_big + i), n_events - 1);
             unsigned r0;
             const unsigned nr = roads_of(e, r0);
-            p2_event(d, e, r0, nr, smem, n_comb);
+            p2_event(d, r0, nr, smem, list, n_comb);
         }
         __syncthreads();   // the shared memory becomes the warps' regions
     }
@@ -1339,7 +1489,7 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
             unsigned r0;
             const unsigned nr = roads_of(e, r0);
             if (nr && nr <= (unsigned)P2W_ROADS)   // the others were listed
-                p2_warp(d, r0, nr, w, n_comb);
+                p2_warp(d, r0, nr, w, list, n_comb);
             if (n_events <= n_warps)
                 break;
             unsigned ne = 0;
@@ -1348,9 +1498,7 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
             e = __shfl_sync(FULL_MASK, ne, 0);
         }
     }
-    n_comb = block_sum(n_comb);
-    if (threadIdx.x == 0 && n_comb)
-        atomicAdd(&d.ctrl->n_comb, n_comb);
+    p2_finish(d, list, n_comb);
 }
 
 // ---------------------------------------------------------------------------
@@ -1495,14 +1643,6 @@ constexpr unsigned GROUP_HITS = 128;   // hits of a warp's roads at most (sixtee
 struct P3Group {
     int4 A[GROUP_HITS];   // a road's hits in role order: chi-square partial sums (x, y, z) and comb
                           // part (w); role a also carries curvature, phi, 4096 k and the road bits
-};
-
-// A road as a group reads it, 16 bytes in shared memory: RoadRec::pk, the
-// fitted slots by falling hit count (perm), and its index.
-struct alignas(16) RoadItem {
-    uint32_t g, pk;
-    int16_t curv, phi;
-    uint16_t set, perm;
 };
 
 // The shape of a class and one lane's view of its group's road.
@@ -1698,9 +1838,9 @@ constexpr unsigned TS = 9;
 
 // The float pass's partials by role (see box_float).
 struct P3Float {
-    float4 hit[4][8];      // (x, y, z): a quarter of the components' sums / 4096, the first role less 0.5
-    float2 c[8][4];        // role c again, each component twice
-    float ex[8], ey[8], ez[8];   // role e again, by component
+    float4 hit[4][8];            // (x, y, z): the components' partials / 4096, the first role's less 0.5
+    ulonglong2 c[8][2];          // role c again, each component as a pair of equals
+    ulonglong2 e[2][3];          // role e again, hits 4 i .. 4 i + 3 by component, in pairs
 };
 
 struct P3Box {
@@ -1936,17 +2076,18 @@ __device__ __forceinline__ unsigned box_tab(const BoxShape &sh, unsigned p, unsi
 // each) of numbers below 2^19.  So | |v| - |a| | <= sqrt(3) 0.62 < 1.075, and
 // the float c of |v|^2 is off by a relative 2.5e-7 at most.  Hence, for the
 // chi-squares X of two fits with floats c:
-//   X1 <= X2  =>  c1 <= float_thr(c2)           (near: not certainly larger)
+//   X1 <= X2  =>  c1 <= c2 + 4.3 sqrt(c2) + 4.7 and a little  (near: not certainly larger)
 //   X <= cut  =>  c <= float_hi,   X > cut  =>  c >= float_lo
 //
 // Lane (x, yl) holds hit x of slot a (eight) and hits yl, yl + 4 of slot b and
 // runs over the hits z and w of slots c and e.  The passing fits are those
-// below float_lo; a fit in [float_lo, float_hi] (one road in twenty) makes the
+// below float_lo; a fit in [float_lo, float_hi] (one road in thirty) makes the
 // warp count again in whole numbers.  A pair (x, y) is a candidate when its
 // lowest row is near the minima of tables (a, c) and (b, c) there, which are
-// shuffle minima; each candidate's fits that share two hits with it (about
-// 320) are then taken in float, and only if one is near the candidate without
-// being certainly lower do the whole keys of box_min2 decide.
+// shuffle minima (1.2 a road).  A candidate's lowest fit is chosen by whole
+// keys among those near the lowest; it survives when none of the fits that
+// share two hits with it (about 320) has a lower whole key, of which only the
+// near ones are made.
 //
 // Bound: issue slots, nine instructions per fit; in whole numbers (three
 // sums, floors and squares of 64 bits, 64-bit keys and minima) it took 48.
@@ -1956,26 +2097,38 @@ constexpr long long FLOAT_CUT = 1ll << 24;   // a smaller cut's band [lo, hi] is
 constexpr float FLOAT_PAD = 1e18f;           // component of a missing hit: its fits are far above every cut
 constexpr unsigned FLOAT_CANDS = 8;          // candidates the float pass follows up (more: the integer passes)
 
-// two floats, added and multiplied by one instruction each
-__device__ __forceinline__ float2 f2_add(float2 a, float2 b)
+// Two floats in one 64-bit register pair (kept packed from load to result:
+// packing at every operation cost more moves than the operations), added and
+// multiplied by one instruction each.
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 f2_pack(float x, float y)
 {
-    float2 r;
-    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; add.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
     return r;
 }
-__device__ __forceinline__ float2 f2_mul(float2 a, float2 b)
+__device__ __forceinline__ float2 f2_get(f2 a)
 {
     float2 r;
-    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mul.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
     return r;
 }
-__device__ __forceinline__ float2 f2_fma(float2 a, float2 b, float2 c)
+__device__ __forceinline__ f2 f2_add(f2 a, f2 b)
 {
-    float2 r;
-    asm("{ .reg .b64 x, y, z, w; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mov.b64 w, {%6, %7}; fma.rn.f32x2 z, x, y, w; mov.b64 {%0, %1}, z; }"
-        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b)
+{
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c)
+{
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
 __device__ __forceinline__ float sqrt_approx(float x)
@@ -1985,10 +2138,14 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return r;
 }
 
-// At least c2 + 4.3 sqrt(c2) + 4.7 and a little: what a fit not above c2 stays
-// below.  4.32 sqrt(c2) <= e c2 + 4.67 / e for every e; e = 9 / sqrt(cut) makes
-// that equal near 0.06 cut, where a road's minima lie (eps = 1.000002 + e, off =
-// 4.8 + 0.53 sqrt(cut)).
+// What a fit not above one of float c2 stays below ...
+__device__ __forceinline__ float float_near(float c2)
+{
+    return fmaf(c2, 1.000002f, fmaf(4.32f, sqrt_approx(c2), 4.8f));
+}
+// ... and a looser bound without a root, for the pass over the fits: 4.32
+// sqrt(c2) <= e c2 + 4.67 / e for every e; e = 5 / sqrt(cut) makes that equal
+// near 0.2 cut (eps = 1.000002 + e, off = 4.8 + 0.94 sqrt(cut)).
 #define float_thr(c2) fmaf((c2), eps, off)
 
 // float chi-square of a fit given by its four partials
@@ -1998,23 +2155,74 @@ __device__ __forceinline__ float float_chi(const float4 &a, const float4 &b, con
     return fmaf(z, z, fmaf(y, y, x * x));
 }
 
-// The hits z and w (z << 3 | w) of slots c and e of the pair (x, y)'s fit whose
-// comb bits are those of `low` (the fit exists: it is the pair's minimum).
-__device__ __forceinline__ unsigned box_arg(const P3Box &B, const BoxShape &sh, unsigned x, unsigned y, unsigned low)
+// One lane's view of a road's fits: passing ones (below the band from `lo`),
+// the lowest place in the band, and of each of its pairs the lowest row and
+// the lowest row near the minima of tables (a, c) and (b, c).
+struct FloatPass {
+    unsigned np, near_cut;
+    float q[2], qok[2];
+};
+
+// TWO: slot b has more than four hits (the lane's second y); WIDE: slot e has.
+template <bool TWO, bool WIDE>
+__device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, unsigned lo, float eps, float off)
 {
-    const unsigned base = (unsigned)(B.A[sh.ra][x].w + B.A[sh.rb][y].w);
-    const unsigned lane = lane_id();
-    unsigned hit = 0;
-    for (unsigned i = 0; i < 2; ++i) {
-        const unsigned z = (lane >> 3) + 4 * i, w = lane & 7u;
-        if (z < sh.mc && w < sh.me && ((base + (unsigned)(B.A[sh.rc][z].w + B.A[sh.re][w].w) - low) & 0x7FFFu) == 0)
-            hit = z << 3 | w;
+    constexpr unsigned NJ = TWO ? 2 : 1, NI = WIDE ? 2 : 1;
+    const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
+    FloatPass f{0u, ~0u, {3e38f, 3e38f}, {3e38f, 3e38f}};
+    f2 px[NJ], py[NJ], pz[NJ];
+#pragma unroll
+    for (unsigned j = 0; j < NJ; ++j) {
+        const float4 a = F.hit[0][x], b = F.hit[1][yl + 4 * j];
+        px[j] = f2_pack(a.x + b.x, a.x + b.x);
+        py[j] = f2_pack(a.y + b.y, a.y + b.y);
+        pz[j] = f2_pack(a.z + b.z, a.z + b.z);
     }
-    return __reduce_max_sync(FULL_MASK, hit);
+#pragma unroll 1
+    for (unsigned z = 0; z < mc; ++z) {
+        const ulonglong2 cxy = F.c[z][0];
+        const f2 cz = F.c[z][1].x;
+        float rz[NJ];
+#pragma unroll
+        for (unsigned i = 0; i < NI; ++i) {
+            const ulonglong2 ex = F.e[i][0], ey = F.e[i][1], ez = F.e[i][2];
+#pragma unroll
+            for (unsigned j = 0; j < NJ; ++j) {
+                const f2 zx = f2_add(px[j], cxy.x), zy = f2_add(py[j], cxy.y), zz = f2_add(pz[j], cz);
+#pragma unroll
+                for (unsigned h = 0; h < 2; ++h) {
+                    const f2 vx = f2_add(zx, h ? ex.y : ex.x), vy = f2_add(zy, h ? ey.y : ey.x),
+                             vz = f2_add(zz, h ? ez.y : ez.x);
+                    const float2 c = f2_get(f2_fma(vz, vz, f2_fma(vy, vy, f2_mul(vx, vx))));
+                    const unsigned d0 = __float_as_uint(c.x) - lo, d1 = __float_as_uint(c.y) - lo;
+                    f.np += d0 >> 31;
+                    f.np += d1 >> 31;
+                    f.near_cut = min(f.near_cut, min(d0, d1));
+                    rz[j] = i + h ? fminf(rz[j], fminf(c.x, c.y)) : fminf(c.x, c.y);
+                }
+            }
+        }
+        float ac = TWO ? fminf(rz[0], rz[NJ - 1]) : rz[0];   // (a, c) at x, z
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 8));
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 16));
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            float bc = rz[j];   // (b, c) at y, z
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 1));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 2));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 4));
+            f.q[j] = fminf(f.q[j], rz[j]);
+            f.qok[j] = rz[j] <= float_thr(fminf(ac, bc)) ? fminf(f.qok[j], rz[j]) : f.qok[j];
+        }
+    }
+    return f;
 }
 
-// Fit road g (record rec) with one warp; false when it is left to the integer
-// passes.  The shape's slots are roles here, by falling hit count.
+// Fit road g with one warp; false when it is left to the integer passes.  The
+// shape's slots are roles here, by falling hit count.  Hits that repeat a
+// coordinate need nothing special: the fits of the later hit are the earlier
+// one's with a higher comb, so they tie in float, lose in whole keys, and what
+// they drop or publish the earlier ones drop or publish too.
 __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
     P3Box &B = *reinterpret_cast<P3Box *>(region);
@@ -2022,8 +2230,6 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
     const unsigned lane = lane_id();
     const RoadRec rec = ldcg(d.roads + g);
     const uint32_t pk = rec.pk;
-    if (((pk >> 23) & 1u) || ((rec.fit >> 11) & 1u))   // publishes, or repeats a coordinate
-        return false;
     const unsigned excl = min((pk >> 20) & 7u, 4u), nf = fitted_counts(pk);
     BoxShape sh;
     sh.ra = 0;
@@ -2065,85 +2271,46 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
         }
         F.hit[role][k] = v;
         if (role == 2) {
-            F.c[k][0] = make_float2(v.x, v.x);
-            F.c[k][1] = make_float2(v.y, v.y);
-            F.c[k][2] = make_float2(v.z, v.z);
+            F.c[k][0] = ulonglong2{f2_pack(v.x, v.x), f2_pack(v.y, v.y)};
+            F.c[k][1].x = f2_pack(v.z, v.z);
         }
         if (role == 3) {
-            F.ex[k] = v.x;
-            F.ey[k] = v.y;
-            F.ez[k] = v.z;
+            float *e = reinterpret_cast<float *>(&F.e[k >> 2][0]) + (k & 3u);
+            e[0] = v.x;
+            e[4] = v.y;
+            e[8] = v.z;
         }
     }
     __syncwarp();
     // the cut's band
     const float cut = (float)min(d.cut, 1ll << 38), root = sqrt_approx(cut);
     const float band = fmaf(2.2f, root, 8.f);
-    const float eps = 1.000002f + 9.f / root, off = fmaf(0.53f, root, 4.8f);   // of float_thr
+    const float eps = 1.000002f + 5.f / root, off = fmaf(0.94f, root, 4.8f);   // of float_thr
     const float float_lo = cut * 0.999999f - band, float_hi = cut * 1.000001f + band;
     const unsigned lo = __float_as_uint(float_lo), width = __float_as_uint(float_hi) + 1 - lo;
 
     const unsigned x = lane & 7u, yl = lane >> 3;
-    float2 px[2], py[2], pz[2];
-#pragma unroll
-    for (unsigned j = 0; j < 2; ++j) {
-        const float4 a = F.hit[0][x], b = F.hit[1][yl + 4 * j];
-        px[j] = make_float2(a.x + b.x, a.x + b.x);
-        py[j] = make_float2(a.y + b.y, a.y + b.y);
-        pz[j] = make_float2(a.z + b.z, a.z + b.z);
-    }
-    unsigned np = 0, near_cut = ~0u;
-    float q[2] = {3e38f, 3e38f}, qok[2] = {3e38f, 3e38f};   // a pair's lowest row, and its lowest near one
-    const unsigned nw = (sh.me + 1) / 2, nj = sh.mb > 4 ? 2u : 1u;
-    for (unsigned z = 0; z < sh.mc; ++z) {
-        const float2 cx = F.c[z][0], cy = F.c[z][1], cz = F.c[z][2];
-        float rz[2] = {3e38f, 3e38f};
-#pragma unroll
-        for (unsigned j = 0; j < 2; ++j) {
-            if (j >= nj)
-                break;
-            const float2 zx = f2_add(px[j], cx), zy = f2_add(py[j], cy), zz = f2_add(pz[j], cz);
-#pragma unroll
-            for (unsigned h = 0; h < 4; ++h) {
-                if (h >= nw)
-                    break;
-                const float2 vx = f2_add(zx, *reinterpret_cast<const float2 *>(F.ex + 2 * h));
-                const float2 vy = f2_add(zy, *reinterpret_cast<const float2 *>(F.ey + 2 * h));
-                const float2 vz = f2_add(zz, *reinterpret_cast<const float2 *>(F.ez + 2 * h));
-                const float2 c = f2_fma(vz, vz, f2_fma(vy, vy, f2_mul(vx, vx)));
-                const unsigned d0 = __float_as_uint(c.x) - lo, d1 = __float_as_uint(c.y) - lo;
-                np += d0 >> 31;
-                np += d1 >> 31;
-                near_cut = min(near_cut, min(d0, d1));
-                rz[j] = fminf(rz[j], fminf(c.x, c.y));
-            }
-        }
-        float ac = fminf(rz[0], rz[1]);   // (a, c) at x, z
-        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 8));
-        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 16));
-#pragma unroll
-        for (unsigned j = 0; j < 2; ++j) {
-            if (j >= nj)
-                break;
-            float bc = rz[j];   // (b, c) at y, z
-            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 1));
-            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 2));
-            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 4));
-            q[j] = fminf(q[j], rz[j]);
-            qok[j] = rz[j] <= float_thr(fminf(ac, bc)) ? fminf(qok[j], rz[j]) : qok[j];
-        }
-    }
+    FloatPass f;
+    if (sh.mb > 4 && sh.me > 4)
+        f = float_pass<true, true>(F, sh.mc, lo, eps, off);
+    else if (sh.mb > 4)
+        f = float_pass<true, false>(F, sh.mc, lo, eps, off);
+    else if (sh.me > 4)
+        f = float_pass<false, true>(F, sh.mc, lo, eps, off);
+    else
+        f = float_pass<false, false>(F, sh.mc, lo, eps, off);
+    unsigned np = f.np;
     unsigned cand[2], n_cand = 0;
 #pragma unroll
     for (unsigned j = 0; j < 2; ++j) {
-        cand[j] = __ballot_sync(FULL_MASK, qok[j] <= float_thr(q[j]) && q[j] <= float_hi);
+        cand[j] = __ballot_sync(FULL_MASK, f.qok[j] <= float_thr(f.q[j]) && f.q[j] <= float_hi);
         n_cand += __popc(cand[j]);
     }
     if (n_cand > FLOAT_CANDS)
         return false;
-    if (__any_sync(FULL_MASK, near_cut < width)) {   // count in whole numbers
+    if (__any_sync(FULL_MASK, f.near_cut < width)) {   // count in whole numbers
         np = 0;
-        for (unsigned j = 0; j < nj; ++j) {
+        for (unsigned j = 0; j < 2; ++j) {
             const unsigned y = yl + 4 * j;
             if (x >= sh.ma || y >= sh.mb)
                 continue;
@@ -2168,60 +2335,58 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
         for (unsigned bits = cand[j]; bits; bits &= bits - 1) {
             const unsigned src = __ffs(bits) - 1, cx = src & 7u, cy = (src >> 3) + 4 * j;
             const float4 ha = F.hit[0][cx], hb = F.hit[1][cy];
-            // the pair's lowest fit
+            const auto key_of = [&](unsigned a, unsigned b, unsigned c, unsigned e) {
+                bool pass;
+                return box_key(add4(add4(B.A[0][a], B.A[1][b]), add4(B.A[2][c], B.A[3][e])), d.cut, pass);
+            };
+            // the pair's lowest fit: whole keys of the fits near the lowest float
             const float c0 = float_chi(ha, hb, F.hit[2][u], F.hit[3][v]);
             const float c1 = float_chi(ha, hb, F.hit[2][u + 4], F.hit[3][v]);
-            const float cf = __uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(fminf(c0, c1))));
-            const float thr = float_thr(cf);
-            const unsigned n0 = __ballot_sync(FULL_MASK, c0 <= thr), n1 = __ballot_sync(FULL_MASK, c1 <= thr);
-            unsigned cz, cw;
-            int verdict = -1;   // 1 survives, 0 dropped, -1 undecided
-            if (__popc(n0) + __popc(n1) == 1 && cf < float_lo) {
-                const unsigned at = __ffs(n0 | n1) - 1;
-                cz = (at >> 3) + (n0 ? 0u : 4u);
-                cw = at & 7u;
-                const float4 hc = F.hit[2][cz], he = F.hit[3][cw];
-                float m = 3e38f;   // the lowest other fit that shares two hits with it
+            float thr = float_near(__uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(fminf(c0, c1)))));
+            unsigned long long key = c0 <= thr ? key_of(cx, cy, u, v) : NO_KEY;
+            bool second = false;
+            if (c1 <= thr) {
+                const unsigned long long k1 = key_of(cx, cy, u + 4, v);
+                second = k1 < key;
+                key = umin64(key, k1);
+            }
+            const unsigned kh = __reduce_min_sync(FULL_MASK, (unsigned)(key >> 32));
+            const unsigned kl = __reduce_min_sync(FULL_MASK, (unsigned)(key >> 32) == kh ? (unsigned)key : ~0u);
+            const unsigned long long kf = ((unsigned long long)kh << 32) | kl;
+            if (kf == NO_KEY)
+                continue;   // no passing fit
+            const unsigned at = __ffs(__ballot_sync(FULL_MASK, key == kf)) - 1;   // (keys differ by comb)
+            const unsigned cz = (at >> 3) + (__shfl_sync(FULL_MASK, second, at) ? 4u : 0u), cw = at & 7u;
+            key = kf;
+            // the fits that share two hits with it, two of each of the other
+            // five tables per lane; bit 5 i + t of `near`: not certainly larger
+            const float4 hc = F.hit[2][cz], he = F.hit[3][cw];
+            thr = float_near(float_chi(ha, hb, hc, he));
+            unsigned near = 0;
 #pragma unroll
-                for (unsigned i = 0; i < 2; ++i) {
-                    const unsigned w = u + 4 * i;
-                    const float4 a = F.hit[0][w], b = F.hit[1][w], bv = F.hit[1][v], c = F.hit[2][w], e = F.hit[3][v];
-                    const float ac = float_chi(ha, b, hc, e), bc = float_chi(a, hb, hc, e);
-                    const float ae = float_chi(ha, bv, c, he), be = float_chi(F.hit[0][v], hb, c, he);
-                    const float ce = float_chi(a, bv, hc, he);
-                    m = fminf(m, w == cy && v == cw ? 3e38f : ac);
-                    m = fminf(m, w == cx && v == cw ? 3e38f : bc);
-                    m = fminf(m, v == cy && w == cz ? 3e38f : ae);
-                    m = fminf(m, v == cx && w == cz ? 3e38f : be);
-                    m = fminf(m, w == cx && v == cy ? 3e38f : ce);
-                }
-                m = __uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(m)));
-                verdict = m > thr ? 1 : float_thr(m) < cf ? 0 : -1;
+            for (unsigned i = 0; i < 2; ++i) {
+                const unsigned w = u + 4 * i;
+                const float4 a = F.hit[0][w], b = F.hit[1][w], bv = F.hit[1][v], c = F.hit[2][w], e = F.hit[3][v];
+                near |= (float_chi(ha, b, hc, e) <= thr && !(w == cy && v == cw)) ? 1u << (5 * i) : 0u;
+                near |= (float_chi(a, hb, hc, e) <= thr && !(w == cx && v == cw)) ? 2u << (5 * i) : 0u;
+                near |= (float_chi(ha, bv, c, he) <= thr && !(v == cy && w == cz)) ? 4u << (5 * i) : 0u;
+                near |= (float_chi(F.hit[0][v], hb, c, he) <= thr && !(v == cx && w == cz)) ? 8u << (5 * i) : 0u;
+                near |= (float_chi(a, bv, hc, he) <= thr && !(w == cx && v == cy)) ? 16u << (5 * i) : 0u;
             }
-            unsigned long long key = NO_KEY;
-            if (verdict == 1) {
-                bool pass;
-                key = box_key(add4(add4(B.A[sh.ra][cx], B.A[sh.rb][cy]), add4(B.A[sh.rc][cz], B.A[sh.re][cw])), d.cut,
-                              pass);
-            } else if (verdict < 0) {   // whole keys: the pair's minimum against the other five tables
-                key = box_min2<false>(d, B, sh, sh.ra, cx, sh.rb, cy);
-                if (key != NO_KEY) {
-                    const unsigned t = box_arg(B, sh, cx, cy, (unsigned)key);
-                    cz = t >> 3;
-                    cw = t & 7u;
-                    bool ok = box_min2<false>(d, B, sh, sh.ra, cx, sh.rc, cz) == key;
-                    ok = ok && box_min2<false>(d, B, sh, sh.rb, cy, sh.rc, cz) == key;
-                    ok = ok && box_min2<false>(d, B, sh, sh.ra, cx, sh.re, cw) == key;
-                    ok = ok && box_min2<false>(d, B, sh, sh.rb, cy, sh.re, cw) == key;
-                    ok = ok && box_tce<false>(d, B, sh, cz, cw) == key;
-                    key = ok ? key : NO_KEY;
+            bool kill = false;
+            while (__any_sync(FULL_MASK, near != 0u)) {   // in whole keys, one per lane at a time
+                if (near) {
+                    const unsigned q = __ffs(near) - 1, t = q < 5 ? q : q - 5, w = u + (q < 5 ? 0u : 4u);
+                    kill = kill || key_of(t == 0 || t == 2 ? cx : t == 3 ? v : w, t == 1 || t == 3 ? cy : t == 0 ? w : v,
+                                          t == 2 || t == 3 ? w : cz, t < 2 ? v : cw) < kf;
+                    near &= near - 1;
                 }
             }
-            if (key != NO_KEY) {
-                if (lane == n_surv)
-                    mine = key;
-                ++n_surv;
-            }
+            if (__any_sync(FULL_MASK, kill))
+                continue;
+            if (lane == n_surv)
+                mine = key;
+            ++n_surv;
         }
     // in comb order
     unsigned rank = 0;
@@ -2233,6 +2398,15 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
         d.surv_cnt[g] = (uint8_t)n_surv;
         if (n_surv)
             atomicAdd(&d.rchunk_sum[g / ROAD_CHUNK], n_surv);
+    }
+    if ((pk >> 23) & 1u) {   // a cross-road candidate: its hits lie as a group's of this shape would
+        GroupRoad<3, 2, 2, 8> r;
+        r.it = RoadItem{g, pk, rec.curv, rec.phi, rec.set, (uint16_t)(rec.fit & 0xFFu)};
+        r.hit = &B.A[0][0];
+        r.nf = nf;
+        r.excl = excl;
+        r.cb = 0;
+        group_publish<false>(d, r, true);
     }
     __syncwarp();
     return true;
@@ -2571,35 +2745,24 @@ __device__ __forceinline__ void box_road(const Dev &d, unsigned char *region, un
         box_integer<PLAIN>(d, region, g, npass);
 }
 
-constexpr size_t P3_BOX_BYTES = (sizeof(P3Box) + 15) / 16 * 16;   // a warp's region of the box path
 
-// The group path's shared memory: a slice of the roads, sorted.
-constexpr unsigned P3_ROADS = 2 * BLOCK;      // roads of a slice at most
-constexpr unsigned P3_BUCKETS = 16 * N_GROUP_CLS;
-struct P3Slice {
-    P3Group warp[WARPS];
-    RoadItem item[P3_ROADS];
-    unsigned n[P3_BUCKETS];                      // roads of each bucket, then its first place
-    unsigned end[2 * N_GROUP_CLS];               // place after each half class's last road
-    unsigned csum[P3_ROADS / ROAD_CHUNK + 2];    // survivors of the slice's road chunks
-    unsigned q;                                  // steps handed out
-    unsigned g0, sh;                             // first road; the shift of the 32-bit words
-    // what every step reads of the kernel's argument (a load through its
-    // address takes an L1 miss)
+// Shared memory of P3: what every step reads of the kernel's argument (a load
+// through the argument's address takes an L1 miss), then a region per warp, a
+// group step's hits or a box road.
+struct P3Shared {
     const uint16_t *coords;
     const int4 *fitc;
     unsigned long long *surv_pool;
     uint8_t *surv_cnt;
+    uint32_t *rchunk_sum;
     long long cut;
     size_t max_roads;
+    unsigned sh;                       // the shift of the 32-bit words
+    unsigned n[2 * N_GROUP_CLS];       // roads of each half class
+    unsigned end[2 * N_GROUP_CLS];     // steps up to and with each half class
 };
-static_assert(offsetof(P3Slice, item) % 16 == 0, "16-byte items");
-// the slice's roads left to the box path, after the warps' regions of that path
-struct P3Redo {
-    uint16_t road[P3_ROADS];
-    unsigned n;
-};
-constexpr size_t P3_REDO = WARPS * P3_BOX_BYTES > sizeof(P3Slice) ? WARPS * P3_BOX_BYTES : (sizeof(P3Slice) + 15) / 16 * 16;
+constexpr size_t P3_SHARED_BYTES = (sizeof(P3Shared) + 15) / 16 * 16;
+constexpr size_t P3_WARP_BYTES = ((sizeof(P3Box) > sizeof(P3Group) ? sizeof(P3Box) : sizeof(P3Group)) + 15) / 16 * 16;
 
 // The classes' shapes (lanes of slot a, of slot b, hits of b per lane, hits of
 // e).  Most roads of classes 2 and 4 have two hits at most in slot e: they
@@ -2612,23 +2775,28 @@ using GroupCls3 = GroupRoad<3, 0, 2, 2>;    // (8, 2): 4
 using GroupCls4 = GroupRoad<3, 1, 2, 2>;    // (8, 4): 2
 using GroupCls4e = GroupRoad<3, 1, 2, 4>;
 
-// Fit the roads first .. first + ROADS - 1 of the slice's list (below n) with
-// one warp; returns the lane's passing combinations.  Not inlined: a register
+// Fit roads first .. first + ROADS - 1 of a list of n (from the end of
+// the class's array when `back`) with one warp; adds the lane's passing
+// combinations to np.  Returns the roads with a tie, bit by lane of their
+// groups' first lanes, which are left to the box path.  Not inlined: a register
 // allocation per class (in one function the five classes spilled 220 bytes).
 template <bool PLAIN, class Road>
-__device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, unsigned first, unsigned n)
+__device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, const RoadItem *list, int step,
+                                            unsigned left, unsigned &npass)
 {
-    P3Slice &S = *reinterpret_cast<P3Slice *>(smem);
-    const unsigned sh = S.sh, g0 = S.g0;
+    const P3Shared &S = *reinterpret_cast<const P3Shared *>(smem);
+    const unsigned sh = S.sh;
     constexpr unsigned A = Road::A, YL = Road::YL, YN = Road::YN, B = Road::B, W = Road::W, G = Road::G,
                        HITS = Road::HITS;
     const unsigned lane = lane_id(), gl = lane % G, gi = lane / G;
     const unsigned gmask = G == 32 ? FULL_MASK : ((1u << (G & 31u)) - 1u) << (gi * G);
     Road r;
-    const bool on = first + gi < n;
+    const bool on = gi < left;
     r.it = RoadItem{};
-    if (on)
-        r.it = S.item[first + gi];
+    if (on) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(list + step * (int)gi));
+        memcpy(&r.it, &v, sizeof v);
+    }
     const uint32_t pk = r.it.pk;
     const size_t g = r.it.g;
     r.excl = min((pk >> 20) & 7u, 4u);
@@ -2640,7 +2808,7 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, u
     r.yl = gl / A;
     r.live = r.x < r.m(r.slot(0));
     r.cb = PLAIN && on ? ldcg(d.comb_off + g) : 0ull;
-    int4 *hit = S.warp[warp_id()].A + gi * HITS;
+    int4 *hit = reinterpret_cast<P3Group *>(smem + P3_SHARED_BYTES + warp_id() * P3_WARP_BYTES)->A + gi * HITS;
     r.hit = hit;
     __syncwarp();   // the table's previous readers are done
     {
@@ -2828,176 +2996,122 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, u
     for (unsigned j = 0; j < YN; ++j)
         if (f.surv[j])
             S.surv_pool[f.rank[j] * S.max_roads + g] = f.key[j];
-    if (on && gl == 0) {
-        if (tied) {
-            P3Redo &R = *reinterpret_cast<P3Redo *>(smem + P3_REDO);
-            R.road[atomicAdd(&R.n, 1u)] = (uint16_t)(g - g0);
-        } else {
-            S.surv_cnt[g] = (uint8_t)f.cnt;
-            if (f.cnt)
-                atomicAdd(&S.csum[g / ROAD_CHUNK - g0 / ROAD_CHUNK], f.cnt);
-        }
+    if (on && gl == 0 && !tied) {
+        S.surv_cnt[g] = (uint8_t)f.cnt;
+        if (f.cnt)
+            atomicAdd(&S.rchunk_sum[g / ROAD_CHUNK], f.cnt);
     }
-    np = tied ? 0u : np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
+    npass += tied ? 0u : np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
     const bool publish = ((pk >> 23) & 1u) && !tied;
     if (__any_sync(FULL_MASK, publish)) {   // on a copy, so that the road stays in registers
         const Road rc = r;
         group_publish<PLAIN>(d, rc, publish);
     }
-    return np;
+    __syncwarp();   // (the warp's memory may be the box path's next)
+    return __ballot_sync(FULL_MASK, tied && gl == 0);
 }
 
-// The group path: every CTA takes an equal share of the roads, P3_ROADS at
-// most at a time, and sorts them in shared memory by class, widest first, and
-// by the hits of slots c and e, so that a warp's roads loop alike.  (Lists of
-// the whole batch in device memory, with an atomic per class and warp, made
-// the flag stage of 10,000 events wait 8 us on the counters.)  A step is one
-// warp's roads of one class; the warps claim the steps from a queue in shared
-// memory.  Not inlined: the stages before and after it keep a register
-// allocation of their own (inlined, the decode and the box path took 10 % and
-// 3 % longer).
-template <bool PLAIN>
-__device__ __noinline__ void p3_groups(const Dev &d, unsigned char *smem, unsigned n_roads, unsigned long long &npass)
+// Step s (of the sequence over all half classes) if it is of half class SEG,
+// and then its roads with ties.
+template <bool PLAIN, class Road, unsigned SEG>
+__device__ __forceinline__ void group_step(const Dev &d, unsigned char *smem, unsigned s, unsigned &np,
+                                           unsigned long long &npass)
 {
-    P3Slice &S = *reinterpret_cast<P3Slice *>(smem);
-    P3Redo &R = *reinterpret_cast<P3Redo *>(smem + P3_REDO);
-    const unsigned lane = lane_id();
-    const unsigned lo = (unsigned)((unsigned long long)n_roads * blockIdx.x / gridDim.x);
-    const unsigned hi = (unsigned)((unsigned long long)n_roads * (blockIdx.x + 1) / gridDim.x);
-    const unsigned cl = max((unsigned)d.run_roads / 8, 1u);
-    const unsigned parts = (hi - lo + P3_ROADS - 1) / P3_ROADS;
-    unsigned long long np = 0;
-    for (unsigned part = 0; part < parts; ++part) {
-        const unsigned g0 = lo + (unsigned)((unsigned long long)(hi - lo) * part / parts);
-        const unsigned g1 = lo + (unsigned)((unsigned long long)(hi - lo) * (part + 1) / parts);
-        // counting sort, two roads per thread
-        for (unsigned i = threadIdx.x; i < P3_BUCKETS; i += BLOCK)
-            S.n[i] = 0;
-        if (threadIdx.x < P3_ROADS / ROAD_CHUNK + 2)
-            S.csum[threadIdx.x] = 0;
-        if (threadIdx.x == 0) {
-            S.q = R.n = 0;
-            S.g0 = g0;
+    const P3Shared &S = *reinterpret_cast<const P3Shared *>(smem);
+    const unsigned first = (s - (SEG ? S.end[SEG - 1] : 0u)) * Road::ROADS;
+    const RoadItem *list = d.items + list_at(d, SEG, first);
+    constexpr int dir = (SEG & 1u) ? 1 : -1;
+    for (unsigned tied = group_item<PLAIN, Road>(d, smem, list, dir, S.n[SEG] - first, np); tied; tied &= tied - 1) {
+        const unsigned gi = (__ffs(tied) - 1) / Road::G;
+        box_road<PLAIN>(d, smem + P3_SHARED_BYTES + warp_id() * P3_WARP_BYTES, ldcg(&list[dir * (int)gi].g), npass);
+    }
+}
+
+// The roads of the box path (n_box of them), one warp each.
+template <bool PLAIN>
+__device__ __noinline__ void p3_boxes(const Dev &d, unsigned char *smem, unsigned n_box, int qbox,
+                                      unsigned long long &npass)
+{
+    const unsigned n_warps = gridDim.x * WARPS, wi = warp_id() * gridDim.x + blockIdx.x;
+    Share w(n_box, n_warps, 1, &d.ctrl->q[qbox]);
+    unsigned i = w.first(wi), g = i < n_box ? ldcg(d.box_list + i) : 0u;
+    while (i < n_box) {   // the next road is claimed and looked up ahead
+        const unsigned ni = w.next(i), ng = ni < n_box ? ldcg(d.box_list + ni) : 0u;
+        box_road<PLAIN>(d, smem + P3_SHARED_BYTES + warp_id() * P3_WARP_BYTES, min(g, d.max_roads - 1), npass);
+        i = ni;
+        g = ng;
+    }
+}
+
+// P3: the roads listed in P2, the group path's first: a step is one warp's roads
+// of one half class, widest first (neighbouring warp indices lie on different
+// SMs); then those of the box path, one warp each, whose queue evens out the
+// warps' first steps of a class (its code comes from L2 once per SM: 16 k
+// cycles against 8 k later).  Each warp works in its own region of shared
+// memory, so no part of P3 waits for the whole CTA.  Not inlined: the stages
+// before and after it keep a register allocation of their own (inlined, the
+// decode and the box path took 10 % and 3 % longer).
+template <bool PLAIN>
+__device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbox, int qgroup)
+{
+    P3Shared &S = *reinterpret_cast<P3Shared *>(smem);
+    unsigned long long npass = 0;
+    const unsigned n_box = min(ldcg(&d.ctrl->n_box), d.max_roads);
+    if (warp_id() == 0) {
+        const unsigned lane = lane_id();
+        // roads per step of the half classes: 2, 2, -, 4, 4, 4, -, 8, -, 16
+        static_assert(GroupCls4e::ROADS == 2 && GroupCls4::ROADS == 2 && GroupCls3::ROADS == 4 &&
+                          GroupCls2e::ROADS == 4 && GroupCls2::ROADS == 4 && GroupCls1::ROADS == 8 &&
+                          GroupCls0::ROADS == 16, "roads per step");
+        const unsigned per = lane < 2 ? 2u : lane < 6 ? 4u : lane < 8 ? 8u : 16u;
+        const unsigned n = lane < 2 * N_GROUP_CLS ? min(ldcg(&d.ctrl->n_seg[lane]), d.max_roads) : 0u;
+        unsigned inc = (n + per - 1) / per;
+#pragma unroll
+        for (unsigned o = 1; o < 16; o <<= 1) {
+            const unsigned u = __shfl_up_sync(FULL_MASK, inc, o);
+            inc += lane >= o ? u : 0u;
+        }
+        if (lane < 2 * N_GROUP_CLS) {
+            S.n[lane] = n;
+            S.end[lane] = inc;
+        }
+        if (lane == 0) {
             S.coords = d.coords;
             S.fitc = d.fitc;
             S.surv_pool = d.surv_pool;
             S.surv_cnt = d.surv_cnt;
+            S.rchunk_sum = d.rchunk_sum;
             S.cut = d.cut;
             S.max_roads = d.max_roads;
             // the shift that brings the cut below 2^31 (a chi-square is below 2^38)
             const unsigned long long cut = min((unsigned long long)max(d.cut, 0ll), (1ull << 38) - 1);
             S.sh = cut >> 31 ? 33 - __clzll((long long)cut) : 0u;
         }
-        __syncthreads();
-        RoadItem it[2];
-        unsigned bucket[2], place[2];
-#pragma unroll
-        for (unsigned h = 0; h < 2; ++h) {
-            const unsigned g = g0 + h * BLOCK + threadIdx.x;
-            bucket[h] = P3_BUCKETS;
-            if (g < g1) {
-                const RoadRec r = ldcg(d.roads + g);
-                const unsigned perm = r.fit & 0xFFu, cls = (r.fit >> 8) & 7u;
-                it[h] = RoadItem{g, r.pk, r.curv, r.phi, r.set, (uint16_t)perm};
-                if (cls < N_GROUP_CLS) {   // a fitted road has 1 .. 4 hits in slots c and e
-                    const unsigned nf = fitted_counts(r.pk);
-                    const unsigned mc = (nf >> (4 * ((perm >> 4) & 3u))) & 15u, me = (nf >> (4 * (perm >> 6))) & 15u;
-                    bucket[h] = 16 * (N_GROUP_CLS - 1 - cls) + (me > 2 ? 0u : 8u) + 2 * ((4 - mc) & 3u) + (me & 1u);
-                    place[h] = atomicAdd(&S.n[bucket[h]], 1u);
-                }
-            }
-        }
-        __syncthreads();
-        if (warp_id() == 0) {   // first places: an exclusive scan of the counts, class by class
-            unsigned run = 0;
-#pragma unroll
-            for (unsigned c = 0; c < N_GROUP_CLS; ++c) {
-                const unsigned v = lane < 16 ? S.n[16 * c + lane] : 0u;
-                unsigned inc = v;
-#pragma unroll
-                for (unsigned o = 1; o < 16; o <<= 1) {
-                    const unsigned u = __shfl_up_sync(FULL_MASK, inc, o);
-                    inc += lane >= o ? u : 0u;
-                }
-                if (lane < 16)
-                    S.n[16 * c + lane] = run + inc - v;
-                if (lane == 7 || lane == 15)
-                    S.end[2 * c + (lane >> 3)] = run + inc;
-                run += __shfl_sync(FULL_MASK, inc, 15);
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (unsigned h = 0; h < 2; ++h)
-            if (bucket[h] < P3_BUCKETS)
-                S.item[S.n[bucket[h]] + place[h]] = it[h];
-        __syncthreads();
-        // steps of the classes 4, 3, .. 0
-        const auto steps = [&](unsigned i, unsigned roads) {
-            return (S.end[i] - (i ? S.end[i - 1] : 0u) + roads - 1) / roads;
-        };
-        const unsigned e4e = steps(0, GroupCls4e::ROADS), e4 = e4e + steps(1, GroupCls4::ROADS),
-                       e3 = e4 + steps(3, GroupCls3::ROADS), e2e = e3 + steps(4, GroupCls2e::ROADS),
-                       e2 = e2e + steps(5, GroupCls2::ROADS), e1 = e2 + steps(7, GroupCls1::ROADS),
-                       e0 = e1 + steps(9, GroupCls0::ROADS);
-        for (;;) {
-            unsigned s0 = 0;
-            if (lane == 0)
-                s0 = atomicAdd(&S.q, cl);
-            s0 = __shfl_sync(FULL_MASK, s0, 0);
-            if (s0 >= e0)
-                break;
-            for (unsigned s = s0; s < min(s0 + cl, e0); ++s) {
-                if (s < e4e)
-                    np += group_item<PLAIN, GroupCls4e>(d, smem, s * GroupCls4e::ROADS, S.end[0]);
-                else if (s < e4)
-                    np += group_item<PLAIN, GroupCls4>(d, smem, S.end[0] + (s - e4e) * GroupCls4::ROADS, S.end[1]);
-                else if (s < e3)
-                    np += group_item<PLAIN, GroupCls3>(d, smem, S.end[2] + (s - e4) * GroupCls3::ROADS, S.end[3]);
-                else if (s < e2e)
-                    np += group_item<PLAIN, GroupCls2e>(d, smem, S.end[3] + (s - e3) * GroupCls2e::ROADS, S.end[4]);
-                else if (s < e2)
-                    np += group_item<PLAIN, GroupCls2>(d, smem, S.end[4] + (s - e2e) * GroupCls2::ROADS, S.end[5]);
-                else if (s < e1)
-                    np += group_item<PLAIN, GroupCls1>(d, smem, S.end[6] + (s - e2) * GroupCls1::ROADS, S.end[7]);
-                else
-                    np += group_item<PLAIN, GroupCls0>(d, smem, S.end[8] + (s - e1) * GroupCls0::ROADS, S.end[9]);
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < P3_ROADS / ROAD_CHUNK + 2 && S.csum[threadIdx.x])
-            atomicAdd(&d.rchunk_sum[g0 / ROAD_CHUNK + threadIdx.x], S.csum[threadIdx.x]);
-        __syncthreads();   // the slice's memory becomes the warps' regions, then is refilled
-        for (unsigned i = warp_id(); i < R.n; i += WARPS)
-            box_road<PLAIN>(d, smem + warp_id() * P3_BOX_BYTES, g0 + R.road[i], np);
-        __syncthreads();
     }
-    npass += np;
-}
-
-// P3: the group path's roads, then the roads listed in P2 for the box path
-// (one warp each, a warp's first by its own index, neighbouring indices on
-// different SMs, the rest from a queue, which evens out the group path's
-// shares too).
-template <bool PLAIN>
-__device__ void p3_phase(const Dev &d, unsigned char *smem, unsigned n_roads, int qbox)
-{
-    unsigned long long npass = 0;
-    const unsigned n_box = min(ldcg(&d.ctrl->n_box), d.max_roads);
-    p3_groups<PLAIN>(d, smem, n_roads, npass);
-    __syncthreads();   // the shared memory becomes the warps' regions
-    unsigned char *region = smem + warp_id() * P3_BOX_BYTES;
-    const unsigned n_warps = gridDim.x * WARPS;
-    for (unsigned i = warp_id() * gridDim.x + blockIdx.x; i < n_box;) {
-        box_road<PLAIN>(d, region, min(ldcg(d.box_list + i), d.max_roads - 1), npass);
-        if (n_box <= n_warps)
-            break;
-        unsigned ni = 0;
-        if (lane_id() == 0)
-            ni = n_warps + atomicAdd(&d.ctrl->q[qbox], 1u);
-        i = __shfl_sync(FULL_MASK, ni, 0);
+    __syncthreads();
+    const unsigned n_warps = gridDim.x * WARPS, wi = warp_id() * gridDim.x + blockIdx.x;
+    const unsigned steps = S.end[2 * N_GROUP_CLS - 1];
+    unsigned np = 0;
+    Share w(steps, n_warps, max((unsigned)d.run_roads / 8, 1u), &d.ctrl->q[qgroup]);
+    for (unsigned s = w.first(wi); s < steps; s = w.next(s)) {
+        if (s < S.end[0])
+            group_step<PLAIN, GroupCls4e, 0>(d, smem, s, np, npass);
+        else if (s < S.end[1])
+            group_step<PLAIN, GroupCls4, 1>(d, smem, s, np, npass);
+        else if (s < S.end[3])
+            group_step<PLAIN, GroupCls3, 3>(d, smem, s, np, npass);
+        else if (s < S.end[4])
+            group_step<PLAIN, GroupCls2e, 4>(d, smem, s, np, npass);
+        else if (s < S.end[5])
+            group_step<PLAIN, GroupCls2, 5>(d, smem, s, np, npass);
+        else if (s < S.end[7])
+            group_step<PLAIN, GroupCls1, 7>(d, smem, s, np, npass);
+        else
+            group_step<PLAIN, GroupCls0, 9>(d, smem, s, np, npass);
     }
-    npass = block_sum(npass);
+    __syncwarp();
+    p3_boxes<PLAIN>(d, smem, n_box, qbox, npass);
+    npass = block_sum(npass + np);
     if (!PLAIN && threadIdx.x == 0 && npass)
         atomicAdd(&d.ctrl->n_pass, npass);
 }
@@ -3435,7 +3549,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 2 : 768 / BLOCK) k_persi
     if (fault)
         return;
 
-    p3_phase<false>(d, smem, bt.n_roads, Q_BOX);
+    p3_phase<false>(d, smem, Q_BOX, Q_GROUP);
     if (d.skip_arrival == 2 && blockIdx.x == 0)
         return;   // test hook: this CTA leaves after publishing, the others' waits run out
     if (!grid_sync(d, 4, flags))
@@ -3600,7 +3714,7 @@ __global__ void __launch_bounds__(BLOCK) k_warrior_plain(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem[];
     if (stop_after_unpack(d))
         return;
-    p3_phase<true>(d, smem, min(ldcg(&d.ctrl->n_roads), d.max_roads), Q_BOX);
+    p3_phase<true>(d, smem, Q_BOX, Q_GROUP);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p4(Dev d)
@@ -3657,11 +3771,8 @@ __global__ void __launch_bounds__(BLOCK) k_export_roads(Dev d)
 // ---------------------------------------------------------------------------
 
 static size_t p1_smem() { return WARPS * sizeof(P1Warp); }
-static size_t p2_smem() { return sizeof(P2Smem) > WARPS * P2W_BYTES ? sizeof(P2Smem) : WARPS * P2W_BYTES; }
-static size_t p3_smem()
-{
-    return P3_REDO + sizeof(P3Redo);
-}
+static size_t p2_smem() { return P2_LIST_AT + sizeof(P2List); }
+static size_t p3_smem() { return P3_SHARED_BYTES + WARPS * P3_WARP_BYTES; }
 
 size_t persistent_smem_bytes()
 {

@@ -42,7 +42,8 @@ constexpr size_t OFF_ROADS = OFF_EV + up256(2 * sizeof(uint32_t) * S_EVENTS);
 constexpr size_t OFF_COORDS = OFF_ROADS + up256(sizeof(RoadRec) * S_ROADS);
 constexpr size_t OFF_XMASK = OFF_COORDS + up256(sizeof(uint16_t) * 40 * S_ROADS);
 constexpr size_t OFF_BOX = OFF_XMASK + up256(sizeof(unsigned long long) * S_ROADS);
-constexpr size_t OFF_CAND = OFF_BOX + up256(sizeof(uint32_t) * S_ROADS);
+constexpr size_t OFF_ITEMS = OFF_BOX + up256(sizeof(uint32_t) * S_ROADS);
+constexpr size_t OFF_CAND = OFF_ITEMS + up256(sizeof(RoadItem) * N_GROUP_CLS * S_ROADS);
 constexpr size_t OFF_FITC = OFF_CAND + up256(sizeof(uint32_t) * (S_ROADS / 32 + 1));
 constexpr size_t OFF_SURV = OFF_FITC + up256(sizeof(int4) * SET_INT4 * N_SETS);
 constexpr size_t OFF_SCNT = OFF_SURV + up256(sizeof(unsigned long long) * SURV_SLOTS * S_ROADS);
@@ -128,6 +129,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     d.coords = reinterpret_cast<uint16_t *>(b + OFF_COORDS);
     d.xmask = reinterpret_cast<unsigned long long *>(b + OFF_XMASK);
     d.box_list = reinterpret_cast<uint32_t *>(b + OFF_BOX);
+    d.items = reinterpret_cast<RoadItem *>(b + OFF_ITEMS);
     d.cand_bits = reinterpret_cast<uint32_t *>(b + OFF_CAND);
     d.fitc = reinterpret_cast<int4 *>(b + OFF_FITC);
     d.surv_pool = reinterpret_cast<unsigned long long *>(b + OFF_SURV);

@@ -118,6 +118,7 @@ struct Dev {
     uint32_t *span_ee, *span_ep, *span_seg;   // [MAX_SPANS + MAX_GRID] per word span (one per warp),
                                               // then per CTA (its spans together): EE and EP words,
                                               // EP words since its last EE (SEG_EE set when it holds one)
+    uint2 *wmask;                             // [max_words / 32 + 1] EP and EE masks of 32 words
     uint32_t *ev_road_end;                    // [max_events] roads up to the end of each event
     uint32_t *ev_big;                         // [max_events] events of more than P2W_ROADS roads
     RoadRec *roads;                                               // [max_roads]

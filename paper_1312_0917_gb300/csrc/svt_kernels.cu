@@ -415,9 +415,9 @@ enum { Q_P2 = 0, Q_BOX, Q_GROUP, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
 // its last EE, and checks every word's fields.  P1 gives each warp the counts
 // of the spans before its own (every CTA sums them itself, no CTA scans for
 // the others) and decodes the roads whose header lies in the warp's span.
-// Ballots over the EP and EE bits of a window (lane i: word i) find the roads
-// that start in it, with their road index, event and place in the event;
-// each road is then walked by one lane from its header to its EP word,
+// P0 keeps the EP and EE masks of every window (bit i: word i); they give P1
+// the roads that start in it, with their road index, event and place in the
+// event; each road is then taken by one lane from its header to its EP word,
 // which checks the grammar and ranks each hit in its layer.  A warp follows
 // its last road past the end of its span.
 // ---------------------------------------------------------------------------
@@ -476,38 +476,70 @@ __device__ unsigned block_seg_fold(unsigned v)
     return r;
 }
 
+// Nonzero when !word_ok(w), without branches.
+__device__ __forceinline__ uint32_t word_bad(uint32_t w)
+{
+    const uint32_t t = (w >> 27) & 7u;
+    const uint32_t allowed = t == 7 ? 0x3FFu : t > 4 ? 0xFFFFu : 0xFFFu;
+    const uint32_t pair = w & (w >> 1);   // wedge >= 12: bits 2 and 3; barrel >= 6: bits 5 and 6;
+    const uint32_t head = (pair & 0x24u) | ((w | (w >> 1)) & (w >> 2) & 0x80u);   // excl >= 5: bit 9 and 8 or 7
+    return (w & 0x07FFFFFFu & ~allowed) | (w & ~(w << 1) & 0x80000000u) | (t == 7 ? head : 0u);
+}
+
+// P0 of one warp's span.  A window's EP and EE masks (32 words each) are kept
+// for P1, which then finds the roads without reading the words; the counts are
+// taken from the masks, a window per lane.  Bound: the words' latency, then
+// issue slots (22 instructions a window; 73 when every window was counted and
+// checked by itself).
 __device__ void scan_count(const Dev &d)
 {
     const unsigned lane = lane_id(), sp = blockIdx.x * WARPS + warp_id();
     unsigned long long a, e;
     span_of(d, sp, a, e);
     unsigned ee = 0, ep = 0, seg = 0;
-    unsigned long long bad = ~0ull;
+    uint32_t bad = 0;
     constexpr unsigned UNROLL = 8;   // windows whose loads are in flight together
     for (unsigned long long base = a; base < e; base += UNROLL * WIN) {
         uint32_t w[UNROLL];
 #pragma unroll
         for (unsigned k = 0; k < UNROLL; ++k) {
             const unsigned long long i = base + k * WIN + lane;
-            w[k] = i < e ? __ldg(d.words + i) : 0u;
+            w[k] = i < e ? __ldg(d.words + i) : 0u;   // (0 is a valid word)
         }
+        unsigned pm = 0, em = 0;   // lane k: window k's masks
 #pragma unroll
         for (unsigned k = 0; k < UNROLL; ++k) {
-            const unsigned long long i = base + k * WIN + lane;
-            const unsigned em = __ballot_sync(FULL_MASK, w[k] >> 31);
-            const unsigned pm = __ballot_sync(FULL_MASK, (w[k] >> 30) & 1u);
-            ee += __popc(em);
-            ep += __popc(pm);
-            seg = seg_join(seg, seg_window(em, pm));
-            if (i < e && bad == ~0ull && !word_ok(w[k]))
-                bad = i;
+            const unsigned m = __ballot_sync(FULL_MASK, (w[k] >> 30) & 1u), n = __ballot_sync(FULL_MASK, w[k] >> 31);
+            pm = lane == k ? m : pm;
+            em = lane == k ? n : em;
+            bad |= word_bad(w[k]);
+        }
+        if (lane < UNROLL && base + lane * WIN < e)
+            d.wmask[base / WIN + lane] = make_uint2(pm, em);
+        const unsigned total = __reduce_add_sync(FULL_MASK, __popc(pm));
+        ep += total;
+        const unsigned last = __ballot_sync(FULL_MASK, em != 0u);
+        if (last) {   // EP words after the last EE
+            const unsigned lw = 31 - __clz(last);
+            ee += __reduce_add_sync(FULL_MASK, __popc(em));
+            seg = SEG_EE | __reduce_add_sync(FULL_MASK, lane == lw  ? seg_window(em, pm) & ~SEG_EE
+                                                        : lane > lw ? __popc(pm)
+                                                                    : 0u);
+        } else {
+            seg += total;   // (the flag in the top bit stays)
         }
     }
-    bad = warp_min_u64(bad);
+    if (__any_sync(FULL_MASK, bad != 0u)) {   // the first bad word, one window at a time
+        unsigned long long first = ~0ull;
+        for (unsigned long long i = a + lane; i < e && first == ~0ull; i += WIN)
+            if (!word_ok(__ldg(d.words + i)))
+                first = i;
+        first = warp_min_u64(first);
+        if (lane == 0)
+            report(d, (first << 8) | RANK_BAD);
+    }
     __shared__ unsigned s_cnt[3][WARPS];
     if (lane == 0) {
-        if (bad != ~0ull)
-            report(d, (bad << 8) | RANK_BAD);
         d.span_ee[sp] = ee;
         d.span_ep[sp] = ep;
         d.span_seg[sp] = seg;
@@ -530,19 +562,18 @@ __device__ void scan_count(const Dev &d)
     }
 }
 
-// P1 of one warp.  A ballot scan of the span finds the roads that start in
-// it (the word after an EP word) with their road index, event and place in
-// the event, and queues them in shared memory; each batch of 32 queued roads
-// is decoded one road per lane, the lane walking its road's words from the
-// header to the EP word (past the span's end if need be).  Each lane builds
-// its road's coordinate row in shared memory; the batch's rows (consecutive
-// roads) are then copied out with 16-byte stores.
-constexpr unsigned P1_AHEAD = 4;                  // windows scanned per step (loads in flight together)
-constexpr unsigned P1_Q = (P1_AHEAD + 1) * WIN;  // queued road starts per warp
+// P1 of one warp.  P0's masks of 32 windows, one per lane, give the roads that
+// start in them (the word after an EP word) with their road index, event and
+// place in the event; the starts are listed in shared memory, and each batch
+// of 32 is decoded one road per lane: the lane takes its road's words from the
+// header to the EP word, which may lie past the step's windows.  Each lane
+// builds its road's coordinate row in shared memory; the batch's rows
+// (consecutive roads) are then copied out with 16-byte stores.
+constexpr unsigned P1_WORDS = WIN * WIN;   // words of a step
 struct P1Warp {
     uint16_t row[WIN][40];           // coordinate rows of the batch's roads
-    uint32_t pos[P1_Q], g[P1_Q], ev[P1_Q], rie[P1_Q];   // queued roads: first word, index, event,
-                                                         // roads of the event before it
+    uint32_t start[P1_WORDS];        // a road's first word from the step's (10 bits), roads of the event
+                                     // before it (10 bits, at most 1023), events of the step before it
 };
 static_assert(sizeof(P1Warp) % 16 == 0, "warp regions of 16-byte multiples");
 
@@ -550,95 +581,140 @@ static_assert(sizeof(P1Warp) % 16 == 0, "warp regions of 16-byte multiples");
 // its first MAX_ROAD_WORDS words (a ninth hit on some layer at the latest)
 constexpr unsigned MAX_ROAD_WORDS = 3 + N_LAYERS * MAX_HITS + 1;
 
-// Decode queued roads [off, off + cnt) (cnt <= 32) one per lane; returns the
-// batch's first fault (encoded as in Ctrl::err_inv, ~0 when none).
-__device__ __forceinline__ unsigned long long decode_batch(const Dev &d, P1Warp &q, unsigned off, unsigned cnt,
+// A complete road's record, and its event's end when it is the last one.
+__device__ __forceinline__ void put_road(const Dev &d, unsigned g, unsigned ev, unsigned rie, uint32_t hdr, uint32_t cw,
+                                         uint32_t pw, unsigned cnt4, bool ee, unsigned n_events)
+{
+    const unsigned wedge = min(hdr & 15u, 11u), barrel = min((hdr >> 4) & 7u, 5u);
+    const unsigned excl = min((hdr >> 7) & 7u, 4u);
+    RoadRec r;
+    r.event = ev;
+    r.pk = cnt4 | (excl << 20) | (min(rie, 255u) << 24);   // the hit counts, four bits per layer
+    r.curv = (int16_t)(cw & 0xFFFFu);
+    r.phi = (int16_t)(pw & 0xFFFFu);
+    r.set = (uint16_t)((wedge * 6 + barrel) * 5 + excl);
+    r.fit = 0;
+    d.roads[g] = r;
+    if (ee && ev < d.max_events) {   // the event's last road
+        d.ev_road_end[ev] = g + 1;
+        if (rie + 1 > (unsigned)P2W_ROADS)   // P2 takes this event with a whole CTA
+            d.ev_big[atomicAdd(&d.ctrl->n_big_ev, 1u)] = ev;
+        if (ev + 1 == n_events)
+            d.ctrl->n_roads = g + 1;
+    }
+}
+
+// The lane's road, word by word, with every rule of the grammar and the limits
+// in order (a batch with a road that breaks one or does not end): true when it
+// is complete; err: its first fault (encoded as in Ctrl::err_inv, ~0 when none).
+__device__ __noinline__ bool walk_road(const Dev &d, uint16_t *row, unsigned long long start, unsigned g, unsigned ev,
+                                       unsigned rie, unsigned n_events, unsigned long long &err)
+{
+    unsigned cnt4 = 0;   // hits so far, layer l in bits 4 l .. 4 l + 3 (at most MAX_HITS)
+    uint32_t hdr = 0, cw = 0, pw = 0;
+    for (unsigned k = 0; k < MAX_ROAD_WORDS; ++k) {
+        const unsigned long long p = start + k;
+        if (p >= d.n_words)
+            return false;
+        const uint32_t w = __ldg(d.words + p);
+        const unsigned type = (w >> 27) & 7u;
+        const bool ep = (w >> 30) & 1u;
+        bool bad;
+        if (k == 0) {
+            bad = type != 7 || ep;
+            hdr = w;
+            if (!bad && rie >= (unsigned)MAX_ROADS_EV)
+                err = (p << 8) | RANK_LIMIT;
+        } else if (k == 1) {
+            bad = type != 5 || ep;
+            cw = w;
+        } else if (k == 2) {
+            bad = type != 6;
+            pw = w;
+        } else {
+            bad = type > 4;
+            if (!bad) {
+                const unsigned r = (cnt4 >> (4 * type)) & 15u;
+                if (r >= (unsigned)MAX_HITS) {
+                    err = (p << 8) | RANK_LIMIT;
+                } else {
+                    row[type * 8 + r] = (uint16_t)(w & 0xFFFu);
+                    cnt4 += 1u << (4 * type);
+                }
+            }
+        }
+        if (bad)
+            err = (p << 8) | RANK_BAD;
+        if (err != ~0ull)
+            return false;
+        if (ep) {
+            if (g < d.max_roads)
+                put_road(d, g, ev, rie, hdr, cw, pw, cnt4, (w >> 31) != 0, n_events);
+            return true;
+        }
+    }
+    return false;
+}
+
+// Decode the lane's road (have: there is one) of `len` words from `start`;
+// returns the batch's first fault.  A road's length is known, so its words
+// need no test for the end, and a rule's break is only noted: the batch is then
+// walked again word by word.
+__device__ __forceinline__ unsigned long long decode_batch(const Dev &d, P1Warp &q, bool have, unsigned long long start,
+                                                           unsigned len, unsigned g, unsigned ev, unsigned rie,
                                                            unsigned n_events)
 {
     const unsigned lane = lane_id();
+    uint16_t *row = q.row[lane];
     unsigned long long err = ~0ull;
-    bool done = false;   // a complete road (its EP word seen)
-    unsigned g = 0;
-    if (lane < cnt) {
-        const unsigned start = q.pos[off + lane], ev = q.ev[off + lane], rie = q.rie[off + lane];
-        g = q.g[off + lane];
-        uint16_t *row = q.row[lane];
-        unsigned cnt4 = 0;   // hits so far, layer l in bits 4 l .. 4 l + 3 (at most MAX_HITS)
-        uint32_t hdr = 0, cw = 0, pw = 0;
-        bool ee = false;
-        for (unsigned k0 = 0; k0 < MAX_ROAD_WORDS && !done && err == ~0ull; k0 += 8) {
-            uint32_t w4[8];
+    bool done = have;
+    unsigned cnt4 = 0;   // hits so far, four bits per layer
+    uint32_t w[8], hdr = 0, cw = 0, pw = 0, last = 0;
+    bool bad = have && (len < 3 || len >= MAX_ROAD_WORDS || rie >= (unsigned)MAX_ROADS_EV);
+    const unsigned n = bad || !have ? 0u : len;
+    const uint32_t *words = d.words + start;
+    const unsigned most = __reduce_max_sync(FULL_MASK, n);
+    for (unsigned k0 = 0; k0 < most; k0 += 8) {
 #pragma unroll
-            for (unsigned u = 0; u < 8; ++u) {   // eight loads in flight
-                const unsigned long long p = (unsigned long long)start + k0 + u;
-                w4[u] = p < d.n_words ? __ldg(d.words + p) : 0u;
+        for (unsigned u = 0; u < 8; ++u)   // eight loads in flight
+            w[u] = k0 + u < n ? __ldg(words + k0 + u) : 0xFFFFFFFFu;
+#pragma unroll
+        for (unsigned u = 0; u < 8; ++u) {
+            if (k0 == 0 && u < 3) {
+                if (u == 0)
+                    hdr = w[0];
+                else if (u == 1)
+                    cw = w[1];
+                else
+                    pw = w[2];
+                continue;
             }
-#pragma unroll
-            for (unsigned u = 0; u < 8; ++u) {
-                const unsigned k = k0 + u;
-                const unsigned long long p = (unsigned long long)start + k;
-                if (done || err != ~0ull || k >= MAX_ROAD_WORDS || p >= d.n_words)
-                    break;
-                const uint32_t w = w4[u];
-                const unsigned type = (w >> 27) & 7u;
-                const bool ep = (w >> 30) & 1u;
-                bool bad;
-                if (k == 0) {
-                    bad = type != 7 || ep;
-                    hdr = w;
-                    if (!bad && rie >= (unsigned)MAX_ROADS_EV)
-                        err = (p << 8) | RANK_LIMIT;
-                } else if (k == 1) {
-                    bad = type != 5 || ep;
-                    cw = w;
-                } else if (k == 2) {
-                    bad = type != 6;
-                    pw = w;
-                } else {
-                    bad = type > 4;
-                    if (!bad) {
-                        const unsigned r = (cnt4 >> (4 * type)) & 15u;
-                        if (r >= (unsigned)MAX_HITS) {
-                            err = (p << 8) | RANK_LIMIT;
-                        } else {
-                            row[type * 8 + r] = (uint16_t)(w & 0xFFFu);
-                            cnt4 += 1u << (4 * type);
-                        }
-                    }
-                }
-                if (bad)
-                    err = (p << 8) | RANK_BAD;
-                else if (ep && err == ~0ull) {
-                    done = true;
-                    ee = (w >> 31) != 0;
-                }
+            if (k0 + u < n) {
+                const unsigned type = (w[u] >> 27) & 7u, sh = 4 * type, r = (cnt4 >> (sh & 31u)) & 15u;
+                const bool fits = (type <= 4) & (r < (unsigned)MAX_HITS);
+                bad = bad | !fits;
+                if (fits)
+                    row[type * 8 + r] = (uint16_t)w[u];
+                cnt4 += 1u << (sh & 31u);
+                last = w[u];
             }
         }
-        if (done && g < d.max_roads) {   // a complete road: its record
-            const unsigned pk = cnt4;   // the hit counts, four bits per layer
-            const unsigned wedge = min(hdr & 15u, 11u), barrel = min((hdr >> 4) & 7u, 5u);
-            const unsigned excl = min((hdr >> 7) & 7u, 4u);
-            RoadRec r;
-            r.event = ev;
-            r.pk = pk | (excl << 20) | (min(rie, 255u) << 24);
-            r.curv = (int16_t)(cw & 0xFFFFu);
-            r.phi = (int16_t)(pw & 0xFFFFu);
-            r.set = (uint16_t)((wedge * 6 + barrel) * 5 + excl);
-            r.fit = 0;
-            d.roads[g] = r;
-            if (ee && ev < d.max_events) {   // the event's last road
-                d.ev_road_end[ev] = g + 1;
-                if (rie + 1 > (unsigned)P2W_ROADS)   // P2 takes this event with a whole CTA
-                    d.ev_big[atomicAdd(&d.ctrl->n_big_ev, 1u)] = ev;
-                if (ev + 1 == n_events)
-                    d.ctrl->n_roads = g + 1;
-            }
-        }
+    }
+    if (n) {
+        last = n == 3 ? pw : last;
+        bad = bad | (((hdr >> 27) & 7u) != 7) | (((cw >> 27) & 7u) != 5) | (((pw >> 27) & 7u) != 6);
+    }
+    if (__any_sync(FULL_MASK, bad)) {
+        if (have)
+            done = walk_road(d, row, start, g, ev, rie, n_events, err);
+    } else if (have && g < d.max_roads) {
+        put_road(d, g, ev, rie, hdr, cw, pw, cnt4, (last >> 31) != 0, n_events);
     }
     __syncwarp();
     // the rows of the batch's complete roads (consecutive road indices from
     // the first lane's), five 16-byte words each
     const unsigned g0 = __shfl_sync(FULL_MASK, g, 0), dm = __ballot_sync(FULL_MASK, done);
+    const unsigned cnt = __popc(__ballot_sync(FULL_MASK, have));
     const uint4 *src = reinterpret_cast<const uint4 *>(&q.row[0][0]);
     uint4 *dst = reinterpret_cast<uint4 *>(d.coords + (size_t)g0 * 40);
     for (unsigned i = lane; i < cnt * N_LAYERS; i += WIN) {
@@ -656,70 +732,79 @@ __device__ __forceinline__ unsigned long long decode_batch(const Dev &d, P1Warp 
 __device__ void decode_span(const Dev &d, P1Warp &q, unsigned long long a, unsigned long long e, unsigned g,
                             unsigned ev, unsigned rie, unsigned n_events)
 {
-    const unsigned lane = lane_id(), lt = lanemask_lt();
-    bool prev_ep = a == 0 || ((__ldg(d.words + a - 1) >> 30) & 1u);   // word a starts a road
-    unsigned qn = 0;
+    const unsigned lane = lane_id();
+    if (a >= e)
+        return;
+    const unsigned w_end = (unsigned)((e + WIN - 1) / WIN), w_all = (unsigned)((d.n_words + WIN - 1) / WIN);
+    unsigned W = (unsigned)(a / WIN);
+    unsigned ends = W == 0 ? 1u : __ldcg(&d.wmask[W - 1].x) >> 31;   // the step's first word starts a road
     unsigned long long err = ~0ull;
-    for (unsigned long long W0 = a;; W0 += P1_AHEAD * WIN) {
-        const bool more = W0 < e && err == ~0ull;
-        if (more) {   // P1_AHEAD windows: their road starts join the queue
-            uint32_t wds[P1_AHEAD];
+    for (; W < w_end && err == ~0ull; W += WIN) {
+        // the step's windows, one per lane
+        const unsigned win = W + lane;
+        const uint2 m = win < w_end ? __ldcg(&d.wmask[win]) : make_uint2(0u, 0u);
+        const unsigned pm = m.x, em = m.y, up = __shfl_up_sync(FULL_MASK, pm, 1);
+        const unsigned pe = lane ? up >> 31 : ends;
+        const unsigned long long base = (unsigned long long)W * WIN, left = win < w_end ? d.n_words - base - lane * WIN : 0;
+        const unsigned in = left >= WIN ? FULL_MASK : (1u << (unsigned)left) - 1u;
+        unsigned sm = ((pm << 1) | pe) & in;   // roads start
+        // EP and EE words of the windows before, and EP words since the last EE
+        const unsigned own = __popc(pm) | __popc(em) << 16;
+        unsigned inc = own, seg = seg_window(em, pm);
 #pragma unroll
-            for (unsigned k = 0; k < P1_AHEAD; ++k) {
-                const unsigned long long i = W0 + k * WIN + lane;
-                wds[k] = i < e ? __ldg(d.words + i) : 0u;
+        for (unsigned o = 1; o < 32; o <<= 1) {
+            const unsigned u = __shfl_up_sync(FULL_MASK, inc, o), v = __shfl_up_sync(FULL_MASK, seg, o);
+            if (lane >= o) {
+                inc += u;
+                seg = seg_join(v, seg);
             }
-#pragma unroll
-            for (unsigned k = 0; k < P1_AHEAD; ++k) {
-                const unsigned long long i = W0 + k * WIN + lane;
-                const bool in = i < e;
-                const uint32_t wd = wds[k];
-                const unsigned pm = __ballot_sync(FULL_MASK, in && ((wd >> 30) & 1u));
-                const unsigned em = __ballot_sync(FULL_MASK, in && (wd >> 31));
-                const unsigned sm = ((pm << 1) | (prev_ep ? 1u : 0u)) & __ballot_sync(FULL_MASK, in);
-                if ((sm >> lane) & 1u) {   // a road starts at this word
-                    const unsigned j = qn + __popc(sm & lt), em_lt = em & lt;
-                    q.pos[j] = (uint32_t)i;
-                    q.g[j] = g + __popc(pm & lt);
-                    q.ev[j] = ev + __popc(em & lt);
-                    q.rie[j] = em_lt ? __popc(pm & lt & ~((2u << (31 - __clz(em_lt))) - 1u)) : rie + __popc(pm & lt);
-                }
-                qn += __popc(sm);
-                g += __popc(pm);
-                ev += __popc(em);
-                rie = em ? (unsigned)__popc((pm >> (31 - __clz(em))) >> 1) : rie + __popc(pm);
-                prev_ep = (pm >> 31) & 1u;
-            }
-            __syncwarp();
         }
-        // full batches of 32 roads, and at the end the rest
-        unsigned off = 0;
-        while (err == ~0ull && (qn - off >= WIN || (!more && qn > off))) {
-            const unsigned c = min(qn - off, WIN);
-            err = decode_batch(d, q, off, c, n_events);
-            off += c;
+        unsigned before = __shfl_up_sync(FULL_MASK, seg, 1);
+        before = seg_join(rie, lane ? before : 0u) & ~SEG_EE;
+        const unsigned ex = inc - own;
+        const unsigned n_start = __reduce_add_sync(FULL_MASK, __popc(sm));
+        unsigned at = ends + (ex & 0xFFFFu) - pe;   // place of the lane's first start
+        const unsigned g_first = g + 1 - ends;
+        unsigned last_start = 0;
+        while (sm) {
+            const unsigned b = __ffs(sm) - 1, lt = (1u << b) - 1u, el = em & lt;
+            const unsigned r = el ? __popc(pm & lt & ~((2u << (31 - __clz(el))) - 1u)) : before + __popc(pm & lt);
+            last_start = lane * WIN + b;
+            q.start[at++] = last_start | min(r, 1023u) << 10 | ((ex >> 16) + __popc(el)) << 20;
+            sm &= sm - 1;
         }
-        if (!more || err != ~0ull)
-            break;
-        if (off) {   // fewer than 32 left: to the front of the queue
-            const unsigned rest = qn - off;
-            uint32_t p0 = 0, p1 = 0, p2 = 0, p3 = 0;
-            if (lane < rest) {
-                p0 = q.pos[off + lane];
-                p1 = q.g[off + lane];
-                p2 = q.ev[off + lane];
-                p3 = q.rie[off + lane];
+        // the word after the last road's end (the first EP from its start on,
+        // within the step or the two windows after it)
+        last_start = __reduce_max_sync(FULL_MASK, last_start);
+        unsigned end = ~0u;
+        {
+            const unsigned ls = last_start, lw = ls / WIN;
+            const unsigned c = lane < lw ? 0u : lane == lw ? pm & ~((1u << (ls % WIN)) - 1u) : pm;
+            if (c)
+                end = lane * WIN + __ffs(c);
+            const unsigned after = min(W + WIN, w_end) + lane;
+            if (lane < 2 && after < w_all) {
+                const unsigned p2 = __ldcg(&d.wmask[after].x);
+                if (p2)
+                    end = min(end, (after - W) * WIN + __ffs(p2));
             }
-            __syncwarp();
-            if (lane < rest) {
-                q.pos[lane] = p0;
-                q.g[lane] = p1;
-                q.ev[lane] = p2;
-                q.rie[lane] = p3;
-            }
-            qn = rest;
-            __syncwarp();
+            end = __reduce_min_sync(FULL_MASK, end);
         }
+        __syncwarp();
+        for (unsigned off = 0; off < n_start && err == ~0ull; off += WIN) {
+            const unsigned i = off + lane;
+            const bool have = i < n_start;
+            const unsigned s = have ? q.start[i] : 0u, pos = s & 1023u;
+            const unsigned next = i + 1 < n_start ? q.start[i + 1] & 1023u : end;
+            err = decode_batch(d, q, have, base + pos, next == ~0u ? MAX_ROAD_WORDS : next - pos, g_first + i,
+                               ev + (s >> 20), (s >> 10) & 1023u, n_events);
+        }
+        __syncwarp();   // the list is refilled next
+        const unsigned tot = __shfl_sync(FULL_MASK, inc, 31);
+        rie = seg_join(rie, __shfl_sync(FULL_MASK, seg, 31)) & ~SEG_EE;
+        g += tot & 0xFFFFu;
+        ev += tot >> 16;
+        ends = __shfl_sync(FULL_MASK, pm, 31) >> 31;   // (a step that is not full is the span's last)
     }
     if (lane == 0 && err != ~0ull)
         report(d, err);   // the first fault of the batch is its status

@@ -37,7 +37,8 @@ constexpr size_t OFF_CTRL = 0;
 constexpr size_t OFF_CONSTS = OFF_CTRL + up256(sizeof(Ctrl));
 constexpr unsigned S_SPANS = MAX_SPANS + MAX_GRID;   // per-warp word spans, then per-CTA totals
 constexpr size_t OFF_SPAN = OFF_CONSTS + up256(sizeof(svt_const_set) * N_SETS);    // 3 x [S_SPANS] u32
-constexpr size_t OFF_EV = OFF_SPAN + up256(3 * sizeof(uint32_t) * S_SPANS);         // 2 x [S_EVENTS] u32
+constexpr size_t OFF_WMASK = OFF_SPAN + up256(3 * sizeof(uint32_t) * S_SPANS);      // [S_WORDS / 32 + 1] uint2
+constexpr size_t OFF_EV = OFF_WMASK + up256(sizeof(uint2) * (S_WORDS / 32 + 1));         // 2 x [S_EVENTS] u32
 constexpr size_t OFF_ROADS = OFF_EV + up256(2 * sizeof(uint32_t) * S_EVENTS);
 constexpr size_t OFF_COORDS = OFF_ROADS + up256(sizeof(RoadRec) * S_ROADS);
 constexpr size_t OFF_XMASK = OFF_COORDS + up256(sizeof(uint16_t) * 40 * S_ROADS);
@@ -123,6 +124,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     d.span_ee = span;
     d.span_ep = span + S_SPANS;
     d.span_seg = span + 2 * S_SPANS;
+    d.wmask = reinterpret_cast<uint2 *>(b + OFF_WMASK);
     d.ev_road_end = reinterpret_cast<uint32_t *>(b + OFF_EV);
     d.ev_big = d.ev_road_end + S_EVENTS;
     d.roads = reinterpret_cast<RoadRec *>(b + OFF_ROADS);

@@ -1281,19 +1281,22 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
             s.rep[k] = 1;
     }
     __syncthreads();
-    // signatures of the shared coordinates; roads with >= 3 such layers
+    // signatures of the shared coordinates, a layer of a road per thread
+    for (unsigned i = threadIdx.x; i < nr * N_LAYERS; i += BLOCK) {
+        const unsigned k = i / N_LAYERS, l = i - k * N_LAYERS, n = (s.rec[k].pk >> (4 * l)) & 15u;
+        const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
+        unsigned long long sg = 0;
+        for (unsigned m = multi_row(s.multi[l], q, n, MAX_HITS); m; m &= m - 1)
+            sg |= 1ull << sig_bit(row_at(q, __ffs(m) - 1));
+        s.sig[k][l] = sg;
+    }
+    __syncthreads();
+    // roads with >= 3 such layers
     for (unsigned k = threadIdx.x; k < nr; k += BLOCK) {
         unsigned layers = 0;
 #pragma unroll
-        for (unsigned l = 0; l < N_LAYERS; ++l) {
-            const unsigned n = (s.rec[k].pk >> (4 * l)) & 15u;
-            unsigned long long sg = 0;
-            const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
-            for (unsigned m = multi_row(s.multi[l], q, n, MAX_HITS); m; m &= m - 1)
-                sg |= 1ull << sig_bit(row_at(q, __ffs(m) - 1));
-            s.sig[k][l] = sg;
-            layers += sg != 0;
-        }
+        for (unsigned l = 0; l < N_LAYERS; ++l)
+            layers += s.sig[k][l] != 0;
         if (layers >= 3)
             s.elig[atomicAdd(&s.n_elig, 1u)] = (uint16_t)k;
     }

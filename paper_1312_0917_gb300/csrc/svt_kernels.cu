@@ -569,10 +569,13 @@ __device__ void scan_count(const Dev &d)
 // header to the EP word, which may lie past the step's windows.  Each lane
 // builds its road's coordinate row in shared memory; the batch's rows
 // (consecutive roads) are then copied out with 16-byte stores.
-constexpr unsigned P1_WORDS = WIN * WIN;   // words of a step
+// Roads listed of a step's 1024 words.  A road has three words at least, so a
+// step of more starts than this has a road that is too short among the listed
+// ones, and its fault is the batch's.
+constexpr unsigned P1_STARTS = 384;
 struct P1Warp {
     uint16_t row[WIN][40];           // coordinate rows of the batch's roads
-    uint32_t start[P1_WORDS];        // a road's first word from the step's (10 bits), roads of the event
+    uint32_t start[P1_STARTS];       // a road's first word from the step's (10 bits), roads of the event
                                      // before it (10 bits, at most 1023), events of the step before it
 };
 static_assert(sizeof(P1Warp) % 16 == 0, "warp regions of 16-byte multiples");
@@ -770,7 +773,9 @@ __device__ void decode_span(const Dev &d, P1Warp &q, unsigned long long a, unsig
             const unsigned b = __ffs(sm) - 1, lt = (1u << b) - 1u, el = em & lt;
             const unsigned r = el ? __popc(pm & lt & ~((2u << (31 - __clz(el))) - 1u)) : before + __popc(pm & lt);
             last_start = lane * WIN + b;
-            q.start[at++] = last_start | min(r, 1023u) << 10 | ((ex >> 16) + __popc(el)) << 20;
+            if (at < P1_STARTS)
+                q.start[at] = last_start | min(r, 1023u) << 10 | ((ex >> 16) + __popc(el)) << 20;
+            ++at;
             sm &= sm - 1;
         }
         // the word after the last road's end (the first EP from its start on,
@@ -791,11 +796,14 @@ __device__ void decode_span(const Dev &d, P1Warp &q, unsigned long long a, unsig
             end = __reduce_min_sync(FULL_MASK, end);
         }
         __syncwarp();
-        for (unsigned off = 0; off < n_start && err == ~0ull; off += WIN) {
+        if (n_start > P1_STARTS)
+            end = ~0u;
+        const unsigned n_list = min(n_start, P1_STARTS);
+        for (unsigned off = 0; off < n_list && err == ~0ull; off += WIN) {
             const unsigned i = off + lane;
-            const bool have = i < n_start;
+            const bool have = i < n_list;
             const unsigned s = have ? q.start[i] : 0u, pos = s & 1023u;
-            const unsigned next = i + 1 < n_start ? q.start[i + 1] & 1023u : end;
+            const unsigned next = i + 1 < n_list ? q.start[i + 1] & 1023u : end;
             err = decode_batch(d, q, have, base + pos, next == ~0u ? MAX_ROAD_WORDS : next - pos, g_first + i,
                                ev + (s >> 20), (s >> 10) & 1023u, n_events);
         }
@@ -893,7 +901,6 @@ constexpr unsigned P2_PAIRS = 1024;   // road pairs queued for the exact test (m
 
 struct P2Smem {
     RoadRec rec[MAX_ROADS_EV];
-    uint16_t coord[MAX_ROADS_EV][40];     // [road][layer * 8 + hit]
     unsigned long long sig[MAX_ROADS_EV][N_LAYERS];   // signatures of a road's shared coordinates
     uint32_t seen[N_LAYERS][128];         // coordinate bitmaps of the event
     uint32_t multi[N_LAYERS][128];
@@ -904,7 +911,6 @@ struct P2Smem {
     uint8_t rep[MAX_ROADS_EV];            // a coordinate repeated within a layer of the road
     unsigned n_elig, n_cp;
 };
-static_assert(offsetof(P2Smem, coord) % 16 == 0 && offsetof(P2Smem, rec) % 16 == 0, "16-byte rows");
 
 // signature bit of a coordinate: a multiplicative hash into 0..63
 __device__ __forceinline__ unsigned sig_bit(unsigned v) { return (v * 0x9E3779B1u) >> 26; }
@@ -1009,7 +1015,7 @@ __device__ __forceinline__ unsigned multi_row(const uint32_t *multi, const uint4
 // coordinate and the hits involved; with three or more such layers, the
 // shared hits of both roads are marked.  Only coordinates present in two
 // roads can be common.
-__device__ void pair_exact(P2Smem &s, unsigned r, unsigned t)
+__device__ void pair_exact(P2Smem &s, const uint16_t *co, unsigned r, unsigned t)
 {
     const uint32_t pr = s.rec[r].pk, pt = s.rec[t].pk;
     unsigned lo_r = 0, lo_t = 0, hi_r = 0, hi_t = 0, layers = 0;
@@ -1018,11 +1024,11 @@ __device__ void pair_exact(P2Smem &s, unsigned r, unsigned t)
         const unsigned nr = (pr >> (4 * l)) & 15u, nt = (pt >> (4 * l)) & 15u;   // <= MAX_HITS
         unsigned br = 0, bt = 0;
         for (unsigned x = 0; x < nr; ++x) {
-            const unsigned v = s.coord[r][l * 8 + x];
+            const unsigned v = co[r * 40 + l * 8 + x];
             if (!is_multi(s, l, v))
                 continue;
             for (unsigned y = 0; y < nt; ++y)
-                if (s.coord[t][l * 8 + y] == v) {
+                if (co[t * 40 + l * 8 + y] == v) {
                     br |= 1u << x;
                     bt |= 1u << y;
                 }
@@ -1047,7 +1053,7 @@ __device__ void pair_exact(P2Smem &s, unsigned r, unsigned t)
 // The exact test of pair_exact by a whole warp: lane 8 l + x (then lane x
 // for layer 4) takes hit x of road r on layer l and compares it with road t's
 // hits on that layer.
-__device__ void pair_exact_warp(P2Smem &s, unsigned r, unsigned t)
+__device__ void pair_exact_warp(P2Smem &s, const uint16_t *co, unsigned r, unsigned t)
 {
     const unsigned lane = lane_id();
     const uint32_t pr = s.rec[r].pk, pt = s.rec[t].pk;
@@ -1058,10 +1064,10 @@ __device__ void pair_exact_warp(P2Smem &s, unsigned r, unsigned t)
         const unsigned nr = (pr >> (4 * l)) & 15u, nt = (pt >> (4 * l)) & 15u;   // <= MAX_HITS
         unsigned br = 0, bt = 0;
         if (x < nr && (!pass || lane < 8)) {
-            const unsigned v = s.coord[r][l * 8 + x];
+            const unsigned v = co[r * 40 + l * 8 + x];
             if (is_multi(s, l, v))
                 for (unsigned y = 0; y < nt; ++y)
-                    if (s.coord[t][l * 8 + y] == v) {
+                    if (co[t * 40 + l * 8 + y] == v) {
                         br = 1u << x;
                         bt |= 1u << y;
                     }
@@ -1248,18 +1254,16 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
                          unsigned long long &n_comb)
 {
     P2Smem &s = *reinterpret_cast<P2Smem *>(smem);
-    // the event's roads: records and coordinate rows (16-byte loads)
+    // the event's roads: records; the coordinate rows stay in global memory (they
+    // are written before this stage, so that loads may use L1, which has what
+    // shared memory leaves)
+    const uint16_t *co = d.coords + (size_t)r0 * 40;
+    const uint4 *rows = reinterpret_cast<const uint4 *>(co);
     for (unsigned k = threadIdx.x; k < nr; k += BLOCK) {
         s.rec[k] = ldcg(d.roads + r0 + k);
         s.rep[k] = 0;
         s.xlo[k] = 0;
         s.xhi[k] = 0;
-    }
-    {
-        const uint4 *src = reinterpret_cast<const uint4 *>(d.coords + (size_t)r0 * 40);
-        uint4 *dst = reinterpret_cast<uint4 *>(&s.coord[0][0]);
-        for (unsigned i = threadIdx.x; i < nr * N_LAYERS; i += BLOCK)
-            dst[i] = ldcg(src + i);
     }
     for (unsigned i = threadIdx.x; i < N_LAYERS * 128; i += BLOCK) {
         (&s.seen[0][0])[i] = 0;
@@ -1275,7 +1279,7 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
     for (unsigned i0 = threadIdx.x - lane_id(); i0 < nr * N_LAYERS; i0 += BLOCK) {
         const unsigned i = min(i0 + lane_id(), nr * N_LAYERS - 1), k = i / N_LAYERS, l = i - k * N_LAYERS;
         const unsigned n = i0 + lane_id() == i ? (s.rec[k].pk >> (4 * l)) & 15u : 0u;   // <= MAX_HITS
-        const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
+        const uint4 q = rows[i];
         const unsigned again = see_row(s.seen[l], q, n, __reduce_max_sync(FULL_MASK, n));
         if (again && seen_again(s.multi[l], q, again))
             s.rep[k] = 1;
@@ -1284,7 +1288,7 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
     // signatures of the shared coordinates, a layer of a road per thread
     for (unsigned i = threadIdx.x; i < nr * N_LAYERS; i += BLOCK) {
         const unsigned k = i / N_LAYERS, l = i - k * N_LAYERS, n = (s.rec[k].pk >> (4 * l)) & 15u;
-        const uint4 q = *reinterpret_cast<const uint4 *>(&s.coord[k][l * 8]);
+        const uint4 q = rows[i];
         unsigned long long sg = 0;
         for (unsigned m = multi_row(s.multi[l], q, n, MAX_HITS); m; m &= m - 1)
             sg |= 1ull << sig_bit(row_at(q, __ffs(m) - 1));
@@ -1316,13 +1320,13 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
                 if (k < P2_PAIRS)
                     s.cp[k] = r | (t << 16);
                 else
-                    pair_exact(s, r, t);
+                    pair_exact(s, co, r, t);
             }
         }
     }
     __syncthreads();
     for (unsigned k = warp_id(); k < min(s.n_cp, P2_PAIRS); k += WARPS)
-        pair_exact_warp(s, s.cp[k] & 0xFFFFu, s.cp[k] >> 16);
+        pair_exact_warp(s, co, s.cp[k] & 0xFFFFu, s.cp[k] >> 16);
     __syncthreads();
     // the road records: candidate bit and fit path
     for (unsigned k0 = threadIdx.x - lane_id(); k0 < nr; k0 += BLOCK) {
@@ -1919,7 +1923,7 @@ __device__ __noinline__ void group_publish(const Dev &d, const Road &r, bool pub
 // pair has at most one candidate and a road at most 64 survivors.
 // ---------------------------------------------------------------------------
 
-enum { T_AB = 0, T_CE, T_AC, T_BC, T_AE, T_BE, N_TAB };
+enum { T_AB = 0, T_CE, T_AE, T_BE, T_AC, T_BC };
 // table row stride: rows 9 entries apart put the entries [u][v] of
 // different u in different banks
 constexpr unsigned TS = 9;
@@ -1934,12 +1938,10 @@ struct P3Float {
 struct P3Box {
     union {
         struct {
-            unsigned long long T[2][8 * TS];   // T_ab, T_ce: [u * TS + v] (u: the first role's hit);
-                                               // T_ce only where needed (box_tce)
-            unsigned H[2][4][8 * TS];          // T_ac, T_bc of pass 0 and pass 1: high words; T_ae,
-                                               // T_be: the entries taken on demand for the publish
-                                               // step (pass 0)
-            unsigned L[2][4][8 * TS];          // and low words (of the keys with the minimum high word)
+            unsigned long long T[4][8 * TS];   // T_ab, T_ce, T_ae, T_be: [u * TS + v] (u: the first
+                                               // role's hit); the last three only where needed
+            unsigned H[2][2][8 * TS];          // T_ac, T_bc of pass 0 and pass 1: high words
+            unsigned L[2][2][8 * TS];          // and low words (of the keys with the minimum high word)
         };
         P3Float F;
     };
@@ -1963,9 +1965,9 @@ __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsig
 // smaller of the two passes' (high, low) entries
 __device__ __forceinline__ unsigned long long box_get(const P3Box &B, unsigned tab, unsigned idx)
 {
-    if (tab < 2)
+    if (tab < T_AC)
         return B.T[tab][idx];
-    const unsigned t = tab - 2;
+    const unsigned t = tab - T_AC;
     return umin64(((unsigned long long)B.H[0][t][idx] << 32) | B.L[0][t][idx],
                   ((unsigned long long)B.H[1][t][idx] << 32) | B.L[1][t][idx]);
 }
@@ -2077,13 +2079,13 @@ __device__ void box_pass(const Dev &d, P3Box &B, const BoxShape &sh, unsigned p,
         rz = cut_min(rz);
         const unsigned q = p & 1u;
         if (act) {
-            fold_hi(B, q, T_AC - 2, x * TS + z, rz);
-            fold_hi(B, q, T_BC - 2, y * TS + z, rz);
+            fold_hi(B, q, T_AC - T_AC, x * TS + z, rz);
+            fold_hi(B, q, T_BC - T_AC, y * TS + z, rz);
         }
         __syncwarp();
         if (act) {
-            fold_lo(B, q, T_AC - 2, x * TS + z, rz);
-            fold_lo(B, q, T_BC - 2, y * TS + z, rz);
+            fold_lo(B, q, T_AC - T_AC, x * TS + z, rz);
+            fold_lo(B, q, T_BC - T_AC, y * TS + z, rz);
         }
     }
     if (act)
@@ -2565,9 +2567,9 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
         }
         B.A[j][k] = a;
     }
-    for (unsigned i = lane; i < 2 * 8 * TS; i += 32)
+    for (unsigned i = lane; i < 4 * 8 * TS; i += 32)
         (&B.T[0][0])[i] = NO_KEY;
-    for (unsigned i = lane; i < 2 * 2 * 4 * 8 * TS; i += 32)   // H and L
+    for (unsigned i = lane; i < 2 * 2 * 2 * 8 * TS; i += 32)   // H and L
         (&B.H[0][0][0])[i] = 0xFFFFFFFFu;
     // roles: the pair (a, b) that needs the fewest lane steps, then c before
     // e with e (the unrolled inner loop) the larger
@@ -2738,12 +2740,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
                             const unsigned kp = B.rank[sp][__ffs(bp) - 1], w = B.rank[sh.re][__ffs(be) - 1];
                             const unsigned long long m = box_min2<PLAIN>(d, B, sh, sp, kp, sh.re, w);
                             if (lane == 0) {
-                                if (q == 2) {
-                                    B.T[T_CE][kp * TS + w] = m;
-                                } else {   // read by box_get as the first pass's entry
-                                    B.H[0][q == 0 ? T_AE - 2 : T_BE - 2][kp * TS + w] = (unsigned)(m >> 32);
-                                    B.L[0][q == 0 ? T_AE - 2 : T_BE - 2][kp * TS + w] = (unsigned)m;
-                                }
+                                B.T[q == 0 ? T_AE : q == 1 ? T_BE : T_CE][kp * TS + w] = m;
                             }
                         }
                 }
@@ -3281,11 +3278,11 @@ __device__ __forceinline__ unsigned coord_of(const uint4 &r, unsigned d)
 }
 
 // The track of key `key` of road g (record rec, coordinate row rw: the
-// road's 40 coordinates as five 16-byte words), written to output slot pos.
+// road's 40 coordinates as five 16-byte words), written to *out.
 // The loops are unrolled (registers, no local arrays).
 template <bool PLAIN>
 __device__ void build_track(const Dev &d, unsigned g, const RoadRec &rec, const uint4 (&rw)[N_LAYERS],
-                            unsigned long long key, unsigned long long pos)
+                            unsigned long long key, svt_track *out)
 {
     int F[3][6], q[3];
     if (!PLAIN) {   // six 16-byte loads of the set's F and q
@@ -3347,8 +3344,7 @@ __device__ void build_track(const Dev &d, unsigned g, const RoadRec &rec, const 
             t.p[k] = (acc >> 12) + q[k];
         }
     }
-    if (pos < d.max_tracks)
-        d.tracks[pos] = t;
+    *out = t;
 }
 
 // Track of survivor idx of road g, written to output slot pos: the road's
@@ -3365,7 +3361,8 @@ __device__ void emit_track(const Dev &d, unsigned g, unsigned idx, unsigned long
 #pragma unroll
     for (unsigned l = 0; l < N_LAYERS; ++l)
         rw[l] = ldcg(row + l);
-    build_track<PLAIN>(d, g, rec, rw, key, pos);
+    if (pos < d.max_tracks)
+        build_track<PLAIN>(d, g, rec, rw, key, d.tracks + pos);
 }
 
 // road of survivor i of a chunk: the last r with s_first[r] <= i (a road
@@ -3435,154 +3432,86 @@ __device__ void p4_cand_phase(const Dev &d, unsigned n_roads)
     }
 }
 
-// P5 of the persistent kernel: the tracks in road order, split evenly over
-// the CTAs.  Every CTA scans the chunk totals itself (no CTA scans for the
-// others) and takes survivors [S b / grid, S (b + 1) / grid) of the S in all.
-// The survivor counts of the roads that hold them are loaded at once, eight
-// roads per thread (P5_GROUP chunks at a time), and scanned into a table of
-// first survivors, which places each survivor at its road.
-constexpr unsigned P5_PER_THREAD = 8;
-constexpr unsigned P5_ROADS = BLOCK * P5_PER_THREAD;
-constexpr unsigned P5_GROUP = P5_ROADS / ROAD_CHUNK;   // chunks per pass
-static_assert(P5_ROADS % ROAD_CHUNK == 0, "whole chunks per pass");
-static_assert(P5_GROUP <= 32, "a lane per chunk of a pass");
-
-constexpr unsigned P5_STAGE = 448;   // roads whose records and coordinates are staged at once
-
+// P5 of the persistent kernel: the tracks in road order.  Every CTA takes an
+// equal share of the roads; the chunk totals and the counts before its share,
+// which every CTA sums itself, give its first track's place.  A road's count,
+// record, coordinate row and first key do not depend on each other: they are
+// loaded together, a road per thread, and a scan of the counts places the
+// tracks, which are gathered in shared memory and written out as one stretch.
+// Bound: two trips to L2 and the writes (a search for the road of each of an
+// equal share of the tracks took four trips and wrote each track's five words
+// 40 bytes apart).
+constexpr unsigned P5_TRACKS = 2 * BLOCK;   // tracks gathered at most (more: written by their thread)
 struct P5Smem {
-    unsigned first[P5_ROADS + 1];   // first survivor of each road of the pass, from its start
-    unsigned long long at[2];       // the chunk holding survivor lo, and its first survivor
-    RoadRec rec[P5_STAGE];          // staged roads: records
-    uint4 row[P5_STAGE * N_LAYERS]; // and coordinate rows
+    svt_track track[P5_TRACKS];
 };
-
-// the last road r of [lo, hi) with first[r] <= k (the road of survivor k)
-__device__ __forceinline__ unsigned p5_road(const unsigned *first, unsigned lo, unsigned hi, unsigned k)
-{
-    while (hi - lo > 1) {
-        const unsigned mid = (lo + hi) >> 1;
-        if (first[mid] <= k)
-            lo = mid;
-        else
-            hi = mid;
-    }
-    return lo;
-}
-
-// survivor counts of roads g .. g + 7 (0 from n_roads on), one byte each
-__device__ __forceinline__ unsigned long long load_counts8(const Dev &d, unsigned g, unsigned n_roads)
-{
-    if (g + P5_PER_THREAD <= n_roads)
-        return ldcg(reinterpret_cast<const unsigned long long *>(d.surv_cnt + g));
-    unsigned long long v = 0;
-    for (unsigned k = 0; k < P5_PER_THREAD && g + k < n_roads; ++k)
-        v |= (unsigned long long)ldcg(d.surv_cnt + g + k) << (8 * k);
-    return v;
-}
 
 __device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads)
 {
     P5Smem &s = *reinterpret_cast<P5Smem *>(smem);
     const unsigned n_chunks = min((n_roads + ROAD_CHUNK - 1) / ROAD_CHUNK, d.max_chunks_r);
-    // each thread sums a contiguous range of chunk totals
-    const unsigned per = (n_chunks + BLOCK - 1) / BLOCK;
-    const unsigned c0 = min(threadIdx.x * per, n_chunks), c1 = min(c0 + per, n_chunks);
-    unsigned long long mine = 0;
-    for (unsigned c = c0; c < c1; ++c)
-        mine += ldcg(d.rchunk_sum + c);
-    unsigned long long S;
-    const unsigned long long ex = block_excl_scan(mine, &S);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        d.ctrl->n_out = S;
-        if (S > d.max_tracks)
-            raise_flag(d, FLAG_CAPACITY);
+    const unsigned lo = (unsigned)((unsigned long long)n_roads * blockIdx.x / gridDim.x);
+    const unsigned hi = (unsigned)((unsigned long long)n_roads * (blockIdx.x + 1) / gridDim.x);
+    const unsigned c_lo = lo / ROAD_CHUNK;
+    unsigned long long all = 0, before = 0;   // survivors of the batch, and of the roads before lo
+    for (unsigned c = threadIdx.x; c < n_chunks; c += BLOCK) {
+        const unsigned t = ldcg(d.rchunk_sum + c);
+        all += t;
+        before += c < c_lo ? t : 0u;
     }
-    if (S > d.max_tracks)
-        return;
-    const unsigned long long lo = S * blockIdx.x / gridDim.x, hi = S * (blockIdx.x + 1) / gridDim.x;
-    if (lo == hi)
-        return;
-    // the chunk holding survivor lo lies in one thread's range
-    if (ex <= lo && lo < ex + mine) {
-        unsigned c = c0;
-        unsigned long long pre = ex;
-        for (unsigned long long t = ldcg(d.rchunk_sum + c); pre + t <= lo; t = ldcg(d.rchunk_sum + c)) {
-            pre += t;
-            ++c;
-        }
-        s.at[0] = c;
-        s.at[1] = pre;
-    }
-    __syncthreads();
-    unsigned c = (unsigned)s.at[0];
-    unsigned long long pre = s.at[1];   // first survivor of chunk c
-    while (pre < hi && c < n_chunks) {
-        const unsigned g0 = c * ROAD_CHUNK, gt = g0 + threadIdx.x * P5_PER_THREAD;
-        const unsigned long long cnt8 = load_counts8(d, gt, n_roads);
-        unsigned mysum = 0;
+    for (unsigned g = c_lo * ROAD_CHUNK + threadIdx.x; g < lo; g += BLOCK)
+        before += ldcg(d.surv_cnt + g);
+    bool summed = false;
+    for (unsigned r0 = lo; r0 < hi || !summed; r0 += BLOCK) {
+        const unsigned g = r0 + threadIdx.x;
+        unsigned cnt = 0;
+        RoadRec rec{};
+        unsigned long long key = 0;
+        uint4 rw[N_LAYERS];
+        if (g < hi) {
+            cnt = ldcg(d.surv_cnt + g);
+            rec = ldcg(d.roads + g);
+            key = ldcg(d.surv_pool + surv_at(d, g, 0));   // (unspecified when there is none)
+            const uint4 *row = reinterpret_cast<const uint4 *>(d.coords + (size_t)g * 40);
 #pragma unroll
-        for (unsigned k = 0; k < P5_PER_THREAD; ++k)
-            mysum += (unsigned)(cnt8 >> (8 * k)) & 0xFFu;
-        unsigned long long tot;
-        unsigned run = (unsigned)block_excl_scan(mysum, &tot);
-#pragma unroll
-        for (unsigned k = 0; k < P5_PER_THREAD; ++k) {
-            s.first[threadIdx.x * P5_PER_THREAD + k] = run;
-            run += (unsigned)(cnt8 >> (8 * k)) & 0xFFu;
+            for (unsigned l = 0; l < N_LAYERS; ++l)
+                rw[l] = row[l];
         }
-        if (warp_id() == 0) {   // the counts and the chunk totals agree (a lane per chunk)
-            const unsigned k = lane_id();
-            const unsigned long long chk =
-                warp_sum(k < P5_GROUP && c + k < n_chunks ? ldcg(d.rchunk_sum + c + k) : 0ull);
-            if (k == 0) {
-                s.first[P5_ROADS] = (unsigned)tot;
-                if (chk != tot)
-                    raise_flag(d, FLAG_INTERNAL);
+        if (!summed) {
+            block_sum2(all, before);
+            summed = true;
+            if (blockIdx.x == 0 && threadIdx.x == 0) {
+                d.ctrl->n_out = all;
+                if (all > d.max_tracks)
+                    raise_flag(d, FLAG_CAPACITY);
             }
+            if (all > d.max_tracks)
+                return;
         }
-        __syncthreads();
-        const unsigned long long a = lo > pre ? lo : pre, b = hi < pre + tot ? hi : pre + tot;
-        if (a < b) {
-            // survivors ka .. kb of the pass lie in roads r_lo .. r_hi; their
-            // records and coordinate rows are staged with coalesced loads,
-            // P5_STAGE roads at a time
-            const unsigned ka = (unsigned)(a - pre), kb = (unsigned)(b - 1 - pre);
-            const unsigned r_lo = p5_road(s.first, 0, P5_ROADS, ka), r_hi = p5_road(s.first, 0, P5_ROADS, kb);
-            for (unsigned rb = r_lo; rb <= r_hi; rb += P5_STAGE) {
-                const unsigned re = min(rb + P5_STAGE, r_hi + 1), nr = re - rb;
-                // the thread's first survivor of the stage: its key is loaded
-                // together with the stage
-                const unsigned k0 = max(ka, s.first[rb]), k1 = min(kb + 1, s.first[re]);
-                const unsigned kf = k0 + threadIdx.x;
-                unsigned rf = 0;
-                unsigned long long keyf = 0;
-                if (kf < k1) {
-                    rf = p5_road(s.first, rb, re, kf);
-                    keyf = ldcg(d.surv_pool + surv_at(d, g0 + rf, kf - s.first[rf]));
-                }
-                for (unsigned j = threadIdx.x; j < nr; j += BLOCK)
-                    s.rec[j] = ldcg(d.roads + g0 + rb + j);
-                const uint4 *rows = reinterpret_cast<const uint4 *>(d.coords + (size_t)(g0 + rb) * 40);
-                for (unsigned j = threadIdx.x; j < nr * N_LAYERS; j += BLOCK)
-                    s.row[j] = ldcg(rows + j);
-                __syncthreads();
-                for (unsigned k = kf; k < k1; k += BLOCK) {
-                    const unsigned r = k == kf ? rf : p5_road(s.first, rb, re, k), g = g0 + r;
-                    const unsigned long long key =
-                        k == kf ? keyf : ldcg(d.surv_pool + surv_at(d, g, k - s.first[r]));
-                    uint4 rw[N_LAYERS];
-#pragma unroll
-                    for (unsigned l = 0; l < N_LAYERS; ++l)
-                        rw[l] = s.row[(r - rb) * N_LAYERS + l];
-                    build_track<false>(d, g, s.rec[r - rb], rw, key, pre + k);
-                }
-                __syncthreads();   // the stage is refilled next
-            }
+        unsigned tot;
+        const unsigned at = block_excl_scan32(cnt, &tot);
+        const bool gather = tot <= P5_TRACKS;
+        svt_track *out = gather ? s.track : d.tracks + before;
+        for (unsigned i = 0; i < cnt; ++i) {
+            if (i)
+                key = ldcg(d.surv_pool + surv_at(d, g, i));
+            if (gather || before + at + i < d.max_tracks)
+                build_track<false>(d, g, rec, rw, key, out + at + i);
         }
-        pre += tot;
-        c += P5_GROUP;
-        __syncthreads();   // the table is refilled next
+        if (gather) {
+            __syncthreads();
+            static_assert(sizeof(svt_track) % 8 == 0, "whole words");
+            const unsigned long long *src = reinterpret_cast<const unsigned long long *>(s.track);
+            unsigned long long *dst = reinterpret_cast<unsigned long long *>(d.tracks + before);
+            for (unsigned i = threadIdx.x; i < tot * (sizeof(svt_track) / 8); i += BLOCK)
+                dst[i] = src[i];
+            __syncthreads();
+        }
+        before += tot;
     }
+    // the roads' counts and the chunk totals agree
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && before != all)
+        raise_flag(d, FLAG_INTERNAL);
 }
 
 // Leave the group table empty: every claimed slot (its bit) is cleared, with

@@ -53,10 +53,9 @@ void drop_graph(svt_ctx *c)
     c->g_mode = -1;
 }
 
+// the last batch's control block, which its kernel wrote to h_ctrl
 int read_ctrl(svt_ctx *c, cudaStream_t s)
 {
-    if (cudaMemcpyAsync(c->h_ctrl, c->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-        return SVT_E_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess)
         return SVT_E_CUDA;
     if (c->h_ctrl->flags & FLAG_TIMEOUT)
@@ -73,35 +72,40 @@ int ensure_plain_buffers(svt_ctx *c)
     return SVT_OK;
 }
 
-// Clear the group table on s if a batch stopped before leaving it empty.
+// Clear the group table and the control block on s if a batch stopped before
+// leaving them empty.
 cudaError_t clear_if_dirty(svt_ctx *c, cudaStream_t s)
 {
     if (!c->hash_dirty)
         return cudaSuccess;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(c->d.hash, 0, sizeof(HashSlot) * (size_t)(c->d.hash_mask + 1), s)) ||
+    if ((e = cudaMemsetAsync(c->d.ctrl, 0, sizeof(Ctrl), s)) ||
+        (e = cudaMemsetAsync(c->d.hash, 0, sizeof(HashSlot) * (size_t)(c->d.hash_mask + 1), s)) ||
         (e = cudaMemsetAsync(c->d.hash_bits, 0, sizeof(uint32_t) * (c->d.hash_mask / 32 + 1), s)))
         return e;
     c->hash_dirty = false;
     return cudaSuccess;
 }
 
-// enqueue one batch (ctrl reset + kernels) on s
+// enqueue one batch's kernels on s
 cudaError_t enqueue(svt_ctx *c, int mode, cudaStream_t s, int *launches)
 {
     Dev d = c->d;
     d.wait_ns = c->wait_ns;
     d.skip_arrival = mode == SVT_PERSISTENT ? c->skip_arrival : 0;
-    cudaError_t e = cudaMemsetAsync(c->d.ctrl, 0, sizeof(Ctrl), s);
-    if (e || (e = clear_if_dirty(c, s)))
+    cudaError_t e = clear_if_dirty(c, s);
+    if (e)
         return e;
     if (mode == SVT_PLAIN) {
-        if ((e = launch_unpack_plain(d, s, launches)))
-            return e;
-        return launch_fit_plain(d, s, launches);
+        if (!(e = launch_unpack_plain(d, s, launches)))
+            e = launch_fit_plain(d, s, launches);
+    } else {
+        c->skip_arrival = 0;   // the test hook holds for one persistent launch
+        e = launch_persistent(c->block, d, s, c->blocks_per_sm, c->max_ctas, launches);
     }
-    c->skip_arrival = 0;   // the test hook holds for one persistent launch
-    return launch_persistent(c->block, d, s, c->blocks_per_sm, c->max_ctas, launches);
+    if (e)
+        c->hash_dirty = true;   // nothing says how much of the batch ran
+    return e;
 }
 
 }  // namespace
@@ -167,7 +171,7 @@ int svt_create(svt_ctx **out, int device, const svt_limits *lim)
     d.small_n4 = N4_SMALL_MAX;
     d.run_roads = RUN_ROADS;
     bool ok =
-        !dalloc(c, &d.ctrl, 1) && !dalloc(c, const_cast<svt_const_set **>(&d.consts), N_SETS) &&
+        !dalloc(c, &d.ctrl, 1) && !dalloc(c, &d.last, 1) && !dalloc(c, const_cast<svt_const_set **>(&d.consts), N_SETS) &&
         !dalloc(c, &d.span_ee, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.span_ep, MAX_SPANS + MAX_GRID) &&
         !dalloc(c, &d.span_seg, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.wmask, L.max_words / 32 + 1) && !dalloc(c, &d.ev_road_end, L.max_events) && !dalloc(c, &d.ev_big, L.max_events) &&
         !dalloc(c, &d.roads, L.max_roads) && !dalloc(c, &d.coords, (size_t)L.max_roads * 40) &&
@@ -181,10 +185,14 @@ int svt_create(svt_ctx **out, int device, const svt_limits *lim)
         !dalloc(c, &d.hash, L.hash_slots) && !dalloc(c, &d.hash_bits, L.hash_slots / 32 + 1) &&
         !dalloc(c, &d.comb_off, L.max_roads) && !dalloc(c, &d.tracks, L.max_tracks) &&
         cudaMallocHost(&c->h_ctrl, sizeof(Ctrl)) == cudaSuccess &&
+        cudaHostGetDevicePointer(reinterpret_cast<void **>(&d.host), c->h_ctrl, 0) == cudaSuccess &&
         cudaMemset(d.hash, 0, sizeof(HashSlot) * (size_t)L.hash_slots) == cudaSuccess &&
         cudaMemset(d.hash_bits, 0, sizeof(uint32_t) * (L.hash_slots / 32 + 1)) == cudaSuccess &&
-        cudaMemset(d.ctrl, 0, sizeof(Ctrl)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
+        cudaMemset(d.ctrl, 0, sizeof(Ctrl)) == cudaSuccess &&
+        cudaMemset(d.last, 0, sizeof(Ctrl)) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess;
     c->dev_tracks = d.tracks;
+    if (ok)
+        std::memset(c->h_ctrl, 0, sizeof(Ctrl));
     if (!ok) {
         free_all(c);
         delete c;
@@ -357,16 +365,16 @@ int svt_get_tracks(svt_ctx *c, svt_track *out, size_t cap, size_t *n_out, void *
     cudaStream_t s = (cudaStream_t)stream;
     if (cudaSetDevice(c->device))
         return SVT_E_CUDA;
-    // The status block and, speculatively, as many tracks as the previous
-    // batch had go out together, so a batch like the one before takes one
-    // synchronisation; the rest (if any) follows once the count is known.
+    // The batch's last kernel wrote the status block to the host.  As many
+    // tracks as the previous batch had are copied ahead of knowing the count,
+    // so a batch like the one before takes one synchronisation; the rest (if
+    // any) follows once the count is known.
     // With a host output buffer the tracks are there already: `out` equal to
     // it takes no copy.
     const bool in_place = c->host_out && out == c->host_out;
     const svt_track *src = c->host_out ? c->host_out : c->d.tracks;
     const size_t spec = out && !in_place ? std::min(cap, (size_t)c->last_n_out) : 0;
-    if (cudaMemcpyAsync(c->h_ctrl, c->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) ||
-        (spec && cudaMemcpyAsync(out, src, spec * sizeof(svt_track), cudaMemcpyDefault, s)) ||
+    if ((spec && cudaMemcpyAsync(out, src, spec * sizeof(svt_track), cudaMemcpyDefault, s)) ||
         cudaStreamSynchronize(s))
         return SVT_E_CUDA;
     if (c->h_ctrl->flags & FLAG_TIMEOUT)
@@ -401,8 +409,14 @@ int svt_get_roads(svt_ctx *c, svt_road *out, size_t cap, size_t *n_out, void *st
     if (!c->roads_valid) {
         int nl = 0;
         Dev d = c->d;
-        if (cudaMemsetAsync(c->d.ctrl, 0, sizeof(Ctrl), s) || launch_unpack_plain(d, s, &nl))
+        // unpacking alone: its control block is copied out and cleared here
+        if (clear_if_dirty(c, s) || launch_unpack_plain(d, s, &nl) ||
+            cudaMemcpyAsync(c->d.last, c->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToDevice, s) ||
+            cudaMemcpyAsync(c->h_ctrl, c->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) ||
+            cudaMemsetAsync(c->d.ctrl, 0, sizeof(Ctrl), s)) {
+            c->hash_dirty = true;
             return SVT_E_CUDA;
+        }
         c->roads_valid = true;
     }
     if (!c->d.road_out && dalloc(c, &c->d.road_out, c->lim.max_roads))

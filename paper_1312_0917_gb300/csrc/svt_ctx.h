@@ -10,7 +10,7 @@ struct svt_ctx {
     int device = 0;
     svt_limits lim{};
     svt::Dev d{};
-    svt::Ctrl *h_ctrl = nullptr;          // pinned mirror of the control block
+    svt::Ctrl *h_ctrl = nullptr;          // pinned: the last batch's control block, written by its kernel
     bool consts_loaded = false;
     bool bound = false;              // a batch is bound by svt_unpack
     bool roads_valid = false;        // the road table holds the bound batch
@@ -21,7 +21,7 @@ struct svt_ctx {
     int last_launches = 0;
     unsigned long long wait_ns = 2000000000ull;
     int skip_arrival = 0;
-    bool hash_dirty = false;         // a batch stopped before clearing its group table
+    bool hash_dirty = false;         // a batch stopped before clearing its group table and control block
     unsigned long long last_n_out = 0;   // tracks of the last batch read (svt_get_tracks' first copy)
     svt_track *dev_tracks = nullptr;     // the context's own track buffer (device memory)
     svt_track *host_out = nullptr;       // host buffer the output stage writes (svt_set_track_output)
@@ -87,11 +87,10 @@ inline int status_of(const Ctrl &c)
     return SVT_OK;
 }
 
-// Enqueue one batch of the words bound to c (control block reset, kernels)
-// on s; adds the kernel launches to *launches.
+// Enqueue the kernels of one batch of the words bound to c on s; adds the kernel launches to *launches.
 cudaError_t ctx_enqueue(svt_ctx *c, int mode, cudaStream_t s, int *launches);
 
-// Status of the batch whose control block is in c->h_ctrl (after a copy).
+// Status of the batch whose control block is in c->h_ctrl.
 int ctx_status(const svt_ctx *c);
 
 // Allocate what `mode` needs beyond svt_create (SVT_PLAIN's per-combination

@@ -54,9 +54,11 @@ inline void fit_words(const svt_const_set *sets, int32_t *out)
     }
 }
 
-// Per-batch control block in device memory; zeroed by the host before each
-// batch.  Queue counters hand out work items; `bar` counts grid-barrier
-// arrivals of the persistent kernel.
+// Per-batch control block in device memory.  It is zero before each batch: the
+// last CTA to leave a batch's last kernel copies it out (Dev::last, Dev::host)
+// and clears it, so a batch needs no memset before its kernel and no copy of
+// its status behind it.  Queue counters hand out work items; `bar` counts
+// grid-barrier arrivals of the persistent kernel.
 struct Ctrl {
     unsigned long long err_inv;   // max over faults of ~((pos << 8) | rank); 0 = none
     unsigned int bar;             // grid barrier arrivals; its polls read the flags with it
@@ -70,11 +72,11 @@ struct Ctrl {
     unsigned int n_box;           // roads of the box path (list length)
     unsigned int n_seg[10];       // roads of each half class of the group path (list lengths)
     unsigned int q[12];           // work-queue heads
-    unsigned int done[4];         // last-block-done counters
+    unsigned int done[4];         // last-block-done counters; [0]: CTAs that left the last kernel
     unsigned long long n_comb, n_pass, n_out;
     unsigned long long pad1[2];
     unsigned long long t_phase[8];   // persistent kernel: globaltimer at its start, after each
-                                     // barrier (block 0) and at the last CTA's exit (max)
+                                     // barrier (block 0) and when the last CTA leaves
 };
 
 // Unpacked road, 16 bytes.  pk: n[l] in bits 4l..4l+3 (l < 5), excluded layer
@@ -110,6 +112,8 @@ struct HashSlot {
 // Everything a kernel needs, passed by value.
 struct Dev {
     Ctrl *ctrl;
+    Ctrl *last, *host;     // what ctrl held at the end of the last batch: in device memory, and in the
+                           // caller's pinned host memory (null: none)
     const svt_const_set *consts;
     const uint32_t *words;
     unsigned long long n_words;

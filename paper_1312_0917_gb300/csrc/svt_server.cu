@@ -440,8 +440,6 @@ bool admit(svt_server *s, const uint32_t *words, size_t n_words, uint64_t parent
               cudaStreamWaitEvent(sl->stream, sl->ev_h2d, 0) == cudaSuccess &&
               svt_unpack(sl->ctx, sl->d_words, n_words, sl->stream) == SVT_OK &&
               ctx_enqueue(sl->ctx, s->cfg.mode, sl->stream, &launches) == cudaSuccess &&
-              cudaMemcpyAsync(sl->ctx->h_ctrl, sl->ctx->d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost,
-                              sl->stream) == cudaSuccess &&
               cudaEventRecord(sl->ev_ctrl, sl->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();

@@ -34,7 +34,8 @@ constexpr size_t up256(size_t b) { return (b + 255) / 256 * 256; }
 
 // byte offsets of the arena's regions
 constexpr size_t OFF_CTRL = 0;
-constexpr size_t OFF_CONSTS = OFF_CTRL + up256(sizeof(Ctrl));
+constexpr size_t OFF_LAST = OFF_CTRL + up256(sizeof(Ctrl));
+constexpr size_t OFF_CONSTS = OFF_LAST + up256(sizeof(Ctrl));
 constexpr unsigned S_SPANS = MAX_SPANS + MAX_GRID;   // per-warp word spans, then per-CTA totals
 constexpr size_t OFF_SPAN = OFF_CONSTS + up256(sizeof(svt_const_set) * N_SETS);    // 3 x [S_SPANS] u32
 constexpr size_t OFF_WMASK = OFF_SPAN + up256(3 * sizeof(uint32_t) * S_SPANS);      // [S_WORDS / 32 + 1] uint2
@@ -112,6 +113,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     }
     Dev d{};
     d.ctrl = reinterpret_cast<Ctrl *>(b + OFF_CTRL);
+    d.last = reinterpret_cast<Ctrl *>(b + OFF_LAST);
     d.consts = reinterpret_cast<const svt_const_set *>(b + OFF_CONSTS);
     d.words = d_words;
     d.n_words = n_words;
@@ -151,20 +153,21 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     d.run_roads = RUN_ROADS;
     d.wait_ns = 2000000000ull;
 
-    // what must start at zero: the control block every batch, the group
-    // table on the first batch and after one that did not finish
+    // what must start at zero and is left so by a batch that completes: the
+    // control block and the group table
     int launches = 0;
     std::vector<int32_t> fw((size_t)N_SETS * SET_INT4 * 4);   // lives until the stream is synchronized below
     fit_words(sets, fw.data());
     if (cudaMemcpyAsync(b + OFF_CONSTS, sets, sizeof(svt_const_set) * N_SETS, cudaMemcpyHostToDevice, s) ||
         cudaMemcpyAsync(d.fitc, fw.data(), sizeof(int32_t) * fw.size(), cudaMemcpyHostToDevice, s) ||
-        cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), s) ||
-        (da->hash_dirty && (cudaMemsetAsync(d.hash, 0, sizeof(HashSlot) * S_HASH, s) ||
+        (da->hash_dirty && (cudaMemsetAsync(d.ctrl, 0, sizeof(Ctrl), s) ||
+                            cudaMemsetAsync(d.hash, 0, sizeof(HashSlot) * S_HASH, s) ||
                             cudaMemsetAsync(d.hash_bits, 0, sizeof(uint32_t) * (S_HASH / 32 + 1), s))) ||
         launch_persistent(256, d, s, 0, 0, &launches))
         return SVT_E_CUDA;
+    da->hash_dirty = true;   // until the batch is known to have finished
     Ctrl h;
-    if (cudaMemcpyAsync(&h, d.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) || cudaStreamSynchronize(s))
+    if (cudaMemcpyAsync(&h, d.last, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) || cudaStreamSynchronize(s))
         return SVT_E_CUDA;
     da->hash_dirty = (h.flags & FLAG_TIMEOUT) != 0;
     const int st = status_of(h);

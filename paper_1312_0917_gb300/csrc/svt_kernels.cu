@@ -31,6 +31,7 @@
 // The block size of every kernel is SVT_BLOCK (256 unless the including
 // file sets it); each block size builds in a namespace of its own, and only
 // the 256-thread build holds the plain pipeline.
+#include <algorithm>
 #include <cstddef>
 
 #include "svt_internal.h"
@@ -1551,10 +1552,16 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2Lis
     __syncwarp();   // the state is refilled for the next event
 }
 
-// P2 over the events.  At most one per CTA: a CTA each.  More: those of more
-// than P2W_ROADS roads (listed in P1) a CTA each from a queue, then every warp takes the other events one at a time, its
-// first by its own index (neighbouring indices on different SMs), the rest
-// from a queue.  One combination-count atomic per CTA.
+// P2 over the events.  At most P2_ROUNDS per CTA: a CTA each.  More: those of
+// more than P2W_ROADS roads (listed in P1) a CTA each from a queue, then every
+// warp takes the other events one at a time, its first by its own index
+// (neighbouring indices on different SMs), the rest from a queue.  An event of
+// 64 roads takes a warp some 18 us whether it is alone or not, a CTA 6 us, so
+// the line is at three: a chain of 400 events of one to eight hits on 152 CTAs
+// 103 us with a warp each, 99 us with a CTA each, 1100 events that share hits
+// on 456 CTAs 89.9 -> 87.3 us, 170 events on 152 CTAs 48.1 -> 40.5 us.  One
+// combination-count atomic per CTA.
+constexpr unsigned P2_ROUNDS = 3;
 constexpr size_t P2_LIST_AT = (sizeof(P2Smem) > WARPS * P2W_BYTES ? sizeof(P2Smem) : WARPS * P2W_BYTES) / 16 * 16 + 16;
 
 // The end of P2 in a CTA: its list goes out, its combinations are counted.
@@ -1590,10 +1597,10 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
         const unsigned r1 = min(ldcg(d.ev_road_end + e), d.max_roads);
         return min(r1 - min(r0, r1), (unsigned)MAX_ROADS_EV);
     };
-    if (n_events <= gridDim.x) {   // few: a CTA each is the shortest time per event
-        if (e0 < n_events) {
+    if (n_events <= P2_ROUNDS * gridDim.x) {   // few: a CTA each is the shortest time per event
+        for (unsigned e = e0; e < n_events; e += gridDim.x) {
             unsigned r0;
-            const unsigned nr = roads_of(e0, r0);
+            const unsigned nr = roads_of(e, r0);
             p2_event(d, r0, nr, smem, list, n_comb);
         }
         p2_finish(d, list, n_comb);
@@ -3885,7 +3892,19 @@ cudaError_t launch_persistent(const Dev &d, cudaStream_t s, int blocks_per_sm, i
     int maxb = persistent_max_blocks_per_sm(dev);
     if (maxb <= 0)
         return cudaErrorInvalidConfiguration;
-    int bps = blocks_per_sm > 0 && blocks_per_sm < maxb ? blocks_per_sm : maxb;
+    // Every CTA costs each barrier an arrival and each stage its first loads and
+    // instructions, so the grid grows with the batch: 256 threads an SM up to 640
+    // words an SM (97k words on 152 SMs), 512 up to 3072 (467k), then all that
+    // fit.  Device time with one, two and three CTAs of 256 an SM, us: one event
+    // of 977 words 27.5 / 28.9 / 30.5, 8k words 24.7 / 26.8 / 30.4, 99k words
+    // 37.1 / 38.4 / 41.7, 155k words 61 / 57 / 61 (shared hits), 495k words
+    // 57.4 / 51.2 / 53.3, 978k words 158 / 119 / 110 (one to eight hits).  Just
+    // below each line no kind of batch was slower than with all that fit.
+    int bps = maxb;
+    if (blocks_per_sm > 0)
+        bps = blocks_per_sm < maxb ? blocks_per_sm : maxb;
+    else if (d.n_words <= 3072ull * sms)
+        bps = std::min(maxb, std::max((d.n_words <= 640ull * sms ? 256 : 512) / BLOCK, 1));
     Dev dd = d;
     void *args[] = {&dd};
     cudaLaunchConfig_t cfg = {};

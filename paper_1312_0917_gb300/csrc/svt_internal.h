@@ -27,8 +27,15 @@ constexpr unsigned long long NO_KEY = ~0ull;
 // truncation is reported at position n_words, after every word
 enum : unsigned { RANK_BAD = 1, RANK_LIMIT = 2, RANK_TRUNC = 3 };
 // FLAG_FAULT: the stream has a fault (err_inv is set); FLAG_GROUPS: the group
-// table has an entry
-enum : unsigned { FLAG_CAPACITY = 1, FLAG_TIMEOUT = 2, FLAG_INTERNAL = 4, FLAG_FAULT = 8, FLAG_GROUPS = 16 };
+// table has an entry; FLAG_CANDS: a road is a cross-road candidate
+enum : unsigned {
+    FLAG_CAPACITY = 1,
+    FLAG_TIMEOUT = 2,
+    FLAG_INTERNAL = 4,
+    FLAG_FAULT = 8,
+    FLAG_GROUPS = 16,
+    FLAG_CANDS = 32
+};
 
 // The kernels' copy of each set's constants as int32 in 16-byte words, 14
 // per set: words 0..5 hold F row by row, then q and three zeros (the output

@@ -1215,6 +1215,8 @@ __device__ __forceinline__ unsigned finish_road(const Dev &d, P2List &list, bool
         if (N > 0 && cand)   // checked against the other roads' groups after the fit
             atomicOr(&d.cand_bits[g >> 5], 1u << (g & 31u));
     }
+    if (__any_sync(FULL_MASK, N > 0 && cand) && lane == 0)
+        raise_flag(d, FLAG_CANDS);
     const unsigned mg = __ballot_sync(FULL_MASK, cls < N_GROUP_CLS), mb = __ballot_sync(FULL_MASK, cls == CLS_BOX);
     unsigned at = 0;
     if (lane == 0 && mg)
@@ -1672,27 +1674,35 @@ constexpr unsigned HASH_PROBES = 64;
 
 __device__ __forceinline__ unsigned hash_probes(const Dev &d) { return min(HASH_PROBES, d.hash_mask + 1); }
 
-__device__ void hash_min(const Dev &d, unsigned long long gk, unsigned long long key)
+__device__ unsigned hash_min(const Dev &d, unsigned long long gk, unsigned long long key)
 {
     unsigned h = hash_slot(gk, d.hash_mask);
-    const unsigned slots = d.hash_mask + 1;
     for (unsigned probe = 0; probe < hash_probes(d); ++probe) {
         unsigned long long prev = atomicCAS(&d.hash[h].key, 0ull, gk);
         if (prev == 0ull) {   // a new slot: marked for clearing (no value awaited)
             atomicOr(&d.hash_bits[h >> 5], 1u << (h & 31u));
-            const unsigned used = atomicAdd(&d.ctrl->hash_used, 1u);
-            if (used == 0)
-                raise_flag(d, FLAG_GROUPS);
-            if (used >= slots - slots / 4)
-                raise_flag(d, FLAG_CAPACITY);
         }
         if (prev == 0ull || prev == gk) {
             atomicMax(&d.hash[h].val_inv, ~key);
-            return;
+            return prev == 0ull;
         }
         h = (h + 1) & d.hash_mask;
     }
     raise_flag(d, FLAG_CAPACITY);
+    return 0;
+}
+
+// The warp's new slots of the group table join the batch's count.
+__device__ void hash_count(const Dev &d, unsigned n)
+{
+    n = __reduce_add_sync(FULL_MASK, n);
+    if (lane_id() == 0 && n) {
+        const unsigned used = atomicAdd(&d.ctrl->hash_used, n), slots = d.hash_mask + 1;
+        if (used == 0)
+            raise_flag(d, FLAG_GROUPS);
+        if (used + n > slots - slots / 4)
+            raise_flag(d, FLAG_CAPACITY);
+    }
 }
 
 // lookup after the table is complete (no writer in flight): a slot's key and
@@ -1852,82 +1862,172 @@ __device__ __forceinline__ void group_rank(GroupFound<YN> &f, unsigned gmask)
     }
 }
 
-// Publish, for each cross-road candidate among the warp's roads (no repeated
-// coordinate in a layer, so every hit is canonical), the minimum key of every
-// group (layer triple, three coordinates) whose three hits are flagged as
-// shared with another road of the event: the road's lanes take its groups.
-template <bool PLAIN, class Road>
-__device__ __noinline__ void group_publish(const Dev &d, const Road &r, bool publish)
+// ---------------------------------------------------------------------------
+// P3, publish: the groups of the cross-road candidates.  A group is a layer
+// triple and three coordinates whose three hits are flagged as shared with
+// another road of the event; the table gets the lowest key of the road's
+// passing fits in it.  This takes a road none of whose layers repeats a
+// coordinate (every hit is canonical).
+//
+// A candidate has few groups (1.7 on average where 60 % of the hits are
+// shared, and one road in five is a candidate), so the candidates of 32 roads
+// put theirs together, one group a lane, and the lane computes its fits anew
+// from the road's coordinates and constants.  Publishing in the fit's own step
+// (two lanes of 32 at work, nearly every step waiting for the mask, the
+// coordinates and the table) took 30 of 68 us of the fit stage for 1501 events
+// that share hits.
+// ---------------------------------------------------------------------------
+
+// flagged hits of layer l: byte l of the mask; groups of triple t
+__device__ __forceinline__ unsigned flagged(unsigned long long xm, unsigned l) { return (unsigned)(xm >> (8 * l)) & 0xFFu; }
+__device__ __forceinline__ unsigned groups_of(unsigned long long xm, unsigned t)
 {
-    const unsigned g = r.it.g, excl = r.excl;
-    if (publish) {
-        const unsigned long long xm = ldcg(d.xmask + g);   // flagged hits of layer l: byte l
-        const unsigned event = ldcg(&d.roads[g].event);
-        unsigned Se = 1;   // comb stride of the excluded layer
-        for (unsigned l = 0; l < excl; ++l)
-            Se *= (r.it.pk >> (4 * l)) & 15u;
-        const auto fl = [xm](unsigned l) { return (unsigned)(xm >> (8 * l)) & 0xFFu; };
-        const auto groups = [&fl](unsigned t) {   // groups of triple t
-            return __popc(fl(triple_l(t, 0))) * __popc(fl(triple_l(t, 1))) * __popc(fl(triple_l(t, 2)));
-        };
-        unsigned total = 0;
+    return __popc(flagged(xm, triple_l(t, 0))) * __popc(flagged(xm, triple_l(t, 1))) *
+           __popc(flagged(xm, triple_l(t, 2)));
+}
+__device__ __forceinline__ unsigned groups_of(unsigned long long xm)
+{
+    unsigned total = 0;
 #pragma unroll
-        for (unsigned t = 0; t < 10; ++t)
-            total += groups(t);
-        for (unsigned gi = lane_id() % Road::G; gi < total; gi += Road::G) {
-            unsigned t = 0, rem = gi;
-            bool found = false;
+    for (unsigned t = 0; t < 10; ++t)
+        total += groups_of(xm, t);
+    return total;
+}
+
+__device__ __forceinline__ int4 mad4(const int4 &b, const int4 &c, int v, unsigned w)
+{
+    return make_int4(b.x + c.x * v, b.y + c.y * v, b.z + c.z * v, b.w + (int)w);
+}
+
+// Publish group gi of road g (record r, flagged hits xm); 1 if it claimed a slot.
+__device__ __noinline__ unsigned publish_group(const Dev &d, unsigned g, const RoadRec &r, unsigned long long xm,
+                                               unsigned gi)
+{
+    const uint32_t pk = r.pk;
+    const unsigned excl = min((pk >> 20) & 7u, 4u);
+    unsigned t = 0, rem = gi;
+    bool found = false;
 #pragma unroll
-            for (unsigned tt = 0; tt < 10; ++tt) {   // the triple of group gi
-                const unsigned c = groups(tt);
-                if (!found) {
-                    if (rem < c) {
-                        t = tt;
-                        found = true;
-                    } else {
-                        rem -= c;
-                    }
-                }
-            }
-            const unsigned lt[3] = {triple_l(t, 0), triple_l(t, 1), triple_l(t, 2)};
-            const unsigned f0 = fl(lt[0]), f1 = fl(lt[1]), f2 = fl(lt[2]);
-            const unsigned p0 = __popc(f0), p1 = __popc(f1);   // at most 8 each: the quotients are divm's
-            const unsigned r1 = divm(rem, c_magic[p0]), r2 = divm(r1, c_magic[p1]);
-            const unsigned dsel[3] = {nth_bit(f0, rem - r1 * p0), nth_bit(f1, r1 - r2 * p1), nth_bit(f2, r2)};
-            // the triple's fitted slots are fixed, the other fitted slots
-            // (one, or two when the triple has the excluded layer) run over
-            // their hits
-            int4 base = make_int4(0, 0, 0, 0);
-            unsigned de = 0, rest = 0xFu;
-#pragma unroll
-            for (unsigned q = 0; q < 3; ++q) {
-                if (lt[q] == excl) {
-                    de = dsel[q];
-                } else {
-                    const unsigned s = lt[q] - (lt[q] > excl);
-                    base = add4(base, r.hit[r.first(s) + dsel[q]]);
-                    rest &= ~(1u << s);
-                }
-            }
-            const unsigned su = __ffs(rest) - 1, sv = 31 - __clz(rest);   // the same slot when one is free
-            const unsigned mv = su == sv ? 1u : r.m(sv);
-            unsigned long long mn = NO_KEY;
-            for (unsigned u = 0; u < r.m(su); ++u) {
-                const int4 bu = add4(base, r.hit[r.first(su) + u]);
-                for (unsigned v = 0; v < mv; ++v) {
-                    const unsigned long long k = r.template key<PLAIN>(d, d.cut, su == sv ? bu : add4(bu, r.hit[r.first(sv) + v]));
-                    mn = k < mn ? k : mn;
-                }
-            }
-            if (mn != NO_KEY) {   // the excluded layer's hit of the group, or its lowest
-                const uint16_t *co = d.coords + (size_t)g * 40;
-                hash_min(d, group_key(event, t, ldcg(co + lt[0] * 8 + dsel[0]), ldcg(co + lt[1] * 8 + dsel[1]),
-                                      ldcg(co + lt[2] * 8 + dsel[2])),
-                         mn + (unsigned long long)de * Se);
+    for (unsigned tt = 0; tt < 10; ++tt) {   // the triple of group gi
+        const unsigned c = groups_of(xm, tt);
+        if (!found) {
+            if (rem < c) {
+                t = tt;
+                found = true;
+            } else {
+                rem -= c;
             }
         }
     }
+    const unsigned lt[3] = {triple_l(t, 0), triple_l(t, 1), triple_l(t, 2)};
+    const unsigned f0 = flagged(xm, lt[0]), f1 = flagged(xm, lt[1]), f2 = flagged(xm, lt[2]);
+    const unsigned p0 = __popc(f0), p1 = __popc(f1);   // at most 8 each: the quotients are divm's
+    const unsigned r1 = divm(rem, c_magic[p0]), r2 = divm(r1, c_magic[p1]);
+    const unsigned dsel[3] = {nth_bit(f0, rem - r1 * p0), nth_bit(f1, r1 - r2 * p1), nth_bit(f2, r2)};
+    // every load in one trip
+    const uint16_t *co = d.coords + (size_t)g * 40;
+    const int4 *cc = d.fitc + SET_INT4 * min((unsigned)r.set, (unsigned)(N_SETS - 1)) + SET_C;
+    unsigned v[3], rest = 0xFu;   // rest: the fitted slots outside the triple
+    int4 ct[3];
+#pragma unroll
+    for (unsigned q = 0; q < 3; ++q) {
+        v[q] = ldcg(co + lt[q] * 8 + dsel[q]);
+        const unsigned sl = min(lt[q] - (lt[q] > excl), 3u);
+        ct[q] = __ldg(cc + sl);
+        rest &= lt[q] == excl ? ~0u : ~(1u << sl);
+    }
+    // one, or two when the triple has the excluded layer (one: u and v the same)
+    const unsigned su = __ffs(rest) - 1, sv = 31 - __clz(rest), Lu = su + (su >= excl), Lv = sv + (sv >= excl);
+    const uint4 hu = ldcg(reinterpret_cast<const uint4 *>(co + Lu * 8)),
+                hv = ldcg(reinterpret_cast<const uint4 *>(co + Lv * 8));
+    const int4 cu = __ldg(cc + su), cv = __ldg(cc + sv), c4 = __ldg(cc + 4), c5 = __ldg(cc + 5), kk = __ldg(cc + 6);
+    const unsigned S1 = pk & 15u, S2 = S1 * ((pk >> 4) & 15u), S3 = S2 * ((pk >> 8) & 15u),
+                   S4 = S3 * ((pk >> 12) & 15u);   // comb strides of the layers
+    const auto stride = [&](unsigned L) { return L == 0 ? 1u : L == 1 ? S1 : L == 2 ? S2 : L == 3 ? S3 : S4; };
+    int4 base = make_int4(c4.x * r.curv + c5.x * r.phi + 4096 * kk.x, c4.y * r.curv + c5.y * r.phi + 4096 * kk.y,
+                          c4.z * r.curv + c5.z * r.phi + 4096 * kk.z, (int)((pk >> 24) << 15));
+#pragma unroll
+    for (unsigned q = 0; q < 3; ++q)   // the excluded layer's hit counts in the comb alone
+        base = mad4(base, ct[q], lt[q] == excl ? 0 : (int)v[q], dsel[q] * stride(lt[q]));
+    const unsigned mu = (pk >> (4 * Lu)) & 15u, mv = su == sv ? 1u : (pk >> (4 * Lv)) & 15u, Su = stride(Lu), Sv = stride(Lv);
+    unsigned long long mn = NO_KEY;
+    for (unsigned a = 0; a < mu; ++a) {
+        const int4 bu = mad4(base, cu, (int)row_at(hu, a), a * Su);
+        for (unsigned b = 0; b < mv; ++b) {
+            bool pass;
+            const unsigned long long k =
+                box_key(su == sv ? bu : mad4(bu, cv, (int)row_at(hv, b), b * Sv), d.cut, pass);
+            mn = k < mn ? k : mn;
+        }
+    }
+    return mn == NO_KEY ? 0u : hash_min(d, group_key(r.event, t, v[0], v[1], v[2]), mn);
+}
+
+// The groups of one road by the whole warp (the box path's roads, which have
+// the most).
+__device__ __noinline__ void publish_road(const Dev &d, unsigned g, const RoadRec &r)
+{
+    const unsigned long long xm = ldcg(d.xmask + g);
+    const unsigned total = groups_of(xm);
+    unsigned fresh = 0;
+    for (unsigned gi = lane_id(); gi < total; gi += 32)
+        fresh += publish_group(d, g, r, xm, gi);
     __syncwarp();
+    hash_count(d, fresh);
+}
+
+// Part `part` of `parts` of the groups of the candidates among roads
+// 32 w .. 32 w + 31 that the group path fits.
+__device__ __forceinline__ void publish_word(const Dev &d, unsigned w, unsigned part, unsigned parts, unsigned n_roads)
+{
+    const unsigned lane = lane_id(), g = w * 32 + lane;
+    const bool cand = ((ldcg(d.cand_bits + w) >> lane) & 1u) && g < n_roads;
+    RoadRec r{};
+    unsigned long long xm = 0;
+    if (cand) {
+        r = ldcg(d.roads + g);
+        xm = ldcg(d.xmask + g);
+    }
+    const unsigned total = cand && ((r.fit >> 8) & 7u) < N_GROUP_CLS ? groups_of(xm) : 0u;
+    unsigned inc = total;   // groups up to and with the lane's road
+#pragma unroll
+    for (unsigned o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(FULL_MASK, inc, o);
+        inc += lane >= o ? u : 0u;
+    }
+    const unsigned all = __shfl_sync(FULL_MASK, inc, 31);
+    unsigned fresh = 0;
+    for (unsigned i0 = 32 * part; i0 < all; i0 += 32 * parts) {
+        const unsigned i = i0 + lane;
+        unsigned src = 0;   // roads whose groups all lie below i
+#pragma unroll
+        for (unsigned o = 16; o; o >>= 1)
+            src += __shfl_sync(FULL_MASK, inc, src + o - 1) <= i ? o : 0u;
+        const unsigned gi = i - __shfl_sync(FULL_MASK, inc - total, src);
+        uint4 v;
+        memcpy(&v, &r, sizeof v);
+        v.x = __shfl_sync(FULL_MASK, v.x, src);
+        v.y = __shfl_sync(FULL_MASK, v.y, src);
+        v.z = __shfl_sync(FULL_MASK, v.z, src);
+        v.w = __shfl_sync(FULL_MASK, v.w, src);
+        RoadRec rs;
+        memcpy(&rs, &v, sizeof v);
+        const unsigned long long xs = __shfl_sync(FULL_MASK, xm, src);
+        if (i < all)
+            fresh += publish_group(d, w * 32 + src, rs, xs, gi);
+        __syncwarp();
+    }
+    hash_count(d, fresh);
+}
+
+// The groups of every word's candidates, a word in as many parts as there are
+// warps for.
+__device__ __noinline__ void publish_words(const Dev &d)
+{
+    const unsigned n_roads = min(ldcg(&d.ctrl->n_roads), d.max_roads), words = (n_roads + 31) / 32;
+    const unsigned n_warps = gridDim.x * WARPS, parts = words ? max(n_warps / words, 1u) : 1u;
+    for (unsigned i = warp_id() * gridDim.x + blockIdx.x; i < words * parts; i += n_warps)
+        publish_word(d, i % words, i / words, parts, n_roads);
 }
 
 // ---------------------------------------------------------------------------
@@ -2530,15 +2630,9 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
         if (n_surv)
             atomicAdd(&d.rchunk_sum[g / ROAD_CHUNK], n_surv);
     }
-    if ((pk >> 23) & 1u) {   // a cross-road candidate: its hits lie as a group's of this shape would
-        GroupRoad<3, 2, 2, 8> r;
-        r.it = RoadItem{g, pk, rec.curv, rec.phi, rec.set, (uint16_t)(rec.fit & 0xFFu)};
-        r.hit = &B.A[0][0];
-        r.nf = nf;
-        r.excl = excl;
-        r.cb = 0;
-        group_publish<false>(d, r, true);
-    }
+    // a cross-road candidate (one that the group path listed is published there)
+    if (((pk >> 23) & 1u) && ((rec.fit >> 8) & 7u) == CLS_BOX)
+        publish_road(d, g, rec);
     __syncwarp();
     return true;
 }
@@ -2742,7 +2836,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     // cross-road candidates: the minimum key of every group (layer triple,
     // three coordinates) whose three hits are canonical and flagged as
     // present in another road of the event
-    if ((pk >> 23) & 1u) {
+    if (((pk >> 23) & 1u) && ((rec.fit >> 8) & 7u) == CLS_BOX) {   // (the group path's are published there)
         // canonical hits of the excluded layer (lanes 0..7)
         unsigned xc = lane;
         const bool xv = lane < sh.ne;
@@ -2754,6 +2848,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
         const unsigned cmx = __ballot_sync(FULL_MASK, xv && xc == lane) & 0xFFu;
         const unsigned long long xm = ldcg(d.xmask + g);
         const unsigned event = rec.event;
+        unsigned fresh = 0;   // slots claimed
         unsigned long long flp = 0;
 #pragma unroll
         for (unsigned l = 0; l < N_LAYERS; ++l) {
@@ -2856,10 +2951,11 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
                     mn += (unsigned long long)de * Se;
             }
             if (mn != NO_KEY)
-                hash_min(d, group_key(event, t, B.co[lt[0] * 8 + dsel[0]], B.co[lt[1] * 8 + dsel[1]],
+                fresh += hash_min(d, group_key(event, t, B.co[lt[0] * 8 + dsel[0]], B.co[lt[1] * 8 + dsel[1]],
                                       B.co[lt[2] * 8 + dsel[2]]),
                          mn);
         }
+        hash_count(d, fresh);
     }
     __syncwarp();
 }
@@ -3128,11 +3224,6 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
             atomicAdd(&S.rchunk_sum[g / ROAD_CHUNK], f.cnt);
     }
     npass += tied ? 0u : np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
-    const bool publish = ((pk >> 23) & 1u) && !tied;
-    if (__any_sync(FULL_MASK, publish)) {   // on a copy, so that the road stays in registers
-        const Road rc = r;
-        group_publish<PLAIN>(d, rc, publish);
-    }
     __syncwarp();   // (the warp's memory may be the box path's next)
     return __ballot_sync(FULL_MASK, tied && gl == 0);
 }
@@ -3177,8 +3268,9 @@ __device__ __noinline__ void p3_boxes(const Dev &d, unsigned char *smem, unsigne
 // memory, so no part of P3 waits for the whole CTA.  Not inlined: the stages
 // before and after it keep a register allocation of their own (inlined, the
 // decode and the box path took 10 % and 3 % longer).
+// cands: the batch has cross-road candidates
 template <bool PLAIN>
-__device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbox, int qgroup)
+__device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbox, int qgroup, bool cands)
 {
     P3Shared &S = *reinterpret_cast<P3Shared *>(smem);
     unsigned long long npass = 0;
@@ -3236,6 +3328,8 @@ __device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbo
             group_step<PLAIN, GroupCls0, 9>(d, smem, s, np, npass);
     }
     __syncwarp();
+    if (cands)
+        publish_words(d);
     p3_boxes<PLAIN>(d, smem, n_box, qbox, npass);
     npass = block_sum(npass + np);
     if (!PLAIN && threadIdx.x == 0 && npass)
@@ -3246,18 +3340,28 @@ __device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbo
 // P4: cross-road hit-warrior and survivor counts, P5: output
 // ---------------------------------------------------------------------------
 
-__device__ unsigned cross_check(const Dev &d, unsigned g, unsigned cnt)
+__device__ unsigned cross_check(const Dev &d, unsigned g, unsigned &cnt)
 {
+    // everything about the road in one trip (the first survivor: unspecified
+    // when there is none), then the lookups
     const RoadRec rec = ldcg(d.roads + g);
     const unsigned long long xm = ldcg(d.xmask + g);
+    unsigned long long key = ldcg(d.surv_pool + surv_at(d, g, 0));
+    uint4 rw[N_LAYERS];
+#pragma unroll
+    for (unsigned l = 0; l < N_LAYERS; ++l)
+        rw[l] = ldcg(reinterpret_cast<const uint4 *>(d.coords + (size_t)g * 40) + l);
+    cnt = ldcg(d.surv_cnt + g);
+    if (!cnt || !((rec.pk >> 23) & 1u))
+        return cnt;
     unsigned n[N_LAYERS];
 #pragma unroll
     for (unsigned l = 0; l < N_LAYERS; ++l)
         n[l] = max(min((rec.pk >> (4 * l)) & 15u, (unsigned)MAX_HITS), 1u);
-    const uint16_t *co = d.coords + (size_t)g * 40;
     unsigned kept = 0;
     for (unsigned i = 0; i < cnt; ++i) {
-        unsigned long long key = ldcg(d.surv_pool + surv_at(d, g, i));
+        if (i)
+            key = ldcg(d.surv_pool + surv_at(d, g, i));
         unsigned t = (unsigned)(key & 0x7FFFu);
         unsigned dl[N_LAYERS], v[N_LAYERS];
 #pragma unroll
@@ -3265,7 +3369,7 @@ __device__ unsigned cross_check(const Dev &d, unsigned g, unsigned cnt)
             const unsigned q = divm(t, c_magic[n[l]]);
             dl[l] = t - q * n[l];
             t = q;
-            v[l] = ldcg(co + l * 8 + dl[l]);
+            v[l] = row_at(rw[l], dl[l]);
         }
         bool dropped = false;
 #pragma unroll
@@ -3289,11 +3393,9 @@ __device__ void p4_item(const Dev &d, unsigned c, unsigned n_roads)
     unsigned g = c * ROAD_CHUNK + threadIdx.x;
     unsigned cnt = 0;
     if (g < n_roads) {
-        cnt = ldcg(d.surv_cnt + g);
-        if (cnt && ((ldcg(&d.roads[g].pk) >> 23) & 1u)) {
-            cnt = cross_check(d, g, cnt);
-            d.surv_cnt[g] = (uint8_t)cnt;
-        }
+        const unsigned kept = cross_check(d, g, cnt);
+        if (kept != cnt)
+            d.surv_cnt[g] = (uint8_t)(cnt = kept);
     }
     unsigned long long tot = block_sum(cnt);
     if (threadIdx.x == 0)
@@ -3462,9 +3564,7 @@ __device__ void p4_cand_phase(const Dev &d, unsigned n_roads)
         const unsigned g = w * 32 + lane;
         if (!((bits >> lane) & 1u) || g >= n_roads)
             continue;   // not a candidate, or a road of the truncated tail (not fitted)
-        const unsigned cnt = ldcg(d.surv_cnt + g);
-        if (!cnt)
-            continue;
+        unsigned cnt;
         const unsigned kept = cross_check(d, g, cnt);
         if (kept != cnt) {
             d.surv_cnt[g] = (uint8_t)kept;
@@ -3608,7 +3708,7 @@ __device__ __forceinline__ bool chain(const Dev &d)
     if (fault)
         return false;
 
-    p3_phase<false>(d, smem, Q_BOX, Q_GROUP);
+    p3_phase<false>(d, smem, Q_BOX, Q_GROUP, flags & FLAG_CANDS);
     if (d.skip_arrival == 2 && blockIdx.x == 0)
         return false;   // test hook: this CTA leaves after publishing, the others' waits run out
     if (!grid_sync(d, 4, flags))
@@ -3778,7 +3878,7 @@ __global__ void __launch_bounds__(BLOCK) k_warrior_plain(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem[];
     if (stop_after_unpack(d))
         return;
-    p3_phase<true>(d, smem, Q_BOX, Q_GROUP);
+    p3_phase<true>(d, smem, Q_BOX, Q_GROUP, ldcg(&d.ctrl->flags) & FLAG_CANDS);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p4(Dev d)

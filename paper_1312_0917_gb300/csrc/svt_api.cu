@@ -173,7 +173,8 @@ int svt_create(svt_ctx **out, int device, const svt_limits *lim)
     bool ok =
         !dalloc(c, &d.ctrl, 1) && !dalloc(c, &d.last, 1) && !dalloc(c, const_cast<svt_const_set **>(&d.consts), N_SETS) &&
         !dalloc(c, &d.span_ee, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.span_ep, MAX_SPANS + MAX_GRID) &&
-        !dalloc(c, &d.span_seg, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.wmask, L.max_words / 32 + 1) && !dalloc(c, &d.ev_road_end, L.max_events) && !dalloc(c, &d.ev_big, L.max_events) &&
+        !dalloc(c, &d.span_seg, MAX_SPANS + MAX_GRID) && !dalloc(c, &d.wmask, L.max_words / 32 + 1) &&
+        !dalloc(c, &d.ev_road_end, L.max_events) && !dalloc(c, &d.ev_big, L.max_events) &&
         !dalloc(c, &d.roads, L.max_roads) && !dalloc(c, &d.coords, (size_t)L.max_roads * 40) &&
         !dalloc(c, &d.xmask, L.max_roads) && !dalloc(c, &d.box_list, L.max_roads) &&
         !dalloc(c, &d.items, (size_t)N_GROUP_CLS * L.max_roads) &&

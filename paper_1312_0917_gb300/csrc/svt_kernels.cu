@@ -441,7 +441,7 @@ __device__ __forceinline__ void stamp(const Dev &d, unsigned k)
 }
 
 // work-queue indices (Ctrl::q)
-enum { Q_P2 = 0, Q_BOX, Q_GROUP, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_FIT, Q_P2W };
+enum { Q_P2 = 0, Q_BOX, Q_GROUP, Q_P4, Q_P5, Q_CNT, Q_CSC, Q_P2W };
 
 // ---------------------------------------------------------------------------
 // P0 / P1: the word stream, one warp per span.  The stream is cut into
@@ -1637,8 +1637,9 @@ __device__ void p2_phase(const Dev &d, unsigned char *smem, Batch &bt)
 }
 
 // ---------------------------------------------------------------------------
-// P3: fit + cut + road-local hit-warrior: runs of roads per warp (the flat
-// path), the roads listed in P2 one per warp (the box path)
+// P3: fit + cut + road-local hit-warrior: roads of like shape several to a warp
+// step (the group path), larger ones a warp each (the box path), then the groups
+// of the cross-road candidates; all three by lists made in P2
 // ---------------------------------------------------------------------------
 
 // the same triples as constants the compiler folds in unrolled loops: layer
@@ -1804,12 +1805,6 @@ struct GroupRoad {
     __device__ unsigned slot(unsigned role) const { return (it.perm >> (2 * role)) & 3u; }
     __device__ unsigned m(unsigned s) const { return (nf >> (4 * s)) & 15u; }
     __device__ unsigned y(unsigned j) const { return yl + j * YL; }
-    __device__ bool has(unsigned j) const { return live && y(j) < mb; }
-    // first hit of fitted slot s in the table
-    __device__ unsigned first(unsigned s) const
-    {
-        return s == slot(0) ? 0u : A + B * (s == slot(1) ? 0u : s == slot(2) ? 1u : 2u);
-    }
     template <bool PLAIN>
     __device__ unsigned long long key(const Dev &d, long long cut, const int4 &s) const
     {
@@ -1825,12 +1820,6 @@ struct GroupRoad {
         return key<PLAIN>(d, cut, add4(add4(hit[x], hit[A + y(j)]), add4(hit[A + B + z], hit[A + 2 * B + w])));
     }
 };
-
-// a fit's hits by role in one word
-__device__ __forceinline__ unsigned pack_fit(unsigned x, unsigned y, unsigned z, unsigned w)
-{
-    return x | (y << 3) | (z << 6) | (w << 9);
-}
 
 // What a lane has found of its road's survivors: those of its pairs (flag,
 // key, place among the road's survivors by comb), and the road's number.
@@ -1879,7 +1868,10 @@ __device__ __forceinline__ void group_rank(GroupFound<YN> &f, unsigned gmask)
 // ---------------------------------------------------------------------------
 
 // flagged hits of layer l: byte l of the mask; groups of triple t
-__device__ __forceinline__ unsigned flagged(unsigned long long xm, unsigned l) { return (unsigned)(xm >> (8 * l)) & 0xFFu; }
+__device__ __forceinline__ unsigned flagged(unsigned long long xm, unsigned l)
+{
+    return (unsigned)(xm >> (8 * l)) & 0xFFu;
+}
 __device__ __forceinline__ unsigned groups_of(unsigned long long xm, unsigned t)
 {
     return __popc(flagged(xm, triple_l(t, 0))) * __popc(flagged(xm, triple_l(t, 1))) *
@@ -1940,7 +1932,8 @@ __device__ __noinline__ unsigned publish_group(const Dev &d, unsigned g, const R
     const unsigned su = __ffs(rest) - 1, sv = 31 - __clz(rest), Lu = su + (su >= excl), Lv = sv + (sv >= excl);
     const uint4 hu = ldcg(reinterpret_cast<const uint4 *>(co + Lu * 8)),
                 hv = ldcg(reinterpret_cast<const uint4 *>(co + Lv * 8));
-    const int4 cu = __ldg(cc + su), cv = __ldg(cc + sv), c4 = __ldg(cc + 4), c5 = __ldg(cc + 5), kk = __ldg(cc + 6);
+    const int4 cu = __ldg(cc + su), cv = __ldg(cc + sv), c4 = __ldg(cc + 4), c5 = __ldg(cc + 5),
+               kk = __ldg(cc + 6);
     const unsigned S1 = pk & 15u, S2 = S1 * ((pk >> 4) & 15u), S3 = S2 * ((pk >> 8) & 15u),
                    S4 = S3 * ((pk >> 12) & 15u);   // comb strides of the layers
     const auto stride = [&](unsigned L) { return L == 0 ? 1u : L == 1 ? S1 : L == 2 ? S2 : L == 3 ? S3 : S4; };
@@ -2060,8 +2053,10 @@ __device__ __noinline__ void publish_words(const Dev &d)
 // atomic minima, and folds through scratch rows or warp shuffles, measured
 // slower.)
 // A fit survives the road-local warrior iff its key is the minimum of all
-// six (see the flat path); it is then the minimum of its pair (x, y), so a
-// pair has at most one candidate and a road at most 64 survivors.
+// six: two fitted hits and a hit of the excluded layer are a group, and a
+// group of three fitted hits lies within the fits of two of them.  It is then
+// the minimum of its pair (x, y), so a pair has at most one candidate and a
+// road at most 64 survivors.
 // ---------------------------------------------------------------------------
 
 enum { T_AB = 0, T_CE, T_AE, T_BE, T_AC, T_BC };
@@ -2967,7 +2962,6 @@ __device__ __forceinline__ void box_road(const Dev &d, unsigned char *region, un
         box_integer<PLAIN>(d, region, g, npass);
 }
 
-
 // Shared memory of P3: what every step reads of the kernel's argument (a load
 // through the argument's address takes an L1 miss), then a region per warp, a
 // group step's hits or a box road.
@@ -3413,13 +3407,6 @@ __device__ void p4_finish(const Dev &d, unsigned n_chunks)
     }
 }
 
-// hit d (0..7) of a layer's eight 16-bit coordinates held in one uint4
-__device__ __forceinline__ unsigned coord_of(const uint4 &r, unsigned d)
-{
-    const unsigned w = d < 4 ? (d < 2 ? r.x : r.y) : (d < 6 ? r.z : r.w);
-    return (w >> (16 * (d & 1u))) & 0xFFFFu;
-}
-
 // The track of key `key` of road g (record rec, coordinate row rw: the
 // road's 40 coordinates as five 16-byte words), written to *out.
 // The loops are unrolled (registers, no local arrays).
@@ -3455,7 +3442,7 @@ __device__ void build_track(const Dev &d, unsigned g, const RoadRec &rec, const 
         const unsigned qq = divm(rest, c_magic[n]);
         const unsigned dl = rest - qq * n;
         rest = qq;
-        v[l] = coord_of(rw[l], dl);
+        v[l] = row_at(rw[l], dl);
     }
     svt_track t;
     t.event = rec.event;

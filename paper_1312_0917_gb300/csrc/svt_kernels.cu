@@ -525,7 +525,7 @@ __device__ __forceinline__ uint32_t word_bad(uint32_t w)
 // for P1, which then finds the roads without reading the words; the counts are
 // taken from the masks, a window per lane.  Bound: the words' latency, then
 // issue slots (22 instructions a window; 73 when every window was counted and
-// checked by itself).
+// checked by itself: 11.9 MB of words 10.8 -> 9.2 us, 16.5 MB 13.9 -> 11.9).
 __device__ void scan_count(const Dev &d)
 {
     const unsigned lane = lane_id(), sp = blockIdx.x * WARPS + warp_id();
@@ -766,7 +766,10 @@ __device__ __forceinline__ unsigned long long decode_batch(const Dev &d, P1Warp 
 
 // P1 for one warp: the roads whose header lies in [a, e).  g, ev: EP and EE
 // words before a; rie: EP words since the last EE before a (roads of the open
-// event).
+// event).  Bound: the walk of a road, a chain of its words per lane.
+// 192,000 roads of 12 hits 27.9 -> 13.7 us, 25,600 of 40 hits 18.9 -> 12.0 (with
+// the stream scanned a second time for the starts, and each road's end found on
+// its walk).
 __device__ void decode_span(const Dev &d, P1Warp &q, unsigned long long a, unsigned long long e, unsigned g,
                             unsigned ev, unsigned rie, unsigned n_events)
 {
@@ -1287,6 +1290,10 @@ __device__ void list_out(const Dev &d, P2List &list)
 }
 
 // Flags of the event of roads r0 .. r0 + nr - 1; adds its combinations to n_comb.
+// Bound: the latency of its steps, each a pass over the event's rows by one
+// CTA (one event of 64 roads 8.0 -> 6.4 us for the stage; 301 events of 96
+// roads 14.5 -> 11.9; 200 events of 128 roads with eight hits a layer 18.4 with
+// 512 threads a CTA, 22.4 with 256, of which the pairs are 6.3).
 __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *smem, P2List &list,
                          unsigned long long &n_comb)
 {
@@ -1449,7 +1456,7 @@ __device__ __noinline__ void p2_pairs(const uint16_t *coords, const RoadRec *roa
 // those per road, pairs of roads whose signatures meet on >= 3 layers tested
 // exactly (a lane per pair).  Bound: latency of one warp's chain, so a layer's
 // rows are loaded while the layer before is worked on, and a layer's atomics
-// are in flight together.
+// are in flight together (3000 events of 64 roads 26.3 -> 19.3 us).
 __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2List &list, unsigned long long &n_comb)
 {
     const unsigned lane = lane_id();
@@ -2025,7 +2032,8 @@ __device__ __noinline__ void publish_words(const Dev &d)
 
 // ---------------------------------------------------------------------------
 // P3, box path: one warp fits one listed road (more distinct fits than
-// small_n4, or a cross-road candidate with a repeated coordinate).
+// small_n4, more than four hits in its second largest slot, or a coordinate
+// repeated within a layer).
 //
 // Hits with one coordinate in one layer are one hit for the warrior (hits
 // are shared by value), and among fits with the same coordinates the lowest
@@ -2448,7 +2456,9 @@ __device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, u
 // shape's slots are roles here, by falling hit count.  Hits that repeat a
 // coordinate need nothing special: the fits of the later hit are the earlier
 // one's with a higher comb, so they tie in float, lose in whole keys, and what
-// they drop or publish the earlier ones drop or publish too.
+// they drop or publish the earlier ones drop or publish too.  Bound: issue slots
+// (two fits an instruction).  The fit stage of 25,600 roads of 8^4 distinct fits:
+// 153.8 -> 82.4 us with it in place of the integer passes.
 __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
     P3Box &B = *reinterpret_cast<P3Box *>(region);
@@ -2996,6 +3006,9 @@ using GroupCls4e = GroupRoad<3, 1, 2, 4>;
 // combinations to np.  Returns the roads with a tie, bit by lane of their
 // groups' first lanes, which are left to the box path.  Not inlined: a register
 // allocation per class (in one function the five classes spilled 220 bytes).
+// Bound: issue slots and the chain from the list to the hits.  The fit stage of
+// 192,000 roads of one to four hits a layer, nearly all of them here: 124.4 ->
+// 67.6 us (a lane per table entry, tables in shared memory, before).
 template <bool PLAIN, class Road>
 __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, const RoadItem *list, int step,
                                             unsigned left, unsigned &npass)
@@ -3568,7 +3581,7 @@ __device__ void p4_cand_phase(const Dev &d, unsigned n_roads)
 // tracks, which are gathered in shared memory and written out as one stretch.
 // Bound: two trips to L2 and the writes (a search for the road of each of an
 // equal share of the tracks took four trips and wrote each track's five words
-// 40 bytes apart).
+// 40 bytes apart: 175,000 tracks 15.1 -> 10.2 us).
 constexpr unsigned P5_TRACKS = 2 * BLOCK;   // tracks gathered at most (more: written by their thread)
 struct P5Smem {
     svt_track track[P5_TRACKS];

@@ -18,11 +18,12 @@ roads x 8 hits on each of 5 layers (838,860,800 combinations).
          svt_get_tracks (D2H of the status block and the tracks), host wall
          clock; two contexts take batches in turn (one batch's copies overlap
          the other's kernel).  p50 / p99 are one batch at a time.
-  roofline  integer multiply-adds: 36 per distinct fit (the fit of one input
+  roofline  multiply-adds: 36 per distinct fit (the fit of one input
          vector x, Sec. II: 18 for p = F x + q, 18 for the chi-square rows;
          combinations that differ only in the excluded layer's hit share x),
-         against the device's multiply-add rate (SMs x 64 lanes x clock; the
-         in-tree measurement beside it).
+         against the device's multiply-add rate (SMs x 128 lanes x clock: the
+         fit's main pass runs them as pairs in single precision, exact where
+         it decides; integer ones have 64 lanes, measured beside it).
   scaled / uneven  the 3000 x 64 and 10,000-event uneven batches: the
          persistent form against the plain per-stage launch (fits/s, p50,
          p99 per batch, device and end to end).
@@ -58,8 +59,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# multiply-add lanes of one GB300 SM (the IMAD rate: half the FP32 lanes)
-IMAD_LANES_PER_SM = 64
+FMA_LANES_PER_SM = 128      # single-precision multiply-adds per SM and clock (integer ones: 64)
 MACS_PER_FIT = 36   # 6 inputs x (3 track parameters + 3 chi-square components)
 HEADLINE = "stress"
 
@@ -343,9 +343,9 @@ def run_serving(B, synth, consts, cut, rates, n_requests, n_slots=8, seed=0, **s
 # (kernels and their header) they were taken on: the bench line reports a
 # figure only while the sources are unchanged.
 NCU_TRAFFIC = {
-    "stress": {"kernels_sha256": "0534c74cb0ab5f09209c952563eeee5892be75a4d1c9d099ab65f7b7abb143bf", "bytes": 5278720},    # 5.279 MB read, 0 B written
-    "scaled": {"kernels_sha256": "0534c74cb0ab5f09209c952563eeee5892be75a4d1c9d099ab65f7b7abb143bf", "bytes": 12697600},   # 12.626 MB read + 71.7 KB written
-    "uneven": {"kernels_sha256": "0534c74cb0ab5f09209c952563eeee5892be75a4d1c9d099ab65f7b7abb143bf", "bytes": 20996096},   # 17.692 MB read + 3.304 MB written
+    "stress": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 5836544},    # 5.744 MB read + 92.4 KB written
+    "scaled": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 16996864},   # 13.885 MB read + 3.112 MB written
+    "uneven": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 36923648},   # 19.202 MB read + 17.722 MB written
 }
 
 
@@ -740,7 +740,7 @@ def gpu_arm(args):
     clk = clocks.summary(t_timed0 - 0.02, t_timed1 + 0.02)
     clk["gpu_section"] = clocks.summary()
     mhz = clk["sm_max_mhz"] or 2070.0
-    peak_macs = sms * IMAD_LANES_PER_SM * mhz * 1e6 / 1e12
+    peak_macs = sms * FMA_LANES_PER_SM * mhz * 1e6 / 1e12
     achieved = MACS_PER_FIT * n_fit4 / (step_ms / 1e3) / 1e12
     line = {
         "metric": "track fits/s", "value": value, "unit": "fits/s", "n_gpus": world,
@@ -758,12 +758,13 @@ def gpu_arm(args):
                               "cross_road_warrior", "output"],
                              [round(x / 1e3, 1) for x in stats["phase_ns"]])),
         "e2e": e2e,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_macs, "unit": "T int32 MAC/s",
+        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_macs, "unit": "T MAC/s",
                      "frac": achieved / peak_macs, "traffic": measured_traffic(args.workload),
-                     "peak_measured": peak["imad"] / 1e12,
+                     "peak_measured": peak["mixed"] / 1e12,
                      "units": "%d distinct fits x %d multiply-adds per launch" % (n_fit4, MACS_PER_FIT),
-                     "note": "peak = SMs x 64 multiply-add lanes x max clock; peak_measured: "
-                             "svt_measure_int_peak (mad.lo.u32 chains on every SM); "
+                     "note": "peak = SMs x 128 single-precision multiply-add lanes x max clock; "
+                             "peak_measured: svt_measure_int_peak, multiply-add and xor "
+                             "alternating on every SM; "
                              "per combination the same time is %.2f T MAC/s"
                              % (MACS_PER_FIT * n_fits / (step_ms / 1e3) / 1e12)},
         "int_peak_tops": {k: round(v / 1e12, 2) for k, v in peak.items()},

@@ -15,7 +15,7 @@ roads x 8 hits on each of 5 layers (838,860,800 combinations).
          written between steps to flush L2.
   e2e    the same metric through the public C ABI from pinned host memory:
          per batch H2D of the words, svt_unpack, svt_fit_events,
-         svt_get_tracks (D2H of the status block and the tracks), host wall
+         svt_get_tracks (the status block and the tracks to the host), host wall
          clock; two contexts take batches in turn (one batch's copies overlap
          the other's kernel).  p50 / p99 are one batch at a time.
   roofline  multiply-adds: 36 per distinct fit (the fit of one input

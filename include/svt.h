@@ -166,9 +166,10 @@ int svt_fit_events(svt_ctx *ctx, int mode, void *stream);
  * (event, road, comb) order, to `out` (host or device memory, capacity `cap`
  * records).  *n_out = number of survivors (also when they do not fit, in
  * which case SVT_E_CAPACITY is returned).  Returns the batch status (a
- * device-detected error is returned here with *n_out = 0).  The status block
- * and as many records as the context's previous batch had are copied in one
- * go (one synchronisation when the count does not grow); when the call
+ * device-detected error is returned here with *n_out = 0).  The batch itself
+ * writes its status to the host; as many records as the context's previous
+ * batch had are copied before the count is known (one synchronisation when
+ * the count does not grow); when the call
  * returns anything but SVT_OK, the contents of `out` are unspecified. */
 int svt_get_tracks(svt_ctx *ctx, svt_track *out, size_t cap, size_t *n_out,
                    void *stream);

@@ -1761,9 +1761,11 @@ __device__ __forceinline__ unsigned nth_bit(unsigned mask, unsigned n)
 // other y, other x, and all its lanes; (a, e) and (b, e) follow after the
 // loop from the minima over z.  No table is kept in memory.  Without two
 // passing fits of one word that meet in a minimum (a tie) the words order the
-// fits as the keys do; a road with a tie (0.3 % of the roads at random: hits
-// that differ by one or two often give the same floors) is left to the box
-// path, which compares whole keys.
+// fits as the keys do.  Hits a strip or two apart often give the same floors,
+// so how many roads have a tie depends on how near their hits lie: 0.2 % with
+// hits anywhere, 8 % within 64 strips, 24 % within 16, 44 % within 8.  The roads
+// with a tie take the step once more, by the same lanes from the hits still in
+// shared memory, with whole keys in place of words (EXACT).
 //
 // Bound: issue slots.  Several hits of slot b per lane (YN = 2) share the
 // road's set-up, the loads and the shuffles of (a, c) and (c, e); with one
@@ -1826,6 +1828,19 @@ struct GroupRoad {
     {
         return key<PLAIN>(d, cut, add4(add4(hit[x], hit[A + y(j)]), add4(hit[A + B + z], hit[A + 2 * B + w])));
     }
+};
+
+// How the group path compares fits: by word, or (EXACT) by whole key; FAIL: no
+// passing fit is as high.
+template <bool EXACT>
+struct FitKey {
+    using type = unsigned;
+    static constexpr unsigned FAIL = 0x80000000u;
+};
+template <>
+struct FitKey<true> {
+    using type = unsigned long long;
+    static constexpr unsigned long long FAIL = NO_KEY;
 };
 
 // What a lane has found of its road's survivors: those of its pairs (flag,
@@ -2635,8 +2650,7 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
         if (n_surv)
             atomicAdd(&d.rchunk_sum[g / ROAD_CHUNK], n_surv);
     }
-    // a cross-road candidate (one that the group path listed is published there)
-    if (((pk >> 23) & 1u) && ((rec.fit >> 8) & 7u) == CLS_BOX)
+    if ((pk >> 23) & 1u)   // a cross-road candidate
         publish_road(d, g, rec);
     __syncwarp();
     return true;
@@ -2841,7 +2855,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     // cross-road candidates: the minimum key of every group (layer triple,
     // three coordinates) whose three hits are canonical and flagged as
     // present in another road of the event
-    if (((pk >> 23) & 1u) && ((rec.fit >> 8) & 7u) == CLS_BOX) {   // (the group path's are published there)
+    if ((pk >> 23) & 1u) {
         // canonical hits of the excluded layer (lanes 0..7)
         unsigned xc = lane;
         const bool xv = lane < sh.ne;
@@ -3001,26 +3015,27 @@ using GroupCls3 = GroupRoad<3, 0, 2, 2>;    // (8, 2): 4
 using GroupCls4 = GroupRoad<3, 1, 2, 2>;    // (8, 4): 2
 using GroupCls4e = GroupRoad<3, 1, 2, 4>;
 
-// Fit roads first .. first + ROADS - 1 of a list of n (from the end of
-// the class's array when `back`) with one warp; adds the lane's passing
-// combinations to np.  Returns the roads with a tie, bit by lane of their
-// groups' first lanes, which are left to the box path.  Not inlined: a register
-// allocation per class (in one function the five classes spilled 220 bytes).
-// Bound: issue slots and the chain from the list to the hits.  The fit stage of
-// 192,000 roads of one to four hits a layer, nearly all of them here: 124.4 ->
-// 67.6 us (a lane per table entry, tables in shared memory, before).
-template <bool PLAIN, class Road>
+// Fit up to ROADS roads of a list (list[0], list[step], .., `left` of them) with
+// one warp; adds the lane's passing combinations to np.  Returns the roads with
+// a tie, bit by lane of their groups' first lanes.  EXACT: those roads (`tied`)
+// again, in whole keys, straight after the call that found them.  Not inlined: a
+// register allocation per class (in one function the five classes spilled 220
+// bytes).  Bound: issue slots and the chain from the list to the hits.  The fit
+// stage of 192,000 roads of one to four hits a layer, nearly all of them here:
+// 124.4 -> 67.6 us (a lane per table entry, tables in shared memory, before).
+template <bool PLAIN, class Road, bool EXACT>
 __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, const RoadItem *list, int step,
-                                            unsigned left, unsigned &npass)
+                                            unsigned left, unsigned tied, unsigned &npass)
 {
+    using Key = typename FitKey<EXACT>::type;
+    constexpr Key FAIL = FitKey<EXACT>::FAIL;
     const P3Shared &S = *reinterpret_cast<const P3Shared *>(smem);
     const unsigned sh = S.sh;
-    constexpr unsigned A = Road::A, YL = Road::YL, YN = Road::YN, B = Road::B, W = Road::W, G = Road::G,
-                       HITS = Road::HITS;
+    constexpr unsigned A = Road::A, YN = Road::YN, B = Road::B, W = Road::W, G = Road::G, HITS = Road::HITS;
     const unsigned lane = lane_id(), gl = lane % G, gi = lane / G;
     const unsigned gmask = G == 32 ? FULL_MASK : ((1u << (G & 31u)) - 1u) << (gi * G);
     Road r;
-    const bool on = gi < left;
+    const bool on = EXACT ? (tied >> (gi * G)) & 1u : gi < left;
     r.it = RoadItem{};
     if (on) {
         const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(list + step * (int)gi));
@@ -3040,7 +3055,7 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
     int4 *hit = reinterpret_cast<P3Group *>(smem + P3_SHARED_BYTES + warp_id() * P3_WARP_BYTES)->A + gi * HITS;
     r.hit = hit;
     __syncwarp();   // the table's previous readers are done
-    {
+    if (!EXACT) {
         // comb strides of the layers
         const unsigned S1 = pk & 15u, S2 = S1 * ((pk >> 4) & 15u), S3 = S2 * ((pk >> 8) & 15u),
                        S4 = S3 * ((pk >> 12) & 15u);
@@ -3095,38 +3110,38 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
 
     // The lane's fits.  A failing or missing fit's word is its own, above
     // every passing one's, so that two equal words are always two passing fits.
+    // (Whole keys of passing fits differ by comb; the others are all NO_KEY.)
     const unsigned mcw = __reduce_max_sync(FULL_MASK, r.mc), mew = __reduce_max_sync(FULL_MASK, r.me);
     const long long cut = S.cut;
     int4 pab[YN];
-    unsigned q[YN], code[YN], cw[YN][W], np = 0;   // a pair's lowest word, its fit and state; minima over z
+    Key q[YN], cw[YN][W];   // a pair's lowest fit; minima over z
+    unsigned code[YN], np = 0;   // the lowest fit's hits and state
     bool tie = false, tie2 = false, tie3 = false, tie4 = false;   // (several: no long chain of one flag)
-    // minimum of t over the lanes that differ in bits [o0, o1) of the lane
-    const auto fold = [](bool &tie, unsigned t, unsigned o0, unsigned o1) {
-#pragma unroll
-        for (unsigned o = o0; o < o1; o <<= 1) {
-            const unsigned u = __shfl_xor_sync(FULL_MASK, t, o);
+    const auto meet = [](bool &tie, Key t, Key u) {
+        if (!EXACT)
             tie = tie | (u == t);
-            t = min(t, u);
-        }
-        return t;
+        return u < t ? u : t;
     };
-    const auto meet = [](bool &tie, unsigned t, unsigned u) {
-        tie = tie | (u == t);
-        return min(t, u);
+    // minimum of t over the lanes that differ in bits [o0, o1) of the lane
+    const auto fold = [&meet](bool &tie, Key t, unsigned o0, unsigned o1) {
+#pragma unroll
+        for (unsigned o = o0; o < o1; o <<= 1)
+            t = meet(tie, t, __shfl_xor_sync(FULL_MASK, t, o));
+        return t;
     };
 #pragma unroll
     for (unsigned j = 0; j < YN; ++j) {
         pab[j] = add4(hit[r.x], hit[A + r.y(j)]);   // unspecified unless the hits exist
-        q[j] = 0xE0000000u | (lane << 8) | j;
+        q[j] = EXACT ? FAIL : (Key)(0xE0000000u | (lane << 8) | j);
         code[j] = 0;
 #pragma unroll
         for (unsigned w = 0; w < W; ++w)
-            cw[j][w] = 0xC0000000u | (lane << 8) | (j * W + w);
+            cw[j][w] = EXACT ? FAIL : (Key)(0xC0000000u | (lane << 8) | (j * W + w));
     }
     for (unsigned z = 0; z < mcw; ++z) {
         const int4 az = hit[A + B + z];
         const unsigned none = 0x80000000u | (lane << 8) | (z << 4);
-        unsigned word[YN][W], rz[YN], ce[W];
+        Key word[YN][W], rz[YN], ce[W];
 #pragma unroll
         for (unsigned w = 0; w < W; ++w) {
             if (w >= 2 && w >= mew) {   // no road of the warp has hit w
@@ -3138,7 +3153,9 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
 #pragma unroll
             for (unsigned j = 0; j < YN; ++j) {
                 const bool in = zw & (r.y(j) < r.mb);
-                if (PLAIN) {
+                if (EXACT) {
+                    word[j][w] = in ? r.template key<PLAIN>(d, cut, add4(pab[j], add4(az, aw))) : FAIL;
+                } else if (PLAIN) {
                     const unsigned long long k =
                         in ? ldcg(d.fit_key + r.cb + (unsigned)(pab[j].w + az.w + aw.w)) : NO_KEY;
                     word[j][w] = k == NO_KEY ? none + (j * W + w) : (unsigned)((k >> 23) >> sh);
@@ -3159,14 +3176,14 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
                 ce[w] = meet(tie3, ce[w], word[j][w]);
             ce[w] = fold(tie3, ce[w], 1, G);
         }
-        unsigned ac = rz[0];   // (a, c) at x, z
+        Key ac = rz[0];   // (a, c) at x, z
 #pragma unroll
         for (unsigned j = 1; j < YN; ++j)
             ac = meet(tie4, ac, rz[j]);
         ac = fold(tie4, ac, A, G);
 #pragma unroll
         for (unsigned j = 0; j < YN; ++j) {
-            const unsigned t = min(ac, fold(tie4, rz[j], 1, A));   // and (b, c) at y, z
+            const Key t = min(ac, fold(tie4, rz[j], 1, A));   // and (b, c) at y, z
             bool ok = false;
             unsigned ws = 0;
 #pragma unroll
@@ -3177,7 +3194,8 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
                 ws = here ? w : ws;
                 ok = here ? ce[w] == rz[j] : ok;
             }
-            tie2 = tie2 | (rz[j] == q[j]);
+            if (!EXACT)
+                tie2 = tie2 | (rz[j] == q[j]);
             if (rz[j] < q[j]) {
                 q[j] = rz[j];
                 code[j] = z << 2 | ws | (ok && t == rz[j] ? 0x80u : 0u);
@@ -3187,7 +3205,7 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
 
     // (a, e) and (b, e), then the survivors
     GroupFound<YN> f;
-    unsigned te[YN];
+    Key te[YN];
 #pragma unroll
     for (unsigned j = 0; j < YN; ++j)
         te[j] = 0;
@@ -3195,29 +3213,29 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
     for (unsigned w = 0; w < W; ++w) {
         if (w >= 2 && w >= mew)
             continue;
-        unsigned ae = cw[0][w];
+        Key ae = cw[0][w];
 #pragma unroll
         for (unsigned j = 1; j < YN; ++j)
             ae = meet(tie3, ae, cw[j][w]);
         ae = fold(tie3, ae, A, G);
 #pragma unroll
         for (unsigned j = 0; j < YN; ++j) {
-            const unsigned t = min(ae, fold(tie4, cw[j][w], 1, A));
+            const Key t = min(ae, fold(tie4, cw[j][w], 1, A));
             te[j] = (code[j] & 3u) == w ? t : te[j];
         }
     }
-    const bool tied = (__ballot_sync(FULL_MASK, tie | tie2 | tie3 | tie4) & gmask) != 0u;   // the road has a tie
+    const bool again = !EXACT && (__ballot_sync(FULL_MASK, tie | tie2 | tie3 | tie4) & gmask) != 0u;   // the road has a tie
     f.cnt = 0;
 #pragma unroll
     for (unsigned j = 0; j < YN; ++j) {
-        f.surv[j] = !tied && code[j] >= 0x80u && te[j] == q[j] && q[j] < 0x80000000u;
-        f.key[j] = NO_KEY;
+        f.surv[j] = !again && code[j] >= 0x80u && te[j] == q[j] && q[j] < FAIL;
+        f.key[j] = EXACT ? (unsigned long long)q[j] : NO_KEY;
         f.rank[j] = 0;
         f.cnt += __popc(__ballot_sync(FULL_MASK, f.surv[j]) & gmask);
     }
 #pragma unroll
     for (unsigned j = 0; j < YN; ++j)
-        if (f.surv[j])
+        if (!EXACT && f.surv[j])
             f.key[j] = r.template key_at<PLAIN>(d, cut, j, (code[j] >> 2) & 3u, code[j] & 3u);
     if (__any_sync(FULL_MASK, f.cnt > 1))
         group_rank(f, gmask);
@@ -3225,30 +3243,29 @@ __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, c
     for (unsigned j = 0; j < YN; ++j)
         if (f.surv[j])
             S.surv_pool[f.rank[j] * S.max_roads + g] = f.key[j];
-    if (on && gl == 0 && !tied) {
+    if (on && gl == 0 && !again) {
         S.surv_cnt[g] = (uint8_t)f.cnt;
         if (f.cnt)
             atomicAdd(&S.rchunk_sum[g / ROAD_CHUNK], f.cnt);
     }
-    npass += tied ? 0u : np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
-    __syncwarp();   // (the warp's memory may be the box path's next)
-    return __ballot_sync(FULL_MASK, tied && gl == 0);
+    if (EXACT)
+        return 0;
+    npass += np * ((pk >> (4 * r.excl)) & 15u);   // once per hit of the excluded layer
+    return __ballot_sync(FULL_MASK, again && gl == 0);
 }
 
 // Step s (of the sequence over all half classes) if it is of half class SEG,
 // and then its roads with ties.
 template <bool PLAIN, class Road, unsigned SEG>
-__device__ __forceinline__ void group_step(const Dev &d, unsigned char *smem, unsigned s, unsigned &np,
-                                           unsigned long long &npass)
+__device__ __forceinline__ void group_step(const Dev &d, unsigned char *smem, unsigned s, unsigned &np)
 {
     const P3Shared &S = *reinterpret_cast<const P3Shared *>(smem);
-    const unsigned first = (s - (SEG ? S.end[SEG - 1] : 0u)) * Road::ROADS;
+    const unsigned first = (s - (SEG ? S.end[SEG - 1] : 0u)) * Road::ROADS, left = S.n[SEG] - first;
     const RoadItem *list = d.items + list_at(d, SEG, first);
     constexpr int dir = (SEG & 1u) ? 1 : -1;
-    for (unsigned tied = group_item<PLAIN, Road>(d, smem, list, dir, S.n[SEG] - first, np); tied; tied &= tied - 1) {
-        const unsigned gi = (__ffs(tied) - 1) / Road::G;
-        box_road<PLAIN>(d, smem + P3_SHARED_BYTES + warp_id() * P3_WARP_BYTES, ldcg(&list[dir * (int)gi].g), npass);
-    }
+    const unsigned tied = group_item<PLAIN, Road, false>(d, smem, list, dir, left, 0u, np);
+    if (tied)
+        group_item<PLAIN, Road, true>(d, smem, list, dir, left, tied, np);
 }
 
 // The roads of the box path (n_box of them), one warp each.
@@ -3320,19 +3337,19 @@ __device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbo
     Share w(steps, n_warps, max((unsigned)d.run_roads / 8, 1u), &d.ctrl->q[qgroup]);
     for (unsigned s = w.first(wi); s < steps; s = w.next(s)) {
         if (s < S.end[0])
-            group_step<PLAIN, GroupCls4e, 0>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls4e, 0>(d, smem, s, np);
         else if (s < S.end[1])
-            group_step<PLAIN, GroupCls4, 1>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls4, 1>(d, smem, s, np);
         else if (s < S.end[3])
-            group_step<PLAIN, GroupCls3, 3>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls3, 3>(d, smem, s, np);
         else if (s < S.end[4])
-            group_step<PLAIN, GroupCls2e, 4>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls2e, 4>(d, smem, s, np);
         else if (s < S.end[5])
-            group_step<PLAIN, GroupCls2, 5>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls2, 5>(d, smem, s, np);
         else if (s < S.end[7])
-            group_step<PLAIN, GroupCls1, 7>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls1, 7>(d, smem, s, np);
         else
-            group_step<PLAIN, GroupCls0, 9>(d, smem, s, np, npass);
+            group_step<PLAIN, GroupCls0, 9>(d, smem, s, np);
     }
     __syncwarp();
     if (cands)

@@ -94,7 +94,7 @@ struct RoadRec {
     int16_t curv, phi;
     uint16_t set;
     uint16_t fit;   // written in P2: the fitted slots by falling hit count, two bits each, the fit
-                    // class in bits 8..10, bit 11: a coordinate repeated within a layer
+                    // class in bits 8..10
 };
 
 // Fit classes of the roads: the group path's

@@ -946,7 +946,6 @@ struct P2Smem {
     uint32_t xhi[MAX_ROADS_EV];           //   >= 3 layers: bit 8 l + d (l < 4), layer 4 in xhi
     uint16_t elig[MAX_ROADS_EV];          // roads with shared coordinates on >= 3 layers
     uint32_t cp[P2_PAIRS];                // road pairs whose signatures meet on >= 3 layers (r | t << 16)
-    uint8_t rep[MAX_ROADS_EV];            // a coordinate repeated within a layer of the road
     unsigned n_elig, n_cp;
 };
 
@@ -1020,19 +1019,15 @@ __device__ __forceinline__ unsigned row_at(const uint4 &q, unsigned x)
 // event's bitmap when the hit set its bit (bit x of `again`): a coordinate
 // of an earlier slot of the same row is a repeat; any other was set by
 // another road and gets the multi bit.  So a coordinate gets the multi bit
-// exactly when two roads hold it.  True when the row repeats a coordinate.
-__device__ __forceinline__ bool seen_again(uint32_t *multi, const uint4 &q, unsigned again)
+// exactly when two roads hold it.
+__device__ __forceinline__ void seen_again(uint32_t *multi, const uint4 &q, unsigned again)
 {
-    bool rep = false;
     for (; again; again &= again - 1) {
         const unsigned x = __ffs(again) - 1;
         const unsigned v = row_at(q, x);
-        if (row_find(q, v) & ((1u << x) - 1u))
-            rep = true;
-        else
+        if (!(row_find(q, v) & ((1u << x) - 1u)))
             atomicOr(&multi[v >> 5], 1u << (v & 31u));
     }
-    return rep;
 }
 
 // hits of a layer (row q, n of them) whose coordinate two roads hold: bit x
@@ -1134,10 +1129,8 @@ __device__ __forceinline__ unsigned fitted_counts(uint32_t pk)
 
 // Fit class of a road with N combinations and N4 distinct fits, and its slots
 // by falling hit count (perm).  The box path takes roads with more than
-// small_n4 distinct fits, with more than four hits on two fitted layers, or
-// with a coordinate repeated within a layer (rep: it works on canonical hits).
-__device__ __forceinline__ unsigned road_class(uint32_t pk, unsigned N, unsigned N4, unsigned small_n4, bool rep,
-                                               unsigned &perm)
+// small_n4 distinct fits or with more than four hits on two fitted layers.
+__device__ __forceinline__ unsigned road_class(uint32_t pk, unsigned N, unsigned N4, unsigned small_n4, unsigned &perm)
 {
     const unsigned nf = fitted_counts(pk);
     unsigned v[4];
@@ -1158,7 +1151,7 @@ __device__ __forceinline__ unsigned road_class(uint32_t pk, unsigned N, unsigned
     const unsigned ma = v[0] >> 2, mb = v[1] >> 2;
     if (N == 0)
         return CLS_NONE;
-    if (rep || N4 > small_n4 || mb > 4)
+    if (N4 > small_n4 || mb > 4)
         return CLS_BOX;
     return ma > 4 ? (mb > 2 ? 4u : 3u) : ma > 2 ? (mb > 2 ? 2u : 1u) : 0u;
 }
@@ -1196,21 +1189,20 @@ __device__ __forceinline__ unsigned road_bucket(uint32_t pk, unsigned perm, unsi
     return 16 * (N_GROUP_CLS - 1 - cls) + (me > 2 ? 0u : 8u) + 2 * ((4 - mc) & 3u) + (me & 1u);
 }
 
-// The end of P2 for road g (record r, flagged hits xm, rep: a coordinate
-// repeated within a layer), one road per lane, by a whole warp (in: the lane
-// has a road): the record's candidate bit and fit path, and the road joins its
-// list.  Returns the road's combinations.
+// The end of P2 for road g (record r, flagged hits xm), one road per lane, by a
+// whole warp (in: the lane has a road): the record's candidate bit and fit path,
+// and the road joins its list.  Returns the road's combinations.
 __device__ __forceinline__ unsigned finish_road(const Dev &d, P2List &list, bool in, unsigned g, RoadRec r,
-                                                unsigned long long xm, bool rep)
+                                                unsigned long long xm)
 {
     const unsigned lane = lane_id(), lt = lanemask_lt();
     const bool cand = xm != 0ull;
     unsigned N, N4, perm;
     road_sizes(r.pk, N, N4);
     N = in ? N : 0u;
-    const unsigned cls = road_class(r.pk, N, N4, (unsigned)d.small_n4, rep, perm);
+    const unsigned cls = road_class(r.pk, N, N4, (unsigned)d.small_n4, perm);
     r.pk |= cand ? (1u << 23) : 0u;
-    r.fit = (uint16_t)(perm | cls << 8 | (rep ? 1u << 11 : 0u));
+    r.fit = (uint16_t)(perm | cls << 8);
     if (in) {
         d.roads[g] = r;
         d.xmask[g] = xm;
@@ -1305,7 +1297,6 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
     const uint4 *rows = reinterpret_cast<const uint4 *>(co);
     for (unsigned k = threadIdx.x; k < nr; k += BLOCK) {
         s.rec[k] = ldcg(d.roads + r0 + k);
-        s.rep[k] = 0;
         s.xlo[k] = 0;
         s.xhi[k] = 0;
     }
@@ -1324,9 +1315,7 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
         const unsigned i = min(i0 + lane_id(), nr * N_LAYERS - 1), k = i / N_LAYERS, l = i - k * N_LAYERS;
         const unsigned n = i0 + lane_id() == i ? (s.rec[k].pk >> (4 * l)) & 15u : 0u;   // <= MAX_HITS
         const uint4 q = rows[i];
-        const unsigned again = see_row(s.seen[l], q, n, __reduce_max_sync(FULL_MASK, n));
-        if (again && seen_again(s.multi[l], q, again))
-            s.rep[k] = 1;
+        seen_again(s.multi[l], q, see_row(s.seen[l], q, n, __reduce_max_sync(FULL_MASK, n)));
     }
     __syncthreads();
     // signatures of the shared coordinates, a layer of a road per thread
@@ -1376,7 +1365,7 @@ __device__ void p2_event(const Dev &d, unsigned r0, unsigned nr, unsigned char *
     for (unsigned k0 = threadIdx.x - lane_id(); k0 < nr; k0 += BLOCK) {
         const unsigned k = min(k0 + lane_id(), nr - 1);
         n_comb += finish_road(d, list, k0 + lane_id() == k, r0 + k, s.rec[k],
-                              ((unsigned long long)s.xhi[k] << 32) | s.xlo[k], s.rep[k] != 0);
+                              ((unsigned long long)s.xhi[k] << 32) | s.xlo[k]);
     }
     __syncthreads();   // the shared arrays are refilled for the next event
 }
@@ -1464,7 +1453,6 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2Lis
     RoadRec rec[2];
     uint4 q[2], next[2];
     unsigned sx[2] = {0u, 0u}, sy[2] = {0u, 0u};   // the roads' signatures (sig_layers)
-    bool rep[2] = {false, false};                  // a coordinate repeated within a layer
 #pragma unroll
     for (unsigned h = 0; h < 2; ++h) {
         const unsigned k = min(32 * h + lane, nr - 1);   // a missing road reads the last one and has no hits
@@ -1495,8 +1483,7 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2Lis
             again[h] = see_row(w.seen, q[h], n[h], most);
 #pragma unroll
         for (unsigned h = 0; h < 2; ++h)
-            if (seen_again(w.multi, q[h], again[h]))
-                rep[h] = true;
+            seen_again(w.multi, q[h], again[h]);
         __syncwarp();
 #pragma unroll
         for (unsigned h = 0; h < 2; ++h) {
@@ -1555,8 +1542,7 @@ __device__ void p2_warp(const Dev &d, unsigned r0, unsigned nr, P2Warp &w, P2Lis
 #pragma unroll
     for (unsigned h = 0; h < 2; ++h) {
         const unsigned k = 32 * h + lane;
-        n_comb += finish_road(d, list, k < nr, r0 + k, rec[h], ((unsigned long long)w.xm[k][1] << 32) | w.xm[k][0],
-                              rep[h]);
+        n_comb += finish_road(d, list, k < nr, r0 + k, rec[h], ((unsigned long long)w.xm[k][1] << 32) | w.xm[k][0]);
     }
     __syncwarp();   // the state is refilled for the next event
 }
@@ -1767,6 +1753,11 @@ __device__ __forceinline__ unsigned nth_bit(unsigned mask, unsigned n)
 // with a tie take the step once more, by the same lanes from the hits still in
 // shared memory, with whole keys in place of words (EXACT).
 //
+// A coordinate repeated within a layer needs nothing of its own.  For the warrior
+// its hits are one hit (hits are shared by value).  The fits of the later hit are
+// the earlier one's with a higher comb: they tie with them, lose to them in whole
+// keys, and what they drop or publish the earlier ones drop or publish too.
+//
 // Bound: issue slots.  Several hits of slot b per lane (YN = 2) share the
 // road's set-up, the loads and the shuffles of (a, c) and (c, e); with one
 // hit per lane a warp step took 700 instructions for half the roads.
@@ -1877,8 +1868,8 @@ __device__ __forceinline__ void group_rank(GroupFound<YN> &f, unsigned gmask)
 // P3, publish: the groups of the cross-road candidates.  A group is a layer
 // triple and three coordinates whose three hits are flagged as shared with
 // another road of the event; the table gets the lowest key of the road's
-// passing fits in it.  This takes a road none of whose layers repeats a
-// coordinate (every hit is canonical).
+// passing fits in it.  (Hits that repeat a coordinate publish the same group
+// with higher keys.)
 //
 // A candidate has few groups (1.7 on average where 60 % of the hits are
 // shared, and one road in five is a candidate), so the candidates of 32 roads
@@ -2047,8 +2038,7 @@ __device__ __noinline__ void publish_words(const Dev &d)
 
 // ---------------------------------------------------------------------------
 // P3, box path: one warp fits one listed road (more distinct fits than
-// small_n4, more than four hits in its second largest slot, or a coordinate
-// repeated within a layer).
+// small_n4, or more than four hits in its second largest slot).
 //
 // Hits with one coordinate in one layer are one hit for the warrior (hits
 // are shared by value), and among fits with the same coordinates the lowest
@@ -2469,9 +2459,7 @@ __device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, u
 
 // Fit road g with one warp; false when it is left to the integer passes.  The
 // shape's slots are roles here, by falling hit count.  Hits that repeat a
-// coordinate need nothing special: the fits of the later hit are the earlier
-// one's with a higher comb, so they tie in float, lose in whole keys, and what
-// they drop or publish the earlier ones drop or publish too.  Bound: issue slots
+// coordinate need nothing special (as in the group path).  Bound: issue slots
 // (two fits an instruction).  The fit stage of 25,600 roads of 8^4 distinct fits:
 // 153.8 -> 82.4 us with it in place of the integer passes.
 __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)

@@ -68,6 +68,16 @@ def test_ties(ctx, orc, consts, lo, hi, width):
     check(ctx, orc, words, consts, cut, mode=B.PLAIN)
 
 
+@pytest.mark.parametrize("lo,hi", SMALL, ids=["%d-%d" % s for s in SMALL])
+def test_repeated_coordinates(ctx, orc, consts, lo, hi):
+    """Layers that hold a coordinate twice or more, fitted and excluded ones."""
+    words = near(batch("near", 4, 40, lo, hi, shared=0.5, seed=hi), 8, distinct=False)
+    cut = p90(orc, words, consts)
+    _, a = check(ctx, orc, words, consts, cut)
+    _, b = check(ctx, orc, words, consts, cut, mode=B.PLAIN)
+    assert a["n_groups"] == b["n_groups"]
+
+
 def test_every_fit_tied(ctx, orc, consts):
     """All chi-squares equal: the comb alone orders a road's fits."""
     flat = {k: v.copy() for k, v in consts.items()}
@@ -84,3 +94,10 @@ def test_ties_cost_one_more_pass(ctx, consts, cuts):
     ctx.load_constants(consts, cuts["scaled"])
     words = batch("apart", 1000, 64, 1, 4)
     assert fit_us(ctx, near(words, 16)) < 3 * fit_us(ctx, words)
+
+
+def test_repeats_cost_one_more_pass(ctx, consts, cuts):
+    """The same for roads of which most hold a coordinate twice."""
+    ctx.load_constants(consts, cuts["scaled"])
+    words = batch("apart", 1000, 64, 1, 4)
+    assert fit_us(ctx, near(words, 16, distinct=False)) < 3 * fit_us(ctx, words)

@@ -2038,38 +2038,34 @@ __device__ __noinline__ void publish_words(const Dev &d)
 
 // ---------------------------------------------------------------------------
 // P3, box path: one warp fits one listed road (more distinct fits than
-// small_n4, or more than four hits in its second largest slot).
+// small_n4, or more than four hits in its second largest slot).  The four fitted
+// slots get roles (a, b, c, e).  A fit survives the road-local warrior iff its
+// key is the minimum of all six pair tables (minima over the fits with the same
+// hits on two slots): two fitted hits and a hit of the excluded layer are a group,
+// and a group of three fitted hits lies within the fits of two of them.  It is
+// then the minimum of its pair (x, y) of slots a and b, so a pair has at most one
+// candidate and a road at most 64 survivors.  box_warp is the fused form;
+// box_plain reads the keys that the plain pipeline's fit kernel stored.
 //
-// Hits with one coordinate in one layer are one hit for the warrior (hits
-// are shared by value), and among fits with the same coordinates the lowest
-// hit index has the lowest comb.  So every pair-table minimum and every
-// road-local survivor takes canonical hits only (the lowest index of each
-// coordinate), and the warp works on the box of canonical fits.  The four
-// fitted slots get roles (a, b, c, e); in pass p, lane t = 32 p + lane takes
-// the pair (x, y) = (t mod m_a, t div m_a) of slots a and b and loops over
-// (z, w) of slots c and e.  Of the six pair tables (minimum key over the
-// fits with the same canonical hits on two slots) that loop makes three:
+// box_plain: hits with one coordinate in one layer are one hit for the warrior
+// (hits are shared by value), and among fits with the same coordinates the
+// lowest hit index has the lowest comb.  So its tables and survivors take
+// canonical hits only (the lowest index of each coordinate), and the warp works
+// on the box of canonical fits; in pass p, lane t = 32 p + lane takes
+// the pair (x, y) = (t mod m_a, t div m_a) and loops over (z, w) of slots c and
+// e.  Of the six tables that loop makes three:
 //   T_ab[x][y]  the lane's minimum over its own fits
 //   T_ac, T_bc  the lane's minimum over w at each z, folded over the lanes
 // A pair's minimum that holds T_ac and T_bc (about one per road) is then
-// checked against the other three, taken on demand by a warp-wide minimum
-// over the other two slots' hits (box_min2), as are the entries the
-// publish step reads:
-//   T_ae, T_be, T_ce  (folding T_ae and T_be in the loop held sixteen more
-//               registers there and measured slower)
+// checked against the other three (T_ae, T_be, T_ce), taken on demand by a
+// warp-wide minimum over the other two slots' hits (box_min2), as are the
+// entries the publish step reads.
 // The lane minima are folded by 32-bit shared-memory atomics without a
 // return value, each pass into tables of its own: the high words first,
 // then, after the warp has synchronised, the low words of the lanes whose
 // high word is the minimum.  That is the exact minimum of the 64-bit keys
 // over the pass (every lane of the pass takes part in the same steps); the
-// survivor check takes the smaller of the two passes' entries.  (64-bit
-// atomic minima, and folds through scratch rows or warp shuffles, measured
-// slower.)
-// A fit survives the road-local warrior iff its key is the minimum of all
-// six: two fitted hits and a hit of the excluded layer are a group, and a
-// group of three fitted hits lies within the fits of two of them.  It is then
-// the minimum of its pair (x, y), so a pair has at most one candidate and a
-// road at most 64 survivors.
+// survivor check takes the smaller of the two passes' entries.
 // ---------------------------------------------------------------------------
 
 enum { T_AB = 0, T_CE, T_AE, T_BE, T_AC, T_BC };
@@ -2077,11 +2073,13 @@ enum { T_AB = 0, T_CE, T_AE, T_BE, T_AC, T_BC };
 // different u in different banks
 constexpr unsigned TS = 9;
 
-// The float pass's partials by role (see box_float).
+// The float passes' partials by role (see box_warp): the components' / 4096, the
+// first role's less 0.5.
 struct P3Float {
-    float4 hit[4][8];            // (x, y, z): the components' partials / 4096, the first role's less 0.5
-    ulonglong2 c[8][2];          // role c again, each component as a pair of equals
-    ulonglong2 e[2][3];          // role e again, hits 4 i .. 4 i + 3 by component, in pairs
+    float4 hit[2][8];            // roles a and b
+    ulonglong2 c[8][2];          // role c, each component as a pair of equals
+    ulonglong2 e[2][3];          // role e, hits 4 i .. 4 i + 3 by component, in pairs
+    float bias[8];               // what the floor pass adds to hit w's x component
 };
 
 struct P3Box {
@@ -2098,9 +2096,7 @@ struct P3Box {
                                        // z) and comb part (w); slot 0 also carries curvature, phi,
                                        // 4096 k and the road bits of the key
     uint16_t co[40];                   // the road's coordinates, [layer * 8 + hit]
-    uint8_t raw[4][8];                 // raw hit index of canonical hit k of slot j
     uint8_t rank[4][8];                // canonical hit (class) of raw hit d of slot j
-    uint8_t mult[4][8];                // raw hits sharing the coordinate of canonical hit k
 };
 static_assert(offsetof(P3Box, A) % 16 == 0 && offsetof(P3Box, co) % 16 == 0 && sizeof(P3Float) % 16 == 0,
               "16-byte rows");
@@ -2108,6 +2104,15 @@ static_assert(offsetof(P3Box, A) % 16 == 0 && offsetof(P3Box, co) % 16 == 0 && s
 __device__ __forceinline__ unsigned long long umin64(unsigned long long a, unsigned long long b)
 {
     return b < a ? b : a;
+}
+
+// the warp's minimum key
+__device__ __forceinline__ unsigned long long warp_min_key(unsigned long long key)
+{
+    const unsigned hi = (unsigned)(key >> 32);
+    const unsigned mh = __reduce_min_sync(FULL_MASK, hi);
+    const unsigned ml = __reduce_min_sync(FULL_MASK, hi == mh ? (unsigned)key : 0xFFFFFFFFu);
+    return ((unsigned long long)mh << 32) | ml;
 }
 
 // entry idx of pair table tab: T_ab and T_ce as stored, the others the
@@ -2150,19 +2155,6 @@ struct BoxShape {
     __device__ unsigned m(unsigned s) const { return (mpk >> (4 * s)) & 15u; }
 };
 
-// Key of the fit with summed partials s (without the comb) and comb part
-// cw, or NO_KEY when it fails the cut or `live` is false.  The comb occupies
-// bits below the chi-square's shifted bits, so it is added, not or-ed.
-__device__ __forceinline__ unsigned long long box_key2(const int4 &s, unsigned cw, long long cut, bool live,
-                                                       bool &ok)
-{
-    const long long chi2 = sq(s.x >> 12) + sq(s.y >> 12) + sq(s.z >> 12);
-    ok = live && chi2 <= cut;
-    const unsigned hi = (unsigned)((unsigned long long)chi2 >> 9);
-    const unsigned lo = ((unsigned)chi2 << 23) + cw;
-    return ok ? ((unsigned long long)hi << 32) | lo : NO_KEY;
-}
-
 // The key of a fit without the cut: chi2 << 23 | cw (the cut is key < kb).
 __device__ __forceinline__ unsigned long long box_key_raw(const int4 &s, unsigned cw)
 {
@@ -2174,58 +2166,26 @@ __device__ __forceinline__ unsigned long long box_key_raw(const int4 &s, unsigne
 
 // One pass over the pairs (x, y) of slots a and b: lane t = 32 p + lane.
 // The inner loop over the hits of slot e has ME (4 or 8, at least me) steps,
-// unrolled and predicated, so a step has no branch.  DUP: the road has
-// repeated coordinates (passing counts are weighted by the raw fits each
-// canonical fit stands for).  T_ce is not made here (see box_tce).
-template <bool PLAIN, bool DUP, unsigned ME, bool FULLW>
-__device__ void box_pass(const Dev &d, P3Box &B, const BoxShape &sh, unsigned p, unsigned &np)
+// unrolled and predicated, so a step has no branch.  FULLW: every lane has a
+// pair and slot e eight hits.  T_ce is not made here (see box_tce).
+template <unsigned ME, bool FULLW>
+__device__ void box_pass(const Dev &d, P3Box &B, const BoxShape &sh, unsigned p)
 {
     const unsigned lane = lane_id();
     const unsigned ma = sh.ma, mb = sh.mb, mc = sh.mc, me = sh.me;
     const unsigned t = p * 32 + lane;
     const bool act = t < ma * mb;
     const unsigned y = act ? divm(t, c_magic[ma]) : 0u, x = act ? t - y * ma : 0u;
-    const int4 pab = add4(B.A[sh.ra][x], B.A[sh.rb][y]);
-    const unsigned wab = DUP ? (unsigned)B.mult[sh.ra][x] * B.mult[sh.rb][y] : 1u;
-    const long long cut = d.cut;
-    // full passes compare raw keys with kb: chi2 <= cut iff key < kb; a
-    // minimum of kb or more means no passing fit (NO_KEY when stored)
-    const unsigned long long kb = cut < 0 ? 0ull : (unsigned long long)(min(cut, 1ll << 40) + 1) << 23;
-    const auto cut_min = [kb](unsigned long long v) { return FULLW && v >= kb ? NO_KEY : v; };
-    const int4 *Ae = B.A[sh.re];
-    bool live[ME];
-#pragma unroll
-    for (unsigned w = 0; w < ME; ++w)
-        live[w] = FULLW || (act && w < me);   // full passes of 8-hit slots e: every lane, every w
+    const int pab = B.A[sh.ra][x].w + B.A[sh.rb][y].w;
     unsigned long long qab = NO_KEY;
     for (unsigned z = 0; z < mc; ++z) {
-        const int4 pz = add4(pab, B.A[sh.rc][z]);
-        const unsigned wz = DUP ? wab * B.mult[sh.rc][z] : 1u;
+        const int pz = pab + B.A[sh.rc][z].w;
         unsigned long long rz = NO_KEY;
 #pragma unroll
-        for (unsigned w = 0; w < ME; ++w) {
-            const int4 aw = Ae[w];
-            unsigned long long key;
-            if (PLAIN) {
-                key = live[w] ? ldcg(d.fit_key + sh.cb + (unsigned)(pz.w + aw.w)) : NO_KEY;
-            } else {
-                const int4 s = make_int4(pz.x + aw.x, pz.y + aw.y, pz.z + aw.z, 0);
-                if (FULLW) {
-                    key = box_key_raw(s, (unsigned)pz.w + (unsigned)aw.w);
-                    np += key < kb;
-                } else {
-                    bool ok;
-                    key = box_key2(s, (unsigned)pz.w + (unsigned)aw.w, cut, live[w], ok);
-                    if (DUP)
-                        np += ok ? wz * B.mult[sh.re][w] : 0u;
-                    else
-                        np += ok;
-                }
-            }
-            rz = umin64(rz, key);
-        }
+        for (unsigned w = 0; w < ME; ++w)
+            if (FULLW || (act && w < me))
+                rz = umin64(rz, ldcg(d.fit_key + sh.cb + (unsigned)(pz + B.A[sh.re][w].w)));
         qab = umin64(qab, rz);
-        rz = cut_min(rz);
         const unsigned q = p & 1u;
         if (act) {
             fold_hi(B, q, T_AC - T_AC, x * TS + z, rz);
@@ -2238,7 +2198,7 @@ __device__ void box_pass(const Dev &d, P3Box &B, const BoxShape &sh, unsigned p,
         }
     }
     if (act)
-        B.T[T_AB][x * TS + y] = cut_min(qab);
+        B.T[T_AB][x * TS + y] = qab;
     __syncwarp();
 }
 
@@ -2247,7 +2207,6 @@ __device__ void box_pass(const Dev &d, P3Box &B, const BoxShape &sh, unsigned p,
 // hits of the other two slots (every lane calls it with the same arguments;
 // the result is the same in every lane).  Gives T_ae, T_be and T_ce, which
 // the passes do not fold.
-template <bool PLAIN>
 __device__ unsigned long long box_min2(const Dev &d, const P3Box &B, const BoxShape &sh, unsigned sp, unsigned kp,
                                        unsigned sq, unsigned kq)
 {
@@ -2255,32 +2214,20 @@ __device__ unsigned long long box_min2(const Dev &d, const P3Box &B, const BoxSh
     const unsigned rest = 0xFu & ~(1u << sp) & ~(1u << sq);
     const unsigned su = __ffs(rest) - 1, sv = 31 - __clz(rest);
     const unsigned mu = sh.m(su), mv = sh.m(sv);
-    const int4 pf = add4(B.A[sp][kp], B.A[sq][kq]);
+    const int pf = B.A[sp][kp].w + B.A[sq][kq].w;
     unsigned long long mn = NO_KEY;
     for (unsigned t = lane; t < mu * mv; t += 32) {
         const unsigned iv = divm(t, c_magic[mu]), iu = t - iv * mu;
-        const int4 s = add4(pf, add4(B.A[su][iu], B.A[sv][iv]));
-        unsigned long long key;
-        if (PLAIN) {
-            key = ldcg(d.fit_key + sh.cb + (unsigned)s.w);
-        } else {
-            bool ok;
-            key = box_key2(s, (unsigned)s.w, d.cut, true, ok);
-        }
-        mn = umin64(mn, key);
+        mn = umin64(mn, ldcg(d.fit_key + sh.cb + (unsigned)(pf + B.A[su][iu].w + B.A[sv][iv].w)));
     }
-    const unsigned hi = (unsigned)(mn >> 32);
-    const unsigned mh = __reduce_min_sync(FULL_MASK, hi);
-    const unsigned ml = __reduce_min_sync(FULL_MASK, hi == mh ? (unsigned)mn : 0xFFFFFFFFu);
-    return ((unsigned long long)mh << 32) | ml;
+    return warp_min_key(mn);
 }
 
 // T_ce[z][w]: the minimum key over every pair (x, y) at hits z, w of slots c and e
-template <bool PLAIN>
 __device__ __forceinline__ unsigned long long box_tce(const Dev &d, const P3Box &B, const BoxShape &sh, unsigned z,
                                                       unsigned w)
 {
-    return box_min2<PLAIN>(d, B, sh, sh.rc, z, sh.re, w);
+    return box_min2(d, B, sh, sh.rc, z, sh.re, w);
 }
 
 // the table holding the minima over slots p and q (p != q) and the index of
@@ -2305,7 +2252,7 @@ __device__ __forceinline__ unsigned box_tab(const BoxShape &sh, unsigned p, unsi
 }
 
 // ---------------------------------------------------------------------------
-// P3, box path, float pass: the road's chi-squares in float, two fits per
+// P3, box path, fused: the road's chi-squares in float, two fits per
 // instruction, with a bound on their error; whole numbers decide only where
 // floats cannot.
 //
@@ -2323,18 +2270,26 @@ __device__ __forceinline__ unsigned box_tab(const BoxShape &sh, unsigned p, unsi
 // below float_lo; a fit in [float_lo, float_hi] (one road in thirty) makes the
 // warp count again in whole numbers.  A pair (x, y) is a candidate when its
 // lowest row is near the minima of tables (a, c) and (b, c) there, which are
-// shuffle minima (1.2 a road).  A candidate's lowest fit is chosen by whole
-// keys among those near the lowest; it survives when none of the fits that
-// share two hits with it (about 320) has a lower whole key, of which only the
-// near ones are made.
+// shuffle minima.  A candidate's lowest fit is found in whole keys; it survives
+// when none of the fits that share two hits with it (about 320) has a lower one.
 //
-// Bound: issue slots, nine instructions per fit; in whole numbers (three
-// sums, floors and squares of 64 bits, 64-bit keys and minima) it took 48.
+// How many candidates there are depends on how near a road's hits lie: of 8^4
+// roads 1 with hits anywhere, 3 within 64 strips, 12 within 16, 29 within 8.  The
+// rows near at the first z say so (as many as there will be candidates): with more
+// than FLOAT_CANDS of them the pass ends there and the floor pass takes its place,
+// whose floats tell apart all but equal chi-squares (two candidates within 8
+// strips); where many are equal (constants of zero), the key pass takes its.
+//
+// Bound: issue slots, nine instructions per fit (14 in the floor pass, 20 in
+// the key pass, whose 64-bit minima have a seventh of the float rate).  The fit
+// stage of 12,800 roads of 8^4 fits: 50 us with hits anywhere, 68 within 16 strips,
+// 78 within 8, 98 with all chi-squares equal; in whole numbers with tables in
+// shared memory alone 84, 85, 90 and 85.
 // ---------------------------------------------------------------------------
 
-constexpr long long FLOAT_CUT = 1ll << 24;   // a smaller cut's band [lo, hi] is a visible share of the fits
+constexpr long long FLOAT_CUT = 1ll << 24;   // a smaller cut's band [lo, hi] is a visible share of the fits: floor pass
 constexpr float FLOAT_PAD = 1e18f;           // component of a missing hit: its fits are far above every cut
-constexpr unsigned FLOAT_CANDS = 8;          // candidates the float pass follows up (more: the integer passes)
+constexpr unsigned FLOAT_CANDS = 8;          // candidates a pass follows up (a candidate takes some 300 instructions)
 
 // Two floats in one 64-bit register pair (kept packed from load to result:
 // packing at every operation cost more moves than the operations), added and
@@ -2377,38 +2332,27 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return r;
 }
 
-// What a fit not above one of float c2 stays below ...
-__device__ __forceinline__ float float_near(float c2)
-{
-    return fmaf(c2, 1.000002f, fmaf(4.32f, sqrt_approx(c2), 4.8f));
-}
-// ... and a looser bound without a root, for the pass over the fits: 4.32
-// sqrt(c2) <= e c2 + 4.67 / e for every e; e = 5 / sqrt(cut) makes that equal
+// What the float of a fit not above one of float c2 stays below, without a root:
+// 4.32 sqrt(c2) <= e c2 + 4.67 / e for every e; e = 5 / sqrt(cut) makes that equal
 // near 0.2 cut (eps = 1.000002 + e, off = 4.8 + 0.94 sqrt(cut)).
 #define float_thr(c2) fmaf((c2), eps, off)
 
-// float chi-square of a fit given by its four partials
-__device__ __forceinline__ float float_chi(const float4 &a, const float4 &b, const float4 &c, const float4 &e)
-{
-    const float x = a.x + b.x + c.x + e.x, y = a.y + b.y + c.y + e.y, z = a.z + b.z + c.z + e.z;
-    return fmaf(z, z, fmaf(y, y, x * x));
-}
-
 // One lane's view of a road's fits: passing ones (below the band from `lo`),
 // the lowest place in the band, and of each of its pairs the lowest row and
-// the lowest row near the minima of tables (a, c) and (b, c).
+// the lowest row near the minima of tables (a, c) and (b, c).  hi: the band's end.
 struct FloatPass {
     unsigned np, near_cut;
     float q[2], qok[2];
+    bool many;   // the pass stopped after the first z: more than FLOAT_CANDS near rows
 };
 
 // TWO: slot b has more than four hits (the lane's second y); WIDE: slot e has.
 template <bool TWO, bool WIDE>
-__device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, unsigned lo, float eps, float off)
+__device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, unsigned lo, float hi, float eps, float off)
 {
     constexpr unsigned NJ = TWO ? 2 : 1, NI = WIDE ? 2 : 1;
     const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
-    FloatPass f{0u, ~0u, {3e38f, 3e38f}, {3e38f, 3e38f}};
+    FloatPass f{0u, ~0u, {3e38f, 3e38f}, {3e38f, 3e38f}, false};
     f2 px[NJ], py[NJ], pz[NJ];
 #pragma unroll
     for (unsigned j = 0; j < NJ; ++j) {
@@ -2453,16 +2397,185 @@ __device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, u
             f.q[j] = fminf(f.q[j], rz[j]);
             f.qok[j] = rz[j] <= float_thr(fminf(ac, bc)) ? fminf(f.qok[j], rz[j]) : f.qok[j];
         }
+        if (z == 0) {
+            unsigned n = 0;
+#pragma unroll
+            for (unsigned j = 0; j < NJ; ++j)
+                n += __popc(__ballot_sync(FULL_MASK, f.qok[j] <= hi));
+            f.many = n > FLOAT_CANDS;
+            if (f.many)
+                break;
+        }
     }
     return f;
 }
 
-// Fit road g with one warp; false when it is left to the integer passes.  The
-// shape's slots are roles here, by falling hit count.  Hits that repeat a
-// coordinate need nothing special (as in the group path).  Bound: issue slots
-// (two fits an instruction).  The fit stage of 25,600 roads of 8^4 distinct fits:
-// 153.8 -> 82.4 us with it in place of the integer passes.
-__device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
+// The same with the components' floors, which floats hold exactly: a chi-square
+// is then off by a relative 1.8e-7 at most, X1 <= X2 => c1 <= c2 FLOOR_EPS, and
+// rows are near only where chi-squares are all but equal.  The floor a of a sum
+// (|a| < 2^19) becomes a float by adding it to the bits of 1.5 2^23.
+constexpr float FLOOR_EPS = 1.0000005f, FLOOR_BIAS = -12582912.f;
+
+template <bool TWO, bool WIDE>
+__device__ __forceinline__ FloatPass floor_pass(const P3Box &B, const BoxShape &sh, unsigned lo, float hi)
+{
+    constexpr unsigned NJ = TWO ? 2 : 1, NI = WIDE ? 4 : 2;
+    const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
+    FloatPass f{0u, ~0u, {3e38f, 3e38f}, {3e38f, 3e38f}, false};
+    const f2 bias = f2_pack(FLOOR_BIAS, FLOOR_BIAS);
+    int4 pab[NJ];
+    bool live[NJ];
+    unsigned np[NJ];
+#pragma unroll
+    for (unsigned j = 0; j < NJ; ++j) {   // (a missing hit's row is unspecified)
+        pab[j] = add4(B.A[0][x], B.A[1][yl + 4 * j]);
+        live[j] = x < sh.ma && yl + 4 * j < sh.mb;
+        np[j] = 0;
+    }
+#pragma unroll 1
+    for (unsigned z = 0; z < sh.mc; ++z) {
+        int4 pz[NJ];
+        float rz[NJ];
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j)
+            pz[j] = add4(pab[j], B.A[2][z]);
+#pragma unroll
+        for (unsigned i = 0; i < NI; ++i) {
+            const int4 a0 = B.A[3][2 * i], a1 = B.A[3][2 * i + 1];
+            const f2 bx = reinterpret_cast<const f2 *>(B.F.bias)[i];   // (a missing hit's: far above every cut)
+            const auto part = [](int s, int t, f2 b) {
+                return f2_add(f2_pack(__int_as_float((s >> 12) + 0x4B400000), __int_as_float((t >> 12) + 0x4B400000)), b);
+            };
+#pragma unroll
+            for (unsigned j = 0; j < NJ; ++j) {
+                const f2 vx = part(pz[j].x + a0.x, pz[j].x + a1.x, bx), vy = part(pz[j].y + a0.y, pz[j].y + a1.y, bias),
+                         vz = part(pz[j].z + a0.z, pz[j].z + a1.z, bias);
+                const float2 c = f2_get(f2_fma(vz, vz, f2_fma(vy, vy, f2_mul(vx, vx))));
+                const unsigned d0 = __float_as_uint(c.x) - lo, d1 = __float_as_uint(c.y) - lo;
+                np[j] += d0 >> 31;
+                np[j] += d1 >> 31;
+                f.near_cut = min(f.near_cut, min(d0, d1));
+                rz[j] = i ? fminf(rz[j], fminf(c.x, c.y)) : fminf(c.x, c.y);
+            }
+        }
+        float ac = 3e38f;   // (a, c) at x, z
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            rz[j] = live[j] ? rz[j] : 3e38f;
+            ac = fminf(ac, rz[j]);
+        }
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 8));
+        ac = fminf(ac, __shfl_xor_sync(FULL_MASK, ac, 16));
+        unsigned n = 0;
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            float bc = rz[j];   // (b, c) at y, z
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 1));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 2));
+            bc = fminf(bc, __shfl_xor_sync(FULL_MASK, bc, 4));
+            f.q[j] = fminf(f.q[j], rz[j]);
+            f.qok[j] = rz[j] <= fminf(ac, bc) * FLOOR_EPS ? fminf(f.qok[j], rz[j]) : f.qok[j];
+            if (z == 0)
+                n += __popc(__ballot_sync(FULL_MASK, f.qok[j] <= hi));
+        }
+        f.many = n > FLOAT_CANDS;
+        if (f.many)
+            break;
+    }
+#pragma unroll
+    for (unsigned j = 0; j < NJ; ++j)
+        f.np += live[j] ? np[j] : 0u;
+    return f;
+}
+
+// The same in whole keys: the lane's passing fits, and of each of its pairs the
+// lowest one and whether tables (a, c) and (b, c) hold it too.  Keys differ by
+// comb, so that a pair has one lowest fit and no two are near.
+struct KeyPass {
+    unsigned np;
+    unsigned long long q[2];
+    bool ok[2];
+};
+
+template <bool TWO>
+__device__ __forceinline__ KeyPass key_pass(const P3Box &B, const BoxShape &sh, long long cut)
+{
+    constexpr unsigned NJ = TWO ? 2 : 1;
+    const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
+    // within a row (x, y, z) the order by (chi2, w) is that by key
+    const unsigned long long rb = (unsigned long long)(min(cut, 1ll << 38) + 1) << 3;   // chi2 <= cut iff below
+    KeyPass f{0u, {NO_KEY, NO_KEY}, {false, false}};
+    int4 pab[NJ];
+    unsigned np[NJ];
+#pragma unroll
+    for (unsigned j = 0; j < NJ; ++j) {
+        pab[j] = add4(B.A[0][x], B.A[1][yl + 4 * j]);
+        np[j] = 0;
+    }
+#pragma unroll 1
+    for (unsigned z = 0; z < sh.mc; ++z) {
+        int4 pz[NJ];
+        unsigned long long rz[NJ];
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            pz[j] = add4(pab[j], B.A[2][z]);
+            rz[j] = NO_KEY;
+        }
+        const auto fit = [&](unsigned w) {
+            const int4 aw = B.A[3][w];
+#pragma unroll
+            for (unsigned j = 0; j < NJ; ++j) {
+                const long long chi2 = sq((pz[j].x + aw.x) >> 12) + sq((pz[j].y + aw.y) >> 12) + sq((pz[j].z + aw.z) >> 12);
+                const unsigned long long key = (unsigned long long)chi2 << 3 | w;
+                np[j] += key < rb;
+                rz[j] = umin64(rz[j], key);
+            }
+        };
+        unsigned w = 0;
+#pragma unroll 1
+        for (; w + 4 <= sh.me; w += 4) {
+#pragma unroll
+            for (unsigned i = 0; i < 4; ++i)
+                fit(w + i);
+        }
+#pragma unroll 1
+        for (; w < sh.me; ++w)
+            fit(w);
+        unsigned long long ac = NO_KEY;   // (a, c) at x, z
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            // (no passing fit, or a pair whose hits do not exist: its sums are unspecified)
+            rz[j] = rz[j] < rb && x < sh.ma && yl + 4 * j < sh.mb
+                        ? (rz[j] >> 3 << 23) + (unsigned)(pz[j].w + B.A[3][(unsigned)rz[j] & 7u].w)
+                        : NO_KEY;
+            ac = umin64(ac, rz[j]);
+        }
+        ac = umin64(ac, __shfl_xor_sync(FULL_MASK, ac, 8));
+        ac = umin64(ac, __shfl_xor_sync(FULL_MASK, ac, 16));
+#pragma unroll
+        for (unsigned j = 0; j < NJ; ++j) {
+            unsigned long long bc = rz[j];   // (b, c) at y, z
+            bc = umin64(bc, __shfl_xor_sync(FULL_MASK, bc, 1));
+            bc = umin64(bc, __shfl_xor_sync(FULL_MASK, bc, 2));
+            bc = umin64(bc, __shfl_xor_sync(FULL_MASK, bc, 4));
+            if (rz[j] < f.q[j]) {   // (keys differ by comb: no two are equal but NO_KEY)
+                f.q[j] = rz[j];
+                f.ok[j] = umin64(ac, bc) == rz[j];
+            }
+        }
+    }
+#pragma unroll
+    for (unsigned j = 0; j < NJ; ++j)
+        f.np += x < sh.ma && yl + 4 * j < sh.mb ? np[j] : 0u;
+    return f;
+}
+
+// Fit road g with one warp.  The shape's slots are roles here, by falling hit
+// count.  Hits that repeat a coordinate need nothing special (as in the group
+// path).  Bound: issue slots (two fits an instruction).  The fit stage of 25,600
+// roads of 8^4 distinct fits: 153.8 -> 82.4 us (whole keys with tables in shared
+// memory before).
+__device__ __noinline__ void box_warp(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
     P3Box &B = *reinterpret_cast<P3Box *>(region);
     P3Float &F = B.F;
@@ -2508,7 +2621,8 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
             v = make_float4(fmaf((float)a.x, 1.f / 4096.f, o), fmaf((float)a.y, 1.f / 4096.f, o),
                             fmaf((float)a.z, 1.f / 4096.f, o), 0.f);
         }
-        F.hit[role][k] = v;
+        if (role < 2)
+            F.hit[role][k] = v;
         if (role == 2) {
             F.c[k][0] = ulonglong2{f2_pack(v.x, v.x), f2_pack(v.y, v.y)};
             F.c[k][1].x = f2_pack(v.z, v.z);
@@ -2518,47 +2632,73 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
             e[0] = v.x;
             e[4] = v.y;
             e[8] = v.z;
+            F.bias[k] = k < sh.me ? FLOOR_BIAS : FLOAT_PAD;
         }
     }
     __syncwarp();
-    // the cut's band
-    const float cut = (float)min(d.cut, 1ll << 38), root = sqrt_approx(cut);
-    const float band = fmaf(2.2f, root, 8.f);
-    const float eps = 1.000002f + 5.f / root, off = fmaf(0.94f, root, 4.8f);   // of float_thr
-    const float float_lo = cut * 0.999999f - band, float_hi = cut * 1.000001f + band;
-    const unsigned lo = __float_as_uint(float_lo), width = __float_as_uint(float_hi) + 1 - lo;
-
-    const unsigned x = lane & 7u, yl = lane >> 3;
+    unsigned cand[2];
+    // what decides: 0 floats, 1 floats of the floors, 2 whole keys
+    unsigned by = d.cut < FLOAT_CUT ? 1u : 0u, width = 0;
+    const float cut = (float)min(d.cut, 1ll << 38);
     FloatPass f;
-    if (sh.mb > 4 && sh.me > 4)
-        f = float_pass<true, true>(F, sh.mc, lo, eps, off);
-    else if (sh.mb > 4)
-        f = float_pass<true, false>(F, sh.mc, lo, eps, off);
-    else if (sh.me > 4)
-        f = float_pass<false, true>(F, sh.mc, lo, eps, off);
-    else
-        f = float_pass<false, false>(F, sh.mc, lo, eps, off);
-    unsigned np = f.np;
-    unsigned cand[2], n_cand = 0;
+    // candidates of a float pass whose chi-squares are near within (eps, off)
+    const auto candidates = [&](float eps, float off, float hi) {
 #pragma unroll
-    for (unsigned j = 0; j < 2; ++j) {
-        cand[j] = __ballot_sync(FULL_MASK, f.qok[j] <= float_thr(f.q[j]) && f.q[j] <= float_hi);
-        n_cand += __popc(cand[j]);
+        for (unsigned j = 0; j < 2; ++j)
+            cand[j] = __ballot_sync(FULL_MASK, f.qok[j] <= float_thr(f.q[j]) && f.q[j] <= hi);
+        return f.many || __popc(cand[0]) + __popc(cand[1]) > FLOAT_CANDS;   // too many
+    };
+    if (by == 0) {
+        // the cut's band
+        const float root = sqrt_approx(cut), band = fmaf(2.2f, root, 8.f);
+        const float eps = 1.000002f + 5.f / root, off = fmaf(0.94f, root, 4.8f);   // of float_thr
+        const float float_lo = cut * 0.999999f - band, float_hi = cut * 1.000001f + band;
+        const unsigned lo = __float_as_uint(float_lo);
+        width = __float_as_uint(float_hi) + 1 - lo;
+        if (sh.mb > 4 && sh.me > 4)
+            f = float_pass<true, true>(F, sh.mc, lo, float_hi, eps, off);
+        else if (sh.mb > 4)
+            f = float_pass<true, false>(F, sh.mc, lo, float_hi, eps, off);
+        else if (sh.me > 4)
+            f = float_pass<false, true>(F, sh.mc, lo, float_hi, eps, off);
+        else
+            f = float_pass<false, false>(F, sh.mc, lo, float_hi, eps, off);
+        by = candidates(eps, off, float_hi);
     }
-    if (n_cand > FLOAT_CANDS)
-        return false;
-    if (__any_sync(FULL_MASK, f.near_cut < width)) {   // count in whole numbers
+    if (by == 1) {
+        const float floor_lo = cut * (2.f - FLOOR_EPS), floor_hi = cut * FLOOR_EPS;
+        const unsigned lo = __float_as_uint(floor_lo);
+        width = __float_as_uint(floor_hi) + 1 - lo;
+        if (sh.mb > 4 && sh.me > 4)
+            f = floor_pass<true, true>(B, sh, lo, floor_hi);
+        else if (sh.mb > 4)
+            f = floor_pass<true, false>(B, sh, lo, floor_hi);
+        else if (sh.me > 4)
+            f = floor_pass<false, true>(B, sh, lo, floor_hi);
+        else
+            f = floor_pass<false, false>(B, sh, lo, floor_hi);
+        by += candidates(FLOOR_EPS, 0.f, floor_hi);
+    }
+    const unsigned x = lane & 7u, yl = lane >> 3;
+    unsigned np = f.np;
+    if (by == 2) {
+        const KeyPass k = sh.mb > 4 ? key_pass<true>(B, sh, d.cut) : key_pass<false>(B, sh, d.cut);
+        np = k.np;
+#pragma unroll
+        for (unsigned j = 0; j < 2; ++j)
+            cand[j] = __ballot_sync(FULL_MASK, k.ok[j]);
+    } else if (__any_sync(FULL_MASK, f.near_cut < width)) {   // count in whole numbers
         np = 0;
         for (unsigned j = 0; j < 2; ++j) {
             const unsigned y = yl + 4 * j;
             if (x >= sh.ma || y >= sh.mb)
                 continue;
-            const int4 pab = add4(B.A[sh.ra][x], B.A[sh.rb][y]);
+            const int4 pab = add4(B.A[0][x], B.A[1][y]);
             for (unsigned z = 0; z < sh.mc; ++z) {
-                const int4 p = add4(pab, B.A[sh.rc][z]);
+                const int4 p = add4(pab, B.A[2][z]);
                 for (unsigned w = 0; w < sh.me; ++w) {
                     bool pass;
-                    box_key(add4(p, B.A[sh.re][w]), d.cut, pass);
+                    box_key(add4(p, B.A[3][w]), d.cut, pass);
                     np += pass;
                 }
             }
@@ -2566,73 +2706,65 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
     }
     npass += (unsigned long long)np * sh.ne;
 
-    // the candidates, one after the other; lane i keeps survivor i
+    // the candidates, one after the other; lane i keeps survivors i and i + 32
     unsigned n_surv = 0;
-    unsigned long long mine = NO_KEY;
+    unsigned long long mine[2] = {NO_KEY, NO_KEY};
     const unsigned u = lane >> 3, v = lane & 7u;   // the lane's two hits of a table: u, u + 4 and v
+    const unsigned long long kb = (unsigned long long)(min(d.cut, 1ll << 38) + 1) << 23;   // chi2 <= cut iff key < kb
     for (unsigned j = 0; j < 2; ++j)
         for (unsigned bits = cand[j]; bits; bits &= bits - 1) {
             const unsigned src = __ffs(bits) - 1, cx = src & 7u, cy = (src >> 3) + 4 * j;
-            const float4 ha = F.hit[0][cx], hb = F.hit[1][cy];
-            const auto key_of = [&](unsigned a, unsigned b, unsigned c, unsigned e) {
-                bool pass;
-                return box_key(add4(add4(B.A[0][a], B.A[1][b]), add4(B.A[2][c], B.A[3][e])), d.cut, pass);
+            const auto key_of = [](const int4 &p, const int4 &q) {   // without the cut
+                const int4 s = add4(p, q);
+                return box_key_raw(s, (unsigned)s.w);
             };
-            // the pair's lowest fit: whole keys of the fits near the lowest float
-            const float c0 = float_chi(ha, hb, F.hit[2][u], F.hit[3][v]);
-            const float c1 = float_chi(ha, hb, F.hit[2][u + 4], F.hit[3][v]);
-            float thr = float_near(__uint_as_float(__reduce_min_sync(FULL_MASK, __float_as_uint(fminf(c0, c1)))));
-            unsigned long long key = c0 <= thr ? key_of(cx, cy, u, v) : NO_KEY;
-            bool second = false;
-            if (c1 <= thr) {
-                const unsigned long long k1 = key_of(cx, cy, u + 4, v);
-                second = k1 < key;
-                key = umin64(key, k1);
-            }
-            const unsigned kh = __reduce_min_sync(FULL_MASK, (unsigned)(key >> 32));
-            const unsigned kl = __reduce_min_sync(FULL_MASK, (unsigned)(key >> 32) == kh ? (unsigned)key : ~0u);
-            const unsigned long long kf = ((unsigned long long)kh << 32) | kl;
-            if (kf == NO_KEY)
-                continue;   // no passing fit
-            const unsigned at = __ffs(__ballot_sync(FULL_MASK, key == kf)) - 1;   // (keys differ by comb)
-            const unsigned cz = (at >> 3) + (__shfl_sync(FULL_MASK, second, at) ? 4u : 0u), cw = at & 7u;
-            key = kf;
-            // the fits that share two hits with it, two of each of the other
-            // five tables per lane; bit 5 i + t of `near`: not certainly larger
-            const float4 hc = F.hit[2][cz], he = F.hit[3][cw];
-            thr = float_near(float_chi(ha, hb, hc, he));
-            unsigned near = 0;
-#pragma unroll
-            for (unsigned i = 0; i < 2; ++i) {
-                const unsigned w = u + 4 * i;
-                const float4 a = F.hit[0][w], b = F.hit[1][w], bv = F.hit[1][v], c = F.hit[2][w], e = F.hit[3][v];
-                near |= (float_chi(ha, b, hc, e) <= thr && !(w == cy && v == cw)) ? 1u << (5 * i) : 0u;
-                near |= (float_chi(a, hb, hc, e) <= thr && !(w == cx && v == cw)) ? 2u << (5 * i) : 0u;
-                near |= (float_chi(ha, bv, c, he) <= thr && !(v == cy && w == cz)) ? 4u << (5 * i) : 0u;
-                near |= (float_chi(F.hit[0][v], hb, c, he) <= thr && !(v == cx && w == cz)) ? 8u << (5 * i) : 0u;
-                near |= (float_chi(a, bv, hc, he) <= thr && !(w == cx && v == cy)) ? 16u << (5 * i) : 0u;
-            }
+            const int4 a = B.A[0][cx], b = B.A[1][cy], ev = B.A[3][v];
+            // the pair's lowest fit and its hits
+            const unsigned long long k0 = key_of(add4(a, b), add4(B.A[2][u], ev)),
+                                     k4 = key_of(add4(a, b), add4(B.A[2][u + 4], ev));
+            const bool in = u < sh.mc & v < sh.me, in4 = u + 4 < sh.mc & v < sh.me;
+            const unsigned long long kf = warp_min_key(umin64(in ? k0 : NO_KEY, in4 ? k4 : NO_KEY));
+            if (kf >= kb)
+                continue;   // it does not pass
+            const unsigned at4 = __ballot_sync(FULL_MASK, in4 & (k4 == kf)),
+                           at = at4 | __ballot_sync(FULL_MASK, in & (k0 == kf));   // (keys differ by comb: one lane)
+            const unsigned cz = ((__ffs(at) - 1) >> 3) + (at4 ? 4u : 0u), cw = (__ffs(at) - 1) & 7u;
+            // tables (a, c) and (b, c), two fits of each per lane, then the others
+            const int4 c = B.A[2][cz], e = B.A[3][cw];
             bool kill = false;
-            while (__any_sync(FULL_MASK, near != 0u)) {   // in whole keys, one per lane at a time
-                if (near) {
-                    const unsigned q = __ffs(near) - 1, t = q < 5 ? q : q - 5, w = u + (q < 5 ? 0u : 4u);
-                    kill = kill || key_of(t == 0 || t == 2 ? cx : t == 3 ? v : w, t == 1 || t == 3 ? cy : t == 0 ? w : v,
-                                          t == 2 || t == 3 ? w : cz, t < 2 ? v : cw) < kf;
-                    near &= near - 1;
-                }
+#pragma unroll
+            for (unsigned i = 0; i < 8; i += 4) {
+                const unsigned w = u + i;
+                kill |= w < sh.mb & v < sh.me & key_of(add4(a, c), add4(B.A[1][w], ev)) < kf;
+                kill |= w < sh.ma & v < sh.me & key_of(add4(b, c), add4(B.A[0][w], ev)) < kf;
             }
             if (__any_sync(FULL_MASK, kill))
                 continue;
-            if (lane == n_surv)
-                mine = key;
+            const int4 cv = B.A[2][v], av = B.A[0][v];
+#pragma unroll
+            for (unsigned i = 0; i < 8; i += 4) {
+                const unsigned w = u + i;
+                kill |= w < sh.mb & v < sh.mc & key_of(add4(a, e), add4(B.A[1][w], cv)) < kf;
+                kill |= w < sh.ma & v < sh.mc & key_of(add4(b, e), add4(B.A[0][w], cv)) < kf;
+                kill |= w < sh.mb & v < sh.ma & key_of(add4(c, e), add4(B.A[1][w], av)) < kf;
+            }
+            if (__any_sync(FULL_MASK, kill))
+                continue;
+            if (lane == (n_surv & 31u))
+                mine[0] = n_surv < 32 ? kf : mine[0], mine[1] = n_surv < 32 ? mine[1] : kf;
             ++n_surv;
         }
     // in comb order
-    unsigned rank = 0;
-    for (unsigned i = 0; i < n_surv; ++i)
-        rank += ((unsigned)__shfl_sync(FULL_MASK, mine, i) & 0x7FFFu) < ((unsigned)mine & 0x7FFFu);
-    if (lane < n_surv)
-        d.surv_pool[surv_at(d, g, rank)] = mine;
+    unsigned rank[2] = {0u, 0u};
+    for (unsigned i = 0; i < n_surv; ++i) {
+        const unsigned other = (unsigned)__shfl_sync(FULL_MASK, i < 32 ? mine[0] : mine[1], i & 31u) & 0x7FFFu;
+        rank[0] += other < ((unsigned)mine[0] & 0x7FFFu);
+        rank[1] += other < ((unsigned)mine[1] & 0x7FFFu);
+    }
+#pragma unroll
+    for (unsigned i = 0; i < 2; ++i)
+        if (lane + 32 * i < n_surv)
+            d.surv_pool[surv_at(d, g, rank[i])] = mine[i];
     if (lane == 0) {
         d.surv_cnt[g] = (uint8_t)n_surv;
         if (n_surv)
@@ -2641,12 +2773,11 @@ __device__ __noinline__ bool box_float(const Dev &d, unsigned char *region, unsi
     if ((pk >> 23) & 1u)   // a cross-road candidate
         publish_road(d, g, rec);
     __syncwarp();
-    return true;
 }
 
-// Fit a listed road with one warp (see above); adds its passing combinations to npass.
-template <bool PLAIN>
-__device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
+// The road-local hit-warrior of the plain pipeline for a listed road, by one warp
+// from the keys the fit kernel stored.
+__device__ __noinline__ void box_plain(const Dev &d, unsigned char *region, unsigned g)
 {
     P3Box &B = *reinterpret_cast<P3Box *>(region);
     const unsigned lane = lane_id();
@@ -2659,7 +2790,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     __syncwarp();
 
     // lane 8 j + h: raw hit h of fitted slot j.  Canonical hits, their ranks
-    // and multiplicities, and the partial sums of the canonical hits.
+    // and comb parts.
     const unsigned j = lane >> 3, h = lane & 7u;
     const unsigned L = j + (j >= excl);
     const unsigned nj = hits_of(pk, L);
@@ -2672,9 +2803,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     }
     const bool canon = valid && cls == h;
     const unsigned cm = __ballot_sync(FULL_MASK, canon);
-    const bool dup = __ballot_sync(FULL_MASK, valid) != cm;
     const unsigned mine = (cm >> (8 * j)) & 0xFFu;
-    const unsigned same = __match_any_sync(FULL_MASK, valid ? j * 8 + cls : 32u + lane);
     const unsigned k = __popc(mine & ((1u << h) - 1u));
     if (valid)
         B.rank[j][h] = (uint8_t)__popc(mine & ((1u << cls) - 1u));
@@ -2684,30 +2813,12 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     for (unsigned s = 0; s < 4; ++s)
         sh.mpk |= (unsigned)__popc((cm >> (8 * s)) & 0xFFu) << (4 * s);
     sh.ne = hits_of(pk, excl);
-    sh.cb = PLAIN ? ldcg(d.comb_off + g) : 0ull;
+    sh.cb = ldcg(d.comb_off + g);
     if (canon) {
         unsigned SL = 1;   // comb stride of layer L
         for (unsigned l = 0; l < L; ++l)
             SL *= hits_of(pk, l);
-        B.raw[j][k] = (uint8_t)h;
-        B.mult[j][k] = (uint8_t)__popc(same);
-        int4 a = make_int4(0, 0, 0, (int)(h * SL));
-        if (!PLAIN) {
-            const int4 *cc = d.fitc + SET_INT4 * min((unsigned)rec.set, (unsigned)(N_SETS - 1)) + SET_C;
-            const int4 cj = __ldg(cc + j);
-            const int hv = B.co[L * 8 + h];
-            a.x = cj.x * hv;
-            a.y = cj.y * hv;
-            a.z = cj.z * hv;
-            if (j == 0) {   // curvature, phi, 4096 * offset and the road bits ride on slot 0
-                const int4 c4 = __ldg(cc + 4), c5 = __ldg(cc + 5), kk = __ldg(cc + 6);
-                a.x += c4.x * rec.curv + c5.x * rec.phi + 4096 * kk.x;
-                a.y += c4.y * rec.curv + c5.y * rec.phi + 4096 * kk.y;
-                a.z += c4.z * rec.curv + c5.z * rec.phi + 4096 * kk.z;
-                a.w += (int)((pk >> 24) << 15);
-            }
-        }
-        B.A[j][k] = a;
+        B.A[j][k] = make_int4(0, 0, 0, (int)(h * SL));
     }
     for (unsigned i = lane; i < 4 * 8 * TS; i += 32)
         (&B.T[0][0])[i] = NO_KEY;
@@ -2746,27 +2857,17 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
     // the loop over the box: every table but T_ce
     const unsigned ma = sh.ma, mb = sh.mb, me = sh.me;
     const unsigned passes = (ma * mb + 31) / 32;   // 1 or 2
-    unsigned np = 0;
     // full passes and all eight hits of slot e (every 8^4 road): no per-step predicate
-    const bool fullw = (ma * mb) % 32 == 0 && me == 8 && !dup;
+    const bool fullw = (ma * mb) % 32 == 0 && me == 8;
     for (unsigned p = 0; p < passes; ++p) {
         if (fullw)
-            box_pass<PLAIN, false, 8, true>(d, B, sh, p, np);
-        else if (me > 4) {
-            if (dup)
-                box_pass<PLAIN, true, 8, false>(d, B, sh, p, np);
-            else
-                box_pass<PLAIN, false, 8, false>(d, B, sh, p, np);
-        } else {
-            if (dup)
-                box_pass<PLAIN, true, 4, false>(d, B, sh, p, np);
-            else
-                box_pass<PLAIN, false, 4, false>(d, B, sh, p, np);
-        }
+            box_pass<8, true>(d, B, sh, p);
+        else if (me > 4)
+            box_pass<8, false>(d, B, sh, p);
+        else
+            box_pass<4, false>(d, B, sh, p);
     }
     __syncwarp();
-    if (!PLAIN)
-        npass += (unsigned long long)np * sh.ne;
 
     // road-local survivors: the minimum of pair (x, y) survives iff it is
     // also the minimum of its other five tables; T_ce (the minimum over all
@@ -2810,9 +2911,9 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
             const unsigned x = e & 7u, y = (e >> 3) & 7u, z = (e >> 6) & 7u, w = e >> 9;
             // T_ae, T_be, T_ce of the candidate, on demand (each one only if
             // the ones before hold the key)
-            bool ok = box_min2<PLAIN>(d, B, sh, sh.ra, x, sh.re, w) == key;
-            ok = ok && box_min2<PLAIN>(d, B, sh, sh.rb, y, sh.re, w) == key;
-            ok = ok && box_tce<PLAIN>(d, B, sh, z, w) == key;
+            bool ok = box_min2(d, B, sh, sh.ra, x, sh.re, w) == key;
+            ok = ok && box_min2(d, B, sh, sh.rb, y, sh.re, w) == key;
+            ok = ok && box_tce(d, B, sh, z, w) == key;
             if (lane == src)
                 sv[p] = ok;
         }
@@ -2881,7 +2982,7 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
                     for (unsigned bp = fl(Lp); bp; bp &= bp - 1)
                         for (unsigned be = fe; be; be &= be - 1) {
                             const unsigned kp = B.rank[sp][__ffs(bp) - 1], w = B.rank[sh.re][__ffs(be) - 1];
-                            const unsigned long long m = box_min2<PLAIN>(d, B, sh, sp, kp, sh.re, w);
+                            const unsigned long long m = box_min2(d, B, sh, sp, kp, sh.re, w);
                             if (lane == 0) {
                                 B.T[q == 0 ? T_AE : q == 1 ? T_BE : T_CE][kp * TS + w] = m;
                             }
@@ -2916,24 +3017,16 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
             unsigned long long mn = NO_KEY;
             if (lt[0] != excl && lt[1] != excl && lt[2] != excl) {
                 // three fitted slots fixed; the fourth runs over its canonical hits
-                int4 base = make_int4(0, 0, 0, 0);
+                int base = 0;
                 unsigned free_slot = 0 + 1 + 2 + 3;
 #pragma unroll
                 for (unsigned q = 0; q < 3; ++q) {
                     const unsigned s = lt[q] - (lt[q] > excl);
                     free_slot -= s;
-                    base = add4(base, B.A[s][B.rank[s][dsel[q]]]);
+                    base += B.A[s][B.rank[s][dsel[q]]].w;
                 }
                 for (unsigned z = 0; z < sh.m(free_slot); ++z) {
-                    const int4 s = add4(base, B.A[free_slot][z]);
-                    unsigned long long key;
-                    if (PLAIN) {
-                        key = ldcg(d.fit_key + sh.cb + (unsigned)s.w);
-                    } else {
-                        bool pass;
-                        key = box_key(s, d.cut, pass);
-                    }
-                    mn = umin64(mn, key);
+                    mn = umin64(mn, ldcg(d.fit_key + sh.cb + (unsigned)(base + B.A[free_slot][z].w)));
                 }
             } else {
                 // the excluded layer in the triple: the pair table of the two
@@ -2970,8 +3063,10 @@ __device__ __noinline__ void box_integer(const Dev &d, unsigned char *region, un
 template <bool PLAIN>
 __device__ __forceinline__ void box_road(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
-    if (PLAIN || d.cut < FLOAT_CUT || !box_float(d, region, g, npass))
-        box_integer<PLAIN>(d, region, g, npass);
+    if (PLAIN)
+        box_plain(d, region, g);
+    else
+        box_warp(d, region, g, npass);
 }
 
 // Shared memory of P3: what every step reads of the kernel's argument (a load

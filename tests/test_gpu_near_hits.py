@@ -7,7 +7,7 @@ import pytest
 
 from paper_1312_0917_gb300 import binding as B
 from gpu_util import torch_words
-from test_gpu_stages import batch, check, p90
+from test_gpu_stages import FLOAT_CUT, batch, check, p90
 
 pytestmark = pytest.mark.gpu
 
@@ -88,6 +88,47 @@ def test_every_fit_tied(ctx, orc, consts):
         check(ctx, orc, words, flat, 1 << 40, mode=B.PLAIN)
 
 
+BIG = [(5, 8), (4, 8), (8, 8)]
+
+
+@pytest.mark.parametrize("width", [8, 16, 64])
+@pytest.mark.parametrize("lo,hi", BIG, ids=["%d-%d" % s for s in BIG])
+def test_near_candidates(ctx, orc, consts, lo, hi, width):
+    """Roads of a warp each, with few and with many fits that floats cannot
+    tell apart, above and below the cut from which floats are used."""
+    words = near(batch("near", 2, 20, lo, hi, shared=0.2, seed=hi), width)
+    cut = p90(orc, words, consts)
+    check(ctx, orc, words, consts, cut)
+    check(ctx, orc, words, consts, cut, mode=B.PLAIN)
+    check(ctx, orc, words, consts, FLOAT_CUT)
+    check(ctx, orc, words, consts, FLOAT_CUT - 1)
+    check(ctx, orc, near(words, width, distinct=False), consts, cut)
+
+
+def test_many_survivors(ctx, orc):
+    """Roads of 8^4 fits of which those with c = a + b and e = a - b have
+    chi-square zero, with a, b in 0..7, c in 0, 2, .. 14 and e in -6, -4, .. 8:
+    one for each of the 32 pairs of like parity, no two with two hits in common,
+    so that all of them survive."""
+    from conftest import zero_consts
+    flat = zero_consts()
+    flat["C"][:, 0, :3] = 4096, 4096, -4096
+    flat["C"][:, 1, :2], flat["C"][:, 1, 3] = (4096, -4096), -4096
+    flat["k"][:, 0], flat["k"][:, 1] = 1000, 2000 + 6
+    words = batch("many", 40, 1, 8, 8, seed=4)
+    kind = (words >> 27) & 7
+    road = np.cumsum(kind == 7) - 1
+    excl = ((words >> 7) & 7)[kind == 7][road]
+    for f, (first, step) in enumerate(((0, 1), (0, 1), (1000, 2), (2000, 2))):   # fitted layers in order
+        for x in range(5):
+            at = np.nonzero((excl == x) & (kind == f + (f >= x)))[0]
+            words[at] = (words[at] & np.uint32(0xFFFFF000)) | (first + step * (np.arange(len(at)) % 8)).astype(np.uint32)
+    want, _ = check(ctx, orc, words, flat, 1 << 40)
+    assert len(want) >= 32 * 40
+    check(ctx, orc, words, flat, 1)
+    check(ctx, orc, words, flat, 1 << 40, mode=B.PLAIN)
+
+
 def test_ties_cost_one_more_pass(ctx, consts, cuts):
     """A tied road takes its warp step twice: with hits 16 strips apart the fit
     stage stays below three times its time with hits anywhere."""
@@ -101,3 +142,14 @@ def test_repeats_cost_one_more_pass(ctx, consts, cuts):
     ctx.load_constants(consts, cuts["scaled"])
     words = batch("apart", 1000, 64, 1, 4)
     assert fit_us(ctx, near(words, 16, distinct=False)) < 3 * fit_us(ctx, words)
+
+
+@pytest.mark.parametrize("kind", ["near", "small_cut"])
+def test_near_candidates_cost_one_pass(ctx, consts, cuts, kind):
+    """Whole keys for every fit take less than twice the pass in floats."""
+    words = batch("apart", 100, 128, 8, 8)
+    ctx.load_constants(consts, cuts["stress"])
+    t = fit_us(ctx, words)
+    if kind == "small_cut":
+        ctx.load_constants(consts, FLOAT_CUT - 1)
+    assert fit_us(ctx, near(words, 16) if kind == "near" else words) < 2 * t

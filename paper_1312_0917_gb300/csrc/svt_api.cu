@@ -58,7 +58,7 @@ int read_ctrl(svt_ctx *c, cudaStream_t s)
 {
     if (cudaStreamSynchronize(s) != cudaSuccess)
         return SVT_E_CUDA;
-    if (c->h_ctrl->flags & FLAG_TIMEOUT)
+    if (c->h_ctrl->flags() & FLAG_TIMEOUT)
         c->hash_dirty = true;   // the batch may have stopped before clearing the table
     return SVT_OK;
 }
@@ -378,7 +378,7 @@ int svt_get_tracks(svt_ctx *c, svt_track *out, size_t cap, size_t *n_out, void *
     if ((spec && cudaMemcpyAsync(out, src, spec * sizeof(svt_track), cudaMemcpyDefault, s)) ||
         cudaStreamSynchronize(s))
         return SVT_E_CUDA;
-    if (c->h_ctrl->flags & FLAG_TIMEOUT)
+    if (c->h_ctrl->flags() & FLAG_TIMEOUT)
         c->hash_dirty = true;   // the batch may have stopped before clearing the table
     int st = status_of(*c->h_ctrl);
     if (st)

@@ -74,15 +74,15 @@ inline bool constants_admissible(const svt_const_set *sets)
 // Status of a batch from its control block (after the kernels).
 inline int status_of(const Ctrl &c)
 {
-    if (c.flags & FLAG_TIMEOUT)
+    if (c.flags() & FLAG_TIMEOUT)
         return SVT_E_TIMEOUT;
-    if (c.flags & FLAG_CAPACITY)
+    if (c.flags() & FLAG_CAPACITY)
         return SVT_E_CAPACITY;
     if (c.err_inv != 0ull) {
         unsigned rank = (unsigned)(~c.err_inv & 0xFFull);
         return rank == RANK_BAD ? SVT_E_BADWORD : rank == RANK_LIMIT ? SVT_E_LIMIT : SVT_E_TRUNCATED;
     }
-    if (c.flags & FLAG_INTERNAL)
+    if (c.flags() & FLAG_INTERNAL)
         return SVT_E_CUDA;
     return SVT_OK;
 }

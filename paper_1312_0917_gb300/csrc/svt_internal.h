@@ -64,12 +64,12 @@ inline void fit_words(const svt_const_set *sets, int32_t *out)
 // Per-batch control block in device memory.  It is zero before each batch: the
 // last CTA to leave a batch's last kernel copies it out (Dev::last, Dev::host)
 // and clears it, so a batch needs no memset before its kernel and no copy of
-// its status behind it.  Queue counters hand out work items; `bar` counts
-// grid-barrier arrivals of the persistent kernel.
+// its status behind it.  Queue counters hand out work items.
 struct Ctrl {
     unsigned long long err_inv;   // max over faults of ~((pos << 8) | rank); 0 = none
-    unsigned int bar;             // grid barrier arrivals; its polls read the flags with it
-    unsigned int flags;           // FLAG_*
+    unsigned long long sync;      // grid barrier arrivals in the low word, FLAG_* in the high word: written
+                                  // and polled by 64-bit operations alone, so that a poll that sees an
+                                  // arrival sees every flag raised before it
     unsigned int n_events;        // complete events (EE words)
     unsigned int n_ep;            // EP words in the stream
     unsigned int has_tail;        // words after the last EE
@@ -84,6 +84,7 @@ struct Ctrl {
     unsigned long long pad1[2];
     unsigned long long t_phase[8];   // persistent kernel: globaltimer at its start, after each
                                      // barrier (block 0) and when the last CTA leaves
+    unsigned flags() const { return (unsigned)(sync >> 32); }
 };
 
 // Unpacked road, 16 bytes.  pk: n[l] in bits 4l..4l+3 (l < 5), excluded layer

@@ -99,7 +99,13 @@ __device__ __forceinline__ RoadRec ldcg(const RoadRec *p)
     return r;
 }
 
-__device__ __forceinline__ void raise_flag(const Dev &d, unsigned f) { atomicOr(&d.ctrl->flags, f); }
+__device__ __forceinline__ void raise_flag(const Dev &d, unsigned f)
+{
+    atomicOr(&d.ctrl->sync, (unsigned long long)f << 32);
+}
+
+// the flags raised before this kernel
+__device__ __forceinline__ unsigned flags_of(const Dev &d) { return (unsigned)(ldcg(&d.ctrl->sync) >> 32); }
 
 // a fault of the stream at word err >> 8 of rank err & 255
 __device__ __forceinline__ void report(const Dev &d, unsigned long long err)
@@ -396,16 +402,13 @@ __device__ bool grid_sync(const Dev &d, unsigned k, unsigned &flags)
     __shared__ unsigned s_flags;
     __syncthreads();
     if (threadIdx.x == 0) {
-        static_assert(offsetof(Ctrl, bar) % 8 == 0 && offsetof(Ctrl, flags) == offsetof(Ctrl, bar) + 4,
-                      "count and flags in one word");
-        const unsigned long long *word = reinterpret_cast<const unsigned long long *>(&d.ctrl->bar);
         __threadfence();
-        atomicAdd(&d.ctrl->bar, 1u);
+        atomicAdd(&d.ctrl->sync, 1ull);
         const unsigned target = k * gridDim.x;
         unsigned long long t0 = 0, v;
         // relaxed polls (the fence below orders what follows); the clock is
         // looked at every 16th poll
-        for (unsigned it = 1; v = ld_relaxed(word), (int)((unsigned)v - target) < 0; ++it) {
+        for (unsigned it = 1; v = ld_relaxed(&d.ctrl->sync), (int)((unsigned)v - target) < 0; ++it) {
             if ((unsigned)(v >> 32) & FLAG_TIMEOUT)
                 break;
             if ((it & 15u) == 0) {
@@ -3852,7 +3855,7 @@ __global__ void __launch_bounds__(BLOCK) k_p1(Dev d)
 __global__ void __launch_bounds__(BLOCK) k_p2(Dev d)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    if (ldcg(&d.ctrl->flags) & (FLAG_CAPACITY | FLAG_FAULT))
+    if (flags_of(d) & (FLAG_CAPACITY | FLAG_FAULT))
         return;
     Batch bt{ldcg(&d.ctrl->n_events), ldcg(&d.ctrl->n_ep), 0u};
     p2_phase(d, smem, bt);
@@ -3860,7 +3863,7 @@ __global__ void __launch_bounds__(BLOCK) k_p2(Dev d)
 
 __device__ __forceinline__ bool stop_after_unpack(const Dev &d)
 {
-    return ldcg(&d.ctrl->flags) & (FLAG_CAPACITY | FLAG_FAULT);
+    return flags_of(d) & (FLAG_CAPACITY | FLAG_FAULT);
 }
 
 // combinations per road -> exclusive offsets (the "combine" stage)
@@ -3978,7 +3981,7 @@ __global__ void __launch_bounds__(BLOCK) k_warrior_plain(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem[];
     if (stop_after_unpack(d))
         return;
-    p3_phase<true>(d, smem, Q_BOX, Q_GROUP, ldcg(&d.ctrl->flags) & FLAG_CANDS);
+    p3_phase<true>(d, smem, Q_BOX, Q_GROUP, flags_of(d) & FLAG_CANDS);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_p4(Dev d)

@@ -141,7 +141,7 @@ void finish(svt_server *s, Slot &sl, int status, size_t n_tracks)
         std::vector<svt_track> tr;
         if (status == SVT_OK && n_tracks)
             tr.assign(sl.h_tracks, sl.h_tracks + n_tracks);
-        if (h.flags & FLAG_TIMEOUT)
+        if (h.flags() & FLAG_TIMEOUT)
             sl.ctx->hash_dirty = true;
         std::lock_guard<std::mutex> lk(s->mu);
         for (auto it = s->parents.begin(); it != s->parents.end(); ++it)
@@ -172,7 +172,7 @@ void finish(svt_server *s, Slot &sl, int status, size_t n_tracks)
         (uint64_t)std::chrono::duration_cast<std::chrono::nanoseconds>(Clock::now() - sl.t_submit).count();
     if (status == SVT_OK && n_tracks)
         r.tracks.assign(sl.h_tracks, sl.h_tracks + n_tracks);
-    if (h.flags & FLAG_TIMEOUT)
+    if (h.flags() & FLAG_TIMEOUT)
         sl.ctx->hash_dirty = true;   // the batch may have stopped before clearing its table
     std::lock_guard<std::mutex> lk(s->mu);
     s->results.push_back(std::move(r));

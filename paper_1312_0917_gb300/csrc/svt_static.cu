@@ -169,7 +169,7 @@ extern "C" int svt_run_static(const uint32_t *d_words, size_t n_words, const svt
     Ctrl h;
     if (cudaMemcpyAsync(&h, d.last, sizeof(Ctrl), cudaMemcpyDeviceToHost, s) || cudaStreamSynchronize(s))
         return SVT_E_CUDA;
-    da->hash_dirty = (h.flags & FLAG_TIMEOUT) != 0;
+    da->hash_dirty = (h.flags() & FLAG_TIMEOUT) != 0;
     const int st = status_of(h);
     // with SVT_E_CAPACITY, the survivors when they did not fit `cap`; 0 when
     // an arena limit (events, roads, group table) was exceeded

@@ -308,15 +308,15 @@ __device__ bool last_block(unsigned *counter, unsigned nblocks)
 // last one copies the control block out, to the host as well, and clears it
 // for the next batch.  A memset in front of the kernel and a copy behind it
 // did this before: two more commands in the stream, 4.0 us of a batch (35.8 ->
-// 31.8 us around a kernel of 21 us).
-__device__ void leave(const Dev &d, bool finished)
+// 31.8 us around a kernel of 21 us).  wrote: thread 0 has, or may have, written the
+// control block since the last barrier (a CTA that has not need not wait here for
+// its tracks to land: 0.5 us).
+__device__ void leave(const Dev &d, bool finished, bool wrote)
 {
     __shared__ unsigned s_last;
     __syncthreads();
     if (threadIdx.x == 0) {
-        // a finished chain's output stage writes the control block in these two
-        // CTAs alone; the others need not wait here for their tracks to land
-        if (!finished || blockIdx.x == 0 || blockIdx.x == gridDim.x - 1)
+        if (wrote)
             __threadfence();
         s_last = atomicAdd(&d.ctrl->done[0], 1u) == gridDim.x - 1;
     }
@@ -3690,8 +3690,10 @@ struct P5Smem {
     svt_track track[P5_TRACKS];
 };
 
-__device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads)
+// Thread 0 alone writes the control block here: `wrote`.
+__device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads, bool &wrote)
 {
+    wrote = false;
     P5Smem &s = *reinterpret_cast<P5Smem *>(smem);
     const unsigned n_chunks = min((n_roads + ROAD_CHUNK - 1) / ROAD_CHUNK, d.max_chunks_r);
     const unsigned lo = (unsigned)((unsigned long long)n_roads * blockIdx.x / gridDim.x);
@@ -3725,6 +3727,7 @@ __device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads)
             block_sum2(all, before);
             summed = true;
             if (blockIdx.x == 0 && threadIdx.x == 0) {
+                wrote = true;
                 d.ctrl->n_out = all;
                 if (all > d.max_tracks)
                     raise_flag(d, FLAG_CAPACITY);
@@ -3754,8 +3757,10 @@ __device__ void p5_phase(const Dev &d, unsigned char *smem, unsigned n_roads)
         before += tot;
     }
     // the roads' counts and the chunk totals agree
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && before != all)
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0 && before != all) {
+        wrote = true;
         raise_flag(d, FLAG_INTERNAL);
+    }
 }
 
 // Leave the group table empty: every claimed slot (its bit) is cleared, with
@@ -3783,9 +3788,11 @@ __device__ void clear_hash(const Dev &d)
 // ---------------------------------------------------------------------------
 
 
-// the whole chain; false: it stopped early (a fault, a limit, a wait that ran out)
-__device__ __forceinline__ bool chain(const Dev &d)
+// The whole chain; false: it stopped early (a fault, a limit, a wait that ran out).
+// wrote: as leave() takes it; true until the output stage says otherwise.
+__device__ __forceinline__ bool chain(const Dev &d, bool &wrote)
 {
+    wrote = true;
     extern __shared__ __align__(16) unsigned char smem[];
     if (d.skip_arrival == 1 && blockIdx.x == 0)
         return false;   // test hook: this CTA never arrives at the first barrier
@@ -3825,7 +3832,7 @@ __device__ __forceinline__ bool chain(const Dev &d)
             return false;
     }
     stamp(d, 5);
-    p5_phase(d, smem, bt.n_roads);
+    p5_phase(d, smem, bt.n_roads, wrote);
     // every lookup is done (barrier above): leave the group table empty
     if (groups)
         clear_hash(d);
@@ -3834,8 +3841,9 @@ __device__ __forceinline__ bool chain(const Dev &d)
 
 __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 2 : 768 / BLOCK) k_persistent(const __grid_constant__ Dev d)
 {
-    const bool finished = chain(d);
-    leave(d, finished);
+    bool wrote;
+    const bool finished = chain(d, wrote);
+    leave(d, finished, wrote);
 }
 
 #if SVT_BLOCK == 256
@@ -4006,7 +4014,7 @@ __global__ void __launch_bounds__(BLOCK) k_p5(Dev d)
             p5_item<true>(d, c, n_roads, s_first);
     // the previous kernels' lookups are done: leave the group table empty
     clear_hash(d);
-    leave(d, false);
+    leave(d, false, true);
 }
 
 __global__ void __launch_bounds__(BLOCK) k_export_roads(Dev d)

@@ -195,8 +195,8 @@ int svt_get_stats(svt_ctx *ctx, svt_stats *out, void *stream);
  * depend on them (every combination of values below gives the same bytes). */
 typedef struct {
     int32_t block;           /* threads per CTA: 128, 256 or 512 (0 = 256) */
-    int32_t blocks_per_sm;   /* resident CTAs per SM (0 = by the words of the batch, at most the
-                              * occupancy maximum of that block size) */
+    int32_t blocks_per_sm;   /* resident CTAs per SM (0, or the occupancy maximum of that block size
+                              * or more = by the words of the batch, at most that maximum) */
     int32_t small_n4;        /* roads with more than this many distinct fits (combinations of the
                               * four fitted layers) take a warp of their own (the box path); the
                               * others are fitted several to a warp (1 .. 256, 0 = 256) */
@@ -211,7 +211,7 @@ typedef struct {
 int svt_set_launch(svt_ctx *ctx, const svt_launch *cfg);
 
 /* The launch settings in use, with the zeros resolved (*out, HOST);
- * blocks_per_sm = 0 as the occupancy maximum. */
+ * blocks_per_sm = 0 as the occupancy maximum (the same setting). */
 int svt_get_launch(svt_ctx *ctx, svt_launch *out);
 
 /* One configuration measured by svt_autotune. */

@@ -188,6 +188,29 @@ using b256::launch_export_roads;
 constexpr int PERSISTENT_BLOCKS[3] = {128, 256, 512};   // the block sizes built
 inline bool persistent_block_ok(int block) { return block == 128 || block == 256 || block == 512; }
 
+// Resident CTAs per SM of a batch of n_words words: `set` (svt_launch::blocks_per_sm)
+// below the occupancy maximum `most`; at 0 or the maximum, by the words.  (Both
+// mean "as many as are of use", so that a setting read back by svt_get_launch,
+// which gives the maximum for 0, is the same setting.)
+//
+// Every CTA costs each barrier an arrival and each stage its first loads and
+// instructions, so the grid grows with the batch: 256 threads an SM up to 640
+// words an SM (97k words on 152 SMs), 512 up to 3072 (467k), then all that
+// fit.  Device time with one, two and three CTAs of 256 an SM, us: one event
+// of 977 words 27.5 / 28.9 / 30.5, 8k words 24.7 / 26.8 / 30.4, 99k words
+// 37.1 / 38.4 / 41.7, 155k words 61 / 57 / 61 (shared hits), 495k words
+// 57.4 / 51.2 / 53.3, 978k words 158 / 119 / 110 (one to eight hits).  Just
+// below each line no kind of batch was slower than with all that fit.
+inline int ctas_per_sm(unsigned long long n_words, int sms, int block, int most, int set)
+{
+    if (set > 0 && set < most)
+        return set;
+    if (n_words > 3072ull * sms)
+        return most;
+    const int few = (n_words <= 640ull * sms ? 256 : 512) / block;
+    return few < 1 ? 1 : few < most ? few : most;
+}
+
 // the persistent kernel at `block` threads per CTA (128, 256 or 512)
 inline cudaError_t launch_persistent(int block, const Dev &d, cudaStream_t s, int blocks_per_sm, int max_ctas,
                                      int *n_launches)

@@ -31,7 +31,6 @@
 // The block size of every kernel is SVT_BLOCK (256 unless the including
 // file sets it); each block size builds in a namespace of its own, and only
 // the 256-thread build holds the plain pipeline.
-#include <algorithm>
 #include <cstddef>
 
 #include "svt_internal.h"
@@ -4103,23 +4102,10 @@ cudaError_t launch_persistent(const Dev &d, cudaStream_t s, int blocks_per_sm, i
     int maxb = persistent_max_blocks_per_sm(dev);
     if (maxb <= 0)
         return cudaErrorInvalidConfiguration;
-    // Every CTA costs each barrier an arrival and each stage its first loads and
-    // instructions, so the grid grows with the batch: 256 threads an SM up to 640
-    // words an SM (97k words on 152 SMs), 512 up to 3072 (467k), then all that
-    // fit.  Device time with one, two and three CTAs of 256 an SM, us: one event
-    // of 977 words 27.5 / 28.9 / 30.5, 8k words 24.7 / 26.8 / 30.4, 99k words
-    // 37.1 / 38.4 / 41.7, 155k words 61 / 57 / 61 (shared hits), 495k words
-    // 57.4 / 51.2 / 53.3, 978k words 158 / 119 / 110 (one to eight hits).  Just
-    // below each line no kind of batch was slower than with all that fit.
-    int bps = maxb;
-    if (blocks_per_sm > 0)
-        bps = blocks_per_sm < maxb ? blocks_per_sm : maxb;
-    else if (d.n_words <= 3072ull * sms)
-        bps = std::min(maxb, std::max((d.n_words <= 640ull * sms ? 256 : 512) / BLOCK, 1));
     Dev dd = d;
     void *args[] = {&dd};
     cudaLaunchConfig_t cfg = {};
-    int grid = sms * bps;
+    int grid = sms * ctas_per_sm(d.n_words, sms, BLOCK, maxb, blocks_per_sm);
     if (max_ctas > 0 && max_ctas < grid)
         grid = max_ctas;
     if (grid > GRID_MAX)   // the word spans (one per warp) and the per-CTA totals are sized for this

@@ -158,7 +158,7 @@ struct Dev {
     svt_road *road_out;                                           // [max_roads] (svt_get_roads)
     long long cut;
     int small_n4;
-    int run_roads;         // claim of a warp of the group path: max(run_roads / 8, 1) warp steps
+    int run_roads;         // how the group path's warp steps are shared out: svt_launch::run_roads
     int skip_arrival;
     unsigned long long wait_ns;
 };

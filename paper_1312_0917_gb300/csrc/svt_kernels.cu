@@ -356,16 +356,16 @@ __device__ __forceinline__ unsigned grab_after_first(const Dev &d, int q)
     return gridDim.x + grab(d, q);
 }
 
-// A warp's items out of n for n_warps warps: three quarters are dealt out in
+// A warp's items out of n for n_warps warps: `quarters` of four are dealt out in
 // turn (warp wi: wi, wi + n_warps, ..), the rest, which evens the warps out,
 // `claim` at a time from queue head q.  (All from the queue, 40,000 claims of
 // one counter were 80 us: L2 takes about one atomic on an address in 2 ns.)
 struct Share {
     unsigned n, n_warps, claim, dealt, left;   // items dealt out; of the last claim, still to do
     unsigned *q;
-    __device__ Share(unsigned n_, unsigned n_warps_, unsigned claim_, unsigned *q_)
+    __device__ Share(unsigned n_, unsigned n_warps_, unsigned quarters, unsigned claim_, unsigned *q_)
         : n(n_), n_warps(n_warps_), claim(claim_),
-          dealt(n_ <= n_warps_ ? n_ : max(n_ / 4 * 3 / n_warps_, 1u) * n_warps_), left(0), q(q_)
+          dealt(n_ <= n_warps_ ? n_ : max(n_ / 4 * quarters / n_warps_, 1u) * n_warps_), left(0), q(q_)
     {
     }
     __device__ unsigned first(unsigned wi) const { return wi < dealt ? wi : ~0u; }   // (dealt is 0 or covers a turn)
@@ -3359,7 +3359,7 @@ __device__ __noinline__ void p3_boxes(const Dev &d, unsigned char *smem, unsigne
                                       unsigned long long &npass)
 {
     const unsigned n_warps = gridDim.x * WARPS, wi = warp_id() * gridDim.x + blockIdx.x;
-    Share w(n_box, n_warps, 1, &d.ctrl->q[qbox]);
+    Share w(n_box, n_warps, 3, 1, &d.ctrl->q[qbox]);
     unsigned i = w.first(wi), g = i < n_box ? ldcg(d.box_list + i) : 0u;
     while (i < n_box) {   // the next road is claimed and looked up ahead
         const unsigned ni = w.next(i), ng = ni < n_box ? ldcg(d.box_list + ni) : 0u;
@@ -3419,7 +3419,8 @@ __device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbo
     const unsigned n_warps = gridDim.x * WARPS, wi = warp_id() * gridDim.x + blockIdx.x;
     const unsigned steps = S.end[2 * N_GROUP_CLS - 1];
     unsigned np = 0;
-    Share w(steps, n_warps, max((unsigned)d.run_roads / 8, 1u), &d.ctrl->q[qgroup]);
+    // (svt_launch::run_roads)
+    Share w(steps, n_warps, d.run_roads < 8 ? 2u : 3u, d.run_roads > 8 ? 2u : 1u, &d.ctrl->q[qgroup]);
     for (unsigned s = w.first(wi); s < steps; s = w.next(s)) {
         if (s < S.end[0])
             group_step<PLAIN, GroupCls4e, 0>(d, smem, s, np);

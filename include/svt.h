@@ -200,9 +200,9 @@ typedef struct {
     int32_t small_n4;        /* roads with more than this many distinct fits (combinations of the
                               * four fitted layers) take a warp of their own (the box path); the
                               * others are fitted several to a warp (1 .. 256, 0 = 256) */
-    int32_t run_roads;       /* how the warp steps of those others are shared out: three quarters dealt
-                              * out and the rest claimed one by one (8), two by two (16), or half of
-                              * them dealt out and half claimed one by one (4) (0 = 8) */
+    int32_t run_roads;       /* how the warp steps of those others are shared out: a quarter (4), half
+                              * (8) or three quarters (16) of them dealt out, the rest claimed one by
+                              * one (0 = 8) */
     int32_t max_ctas;        /* cap on the grid (0 = SMs x blocks_per_sm); the autotuner keeps it */
 } svt_launch;
 

@@ -357,15 +357,19 @@ __device__ __forceinline__ unsigned grab_after_first(const Dev &d, int q)
 }
 
 // A warp's items out of n for n_warps warps: `quarters` of four are dealt out in
-// turn (warp wi: wi, wi + n_warps, ..), the rest, which evens the warps out,
-// `claim` at a time from queue head q.  (All from the queue, 40,000 claims of
-// one counter were 80 us: L2 takes about one atomic on an address in 2 ns.)
+// turn (warp wi: wi, wi + n_warps, ..), the rest, which evens the warps out, one
+// by one from queue head q.  (All from the queue, 40,000 claims of one counter were
+// 80 us: L2 takes about one atomic on an address in 2 ns.)  A half: items take
+// unequal times where some roads are fitted twice.  The fit stage with a half / three
+// quarters dealt out: 96,000 roads of skewed hit counts 38 / 40 us with hits
+// anywhere, 55 / 74 within 64 strips, 63 / 86 within 16; 19,200 roads of one to
+// eight hits within 16 strips 67 / 72; the uneven batch 85 / 84.
 struct Share {
-    unsigned n, n_warps, claim, dealt, left;   // items dealt out; of the last claim, still to do
+    unsigned n, n_warps, dealt;   // items dealt out
     unsigned *q;
-    __device__ Share(unsigned n_, unsigned n_warps_, unsigned quarters, unsigned claim_, unsigned *q_)
-        : n(n_), n_warps(n_warps_), claim(claim_),
-          dealt(n_ <= n_warps_ ? n_ : max(n_ / 4 * quarters / n_warps_, 1u) * n_warps_), left(0), q(q_)
+    __device__ Share(unsigned n_, unsigned n_warps_, unsigned quarters, unsigned *q_)
+        : n(n_), n_warps(n_warps_),
+          dealt(n_ <= n_warps_ ? n_ : max(n_ / 4 * quarters / n_warps_, 1u) * n_warps_), q(q_)
     {
     }
     __device__ unsigned first(unsigned wi) const { return wi < dealt ? wi : ~0u; }   // (dealt is 0 or covers a turn)
@@ -376,14 +380,9 @@ struct Share {
             return i + n_warps;
         if (dealt >= n)
             return ~0u;
-        if (i >= dealt && left) {
-            --left;
-            return i + 1;
-        }
         unsigned c = 0;
         if (lane_id() == 0)
-            c = atomicAdd(q, claim);
-        left = claim - 1;
+            c = atomicAdd(q, 1u);
         return dealt + __shfl_sync(FULL_MASK, c, 0);
     }
 };
@@ -3359,7 +3358,7 @@ __device__ __noinline__ void p3_boxes(const Dev &d, unsigned char *smem, unsigne
                                       unsigned long long &npass)
 {
     const unsigned n_warps = gridDim.x * WARPS, wi = warp_id() * gridDim.x + blockIdx.x;
-    Share w(n_box, n_warps, 3, 1, &d.ctrl->q[qbox]);
+    Share w(n_box, n_warps, 2, &d.ctrl->q[qbox]);
     unsigned i = w.first(wi), g = i < n_box ? ldcg(d.box_list + i) : 0u;
     while (i < n_box) {   // the next road is claimed and looked up ahead
         const unsigned ni = w.next(i), ng = ni < n_box ? ldcg(d.box_list + ni) : 0u;
@@ -3420,7 +3419,7 @@ __device__ __noinline__ void p3_phase(const Dev &d, unsigned char *smem, int qbo
     const unsigned steps = S.end[2 * N_GROUP_CLS - 1];
     unsigned np = 0;
     // (svt_launch::run_roads)
-    Share w(steps, n_warps, d.run_roads < 8 ? 2u : 3u, d.run_roads > 8 ? 2u : 1u, &d.ctrl->q[qgroup]);
+    Share w(steps, n_warps, d.run_roads < 8 ? 1u : d.run_roads > 8 ? 3u : 2u, &d.ctrl->q[qgroup]);
     for (unsigned s = w.first(wi); s < steps; s = w.next(s)) {
         if (s < S.end[0])
             group_step<PLAIN, GroupCls4e, 0>(d, smem, s, np);

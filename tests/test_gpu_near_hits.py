@@ -5,7 +5,7 @@ after the quick pass costs: one more pass of its own kind, not one road at a tim
 import numpy as np
 import pytest
 
-from paper_1312_0917_gb300 import binding as B
+from paper_1312_0917_gb300 import binding as B, synth
 from gpu_util import torch_words
 from test_gpu_stages import FLOAT_CUT, batch, check, p90
 
@@ -135,6 +135,14 @@ def test_ties_cost_one_more_pass(ctx, consts, cuts):
     ctx.load_constants(consts, cuts["scaled"])
     words = batch("apart", 1000, 64, 1, 4)
     assert fit_us(ctx, near(words, 16)) < 3 * fit_us(ctx, words)
+
+
+def test_tied_steps_are_evened_out(ctx, consts, cuts):
+    """Roads of skewed hit counts, four steps a warp, some of them taken twice: the
+    fit stays below twice its time with hits anywhere."""
+    ctx.load_constants(consts, cuts["uneven"])
+    words = synth.make_batch(synth.Config("skew", 3000, ("geom", 32, 1, 256), ("skewed", 8)), seed=1).words
+    assert fit_us(ctx, near(words, 16)) < 2 * fit_us(ctx, words)
 
 
 def test_repeats_cost_one_more_pass(ctx, consts, cuts):

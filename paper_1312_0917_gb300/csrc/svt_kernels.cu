@@ -2283,9 +2283,9 @@ __device__ __forceinline__ unsigned box_tab(const BoxShape &sh, unsigned p, unsi
 //
 // Bound: issue slots, nine instructions per fit (14 in the floor pass, 20 in
 // the key pass, whose 64-bit minima have a seventh of the float rate).  The fit
-// stage of 12,800 roads of 8^4 fits: 50 us with hits anywhere, 68 within 16 strips,
-// 78 within 8, 98 with all chi-squares equal; in whole numbers with tables in
-// shared memory alone 84, 85, 90 and 85.
+// stage of 12,800 roads of 8^4 fits: 50 us with hits anywhere, 69 within 16 strips,
+// 80 within 8, 105 with all chi-squares equal; in whole numbers with tables in
+// shared memory alone 84, 85, 89 and 85.
 // ---------------------------------------------------------------------------
 
 constexpr long long FLOAT_CUT = 1ll << 24;   // a smaller cut's band [lo, hi] is a visible share of the fits: floor pass
@@ -2414,13 +2414,16 @@ __device__ __forceinline__ FloatPass float_pass(const P3Float &F, unsigned mc, u
 // The same with the components' floors, which floats hold exactly: a chi-square
 // is then off by a relative 1.8e-7 at most, X1 <= X2 => c1 <= c2 FLOOR_EPS, and
 // rows are near only where chi-squares are all but equal.  The floor a of a sum
-// (|a| < 2^19) becomes a float by adding it to the bits of 1.5 2^23.
+// (|a| < 2^19) becomes a float by adding it to the bits of 1.5 2^23.  One loop over
+// the pairs of hits of slot e, and one body of the key pass: roads of many shapes
+// meet here (with a body for each, 19,200 roads of one to eight hits within 16
+// strips took 87 us of the fit stage, 72 with these; 8^4 roads 70 and 69).
 constexpr float FLOOR_EPS = 1.0000005f, FLOOR_BIAS = -12582912.f;
 
-template <bool TWO, bool WIDE>
+template <bool TWO>
 __device__ __forceinline__ FloatPass floor_pass(const P3Box &B, const BoxShape &sh, unsigned lo, float hi)
 {
-    constexpr unsigned NJ = TWO ? 2 : 1, NI = WIDE ? 4 : 2;
+    constexpr unsigned NJ = TWO ? 2 : 1;
     const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
     FloatPass f{0u, ~0u, {3e38f, 3e38f}, {3e38f, 3e38f}, false};
     const f2 bias = f2_pack(FLOOR_BIAS, FLOOR_BIAS);
@@ -2439,9 +2442,9 @@ __device__ __forceinline__ FloatPass floor_pass(const P3Box &B, const BoxShape &
         float rz[NJ];
 #pragma unroll
         for (unsigned j = 0; j < NJ; ++j)
-            pz[j] = add4(pab[j], B.A[2][z]);
-#pragma unroll
-        for (unsigned i = 0; i < NI; ++i) {
+            pz[j] = add4(pab[j], B.A[2][z]), rz[j] = 3e38f;
+#pragma unroll 1
+        for (unsigned i = 0; 2 * i < sh.me; ++i) {
             const int4 a0 = B.A[3][2 * i], a1 = B.A[3][2 * i + 1];
             const f2 bx = reinterpret_cast<const f2 *>(B.F.bias)[i];   // (a missing hit's: far above every cut)
             const auto part = [](int s, int t, f2 b) {
@@ -2456,7 +2459,7 @@ __device__ __forceinline__ FloatPass floor_pass(const P3Box &B, const BoxShape &
                 np[j] += d0 >> 31;
                 np[j] += d1 >> 31;
                 f.near_cut = min(f.near_cut, min(d0, d1));
-                rz[j] = i ? fminf(rz[j], fminf(c.x, c.y)) : fminf(c.x, c.y);
+                rz[j] = fminf(rz[j], fminf(c.x, c.y));
             }
         }
         float ac = 3e38f;   // (a, c) at x, z
@@ -2498,21 +2501,18 @@ struct KeyPass {
     bool ok[2];
 };
 
-template <bool TWO>
 __device__ __forceinline__ KeyPass key_pass(const P3Box &B, const BoxShape &sh, long long cut)
 {
-    constexpr unsigned NJ = TWO ? 2 : 1;
+    constexpr unsigned NJ = 2;
     const unsigned x = lane_id() & 7u, yl = lane_id() >> 3;
     // within a row (x, y, z) the order by (chi2, w) is that by key
     const unsigned long long rb = (unsigned long long)(min(cut, 1ll << 38) + 1) << 3;   // chi2 <= cut iff below
     KeyPass f{0u, {NO_KEY, NO_KEY}, {false, false}};
     int4 pab[NJ];
-    unsigned np[NJ];
+    unsigned np[NJ] = {0u, 0u};
 #pragma unroll
-    for (unsigned j = 0; j < NJ; ++j) {
+    for (unsigned j = 0; j < NJ; ++j)
         pab[j] = add4(B.A[0][x], B.A[1][yl + 4 * j]);
-        np[j] = 0;
-    }
 #pragma unroll 1
     for (unsigned z = 0; z < sh.mc; ++z) {
         int4 pz[NJ];
@@ -2522,7 +2522,8 @@ __device__ __forceinline__ KeyPass key_pass(const P3Box &B, const BoxShape &sh, 
             pz[j] = add4(pab[j], B.A[2][z]);
             rz[j] = NO_KEY;
         }
-        const auto fit = [&](unsigned w) {
+#pragma unroll 1
+        for (unsigned w = 0; w < sh.me; ++w) {
             const int4 aw = B.A[3][w];
 #pragma unroll
             for (unsigned j = 0; j < NJ; ++j) {
@@ -2531,17 +2532,7 @@ __device__ __forceinline__ KeyPass key_pass(const P3Box &B, const BoxShape &sh, 
                 np[j] += key < rb;
                 rz[j] = umin64(rz[j], key);
             }
-        };
-        unsigned w = 0;
-#pragma unroll 1
-        for (; w + 4 <= sh.me; w += 4) {
-#pragma unroll
-            for (unsigned i = 0; i < 4; ++i)
-                fit(w + i);
         }
-#pragma unroll 1
-        for (; w < sh.me; ++w)
-            fit(w);
         unsigned long long ac = NO_KEY;   // (a, c) at x, z
 #pragma unroll
         for (unsigned j = 0; j < NJ; ++j) {
@@ -2670,20 +2661,13 @@ __device__ __noinline__ void box_warp(const Dev &d, unsigned char *region, unsig
         const float floor_lo = cut * (2.f - FLOOR_EPS), floor_hi = cut * FLOOR_EPS;
         const unsigned lo = __float_as_uint(floor_lo);
         width = __float_as_uint(floor_hi) + 1 - lo;
-        if (sh.mb > 4 && sh.me > 4)
-            f = floor_pass<true, true>(B, sh, lo, floor_hi);
-        else if (sh.mb > 4)
-            f = floor_pass<true, false>(B, sh, lo, floor_hi);
-        else if (sh.me > 4)
-            f = floor_pass<false, true>(B, sh, lo, floor_hi);
-        else
-            f = floor_pass<false, false>(B, sh, lo, floor_hi);
+        f = sh.mb > 4 ? floor_pass<true>(B, sh, lo, floor_hi) : floor_pass<false>(B, sh, lo, floor_hi);
         by += candidates(FLOOR_EPS, 0.f, floor_hi);
     }
     const unsigned x = lane & 7u, yl = lane >> 3;
     unsigned np = f.np;
     if (by == 2) {
-        const KeyPass k = sh.mb > 4 ? key_pass<true>(B, sh, d.cut) : key_pass<false>(B, sh, d.cut);
+        const KeyPass k = key_pass(B, sh, d.cut);
         np = k.np;
 #pragma unroll
         for (unsigned j = 0; j < 2; ++j)

@@ -110,9 +110,9 @@ typedef struct {
     uint64_t error_word;      /* word position of the first fault (if any) */
     uint64_t phase_ns[6];     /* SVT_PERSISTENT: device time of each stage, from the
                                  first CTA's view of the grid barriers: word scan,
-                                 event scatter, unpack, fit + cut + road-local
-                                 warrior, cross-road warrior, output (to the last
-                                 CTA's exit); 0 when a stage did not complete, and
+                                 road decode, cross-road flags, fit + cut +
+                                 road-local warrior, cross-road warrior, output (to
+                                 the last CTA's exit); 0 when a stage did not complete, and
                                  for SVT_PLAIN */
 } svt_stats;
 
@@ -252,12 +252,12 @@ int svt_last_launch_count(svt_ctx *ctx);
 
 const char *svt_strerror(int code);
 
-/* Integer throughput of `device`, the denominator of the fit's roofline (not
- * a step of the chain): every thread of a grid that fills the device runs
+/* Integer throughput of `device` (not a step of the chain): every thread of a grid that fills the device runs
  * eight independent chains of one operation, timed with CUDA events (best of
  * five launches after a warm-up).  *imad_per_s: 32-bit multiply-adds
  * (mad.lo.u32) per second; *iadd_per_s: 32-bit adds; *mixed_per_s:
- * multiply-adds and xors alternating (two pipes at once).  HOST pointers.
+ * multiply-adds and xors alternating (two pipes at once: the issue rate, one
+ * operation per lane and instruction).  HOST pointers.
  * Allocates one word of device memory for the duration of the call;
  * synchronises the device. */
 int svt_measure_int_peak(int device, double *imad_per_s, double *iadd_per_s, double *mixed_per_s);

@@ -2565,7 +2565,7 @@ __device__ __forceinline__ KeyPass key_pass(const P3Box &B, const BoxShape &sh, 
 // Fit road g with one warp.  The shape's slots are roles here, by falling hit
 // count.  Hits that repeat a coordinate need nothing special (as in the group
 // path).  Bound: issue slots (two fits an instruction).  The fit stage of 25,600
-// roads of 8^4 distinct fits: 153.8 -> 82.4 us (whole keys with tables in shared
+// roads of 8^4 distinct fits: 153.8 -> 80.5 us (whole keys with tables in shared
 // memory before).
 __device__ __noinline__ void box_warp(const Dev &d, unsigned char *region, unsigned g, unsigned long long &npass)
 {
@@ -3090,7 +3090,9 @@ using GroupCls4e = GroupRoad<3, 1, 2, 4>;
 // register allocation per class (in one function the five classes spilled 220
 // bytes).  Bound: issue slots and the chain from the list to the hits.  The fit
 // stage of 192,000 roads of one to four hits a layer, nearly all of them here:
-// 124.4 -> 67.6 us (a lane per table entry, tables in shared memory, before).
+// 124.4 -> 61.7 us (a lane per table entry, tables in shared memory, before).  At
+// 80 registers the shapes with four hits of slot e spill 30 bytes (64 in whole
+// keys), p3_phase and p3_boxes some 70 outside their items.
 template <bool PLAIN, class Road, bool EXACT>
 __device__ __noinline__ unsigned group_item(const Dev &d, unsigned char *smem, const RoadItem *list, int step,
                                             unsigned left, unsigned tied, unsigned &npass)

@@ -18,12 +18,14 @@ roads x 8 hits on each of 5 layers (838,860,800 combinations).
          svt_get_tracks (the status block and the tracks to the host), host wall
          clock; two contexts take batches in turn (one batch's copies overlap
          the other's kernel).  p50 / p99 are one batch at a time.
-  roofline  multiply-adds: 36 per distinct fit (the fit of one input
-         vector x, Sec. II: 18 for p = F x + q, 18 for the chi-square rows;
-         combinations that differ only in the excluded layer's hit share x),
-         against the device's multiply-add rate (SMs x 128 lanes x clock: the
-         fit's main pass runs them as pairs in single precision, exact where
-         it decides; integer ones have 64 lanes, measured beside it).
+  roofline  warp instructions of one launch, as ncu counted them at the default
+         launch settings, per second, against the device's issue rate (SMs x 4
+         schedulers x clock; beside it the rate measured with two alternating
+         pipes).  The kernel forms each hit's share of the chi-square sums once a
+         road, so multiply-adds per fit are no measure of its work; `notional`
+         keeps the figure of 36 a distinct fit (Sec. II: 18 for p = F x + q, 18
+         for the chi-square rows; combinations that differ only in the excluded
+         layer's hit share x) without a peak.
   scaled / uneven  the 3000 x 64 and 10,000-event uneven batches: the
          persistent form against the plain per-stage launch (fits/s, p50,
          p99 per batch, device and end to end).
@@ -59,7 +61,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-FMA_LANES_PER_SM = 128      # single-precision multiply-adds per SM and clock (integer ones: 64)
+SCHEDULERS_PER_SM = 4       # warp instructions per SM and clock at most
 MACS_PER_FIT = 36   # 6 inputs x (3 track parameters + 3 chi-square components)
 HEADLINE = "stress"
 
@@ -338,18 +340,23 @@ def run_serving(B, synth, consts, cut, rates, n_requests, n_slots=8, seed=0, **s
         srv.close()
 
 
-# DRAM bytes (read + write) of one persistent-kernel launch per workload, from
-# the ncu captures summarised under profiles/, with the SHA-256 of the kernel sources
+# DRAM bytes (read + write) and warp instructions of one persistent-kernel launch
+# per workload (default launch settings), from the ncu captures summarised under
+# profiles/, with the SHA-256 of the kernel sources
 # (kernels and their header) they were taken on: the bench line reports a
 # figure only while the sources are unchanged.
 NCU_TRAFFIC = {
-    "stress": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 5836544},    # 5.744 MB read + 92.4 KB written
-    "scaled": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 16996864},   # 13.885 MB read + 3.112 MB written
-    "uneven": {"kernels_sha256": "2090ee01519772749a6a8100b16f6bb6f167eb73c95c1d799e5fac3e919d03e2", "bytes": 36923648},   # 19.202 MB read + 17.722 MB written
+    # 5.319 MB read + 71.9 KB written; 13.930 + 2.257 MB; 18.832 + 16.232 MB
+    "stress": {"kernels_sha256": "30666f4ce5987c8877318a46a40814001b2ebc8582622a2be717d56fc5fed3b7", "bytes": 5390848,
+               "warp_instructions": 75032476},
+    "scaled": {"kernels_sha256": "30666f4ce5987c8877318a46a40814001b2ebc8582622a2be717d56fc5fed3b7", "bytes": 16187648,
+               "warp_instructions": 70444832},
+    "uneven": {"kernels_sha256": "30666f4ce5987c8877318a46a40814001b2ebc8582622a2be717d56fc5fed3b7", "bytes": 35064320,
+               "warp_instructions": 113087533},
 }
 
 
-def measured_traffic(workload: str):
+def measured(workload: str, what: str):
     import hashlib
     h = hashlib.sha256()
     for name in ("svt_kernels.cu", "svt_internal.h"):
@@ -357,8 +364,24 @@ def measured_traffic(workload: str):
             h.update(f.read())
     rec = NCU_TRAFFIC.get(workload)
     if rec and rec["kernels_sha256"] == h.hexdigest():
-        return rec["bytes"]
+        return rec.get(what)
     return None
+
+
+def measured_traffic(workload: str):
+    return measured(workload, "bytes")
+
+
+def issue_roofline(workload: str, ms: float, sms: int, mhz: float, mixed_per_s: float) -> dict:
+    """Warp instructions issued per second against the schedulers' rate.
+    mixed_per_s: the measured operations per second of two alternating pipes,
+    one per lane and instruction."""
+    n = measured(workload, "warp_instructions")
+    peak = sms * SCHEDULERS_PER_SM * mhz * 1e6 / 1e12
+    achieved = n / (ms / 1e3) / 1e12 if n else None
+    return {"bound": "issue", "achieved": achieved, "peak": peak, "unit": "T warp instructions/s",
+            "frac": achieved / peak if n else None, "peak_measured": mixed_per_s / 32 / 1e12,
+            "warp_instructions": n, "traffic": measured_traffic(workload)}
 
 
 # The plain pipeline stores every combination's key (8 bytes) and track
@@ -740,13 +763,11 @@ def gpu_arm(args):
     clk = clocks.summary(t_timed0 - 0.02, t_timed1 + 0.02)
     clk["gpu_section"] = clocks.summary()
     mhz = clk["sm_max_mhz"] or 2070.0
-    peak_macs = sms * FMA_LANES_PER_SM * mhz * 1e6 / 1e12
-    achieved = MACS_PER_FIT * n_fit4 / (step_ms / 1e3) / 1e12
     line = {
         "metric": "track fits/s", "value": value, "unit": "fits/s", "n_gpus": world,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": step_ms,
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "int32/int64", "data": "synthetic (seeded generator, workload shape of the config)",
+        "dtype": "int32/int64 (decisions; fp32 with an error bound where it suffices)", "data": "synthetic (seeded generator, workload shape of the config)",
         "config": {"workload": workload_desc(cfg, n_fits, n_words), "mode": "persistent",
                    "graph": True, "autotuned": tuned, "l2": "256 MB flush written between steps",
                    "parallelism": "replicas" if world > 1 else "single GPU"},
@@ -758,15 +779,9 @@ def gpu_arm(args):
                               "cross_road_warrior", "output"],
                              [round(x / 1e3, 1) for x in stats["phase_ns"]])),
         "e2e": e2e,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_macs, "unit": "T MAC/s",
-                     "frac": achieved / peak_macs, "traffic": measured_traffic(args.workload),
-                     "peak_measured": peak["mixed"] / 1e12,
-                     "units": "%d distinct fits x %d multiply-adds per launch" % (n_fit4, MACS_PER_FIT),
-                     "note": "peak = SMs x 128 single-precision multiply-add lanes x max clock; "
-                             "peak_measured: svt_measure_int_peak, multiply-add and xor "
-                             "alternating on every SM; "
-                             "per combination the same time is %.2f T MAC/s"
-                             % (MACS_PER_FIT * n_fits / (step_ms / 1e3) / 1e12)},
+        "roofline": dict(issue_roofline(args.workload, step_ms, sms, mhz, peak["mixed"]),
+                         notional={"macs_per_distinct_fit": MACS_PER_FIT, "distinct_fits": n_fit4,
+                                   "t_macs_per_s": MACS_PER_FIT * n_fit4 / (step_ms / 1e3) / 1e12}),
         "int_peak_tops": {k: round(v / 1e12, 2) for k, v in peak.items()},
         "gpu_launches": launches * args.steps,
         "clocks": clk,

@@ -1,6 +1,7 @@
-// svt_peak.cu -- svt_measure_int_peak: the integer throughput of the device,
-// the denominator of the fit's roofline (the fit is integer multiply-add work,
-// Sec. II: p_i = f_i . x_i + q_i).  Not a step of the chain.
+// svt_peak.cu -- svt_measure_int_peak: the integer throughput of the device:
+// multiply-adds, adds, and the two pipes in turn, which is one instruction per
+// scheduler and clock (the measured issue rate beside the chain's roofline).
+// Not a step of the chain.
 //
 // Every thread of a grid that fills the device runs CHAINS independent
 // dependency chains of one integer operation (in-line PTX, so that the
